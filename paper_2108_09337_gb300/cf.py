@@ -71,9 +71,11 @@ _SIG = {
     "cf_tourn_select": (_I, [_I, _I, _P, _I, _I, _I, _P, _P, _S, _P]),
     "cf_tourn_select_f32": (_I, [_I, _I, _P, _I, _I, _I, _P, _P, _S, _P]),
     "cf_getrf_workspace_size": (_S, [_I, _OPT]),
+    "cf_getrf_optimal_workspace_size": (_S, [_I, _OPT]),
     "cf_getrf": (_I, [_I, _P, _I, _P, _P, _P, _S, _OPT, _P]),
     "cf_getrf_noalloc": (_I, [_I, _P, _I, _P, _P, _OPT, _P]),
     "cf_potrf_workspace_size": (_S, [_I, _OPT]),
+    "cf_potrf_optimal_workspace_size": (_S, [_I, _OPT]),
     "cf_potrf": (_I, [_I, _P, _I, _P, _P, _S, _OPT, _P]),
     "cf_getrs_workspace_size": (_S, [_I, _I]),
     "cf_getrs": (_I, [_I, _I, _P, _I, _P, _P, _I, _P, _S, _P]),
@@ -218,7 +220,10 @@ def tourn_select(panel: torch.Tensor, leaf_h: int = 128, arity: int = 2) -> torc
 def getrf(A: torch.Tensor, v=None, leaf_h=None, arity=None, work=None, lookahead=None):
     """In-place LU with tournament pivoting.  Returns (ipiv, info) device
     int32 tensors (ipiv 1-based).  lookahead: 1 (default) overlaps step
-    t+1's TournPivot with step t's trailing update, 0 keeps one stream."""
+    t+1's TournPivot with step t's trailing update, 0 keeps one stream.
+    work: at least cf_getrf_workspace_size bytes; from
+    cf_getrf_optimal_workspace_size on (the default buffer's size) the Schur
+    updates run on the tensor cores, below it on the FP64 pipe."""
     assert A.dtype == torch.float64
     n = A.shape[0]
     assert A.shape == (n, n)
@@ -226,7 +231,7 @@ def getrf(A: torch.Tensor, v=None, leaf_h=None, arity=None, work=None, lookahead
     opt = options(v=v, leaf_h=leaf_h, arity=arity, lookahead=lookahead)
     ipiv = torch.empty(max(n, 1), dtype=torch.int32, device=A.device)
     info = torch.zeros(1, dtype=torch.int32, device=A.device)
-    need = _lib.cf_getrf_workspace_size(n, ctypes.byref(opt))
+    need = _lib.cf_getrf_optimal_workspace_size(n, ctypes.byref(opt))
     ws = work if work is not None else _workspace(need, A.device)
     _check("cf_getrf", _lib.cf_getrf(n, _ptr(A), lda, _ptr(ipiv), _ptr(info), _ptr(ws), ws.numel(),
                                      ctypes.byref(opt), _stream()))
@@ -262,7 +267,7 @@ def potrf(A: torch.Tensor, v=None, lookahead=None):
     lda = _ld(A, "A")
     opt = options(v=v, lookahead=lookahead)
     info = torch.zeros(1, dtype=torch.int32, device=A.device)
-    ws = _workspace(_lib.cf_potrf_workspace_size(n, ctypes.byref(opt)), A.device)
+    ws = _workspace(_lib.cf_potrf_optimal_workspace_size(n, ctypes.byref(opt)), A.device)
     _check("cf_potrf", _lib.cf_potrf(n, _ptr(A), lda, _ptr(info), _ptr(ws), ws.numel(),
                                      ctypes.byref(opt), _stream()))
     return info

@@ -1,0 +1,677 @@
+// cf_slice64.cu -- LU-5 / CH-3 of the FP64 path on the tensor cores:
+//     C -= A10 A01   (LU; A10 m x w, A01 w x n)     C -= L10 L10^T   (Cholesky, lower)
+//
+// GB300 runs FP64 at ~2 fused multiply-adds per clock per SM (1.20 TFLOP/s
+// measured), so the update as FP64 code is bound by that pipe; the BF16 tensor
+// cores run 1500 times faster and form the same product exactly from small
+// integers:
+//   * inner scale: rho_j is the largest exponent in row j of A01.  A10's
+//     column j is scaled up and A01's row j down by 2^rho_j (exact; the
+//     product does not change), so that a row scaling of the matrix, which
+//     partial pivoting turns into opposite gradings of A10's columns and
+//     A01's rows, costs no accuracy.  Cholesky needs none (L10 is both sides);
+//   * per row of A10 (column of A01) the elements become integers of at most
+//     62 bits relative to the row's (column's) largest exponent and eight
+//     balanced base-256 digits (the top one in [-64, 64], the others in
+//     [-128, 127]), exact in BF16;
+//   * Q_d = sum_{s+t=d} sum_j d_s e_t, d = 0..7: for every A10 digit s one
+//     chain of tcgen05 MMAs against the A01 digits t = 0..7-s, accumulating
+//     into the TMEM columns of diagonal s + t.  A sum holds at most 128
+//     products of each of at most 8 digit pairs, two of them with a top digit:
+//     at most 7 x 2^21 < 2^24, so the FP32 accumulation is exact in any order;
+//   * C -= 2^(E_i + F_k - 2112) sum_d Q_d 256^(7-d): the 76-bit integer sum is
+//     rounded to FP64 once and subtracted with a second rounding.
+// The error is a few 2^-62 of (max of the row) x (max of the column) per term
+// and one rounding of the sum, where the FP64 loop rounds w partial sums.
+// Every C element's value is a function of its row, its column and the inner
+// exponents alone, so it does not depend on how the update is cut into pieces.
+//
+// Rows (columns) with an infinity, a NaN or scales whose product could leave
+// the normal range flag their tile, and flagged tiles are done by the FP64 loop
+// (k_gemm_flagged), with that loop's results.
+//
+// Kernel layout: persistent CTAs over 128 x 64 tiles of C, column-tile major,
+// so that a CTA's A01 digits (128 KB) stay in shared memory while the A10
+// digits (16 KB tiles, six in flight) stream through from L2; 8 diagonals x 64
+// columns fill the 512 TMEM columns.  Per tile: 36 digit pairs = 9,200 tensor
+// clocks; sixteen epilogue warps combine the diagonals in integers as they
+// leave TMEM (the accumulators are free again after the read), then do the
+// one FP64 operation per element while the next tile's MMAs run.
+#include <climits>
+
+#include <cuda_bf16.h>
+
+#include "cf_common.cuh"
+#include "cf_kernels.cuh"
+#include "cf_slice64.cuh"
+#include "cf_tc.cuh"
+#include "cf_umma.cuh"
+
+namespace cf {
+
+__device__ int g_slice64_status = 0;       // 0 or CF_ERR_TIMEOUT
+
+namespace s64 {
+
+using namespace umma;
+
+constexpr int ND = 8;                  // digits per element
+constexpr int BM = 128, BN = 64, BK = 64;
+constexpr int UMMA_K = 16;
+constexpr int AST = 6;                 // A10 digit tiles in flight
+constexpr int EPI = 16;                // epilogue warps: 4 lane quarters x 4 groups of 16 columns
+constexpr int kThreads = 64 + 32 * EPI;
+constexpr uint32_t kABytes = BM * BK * 2;          // one digit of 128 rows x 64 k
+constexpr uint32_t kBHalf = BN * BK * 2;           // one digit of 64 rows x 64 k
+constexpr uint32_t kBBytes = 2 * ND * kBHalf;      // all digits of 64 columns x 128 k
+constexpr uint32_t kTmemCols = 512;
+constexpr int kCentre = 2046;          // E of a row whose largest scaled element is in [1, 2)
+constexpr int kSpan = 450;             // E and F may be this far from their centres (below), E this far ...
+constexpr int kSpanUp = 900;           // ... above its centre when F <= 0: E + F - 994 - 95 >= 1, E + F - 994 <= 2046
+
+struct Smem {
+    uint64_t afull[AST], aempty[AST];
+    uint64_t bfull, bempty, acc_full, acc_empty, drain;
+    uint32_t tmem_base;
+    int abort_flag;
+};
+
+struct Problem {
+    int m, c0, c1;                     // rows, columns [c0, c1) of the sliced operands
+    int nkb;                           // K blocks of 64 (1 or 2)
+    int lower, same;                   // Cholesky: triangle only; one set of slices for both operands
+    int ct0, ct1, nrt;                 // column tiles of 64, row tiles of 128
+    long long units;
+    const uint8_t *SA, *SB;
+    const int *E, *F;
+    const int *any, *flagA, *flagB;
+    const int *skip;
+    double *C;
+    int ldc;
+};
+
+// Byte offset of the digit-d tile (128 rows x 64 k, 128-byte-swizzled image)
+// of row tile rt and K block kb.
+__host__ __device__ __forceinline__ size_t tile_offset(int rt, int kb, int d) {
+    return (((size_t)rt * 2 + kb) * ND + d) * (size_t)kABytes;
+}
+
+// The units of a CTA: (column tile, row tile) pairs, row tiles fastest.
+struct Walk {
+    int ct, rt;
+    __device__ static int first_rt(const Problem &p, int ct) { return p.lower ? ct / 2 : 0; }
+    __device__ void seek(const Problem &p, long long u) {
+        ct = p.ct0;
+        if (!p.lower) {
+            ct += (int)(u / p.nrt);
+            rt = (int)(u % p.nrt);
+            return;
+        }
+        while (u >= p.nrt - ct / 2) { u -= p.nrt - ct / 2; ++ct; }
+        rt = ct / 2 + (int)u;
+    }
+    __device__ void next(const Problem &p) {
+        if (++rt >= p.nrt) { ++ct; rt = first_rt(p, ct); }
+    }
+};
+
+#define TMEM_LD4(taddr, r, o)                                                                       \
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"                       \
+                 : "=r"(r[o]), "=r"(r[o + 1]), "=r"(r[o + 2]), "=r"(r[o + 3])                       \
+                 : "r"(taddr))
+
+// (hi 2^32 + lo) 2^(e - 2112), |hi| < 2^44, |lo| < 2^48, rounded to nearest (a
+// tie between two doubles goes up in magnitude).  Integer operations only: the
+// FP64 pipe has ~2 lanes per clock and is left to the subtraction.
+__device__ __forceinline__ double scaled_double(long long hi, long long lo, int e) {
+    hi += lo >> 32;
+    unsigned l = (unsigned)lo;
+    const bool neg = hi < 0;
+    if (neg) {                                      // negate the 96-bit number
+        l = 0u - l;
+        hi = -hi - (l != 0u ? 1 : 0);
+    }
+    unsigned long long w = ((unsigned long long)hi << 20) | (l >> 12);
+    unsigned long long x = (unsigned long long)l << 52;
+    if (w == 0) {
+        if (x == 0) return 0.0;
+        w = x;
+        x = 0;
+        e -= 64;
+    }
+    const int lz = __clzll((long long)w);
+    const unsigned long long m = lz ? (w << lz) | (x >> (64 - lz)) : w;
+    // value = m 2^(12 - lz) 2^(e - 2112), m in [2^63, 2^64)
+    const int field = e - 2112 + 12 - lz + 63 + 1023;
+    unsigned long long b = (m >> 11) + ((m >> 10) & 1u);      // 53 bits; a carry moves the exponent up by one
+    b += (unsigned long long)(field - 1) << 52;               // the leading bit adds the missing one
+    return __longlong_as_double((long long)(b | (neg ? 0x8000000000000000ull : 0ull)));
+}
+
+__global__ void __launch_bounds__(kThreads, 1)
+k_update_sliced(Problem p) {
+    if (p.skip != nullptr && *p.skip != 0) return;
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t *base = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t *sB = base;
+    uint8_t *sA = base + kBBytes;
+    Smem &s = *reinterpret_cast<Smem *>(sA + AST * kABytes);
+    volatile int *abort_flag = &s.abort_flag;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long u0 = p.units * blockIdx.x / gridDim.x, u1 = p.units * (blockIdx.x + 1) / gridDim.x;
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < AST; ++i) { mbar_init(&s.afull[i], 1); mbar_init(&s.aempty[i], 1); }
+        mbar_init(&s.bfull, 1);
+        mbar_init(&s.bempty, 1);
+        mbar_init(&s.acc_full, 1);
+        mbar_init(&s.acc_empty, EPI);
+        mbar_init(&s.drain, 1);
+        s.abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s.tmem_base)),
+                     "r"(kTmemCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = s.tmem_base;
+
+    if (warp == 0) {
+        // ------------------------------------------------ copies
+        if (lane == 0 && u0 < u1) {
+            Walk wk;
+            wk.seek(p, u0);
+            int ia = 0, nb = 0, ct = -1;
+            bool ok = true;
+            for (long long u = u0; u < u1 && ok; ++u, wk.next(p)) {
+                if (wk.ct != ct) {
+                    ct = wk.ct;
+                    if (!wait_bounded(&s.bempty, (uint32_t)(nb & 1) ^ 1u, abort_flag, &g_slice64_status)) {
+                        ok = false;
+                        break;
+                    }
+                    mbar_arrive_expect_tx(&s.bfull, (uint32_t)p.nkb * ND * kBHalf);
+                    const uint8_t *S = (p.same ? p.SA : p.SB);
+                    for (int kb = 0; kb < p.nkb; ++kb)
+                        for (int d = 0; d < ND; ++d)
+                            asm volatile(
+                                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, "
+                                "[%3];" ::"r"(smem_u32(sB + (kb * ND + d) * kBHalf)),
+                                "l"(S + tile_offset(ct / 2, kb, d) + (size_t)(ct & 1) * kBHalf), "r"(kBHalf),
+                                "r"(smem_u32(&s.bfull))
+                                : "memory");
+                    ++nb;
+                }
+                for (int kb = 0; kb < p.nkb && ok; ++kb)
+                    for (int d = 0; d < ND; ++d) {
+                        const int st = ia % AST;
+                        if (!wait_bounded(&s.aempty[st], ((uint32_t)(ia / AST) & 1u) ^ 1u, abort_flag,
+                                          &g_slice64_status)) {
+                            ok = false;
+                            break;
+                        }
+                        mbar_arrive_expect_tx(&s.afull[st], kABytes);
+                        asm volatile(
+                            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                                smem_u32(sA + st * kABytes)),
+                            "l"(p.SA + tile_offset(wk.rt, kb, d)), "r"(kABytes), "r"(smem_u32(&s.afull[st]))
+                            : "memory");
+                        ++ia;
+                    }
+            }
+            if (!ok) {
+                // every issued copy must land before the CTA exits
+                for (long long i = 0; nb > 0 && i < kSpinLimit && !mbar_try_wait(&s.bfull, (uint32_t)(nb - 1) & 1u); ++i)
+                    __nanosleep(64);
+                for (int j = (ia > AST ? ia - AST : 0); j < ia; ++j) {
+                    const uint32_t ph = (uint32_t)(j / AST) & 1u;
+                    for (long long i = 0; i < kSpinLimit && !mbar_try_wait(&s.afull[j % AST], ph); ++i)
+                        __nanosleep(64);
+                }
+            }
+        }
+    } else if (warp == 1) {
+        // ------------------------------------------------ MMA issuer
+        if (lane == 0 && u0 < u1) {
+            Walk wk;
+            wk.seek(p, u0);
+            int ia = 0, nb = 0, ct = -1, n = 0;
+            bool ok = true, issued = false;
+            for (long long u = u0; u < u1 && ok; ++u, ++n) {
+                if (wk.ct != ct) {
+                    ct = wk.ct;
+                    if (!wait_bounded(&s.bfull, (uint32_t)nb & 1u, abort_flag, &g_slice64_status)) { ok = false; break; }
+                    ++nb;
+                }
+                if (!wait_bounded(&s.acc_empty, ((uint32_t)n & 1u) ^ 1u, abort_flag, &g_slice64_status)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                for (int kb = 0; kb < p.nkb && ok; ++kb) {
+                    const uint64_t bd = make_sw128_desc(smem_u32(sB + kb * ND * kBHalf));
+                    for (int d = 0; d < ND; ++d) {
+                        const int as = ia % AST;
+                        if (!wait_bounded(&s.afull[as], (uint32_t)(ia / AST) & 1u, abort_flag, &g_slice64_status)) {
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                        const uint64_t ad = make_sw128_desc(smem_u32(sA + as * kABytes));
+                        // A10 digit d times A01 digits t = 0..7-d into the columns of diagonals d..7
+                        const int ncol = BN * (ND - d);
+                        const int n1 = ncol < 256 ? ncol : 256, n2 = ncol - n1;
+                        const uint32_t id1 = make_idesc(true, BM, n1);
+                        const uint32_t id2 = make_idesc(true, BM, n2 > 0 ? n2 : 16);
+                        const uint32_t dst = tmem_base + (uint32_t)(BN * d);
+#pragma unroll
+                        for (int kk = 0; kk < BK / UMMA_K; ++kk) {
+                            const uint32_t acc = (kb > 0 || d > 0 || kk > 0) ? 1u : 0u;
+                            umma_f16(dst, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), id1, acc);
+                            if (n2 > 0)      // 256 rows further: 32 KB
+                                umma_f16(dst + 256, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2 + (256 * 128 >> 4)),
+                                         id2, acc);
+                        }
+                        issued = true;
+                        umma_commit(&s.aempty[as]);
+                        ++ia;
+                    }
+                }
+                if (!ok) break;
+                umma_commit(&s.acc_full);
+                wk.next(p);
+                if (u + 1 < u1 && wk.ct != ct) umma_commit(&s.bempty);
+            }
+            if (issued) {
+                umma_commit(&s.drain);
+                for (long long i = 0; i < kSpinLimit && !mbar_try_wait(&s.drain, 0); ++i) __nanosleep(64);
+            }
+        }
+    } else {
+        // ------------------------------------------------ epilogue (warps 2..17)
+        const int quarter = warp & 3;             // TMEM lanes 32 * quarter ..
+        const int grp = (warp - 2) >> 2;          // columns 16 * grp ..
+        const int any = *p.any;
+        Walk wk;
+        int n = 0;
+        bool ok = true;
+        if (u0 < u1) wk.seek(p, u0);
+        for (long long u = u0; u < u1 && ok; ++u, ++n, wk.next(p)) {
+            const int row = wk.rt * BM + quarter * 32 + lane;
+            const int col0 = wk.ct * BN + grp * 16;
+            const int Ei = row < p.m ? p.E[row] : kCentre;
+            if (lane == 0) ok = wait_bounded(&s.acc_full, (uint32_t)n & 1u, abort_flag, &g_slice64_status);
+            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(grp * 16);
+            double v[16];
+#pragma unroll
+            for (int c = 0; c < 16; c += 4) {
+                uint32_t r[4 * ND];
+#pragma unroll
+                for (int d = 0; d < ND; ++d) TMEM_LD4(taddr + (uint32_t)(d * BN + c), r, 4 * d);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    int S[ND];
+#pragma unroll
+                    for (int d = 0; d < ND; ++d) S[d] = __float2int_rn(__uint_as_float(r[4 * d + q]));
+                    // |S_d| <= d 2^21 (S_0: 2^19): the pairs below fit int32 where they are formed in int32
+                    const long long hi = (long long)(S[0] * 256 + S[1]) * 65536 + (long long)(S[2] * 256 + S[3]);
+                    const long long lo = (long long)S[4] * 16777216 + (long long)S[5] * 65536 +
+                                         ((long long)S[6] * 256 + S[7]);
+                    const int col = col0 + c + q;
+                    const int Fk = p.same ? (col < p.c1 ? p.E[col] - kCentre : 0) : (col < p.c1 ? p.F[col] : 0);
+                    v[c + q] = scaled_double(hi, lo, Ei + Fk);
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&s.acc_empty);
+            if (row >= p.m || (any && (p.flagA[wk.rt] || (p.same ? p.flagA[wk.ct / 2] : p.flagB[wk.ct / 2])))) continue;
+            double *Cp = p.C + (size_t)row + (size_t)col0 * p.ldc;
+            double cv[16];
+#pragma unroll
+            for (int c = 0; c < 16; ++c) {
+                const int col = col0 + c;
+                const bool in = col >= p.c0 && col < p.c1 && (!p.lower || row >= col);
+                cv[c] = in ? Cp[(size_t)c * p.ldc] : 0.0;
+            }
+#pragma unroll
+            for (int c = 0; c < 16; ++c) {
+                const int col = col0 + c;
+                if (col >= p.c0 && col < p.c1 && (!p.lower || row >= col)) Cp[(size_t)c * p.ldc] = cv[c] - v[c];
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 1) {
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols)
+                     : "memory");
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Inner exponents: rho[j] = max over the columns of the exponent field of
+// A01(j, k); zero before.  A warp takes whole columns (w contiguous values).
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) k_inner_exp(const double *__restrict__ U, int ldu, int w, int cols, int *rho) {
+    __shared__ int red[kMaxV];
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x < kMaxV) red[threadIdx.x] = 0;
+    __syncthreads();
+    int f[4] = {0, 0, 0, 0};
+    for (int c = blockIdx.x * 8 + (threadIdx.x >> 5); c < cols; c += gridDim.x * 8) {
+        const double *u = U + (size_t)c * ldu;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int j = lane + 32 * q;
+            if (j < w) {
+                const int e = (int)((__double_as_longlong(u[j]) >> 52) & 0x7FF);
+                if (e != 0x7FF) f[q] = max(f[q], e);
+            }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        if (f[q] > 0) atomicMax(red + lane + 32 * q, f[q]);
+    __syncthreads();
+    if (threadIdx.x < kMaxV && red[threadIdx.x] > 0) atomicMax(rho + threadIdx.x, red[threadIdx.x]);
+}
+
+// ---------------------------------------------------------------------------
+// Digit slices of rows of A10 (A[i + j lda]) and columns of A01 (B[j + i ldb]).
+// CTA: 32 rows x 128 j; the row's largest scaled exponent, the digits, then
+// each slice through shared memory as whole 128-byte tile rows.  Bound by the
+// memory traffic of 24 bytes per element and ~40 integer operations.
+// ---------------------------------------------------------------------------
+constexpr int kRows = 32;
+constexpr int kPitch = 2 * BK + 8;      // BF16 per staged row
+
+__device__ __forceinline__ void digits8(double x, int sh, __nv_bfloat16 (&dg)[ND]) {
+    const long long bits = __double_as_longlong(x);
+    const int f = (int)((bits >> 52) & 0x7FF);
+    const long long mant = bits & ((1ll << 52) - 1);
+    const long long m53 = f == 0 ? mant : (mant | (1ll << 52));
+    long long q;                                   // m53 2^sh, to nearest
+    if (sh >= 0) q = m53 << (sh > 9 ? 9 : sh);
+    else if (-sh >= 60) q = 0;
+    else q = (m53 + (1ll << (-sh - 1))) >> (-sh);
+    if (bits < 0) q = -q;
+    // the seven low digits are the bytes of q + 128 (1 + 256 + ... + 256^6)
+    // less 128 each, the top one what is left above them
+    const long long t = q + 0x0080808080808080ll;
+    const unsigned lo = (unsigned)t, hi = (unsigned)(t >> 32);
+#pragma unroll
+    for (int b = 0; b < 4; ++b) dg[ND - 1 - b] = __float2bfloat16_rn((float)((lo >> (8 * b)) & 255u) - 128.f);
+#pragma unroll
+    for (int b = 0; b < 3; ++b) dg[ND - 5 - b] = __float2bfloat16_rn((float)((hi >> (8 * b)) & 255u) - 128.f);
+    dg[0] = __float2bfloat16_rn((float)(t >> 56));
+}
+
+struct SliceArgs {
+    const double *A, *B;
+    int lda, ldb, rows, cols, w, nkb;
+    int blocks_a;                       // CTAs of the A side; the rest cut B
+    uint8_t *SA, *SB;
+    int *E, *F;
+    const int *rho;                     // null: Cholesky (no inner scale)
+    int *any, *flagA, *flagB;
+    const int *skip;
+};
+
+__global__ void __launch_bounds__(256) k_slice_operands(SliceArgs a) {
+    if (a.skip != nullptr && *a.skip != 0) return;
+    __shared__ double xs[kRows][2 * BK + 1];
+    __shared__ __align__(16) __nv_bfloat16 tile[kRows * kPitch];
+    __shared__ int gmax[8][kRows];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool side_b = (int)blockIdx.x >= a.blocks_a;
+    const int i0 = (side_b ? blockIdx.x - a.blocks_a : blockIdx.x) * kRows;
+    const int m = side_b ? a.cols : a.rows;
+    const int i = i0 + lane, j0 = warp * 16;
+    double x[16];
+    if (!side_b) {
+#pragma unroll
+        for (int c = 0; c < 16; ++c)
+            x[c] = (i < m && j0 + c < a.w) ? a.A[(size_t)i + (size_t)(j0 + c) * a.lda] : 0.0;
+    } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int col = i0 + warp * 4 + q;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int j = lane + 32 * e;
+                xs[warp * 4 + q][j] = (col < m && j < a.w) ? a.B[(size_t)j + (size_t)col * a.ldb] : 0.0;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int c = 0; c < 16; ++c) x[c] = xs[lane][j0 + c];
+    }
+    int g[16];
+    int top = INT_MIN;
+    bool bad = false;
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+        const int f = (int)((__double_as_longlong(x[c]) >> 52) & 0x7FF);
+        int r = 1023;
+        if (a.rho != nullptr && j0 + c < a.w) {
+            r = a.rho[j0 + c];
+            if (r == 0) r = 1023;
+        }
+        g[c] = max(f, 1) + (side_b ? -r : r);
+        bad |= f == 0x7FF;
+        if (x[c] != 0.0) top = max(top, g[c]);
+    }
+    gmax[warp][lane] = top;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 8; ++q) top = max(top, gmax[q][lane]);
+    const int centre = side_b ? 0 : kCentre;
+    if (top == INT_MIN) top = centre;                   // a zero row: all digits zero
+    bad |= top < centre - kSpan || top > centre + (a.rho == nullptr || side_b ? kSpan : kSpanUp);
+    if (i < m) {
+        if (warp == 0) (side_b ? a.F : a.E)[i] = top;
+        if (bad) {
+            atomicOr((side_b ? a.flagB : a.flagA) + i / BM, 1);
+            atomicOr(a.any, 1);
+        }
+    }
+    uint32_t pk[ND][8];
+#pragma unroll
+    for (int c = 0; c < 16; c += 2) {
+        __nv_bfloat16 d0[ND], d1[ND];
+        digits8(x[c], g[c] - top + 9, d0);
+        digits8(x[c + 1], g[c + 1] - top + 9, d1);
+#pragma unroll
+        for (int d = 0; d < ND; ++d) {
+            __nv_bfloat162 h;
+            h.x = d0[d];
+            h.y = d1[d];
+            pk[d][c / 2] = *reinterpret_cast<const uint32_t *>(&h);
+        }
+    }
+    uint8_t *S = side_b ? a.SB : a.SA;
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+        uint4 *sdst = reinterpret_cast<uint4 *>(tile + lane * kPitch + warp * 16);
+        sdst[0] = make_uint4(pk[d][0], pk[d][1], pk[d][2], pk[d][3]);
+        sdst[1] = make_uint4(pk[d][4], pk[d][5], pk[d][6], pk[d][7]);
+        __syncthreads();
+#pragma unroll
+        for (int it = 0; it < 2; ++it) {
+            const int c = tid + 256 * it;
+            const int r = c >> 4, q = c & 15;
+            const int kb = q >> 3, ch = q & 7;
+            const int gi = i0 + r, rl = gi & (BM - 1);
+            if (kb < a.nkb) {       // rows past m: zero digits, inside the padded tile
+                const uint4 v = *reinterpret_cast<const uint4 *>(tile + r * kPitch + q * 8);
+                *reinterpret_cast<uint4 *>(S + tile_offset(gi / BM, kb, d) + (size_t)rl * 128 +
+                                           (size_t)((ch ^ (rl & 7)) * 16)) = v;
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Flagged tiles in FP64: the 64 x 64 tiles of C that lie in a flagged row or
+// column tile.  One element per thread at a time (the flag is rare); nothing
+// flagged: one load per CTA.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256)
+k_gemm_flagged(Problem p, int w, const double *__restrict__ A, int lda, const double *__restrict__ B, int ldb) {
+    if (p.skip != nullptr && *p.skip != 0) return;
+    if (*p.any == 0) return;
+    const int nrt = (p.m + 63) / 64, ct0 = p.c0 / 64, ct1 = (p.c1 + 63) / 64;
+    for (long long t = blockIdx.x; t < (long long)nrt * (ct1 - ct0); t += gridDim.x) {
+        const int rt = (int)(t % nrt), ct = ct0 + (int)(t / nrt);
+        if (!(p.flagA[rt / 2] || (p.same ? p.flagA[ct / 2] : p.flagB[ct / 2]))) continue;
+        for (int e = threadIdx.x; e < 64 * 64; e += 256) {
+            const int i = rt * 64 + (e & 63), j = ct * 64 + (e >> 6);
+            if (i >= p.m || j < p.c0 || j >= p.c1 || (p.lower && i < j)) continue;
+            double acc = 0.0;
+            for (int k = 0; k < w; ++k)
+                acc = fma(A[(size_t)i + (size_t)k * lda],
+                          p.same ? A[(size_t)j + (size_t)k * lda] : B[(size_t)k + (size_t)j * ldb], acc);
+            double *c = p.C + (size_t)i + (size_t)j * p.ldc;
+            *c = *c - acc;
+        }
+    }
+}
+
+}  // namespace s64
+
+// ---------------------------------------------------------------------------
+// Host side
+// ---------------------------------------------------------------------------
+Slice64 slice64_carve(void *work, int rows, int cols) {
+    Slice64 s;
+    s.rows = rows;
+    s.cols = cols;
+    Carver cv(work);
+    const size_t ra = align_up((size_t)rows, s64::BM), rb = align_up((size_t)cols, s64::BM);
+    s.SA = cv.take<uint8_t>(ra * 2 * s64::ND * 128, 1024);
+    s.SB = cols ? cv.take<uint8_t>(rb * 2 * s64::ND * 128, 1024) : nullptr;
+    s.E = cv.take<int>(ra);
+    s.F = cols ? cv.take<int>(rb) : nullptr;
+    s.nflags = 4 + ra / s64::BM + rb / s64::BM;
+    s.head = cv.take<int>(kMaxV + s.nflags);
+    return s;
+}
+
+size_t slice64_bytes(int rows, int cols) {
+    const Slice64 s = slice64_carve(nullptr, rows, cols);
+    Carver cv(nullptr);
+    const size_t ra = align_up((size_t)rows, s64::BM), rb = align_up((size_t)cols, s64::BM);
+    cv.take<uint8_t>(ra * 2 * s64::ND * 128, 1024);
+    if (cols) cv.take<uint8_t>(rb * 2 * s64::ND * 128, 1024);
+    cv.take<int>(ra);
+    if (cols) cv.take<int>(rb);
+    cv.take<int>(kMaxV + s.nflags);
+    return cv.size();
+}
+
+int slice64_begin(const Slice64 &s, const double *A01, int lda, int w, int cols, const int *skip, cudaStream_t st) {
+    (void)skip;
+    CF_CUDA_TRY(cudaMemsetAsync(s.head, 0, sizeof(int) * (kMaxV + s.nflags), st));
+    if (A01 == nullptr || cols <= 0) return CF_OK;
+    const int want = ceil_div(cols, 8), most = 2 * device_sm_count();     // eight columns per CTA and pass
+    s64::k_inner_exp<<<want < most ? want : most, 256, 0, st>>>(A01, lda, w, cols, s.rho());
+    CF_LAUNCH_CHECK();
+    return CF_OK;
+}
+
+int slice64_clear_flags(const Slice64 &s, cudaStream_t st) {
+    CF_CUDA_TRY(cudaMemsetAsync(s.any(), 0, sizeof(int) * s.nflags, st));
+    return CF_OK;
+}
+
+int slice64_operands(const Slice64 &s, const double *A10, int lda, int rows, const double *A01, int ldb, int cols,
+                     int w, const int *skip, cudaStream_t st) {
+    s64::SliceArgs a{};
+    a.A = A10;
+    a.B = A01;
+    a.lda = lda;
+    a.ldb = ldb;
+    a.rows = rows;
+    a.cols = A01 ? cols : 0;
+    a.w = w;
+    a.nkb = ceil_div(w, s64::BK);
+    a.blocks_a = ceil_div(rows, s64::kRows);
+    a.SA = s.SA;
+    a.SB = s.SB;
+    a.E = s.E;
+    a.F = s.F;
+    a.rho = s.cols ? s.rho() : nullptr;
+    a.any = s.any();
+    a.flagA = s.flagA();
+    a.flagB = s.flagB();
+    a.skip = skip;
+    const int blocks = a.blocks_a + ceil_div(a.cols, s64::kRows);
+    if (blocks == 0) return CF_OK;
+    s64::k_slice_operands<<<blocks, 256, 0, st>>>(a);
+    CF_LAUNCH_CHECK();
+    return CF_OK;
+}
+
+int slice64_update(const Slice64 &s, int rows, int c0, int c1, int w, const double *A10, int lda, const double *A01,
+                   int ldb, double *C, int ldc, bool lower, const int *skip, cudaStream_t st) {
+    using namespace s64;
+    if (rows <= 0 || c1 <= c0 || w <= 0) return CF_OK;
+    Problem p{};
+    p.m = rows;
+    p.c0 = c0;
+    p.c1 = c1;
+    p.nkb = ceil_div(w, BK);
+    p.lower = lower ? 1 : 0;
+    p.same = s.cols == 0 ? 1 : 0;
+    p.ct0 = c0 / BN;
+    p.ct1 = ceil_div(c1, BN);
+    p.nrt = ceil_div(rows, BM);
+    p.units = 0;
+    for (int ct = p.ct0; ct < p.ct1; ++ct) p.units += lower ? p.nrt - ct / 2 : p.nrt;
+    p.SA = s.SA;
+    p.SB = s.SB;
+    p.E = s.E;
+    p.F = s.F;
+    p.any = s.any();
+    p.flagA = s.flagA();
+    p.flagB = s.flagB();
+    p.skip = skip;
+    p.C = C;
+    p.ldc = ldc;
+    const int sms = device_sm_count();
+    const size_t smem = 1024 + kBBytes + AST * kABytes + sizeof(Smem);
+    CF_CUDA_TRY(cudaFuncSetAttribute(k_update_sliced, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_update_sliced<<<(int)(p.units < sms ? p.units : sms), kThreads, smem, st>>>(p);
+    CF_LAUNCH_CHECK();
+    k_gemm_flagged<<<sms, 256, 0, st>>>(p, w, A10, lda, A01, ldb);
+    CF_LAUNCH_CHECK();
+    return CF_OK;
+}
+
+int slice64_take_status(cudaStream_t st, int *status) {
+    int h = 0;
+    CF_CUDA_TRY(cudaMemcpyFromSymbolAsync(&h, g_slice64_status, sizeof(int), 0, cudaMemcpyDeviceToHost, st));
+    CF_CUDA_TRY(cudaStreamSynchronize(st));
+    if (h != 0) {
+        const int zero = 0;
+        CF_CUDA_TRY(cudaMemcpyToSymbolAsync(g_slice64_status, &zero, sizeof(int), 0, cudaMemcpyHostToDevice, st));
+        CF_CUDA_TRY(cudaStreamSynchronize(st));
+    }
+    *status = h;
+    return CF_OK;
+}
+
+}  // namespace cf
