@@ -14,6 +14,7 @@
 #include "cf_common.cuh"
 #include "cf_kernels.cuh"
 #include "cf_slice64.cuh"
+#include "cf_solve64.cuh"
 
 namespace cf {
 
@@ -21,11 +22,6 @@ static std::atomic<int> g_last_cuda_error{0};
 static std::atomic<long long> g_launches{0};
 void set_cuda_error(cudaError_t e) { g_last_cuda_error.store((int)e); }
 void count_launches(long long n) { g_launches.fetch_add(n); }
-
-int launch_trsm_left_f64(bool lower, bool unit, bool trans, double *X, int ldx, int w, int cols, const double *Tm,
-                         int ldt, cudaStream_t st);
-int launch_gemm_f64_sub_t(int m, int n, int k, const double *A, int lda, bool trans_a, const double *B, int ldb,
-                          bool trans_b, double *C, int ldc, bool lower, const int *skip, cudaStream_t st);
 
 int resolve_options(const cf_options *in, Opts *o) {
     *o = Opts();
@@ -54,33 +50,6 @@ int resolve_options(const cf_options *in, Opts *o) {
     if (o->gmres_restart < 1 || o->gmres_restart > 256) return CF_ERR_UNSUPPORTED;
     if (o->batch_cps < 0 || o->batch_cps > 8) return CF_ERR_UNSUPPORTED;
     return CF_OK;
-}
-
-// ipiv (1-based interchanges) -> row order: perm[i] = original row now at i.
-__global__ void k_ipiv_to_perm(int n, const int *ipiv, int *perm) {
-    extern __shared__ int sp[];
-    const bool use_smem = (size_t)n * sizeof(int) <= 200 * 1024;
-    int *p = use_smem ? sp : perm;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = i;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < n; ++i) {
-            const int j = ipiv[i] - 1;
-            if (j != i) { const int t = p[i]; p[i] = p[j]; p[j] = t; }
-        }
-    }
-    __syncthreads();
-    if (use_smem)
-        for (int i = threadIdx.x; i < n; i += blockDim.x) perm[i] = p[i];
-}
-
-// Out[i, c] = In[perm[i], c]
-__global__ void k_gather_rows(int n, int nrhs, const int *perm, const double *In, int ldi, double *Out, int ldo) {
-    const size_t tot = (size_t)n * nrhs;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < tot; e += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(e % n), c = (int)(e / n);
-        Out[(size_t)i + (size_t)c * ldo] = In[(size_t)perm[i] + (size_t)c * ldi];
-    }
 }
 
 }  // namespace cf
@@ -464,31 +433,10 @@ extern "C" int cf_getrs(int n, int nrhs, const double *LU, int lda, const int *i
     Carver cv(work);
     int *perm = cv.take<int>(n);
     double *T = cv.take<double>((size_t)n * nrhs);
-    const size_t smem = (size_t)n * sizeof(int) <= 200 * 1024 ? (size_t)n * sizeof(int) : 0;
-    if (smem > 48 * 1024) CF_CUDA_TRY(cudaFuncSetAttribute(k_ipiv_to_perm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_ipiv_to_perm<<<1, 1024, smem, st>>>(n, ipiv, perm);
-    CF_LAUNCH_CHECK();
-    k_gather_rows<<<1024, 256, 0, st>>>(n, nrhs, perm, B, ldb, T, n);
-    CF_LAUNCH_CHECK();
     int rc;
-    const size_t ld = (size_t)lda;
-    const int v = kMaxV;
-    for (int k0 = 0; k0 < n; k0 += v) {                 // L y = P b
-        const int w = v < n - k0 ? v : n - k0;
-        if ((rc = launch_trsm_left_f64(true, true, false, T + k0, n, w, nrhs, LU + k0 + k0 * ld, lda, st))) return rc;
-        if ((rc = launch_gemm_f64_sub_t(n - k0 - w, nrhs, w, LU + (k0 + w) + k0 * ld, lda, false, T + k0, n, false,
-                                        T + k0 + w, n, false, nullptr, st)))
-            return rc;
-    }
-    const int nb = (n + v - 1) / v;
-    for (int b = nb - 1; b >= 0; --b) {                 // U x = y
-        const int k0 = b * v;
-        const int w = v < n - k0 ? v : n - k0;
-        if ((rc = launch_trsm_left_f64(false, false, false, T + k0, n, w, nrhs, LU + k0 + k0 * ld, lda, st))) return rc;
-        if ((rc = launch_gemm_f64_sub_t(k0, nrhs, w, LU + k0 * ld, lda, false, T + k0, n, false, T, n, false, nullptr,
-                                        st)))
-            return rc;
-    }
+    if ((rc = launch_permute_rhs(n, nrhs, ipiv, perm, B, ldb, T, st))) return rc;
+    if ((rc = launch_tri_solve64(0, n, nrhs, LU, lda, T, n, st))) return rc;      // L y = P b
+    if ((rc = launch_tri_solve64(1, n, nrhs, LU, lda, T, n, st))) return rc;      // U x = y
     CF_CUDA_TRY(cudaMemcpy2DAsync(B, sizeof(double) * ldb, T, sizeof(double) * n, sizeof(double) * n, nrhs,
                                   cudaMemcpyDeviceToDevice, st));
     return CF_OK;
@@ -503,27 +451,8 @@ extern "C" int cf_potrs(int n, int nrhs, const double *L, int lda, double *B, in
     if (ldb < (n > 1 ? n : 1)) return -6;
     if (n == 0 || nrhs == 0) return CF_OK;
     int rc;
-    const size_t ld = (size_t)lda, lb = (size_t)ldb;
-    const int v = kMaxV;
-    for (int k0 = 0; k0 < n; k0 += v) {                 // L y = b
-        const int w = v < n - k0 ? v : n - k0;
-        if ((rc = launch_trsm_left_f64(true, false, false, B + k0, ldb, w, nrhs, L + k0 + k0 * ld, lda, st))) return rc;
-        if ((rc = launch_gemm_f64_sub_t(n - k0 - w, nrhs, w, L + (k0 + w) + k0 * ld, lda, false, B + k0, ldb, false,
-                                        B + k0 + w, ldb, false, nullptr, st)))
-            return rc;
-    }
-    const int nb = (n + v - 1) / v;
-    for (int b = nb - 1; b >= 0; --b) {                 // L^T x = y
-        const int k0 = b * v;
-        const int w = v < n - k0 ? v : n - k0;
-        if ((rc = launch_trsm_left_f64(false, false, true, B + k0, ldb, w, nrhs, L + k0 + k0 * ld, lda, st))) return rc;
-        // B[0:k0] -= (L[k0:k0+w, 0:k0])^T B[k0:k0+w]
-        if ((rc = launch_gemm_f64_sub_t(k0, nrhs, w, L + k0, lda, true, B + k0, ldb, false, B, ldb, false, nullptr,
-                                        st)))
-            return rc;
-    }
-    (void)lb;
-    return CF_OK;
+    if ((rc = launch_tri_solve64(2, n, nrhs, L, lda, B, ldb, st))) return rc;     // L y = b
+    return launch_tri_solve64(3, n, nrhs, L, lda, B, ldb, st);                    // L^T x = y
 }
 
 extern "C" int cf_residual(int m, int n, int nrhs, const double *A, int lda, const double *X, int ldx,

@@ -1,0 +1,468 @@
+// cf_solve64.cu -- S-1: the FP64 triangular solves of cf_getrs / cf_potrs and
+// the row order of a list of interchanges.
+//
+// A solve with an n x n triangle is a chain of n dependent steps; its bytes
+// (4 n^2 per direction) and its 2 lanes of FP64 per clock and SM are far from
+// binding for a few right-hand sides.  So the chain is what counts:
+//   * the triangle is cut into super-blocks of 2048 rows.  One thread-block
+//     cluster per right-hand side solves a super-block; its rows beyond take
+//     one product over the whole GPU (launch_residual_f64, k_gemv_t_sub);
+//   * inside the cluster, blocks of 64 rows go round the eight CTAs.  A solved
+//     block is written into every CTA's shared memory (distributed shared
+//     memory, an mbarrier per block), the owner of the next block multiplies
+//     its prefetched tile and substitutes in one warp: two rows per lane, the
+//     pivot's value by shuffle.  No inverse is formed: the operations are
+//     substitution's own, the quotients corrected to
+//     the last bit.
+// The waits are inside a cluster, whose CTAs run at the same time by
+// definition, and bounded.  No workspace: cf_potrs has none.
+#include <cooperative_groups.h>
+
+#include "cf_common.cuh"
+#include "cf_kernels.cuh"
+#include "cf_solve64.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace cf {
+
+__device__ int g_solve64_status = 0;       // 0 or CF_ERR_TIMEOUT
+
+namespace sv {
+
+constexpr int NB = 64;                 // rows of a block
+constexpr int CL = 8;                  // CTAs of a cluster
+constexpr int kSuper = 2048;           // rows of a super-block
+constexpr int MAXB = kSuper / NB;      // blocks
+constexpr int OWN = MAXB / CL;         // blocks of a CTA
+constexpr int LDD = NB + 1;
+constexpr int kThreads = 256;
+
+struct Smem {
+    double D[OWN][NB * LDD];           // diagonal blocks: D[k * LDD + r] = M(r, k)
+    double rinv[OWN][NB];              // 1 / M(k, k)
+    double xs[MAXB][NB];               // solved blocks, in solving order
+    double x0[OWN][NB];                // right-hand side of the CTA's blocks
+    double part[4 * NB];
+    double pub[NB];
+    uint64_t bar[MAXB];
+};
+
+__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void wait_block(uint64_t *bar) {
+    for (long long i = 0; i < (1ll << 22); ++i) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}\n"
+            : "=r"(ok)
+            : "r"(smem_u32(bar))
+            : "memory");
+        if (ok) return;
+        if (i > 64) __nanosleep(20);
+    }
+    atomicExch(&g_solve64_status, CF_ERR_TIMEOUT);
+}
+
+// MODE 0: unit lower, 1: upper, 2: lower, 3: transposed lower (M = T^T)
+template <int MODE>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(kThreads, 1)
+k_tri_solve64(int n, const double *__restrict__ T, int ldt, double *__restrict__ X, int ldx) {
+    constexpr bool FWD = MODE == 0 || MODE == 2, TRANS = MODE == 3, UNIT = MODE == 0;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    Smem &s = *reinterpret_cast<Smem *>(smem_raw);
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nb = (n + NB - 1) / NB;
+    const size_t ld = (size_t)ldt;
+    double *x = X + (size_t)blockIdx.y * ldx;
+    auto row0 = [&](int t) { return (FWD ? t : nb - 1 - t) * NB; };   // first row of the t-th block solved
+
+    if (tid < MAXB) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s.bar[tid])) : "memory");
+    if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    for (int t = rank, o = 0; t < nb; t += CL, ++o) {
+        const int r0 = row0(t), nr = min(NB, n - r0);
+        for (int e = tid; e < NB * NB; e += kThreads) {
+            const int a = e & (NB - 1), b = e >> 6;                   // a runs along the memory
+            const int r = TRANS ? b : a, k = TRANS ? a : b;
+            const bool need = (FWD ? k <= r : k >= r) && r < nr && k < nr && !(UNIT && r == k);
+            double v = (r == k) ? 1.0 : 0.0;                          // rows past the end: identity
+            if (need) v = TRANS ? T[(size_t)(r0 + k) + (size_t)(r0 + r) * ld] : T[(size_t)(r0 + r) + (size_t)(r0 + k) * ld];
+            s.D[o][k * LDD + r] = v;
+        }
+        if (tid < NB) s.x0[o][tid] = tid < nr ? x[r0 + tid] : 0.0;
+    }
+    __syncthreads();
+    if (!UNIT)
+        for (int t = rank, o = 0; t < nb; t += CL, ++o)
+            if (tid < NB) s.rinv[o][tid] = 1.0 / s.D[o][tid * LDD + tid];
+    cl.sync();
+
+    // Partial sums of the CTA's blocks.  Row r, k quarter q (TRANS: eight rows
+    // of a warp, the lane's two k): every load of a tile is coalesced.
+    constexpr int AR = TRANS ? 8 : 1;
+    double acc[OWN][AR];
+#pragma unroll
+    for (int o = 0; o < OWN; ++o)
+#pragma unroll
+        for (int a = 0; a < AR; ++a) acc[o][a] = 0.0;
+
+    auto load_tile = [&](int t, int j, double (&v)[16]) {             // block row t, block column j
+        const int r0 = row0(t), c0 = row0(j);
+        if (TRANS) {
+#pragma unroll
+            for (int a = 0; a < 8; ++a)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int r = r0 + warp * 8 + a, k = c0 + lane + 32 * h;
+                    v[2 * a + h] = (r < n && k < n) ? T[(size_t)k + (size_t)r * ld] : 0.0;
+                }
+        } else {
+            const int r = r0 + (tid & (NB - 1)), k0 = c0 + (tid >> 6) * 16;
+#pragma unroll
+            for (int a = 0; a < 16; ++a) v[a] = (r < n && k0 + a < n) ? T[(size_t)r + (size_t)(k0 + a) * ld] : 0.0;
+        }
+    };
+    auto mac = [&](int t, int j, const double (&v)[16]) {
+        const double *xj = s.xs[j];
+        double sum[AR];
+        if (TRANS) {
+            const double x0 = xj[lane], x1 = xj[lane + 32];
+#pragma unroll
+            for (int a = 0; a < AR; ++a) sum[a] = fma(v[2 * a + 1], x1, v[2 * a] * x0);
+        } else {
+            const double *xq = xj + (tid >> 6) * 16;
+            double s0 = 0.0, s1 = 0.0;                                // two chains
+#pragma unroll
+            for (int a = 0; a < 16; a += 2) {
+                s0 = fma(v[a], xq[a], s0);
+                s1 = fma(v[a + 1], xq[a + 1], s1);
+            }
+            sum[0] = s0 + s1;
+        }
+        const int o = t / CL;
+#pragma unroll
+        for (int q = 0; q < OWN; ++q)
+            if (q == o) {
+#pragma unroll
+                for (int a = 0; a < AR; ++a) acc[q][a] += sum[a];
+            }
+    };
+    // Block t: sum of the parts, substitution, result to every CTA.
+    auto solve_block = [&](int t) {
+        const int o = t / CL, r0 = row0(t);
+        double v[AR];
+#pragma unroll
+        for (int q = 0; q < OWN; ++q)
+            if (q == o) {
+#pragma unroll
+                for (int a = 0; a < AR; ++a) v[a] = acc[q][a];
+            }
+        if (TRANS) {
+            // eight sums over the warp's lanes: halve the values with each exchange
+            double w4[4], w2[2], w1;
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const bool up = lane & 16;
+                const double send = up ? v[a % AR] : v[(a + 4) % AR], keep = up ? v[(a + 4) % AR] : v[a % AR];
+                w4[a] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+            }
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+                const bool up = lane & 8;
+                const double send = up ? w4[a] : w4[a + 2], keep = up ? w4[a + 2] : w4[a];
+                w2[a] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+            }
+            {
+                const bool up = lane & 4;
+                const double send = up ? w2[0] : w2[1], keep = up ? w2[1] : w2[0];
+                w1 = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+            }
+            w1 += __shfl_xor_sync(0xffffffffu, w1, 2);
+            w1 += __shfl_xor_sync(0xffffffffu, w1, 1);
+            if ((lane & 3) == 0) s.part[warp * 8 + ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1)] = w1;
+        } else {
+            s.part[tid] = v[0];
+        }
+        __syncthreads();
+        if (warp == 0) {
+            double a, b;                                              // rows lane and lane + 32
+            if (TRANS) {
+                a = s.x0[o][lane] - s.part[lane];
+                b = s.x0[o][lane + 32] - s.part[lane + 32];
+            } else {
+                a = s.x0[o][lane] - ((s.part[lane] + s.part[NB + lane]) + (s.part[2 * NB + lane] + s.part[3 * NB + lane]));
+                b = s.x0[o][lane + 32] - ((s.part[lane + 32] + s.part[NB + lane + 32]) +
+                                          (s.part[2 * NB + lane + 32] + s.part[3 * NB + lane + 32]));
+            }
+            const double *D = s.D[o];
+#pragma unroll 8
+            for (int q = 0; q < NB; ++q) {
+                const int k = FWD ? q : NB - 1 - q;
+                const bool low = FWD ? q < 32 : q >= 32;              // the pivot is in the lanes' first row
+                double xk = __shfl_sync(0xffffffffu, low ? a : b, k & 31);
+                if (!UNIT) {
+                    // the quotient from the reciprocal, corrected by its exact remainder; a zero, and
+                    // whatever leaves the normal numbers, by the division itself
+                    const double d = D[k * LDD + k], r = s.rinv[o][k];
+                    const double q0 = xk * r;
+                    const double q1 = fma(fma(-q0, d, xk), r, q0);
+                    xk = isfinite(q1) && fabs(q0) > 1e-290 ? q1 : (xk == 0.0 && isfinite(r) && r != 0.0 ? q0 : xk / d);
+                }
+                const double da = D[k * LDD + lane], db = D[k * LDD + lane + 32];
+                if (FWD) {
+                    if (low) a = lane == (k & 31) ? xk : (lane > k ? fma(-da, xk, a) : a);
+                    b = (!low && lane == (k & 31)) ? xk : (lane + 32 > k ? fma(-db, xk, b) : b);
+                } else {
+                    if (!low) b = lane == (k & 31) ? xk : (lane + 32 < k ? fma(-db, xk, b) : b);
+                    a = (low && lane == (k & 31)) ? xk : (lane < k ? fma(-da, xk, a) : a);
+                }
+            }
+            s.pub[lane] = a;
+            s.pub[lane + 32] = b;
+            if (r0 + lane < n) x[r0 + lane] = a;
+            if (r0 + lane + 32 < n) x[r0 + lane + 32] = b;
+        }
+        __syncthreads();
+        {
+            Smem *rs = cl.map_shared_rank(&s, warp);                  // warp q serves CTA q
+            rs->xs[t][lane] = s.pub[lane];
+            rs->xs[t][lane + 32] = s.pub[lane + 32];
+            __syncwarp();
+            if (lane == 0) {
+                uint32_t remote;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(&s.bar[t])), "r"(warp));
+                asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
+            }
+        }
+    };
+
+    if (rank == 0) solve_block(0);
+    // The CTA's tiles: for every solved block j, its own blocks t > j, nearest
+    // first; the next tile's loads are in flight while the current one waits.
+    auto first_own = [&](int j) { return j + 1 + ((rank - (j + 1)) % CL + CL) % CL; };
+    int j = 0, t = first_own(0);
+    while (j < nb - 1 && t >= nb) { ++j; t = first_own(j); }
+    double cur[16], nxt[16];
+    if (j < nb - 1) load_tile(t, j, cur);
+    while (j < nb - 1) {
+        int j2 = j, t2 = t + CL;
+        while (j2 < nb - 1 && t2 >= nb) { ++j2; t2 = first_own(j2); }
+        if (j2 < nb - 1) load_tile(t2, j2, nxt);
+        wait_block(&s.bar[j]);
+        mac(t, j, cur);
+        if (t == j + 1) solve_block(t);
+#pragma unroll
+        for (int a = 0; a < 16; ++a) cur[a] = nxt[a];
+        j = j2;
+        t = t2;
+    }
+    cl.sync();                          // no CTA leaves while others may still write into it
+}
+
+// X[c] -= sum_k L[k + c ldl] Y[k], c < m, k < len, for nrhs columns: a warp per
+// column of L, four right-hand sides at a time.
+__global__ void __launch_bounds__(256)
+k_gemv_t_sub(int m, int len, int nrhs, const double *__restrict__ L, int ldl, const double *__restrict__ Y, int ldy,
+             double *__restrict__ X, int ldx) {
+    const int lane = threadIdx.x & 31;
+    const int c = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (c >= m) return;
+    const double *l = L + (size_t)c * ldl;
+    for (int q0 = 0; q0 < nrhs; q0 += 4) {
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+        const int nq = min(4, nrhs - q0);
+#pragma unroll 4
+        for (int k = lane; k < len; k += 32) {
+            const double a = l[k];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (q < nq) acc[q] = fma(a, Y[(size_t)k + (size_t)(q0 + q) * ldy], acc[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+            if (lane == 0 && q < nq) X[(size_t)c + (size_t)(q0 + q) * ldx] -= acc[q];
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// ipiv (1-based interchanges) -> row order: perm[i] = original row now at i.
+// The interchanges are a chain, but a chunk of 128 of them only permutes its own
+// 128 positions and the at most 128 others it names: one warp per chunk plays it
+// on labels (all chunks at once), then the chunks' permutations are applied in
+// order.  Scratch: 6 bytes per row, the chunk's other positions (int) and the
+// labels of its own and of the other positions (one byte each).
+// ---------------------------------------------------------------------------
+constexpr int CH = 128;
+constexpr size_t kChunkBytes = 6 * CH;
+
+__global__ void __launch_bounds__(32) k_ipiv_chunks(int n, const int *__restrict__ ipiv, unsigned char *scratch) {
+    __shared__ int far_[CH];
+    __shared__ unsigned char lab[2 * CH];
+    const int lane = threadIdx.x, k0 = blockIdx.x * CH, cnt = min(CH, n - k0);
+    for (int q = lane; q < 2 * CH; q += 32) lab[q] = (unsigned char)q;
+    for (int q = lane; q < CH; q += 32) far_[q] = -1;
+    int piv[CH / 32];
+#pragma unroll
+    for (int q = 0; q < CH / 32; ++q) piv[q] = lane + 32 * q < cnt ? ipiv[k0 + lane + 32 * q] - 1 : 0;
+    __syncwarp();
+    int nfar = 0;
+#pragma unroll
+    for (int q = 0; q < CH / 32; ++q)
+        for (int e = 0; e < 32; ++e) {
+            const int i = 32 * q + e;
+            if (i >= cnt) break;
+            const int p = __shfl_sync(0xffffffffu, piv[q], e);
+            int slot = p - k0;
+            if (slot < 0 || slot >= CH) {
+                slot = -1;
+#pragma unroll
+                for (int h = 0; h < CH / 32; ++h) {
+                    const unsigned hit = __ballot_sync(0xffffffffu, lane + 32 * h < nfar && far_[lane + 32 * h] == p);
+                    if (hit && slot < 0) slot = CH + 32 * h + __ffs(hit) - 1;
+                }
+                if (slot < 0) {
+                    if (lane == 0) far_[nfar] = p;
+                    slot = CH + nfar++;
+                    __syncwarp();
+                }
+            }
+            if (lane == 0 && slot != i) {
+                const unsigned char a = lab[i];
+                lab[i] = lab[slot];
+                lab[slot] = a;
+            }
+            __syncwarp();
+        }
+    unsigned char *out = scratch + (size_t)blockIdx.x * kChunkBytes;
+    for (int q = lane; q < cnt; q += 32) {
+        reinterpret_cast<int *>(out)[q] = far_[q];
+        out[4 * cnt + q] = lab[q];
+        out[5 * cnt + q] = lab[CH + q];
+    }
+}
+
+__global__ void __launch_bounds__(1024) k_compose_perm(int n, const unsigned char *__restrict__ scratch, int *perm,
+                                                       int use_smem) {
+    extern __shared__ int sp[];
+    int *p = use_smem ? sp : perm;
+    for (int i = threadIdx.x; i < n; i += 1024) p[i] = i;
+    const int nchunks = (n + CH - 1) / CH;
+    const int q = threadIdx.x;
+    __syncthreads();
+    int pos = -1, src = -1;
+    auto fetch = [&](int c) {           // this thread's place in chunk c and where its new content is
+        const unsigned char *ch = scratch + (size_t)c * kChunkBytes;
+        const int *far_ = reinterpret_cast<const int *>(ch);
+        const int cnt = min(CH, n - c * CH);
+        pos = src = -1;
+        if (q < 2 * CH && (q & (CH - 1)) < cnt) {
+            const int l = ch[(q < CH ? 4 : 5) * cnt + (q & (CH - 1))];
+            if (l != q) {
+                pos = q < CH ? c * CH + q : far_[q - CH];
+                src = l < CH ? c * CH + l : far_[l - CH];
+            }
+        }
+    };
+    fetch(0);
+    for (int c = 0; c < nchunks; ++c) {
+        const int at = pos, v = src >= 0 ? p[src] : 0;
+        __syncthreads();
+        if (at >= 0) p[at] = v;
+        if (c + 1 < nchunks) fetch(c + 1);
+        __syncthreads();
+    }
+    if (use_smem)
+        for (int i = threadIdx.x; i < n; i += 1024) perm[i] = p[i];
+}
+
+// Out[i, c] = In[perm[i], c]
+__global__ void k_gather_rows(int n, int nrhs, const int *perm, const double *In, int ldi, double *Out, int ldo) {
+    const size_t tot = (size_t)n * nrhs;
+    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < tot; e += (size_t)gridDim.x * blockDim.x) {
+        const int i = (int)(e % n), c = (int)(e / n);
+        Out[(size_t)i + (size_t)c * ldo] = In[(size_t)perm[i] + (size_t)c * ldi];
+    }
+}
+
+template <int MODE>
+static int solve_mode(int n, int nrhs, const double *T, int ldt, double *X, int ldx, cudaStream_t st) {
+    constexpr bool FWD = MODE == 0 || MODE == 2;
+    const size_t ld = (size_t)ldt;
+    CF_CUDA_TRY(cudaFuncSetAttribute(k_tri_solve64<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem)));
+    const int ns = ceil_div(n, kSuper);
+    for (int q = 0; q < ns; ++q) {
+        const int k0 = (FWD ? q : ns - 1 - q) * kSuper;
+        const int w = kSuper < n - k0 ? kSuper : n - k0;
+        for (int c0 = 0; c0 < nrhs; c0 += 65535) {
+            const int nc = nrhs - c0 < 65535 ? nrhs - c0 : 65535;
+            k_tri_solve64<MODE><<<dim3(CL, nc), kThreads, sizeof(Smem), st>>>(w, T + k0 + k0 * ld, ldt,
+                                                                            X + k0 + (size_t)c0 * ldx, ldx);
+            CF_LAUNCH_CHECK();
+        }
+        int rc = CF_OK;
+        if (FWD) {
+            const int r0 = k0 + w;
+            rc = launch_residual_f64(n - r0, w, nrhs, T + r0 + k0 * ld, ldt, X + k0, ldx, X + r0, ldx, X + r0, ldx, st);
+        } else if (MODE == 1) {
+            rc = launch_residual_f64(k0, w, nrhs, T + k0 * ld, ldt, X + k0, ldx, X, ldx, X, ldx, st);
+        } else if (k0 > 0) {
+            k_gemv_t_sub<<<ceil_div(k0, 8), 256, 0, st>>>(k0, w, nrhs, T + k0, ldt, X + k0, ldx, X, ldx);
+            CF_LAUNCH_CHECK();
+        }
+        if (rc) return rc;
+    }
+    return CF_OK;
+}
+
+}  // namespace sv
+
+int launch_tri_solve64(int mode, int n, int nrhs, const double *T, int ldt, double *X, int ldx, cudaStream_t st) {
+    if (n <= 0 || nrhs <= 0) return CF_OK;
+    switch (mode) {
+        case 0: return sv::solve_mode<0>(n, nrhs, T, ldt, X, ldx, st);
+        case 1: return sv::solve_mode<1>(n, nrhs, T, ldt, X, ldx, st);
+        case 2: return sv::solve_mode<2>(n, nrhs, T, ldt, X, ldx, st);
+        case 3: return sv::solve_mode<3>(n, nrhs, T, ldt, X, ldx, st);
+        default: return CF_ERR_UNSUPPORTED;
+    }
+}
+
+int launch_permute_rhs(int n, int nrhs, const int *ipiv, int *perm, const double *B, int ldb, double *T, cudaStream_t st) {
+    // the chunks' lists lie in T until the rows are gathered into it
+    const int nchunks = ceil_div(n, sv::CH);
+    unsigned char *scratch = reinterpret_cast<unsigned char *>(T);
+    sv::k_ipiv_chunks<<<nchunks, 32, 0, st>>>(n, ipiv, scratch);
+    CF_LAUNCH_CHECK();
+    const size_t smem = (size_t)n * sizeof(int) <= 200 * 1024 ? (size_t)n * sizeof(int) : 0;
+    if (smem > 48 * 1024)
+        CF_CUDA_TRY(cudaFuncSetAttribute(sv::k_compose_perm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    sv::k_compose_perm<<<1, 1024, smem, st>>>(n, scratch, perm, smem != 0);
+    CF_LAUNCH_CHECK();
+    const size_t tot = (size_t)n * nrhs;
+    const int blocks = tot < 1024 * 256 ? ceil_div((long long)tot, 256) : 1024;
+    sv::k_gather_rows<<<blocks, 256, 0, st>>>(n, nrhs, perm, B, ldb, T, n);
+    CF_LAUNCH_CHECK();
+    return CF_OK;
+}
+
+int solve64_take_status(cudaStream_t st, int *status) {
+    int h = 0;
+    CF_CUDA_TRY(cudaMemcpyFromSymbolAsync(&h, g_solve64_status, sizeof(int), 0, cudaMemcpyDeviceToHost, st));
+    CF_CUDA_TRY(cudaStreamSynchronize(st));
+    if (h != 0) {
+        const int zero = 0;
+        CF_CUDA_TRY(cudaMemcpyToSymbolAsync(g_solve64_status, &zero, sizeof(int), 0, cudaMemcpyHostToDevice, st));
+        CF_CUDA_TRY(cudaStreamSynchronize(st));
+    }
+    *status = h;
+    return CF_OK;
+}
+
+}  // namespace cf
