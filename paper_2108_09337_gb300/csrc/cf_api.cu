@@ -124,14 +124,17 @@ extern "C" size_t cf_getrf_workspace_size(int n, const cf_options *opt) {
     return tourn_ws_bytes(n > 0 ? n : 1, o.leaf_h, o.arity);
 }
 
-// The minimal workspace plus the digit slices of one step's operands, with
-// which the updates run on the tensor cores.
+// A00's LU and its flag.
+static constexpr size_t kLuBytes = sizeof(double) * kMaxV * kMaxV + 1024;
+
+// The minimal workspace plus A00's LU as the tournament leaves it and the digit
+// slices of one step's operands, with which the updates run on the tensor cores.
 extern "C" size_t cf_getrf_optimal_workspace_size(int n, const cf_options *opt) {
     const size_t base = cf_getrf_workspace_size(n, opt);
     Opts o;
     if (base == 0 || resolve_options(opt, &o) != CF_OK) return 0;
-    if (o.v < kSliceMinW || n <= o.v) return base;
-    return align_up(base, 1024) + slice64_bytes(n - o.v, n - o.v);
+    const size_t head = align_up(base, 1024) + kLuBytes;
+    return o.v < kSliceMinW || n <= o.v ? head : head + slice64_bytes(n - o.v, n - o.v);
 }
 
 // LU-6 look-ahead (FP64 path).  Step t runs its panel chain (TournPivot,
@@ -195,10 +198,10 @@ static int getrf_lookahead(int n, double *A, int lda, int *ipiv, int *info, cons
         double *A00 = A + k0 + k0 * ld;
         ep.ipiv = ipiv;
         ep.k0 = k0;
-        if ((rc = launch_tourn<double>(A00, lda, m, w, o.leaf_h, o.arity, ws, ep, sp))) return fail(rc);
+        if ((rc = launch_tourn(A00, lda, m, w, o.leaf_h, o.arity, ws, ep, sp))) return fail(rc);
         if (rest_pending && (rc = L.wait_update())) return fail(rc);
         if ((rc = launch_apply_swaps<double>(A, lda, n, k0, ep, nullptr, sp))) return fail(rc);
-        if ((rc = launch_getf2_nopiv<double>(A00, lda, w, k0, info, sp))) return fail(rc);
+        if ((rc = launch_getf2_nopiv(A00, lda, w, k0, info, ep.lu, ep.lu_ok, sp))) return fail(rc);
         if ((rc = launch_trsm_right_upper<double>(A00 + w, lda, m - w, w, A00, lda, false, nullptr, sp)))
             return fail(rc);
         if ((rc = launch_trsm_left_lower_unit<double>(A00 + w * ld, lda, w, n - k0 - w, A00, lda, sp)))
@@ -314,9 +317,13 @@ extern "C" int cf_getrf(int n, double *A, int lda, int *ipiv, int *info, void *w
     Slice64 slices;
     const Slice64 *sl = nullptr;
     const size_t base = align_up(cf_getrf_workspace_size(n, opt), 1024);
-    if (o.v >= kSliceMinW && n > o.v && lwork >= cf_getrf_optimal_workspace_size(n, opt)) {
-        slices = slice64_carve((char *)work + base, n - o.v, n - o.v);
-        sl = &slices;
+    if (lwork >= cf_getrf_optimal_workspace_size(n, opt)) {
+        ep.lu_ok = (int *)((char *)work + base);
+        ep.lu = (double *)((char *)work + base + 1024);
+        if (o.v >= kSliceMinW && n > o.v) {
+            slices = slice64_carve((char *)work + base + kLuBytes, n - o.v, n - o.v);
+            sl = &slices;
+        }
     }
     if (o.lookahead) return getrf_lookahead(n, A, lda, ipiv, info, o, ws, ep, sl, st);
     const size_t ld = (size_t)lda;
@@ -327,11 +334,11 @@ extern "C" int cf_getrf(int n, double *A, int lda, int *ipiv, int *info, void *w
         ep.ipiv = ipiv;
         ep.k0 = k0;
         // LU-1 TournPivot on A[k0:n, k0:k0+w]
-        if ((rc = launch_tourn<double>(A00, lda, m, w, o.leaf_h, o.arity, ws, ep, st))) return rc;
+        if ((rc = launch_tourn(A00, lda, m, w, o.leaf_h, o.arity, ws, ep, st))) return rc;
         // LU-2 interchanges on all n columns
         if ((rc = launch_apply_swaps<double>(A, lda, n, k0, ep, nullptr, st))) return rc;
         // A00 = L00 U00 (no further pivoting)
-        if ((rc = launch_getf2_nopiv<double>(A00, lda, w, k0, info, st))) return rc;
+        if ((rc = launch_getf2_nopiv(A00, lda, w, k0, info, ep.lu, ep.lu_ok, st))) return rc;
         // LU-3 A10 <- A10 U00^{-1}
         if ((rc = launch_trsm_right_upper<double>(A00 + w, lda, m - w, w, A00, lda, false, nullptr, st))) return rc;
         // LU-4 A01 <- L00^{-1} A01

@@ -36,22 +36,27 @@ struct TournEpilogue {
     int *swap_cnt;            // [1] number of moved rows
     int *swap_dst;            // [2*kMaxV] destination positions (relative to k0)
     int *swap_src;            // [2*kMaxV] source positions (relative to k0)
+    // FP64 tournament, optional: the LU of A00 (ld kMaxV) as the root's
+    // elimination leaves it; lu_ok = 0 where a pivot was exactly zero, whose
+    // step launch_getf2_nopiv takes differently
+    double *lu = nullptr;
+    int *lu_ok = nullptr;
 };
 
 int make_tourn_plan(int m, int w, int h, int arity, TournPlan *plan);
 size_t tourn_ws_bytes(int m, int h, int arity);
 int tourn_ws_carve(void *work, int m, int h, int arity, TournWS *ws, TournEpilogue *ep);
 
-template <typename T>
-int launch_tourn(const T *P, int ldp, int m, int w, int h, int arity, const TournWS &ws, const TournEpilogue &ep,
+int launch_tourn(const double *P, int ldp, int m, int w, int h, int arity, const TournWS &ws, const TournEpilogue &ep,
                  cudaStream_t st);
 template <typename T>
 int launch_apply_swaps(T *A, int lda, int ncols, int k0, const TournEpilogue &ep, int *perm, cudaStream_t st);
 
 // ---- panel kernels (cf_panel.cu)
-// LU of the w x w diagonal block without pivoting (Fig. "prog_rep").
-template <typename T>
-int launch_getf2_nopiv(T *A00, int lda, int w, int kglob, int *info, cudaStream_t st);
+// LU of the w x w diagonal block without pivoting (Fig. "prog_rep"); with
+// lu / lu_ok of the tournament's epilogue only copied where *lu_ok.
+int launch_getf2_nopiv(double *A00, int lda, int w, int kglob, int *info, const double *lu, const int *lu_ok,
+                       cudaStream_t st);
 // A10 <- A10 * U^{-1}: rows x w block X, U upper non-unit w x w (or, with
 // trans_lower, U = L^T for a lower L).  Optional low-precision copy of the
 // result, K-major: lp[(r) * ldlp + c].

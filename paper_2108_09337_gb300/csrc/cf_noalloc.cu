@@ -73,6 +73,12 @@ extern "C" int cf_getrf_noalloc(int n, double *A, int lda, int *ipiv, int *info,
     // The array keeps whatever the previous call left: the arrival counters
     // must start at zero.
     CF_CUDA_TRY(cudaMemsetAsync(ws.counter, 0, ws.counter_bytes, st));
+    // A00's LU beside the tournament's part, where the array has room for it
+    const size_t used = align_up(tourn_ws_bytes(n, o.leaf_h, o.arity), 256);
+    if (used + 256 + sizeof(double) * kMaxV * kMaxV <= kNoAllocScratchBytes) {
+        ep.lu_ok = (int *)((char *)scratch + used);
+        ep.lu = (double *)((char *)scratch + used + 256);
+    }
     const size_t ld = (size_t)lda;
     for (int k0 = 0; k0 < n; k0 += o.v) {
         const int w = o.v < n - k0 ? o.v : n - k0;
@@ -80,9 +86,9 @@ extern "C" int cf_getrf_noalloc(int n, double *A, int lda, int *ipiv, int *info,
         double *A00 = A + k0 + k0 * ld;
         ep.ipiv = ipiv;
         ep.k0 = k0;
-        if ((rc = launch_tourn<double>(A00, lda, m, w, o.leaf_h, o.arity, ws, ep, st))) return rc;
+        if ((rc = launch_tourn(A00, lda, m, w, o.leaf_h, o.arity, ws, ep, st))) return rc;
         if ((rc = launch_apply_swaps<double>(A, lda, n, k0, ep, nullptr, st))) return rc;
-        if ((rc = launch_getf2_nopiv<double>(A00, lda, w, k0, info, st))) return rc;
+        if ((rc = launch_getf2_nopiv(A00, lda, w, k0, info, ep.lu, ep.lu_ok, st))) return rc;
         if ((rc = launch_trsm_right_upper<double>(A00 + w, lda, m - w, w, A00, lda, false, nullptr, st))) return rc;
         if ((rc = launch_trsm_left_lower_unit<double>(A00 + w * ld, lda, w, n - k0 - w, A00, lda, st))) return rc;
         const int right = n - k0 - w;

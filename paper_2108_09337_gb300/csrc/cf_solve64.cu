@@ -442,7 +442,7 @@ int launch_permute_rhs(int n, int nrhs, const int *ipiv, int *perm, const double
     CF_LAUNCH_CHECK();
     const size_t smem = (size_t)n * sizeof(int) <= 200 * 1024 ? (size_t)n * sizeof(int) : 0;
     if (smem > 48 * 1024)
-        CF_CUDA_TRY(cudaFuncSetAttribute(sv::k_compose_perm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        CF_CUDA_TRY(cudaFuncSetAttribute(sv::k_compose_perm, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     sv::k_compose_perm<<<1, 1024, smem, st>>>(n, scratch, perm, smem != 0);
     CF_LAUNCH_CHECK();
     const size_t tot = (size_t)n * nrhs;

@@ -2,21 +2,32 @@
 // Pivoting" and "Pivoting in COnfLUX"; the pivot selection in the I/O-cost proof) and
 // LU-2: the row interchanges that bring the winners to the top.
 //
-// GPU design.  One launch runs a whole tournament.  A thread-block cluster of
-// `arity` CTAs is the unit of work: in the leaf phase each CTA eliminates its
-// own leaf (h consecutive panel rows) in shared memory; in a playoff node the
-// cluster's CTAs each hold one child's candidate rows (original panel values)
-// and eliminate them together, exchanging the per-column argmax through
-// distributed shared memory (one cluster barrier per column).  The cluster
-// that finishes a node last (atomic counter, no spinning) climbs to the
-// parent, so no CTA ever waits for another; the root cluster writes the
-// winners, the LAPACK ipiv and the list of moved rows.
+// GPU design.  One launch per level of the tree: a node (a leaf's rows, or the
+// stacked winners of `arity` children, with their original panel values) is a
+// thread-block cluster of 1 to 16 CTAs that hold its rows in shared memory in
+// equal shares.  The elimination is bound by the FP64 pipe (an element's
+// multiply and subtract take 128 clocks of a quarter SM per 32 lanes), so the
+// cluster size is chosen to put a level on as many SMs as it has: 16 leaves of
+// a 2048-row panel run on 128 SMs, 16 rows each.  Per column:
+//   * the threads that own a row divide by the pivot, update the next column
+//     and take its argmax (redux on the key's bits), which goes straight into
+//     every CTA's slots through distributed shared memory;
+//   * all threads update the other columns, element by element over the rows
+//     still in the race (a list, so that chosen rows cost nothing);
+//   * one cluster barrier; then every warp finds the winner from the slots and
+//     pulls the pivot row from its owner while the multipliers are divided.
+// The eliminated rows of the root's winners are A00's LU, which the root hands
+// to the driver (TournEpilogue::lu).
+//
+// A 2048-row, 128-column panel: 1.0 ms for its three levels (2.5 with one CTA per
+// leaf and all levels in one launch), an 8192-row one 1.9 (3.2).
 //
 // Every elimination step uses separately rounded multiply and subtract and
 // an IEEE division, in the same order as the FP64 oracle, so a tournament on
 // the same panel bytes picks the same pivots bit for bit.
 #include <cooperative_groups.h>
 
+#include <atomic>
 #include <climits>
 
 #include "cf_common.cuh"
@@ -27,268 +38,251 @@ namespace cg = cooperative_groups;
 namespace cf {
 
 constexpr int kTournThreads = 256;
+constexpr int kTournMaxCluster = 16;
 
-template <typename T>
 struct TournSmem {
-    T tile[kMaxV * kMaxV];      // column-major, ld kMaxV: tile[k*kMaxV + r]
-    T prow[kMaxV];              // pivot row of the current column
-    T redv[kTournThreads / 32];
-    int redi[kTournThreads / 32];
-    T slotv[2];                 // this CTA's argmax, by column parity
-    int sloti[2];
-    int used[kMaxV];
-    int order[kMaxV];
-    int rows[kMaxV];            // panel row of each tile row
-    int nrows;
-    int cont;
-    int lab_at[2 * kMaxV];      // root epilogue: swap simulation
+    double prow[kMaxV];                          // pivot row from the current column on
+    double mult[kMaxV];                          // multiplier of each row
+    double slotv[2][4 * kTournMaxCluster];       // candidates of every CTA's warps, by column parity
+    int sloti[2][4 * kTournMaxCluster];          // their stacked positions (-1: none)
+    int act[kMaxV];                              // this CTA's rows still in the race
+    int rows[kMaxV];                             // panel row of each tile row
+    int order[kMaxV];                            // stacked position of each pivot
+    int nact;
+    int hole;                                    // place of the chosen row in act
+    int lab_at[2 * kMaxV];                       // root epilogue: swap simulation
     int where_[2 * kMaxV];
+    int win[kMaxV];
+    int cnt;
+    int bad;
 };
 
-// Key of the argmax: |a|, with NaN ranked below every number but above "no
-// candidate" (-1), exactly as the oracle ranks it.
-template <typename T>
-__device__ __forceinline__ T piv_key(T a) {
-    T x = fabs(a);
-    return (x != x) ? T(-0.5) : x;
+// Rank of a candidate as an unsigned key: |a| by its bits, NaN below every
+// number but above "no candidate" (0), exactly as the oracle ranks it.
+__device__ __forceinline__ unsigned long long piv_key(double a) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(a) & 0x7FFFFFFFFFFFFFFFull;
+    return b > 0x7FF0000000000000ull ? 1ull : b + 2ull;
 }
 
-template <typename T>
-__device__ __forceinline__ void better(T &bv, int &bi, T ov, int oi) {
-    if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
+// Warp maximum of (key, smallest position); every lane gets the position (-1: none).
+__device__ __forceinline__ int warp_best(unsigned long long key, int pos) {
+    const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+    const bool top = hi == mh && lo == ml && key != 0;
+    return (int)__reduce_min_sync(0xffffffffu, top ? (unsigned)pos : 0xffffffffu);
 }
 
-// Masked partial-pivoting selection on the stacked rows held by the CTAs of
-// the cluster (CLUSTERED) or by this CTA alone.  Stacked index of a row =
-// rank * kMaxV + tile row (clustered) or tile row.  Leaves s.order[0..npiv)
-// identical in every participating CTA.
-template <typename T, bool CLUSTERED, int CL>
-__device__ void gepp_select(TournSmem<T> &s, int w, int npiv, int rank) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int base = CLUSTERED ? rank * kMaxV : 0;
-    const int r = tid & (kMaxV - 1);
-    const int half = tid / kMaxV;      // 0 or 1
-    cg::cluster_group cl = cg::this_cluster();
-    for (int j = 0; j < npiv; ++j) {
-        // (1) local argmax of column j over the unused rows.
-        T bv = T(-1);
-        int bi = INT_MAX;
-        if (tid < kMaxV && tid < s.nrows && !s.used[tid]) {
-            bv = piv_key(s.tile[j * kMaxV + tid]);
-            bi = base + tid;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            T ov = __shfl_xor_sync(0xffffffffu, bv, o);
-            int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-            better(bv, bi, ov, oi);
-        }
-        if (lane == 0) { s.redv[warp] = bv; s.redi[warp] = bi; }
-        __syncthreads();
-        if (tid == 0) {
-            T v = s.redv[0];
-            int i = s.redi[0];
-#pragma unroll
-            for (int q = 1; q < kMaxV / 32; ++q) better(v, i, s.redv[q], s.redi[q]);
-            s.slotv[j & 1] = v;
-            s.sloti[j & 1] = i;
-        }
-        if (CLUSTERED) cl.sync(); else __syncthreads();
-        // (2) winner over the cluster (same comparison order everywhere).
-        T gv = T(-1);
-        int gi = INT_MAX;
-        if (CLUSTERED) {
-#pragma unroll
-            for (int q = 0; q < CL; ++q) {
-                TournSmem<T> *rs = cl.map_shared_rank(&s, q);
-                better(gv, gi, rs->slotv[j & 1], rs->sloti[j & 1]);
-            }
-        } else {
-            gv = s.slotv[j & 1];
-            gi = s.sloti[j & 1];
-        }
-        const int owner = CLUSTERED ? gi / kMaxV : rank;
-        const int lrow = CLUSTERED ? gi % kMaxV : gi;
-        // (3) pivot row into local prow; the owner marks the row used.  The
-        // owner's row is final (used rows are never updated again).
-        {
-            TournSmem<T> *os = CLUSTERED ? cl.map_shared_rank(&s, owner) : &s;
-            for (int k = j + tid; k < w; k += kTournThreads) s.prow[k] = os->tile[k * kMaxV + lrow];
-        }
-        if (tid == 0) {
-            s.order[j] = gi;
-            if (owner == rank) s.used[lrow] = 1;
-        }
-        __syncthreads();
-        // (4) eliminate column j from the unused rows.  Column j+1 of row r is
-        // updated by thread r itself (half 0), which is also the thread that
-        // reads it in the next argmax, so no barrier is needed here.
-        const T piv = s.prow[j];
-        if (piv != T(0) && r < s.nrows && !s.used[r]) {
-            const T l = div_rn(s.tile[j * kMaxV + r], piv);
-            for (int k = j + 1 + half; k < w; k += 2)
-                s.tile[k * kMaxV + r] = sub_rn(s.tile[k * kMaxV + r], mul_rn(l, s.prow[k]));
-        }
-    }
-    if (CLUSTERED) cl.sync(); else __syncthreads();
-}
+// Shared memory of the largest share (128 rows x 128 columns): the limit that
+// is set for every launch, whatever the launch takes.
+constexpr size_t kTournMaxSmem = ((sizeof(TournSmem) + 15) & ~(size_t)15) + sizeof(double) * (kMaxV + 1) * kMaxV;
 
-template <typename T>
-__device__ void load_rows(TournSmem<T> &s, const T *__restrict__ P, int ldp, int w, int nrows) {
-    for (int idx = threadIdx.x; idx < kMaxV * w; idx += kTournThreads) {
-        const int k = idx / kMaxV, i = idx % kMaxV;
-        if (i < nrows) s.tile[k * kMaxV + i] = P[(size_t)s.rows[i] + (size_t)k * ldp];
-    }
-    for (int i = threadIdx.x; i < kMaxV; i += kTournThreads) s.used[i] = (i < nrows) ? 0 : 1;
-}
+struct TournLevel {
+    const double *P;
+    int ldp, m, w, h, arity, level, root;
+    int cnt_below, off_below, off;               // nodes of the level below, first node indexes
+    int per, ld;                                 // rows per CTA at most; leading dimension of the tile (odd)
+};
 
 // Root epilogue: LAPACK ipiv and the list of moved rows (relative positions)
 // for bringing the winners, in pivot order, to positions 0..w-1.
-template <typename T>
-__device__ void root_epilogue(TournSmem<T> &s, const int *win, int np, const TournEpilogue &ep) {
-    if (ep.ipiv == nullptr) return;
-    if (threadIdx.x != 0) return;
-    const int w = np;
+__device__ void root_epilogue(TournSmem &s, int w, const TournEpilogue &ep) {
     // Home slot of a label: labels < w live in slot == label; the label of
     // a winner j with win[j] >= w lives in slot w + j.
-    for (int q = 0; q < 2 * w; ++q) { s.lab_at[q] = q; s.where_[q] = q; }
-    for (int j = 0; j < w; ++j) {
-        const int hj = win[j] < w ? win[j] : w + j;
-        const int ps = s.where_[hj];
-        const int p = ps < w ? ps : win[ps - w];
-        ep.ipiv[ep.k0 + j] = ep.k0 + p + 1;
-        if (ps != j) {
-            const int hx = s.lab_at[j];
-            s.lab_at[j] = hj; s.where_[hj] = j;
-            s.lab_at[ps] = hx; s.where_[hx] = ps;
+    for (int q = threadIdx.x; q < 2 * w; q += kTournThreads) { s.lab_at[q] = q; s.where_[q] = q; }
+    if (threadIdx.x == 0) s.cnt = 0;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int j = 0; j < w; ++j) {
+            const int hj = s.win[j] < w ? s.win[j] : w + j;
+            const int ps = s.where_[hj];
+            const int p = ps < w ? ps : s.win[ps - w];
+            ep.ipiv[ep.k0 + j] = ep.k0 + p + 1;
+            if (ps != j) {
+                const int hx = s.lab_at[j];
+                s.lab_at[j] = hj; s.where_[hj] = j;
+                s.lab_at[ps] = hx; s.where_[hx] = ps;
+            }
         }
     }
-    int cnt = 0;
-    for (int q = 0; q < 2 * w; ++q) {
-        if (s.lab_at[q] == q) continue;
+    __syncthreads();
+    for (int q = threadIdx.x; q < 2 * w; q += kTournThreads) {
         const int hq = s.lab_at[q];
-        ep.swap_dst[cnt] = q < w ? q : win[q - w];
-        ep.swap_src[cnt] = hq < w ? hq : win[hq - w];
-        ++cnt;
+        if (hq == q) continue;
+        const int at = atomicAdd(&s.cnt, 1);     // any order: the interchanges are applied as one gather
+        ep.swap_dst[at] = q < w ? q : s.win[q - w];
+        ep.swap_src[at] = hq < w ? hq : s.win[hq - w];
     }
-    *ep.swap_cnt = cnt;
+    __syncthreads();
+    if (threadIdx.x == 0) *ep.swap_cnt = s.cnt;
 }
 
-template <typename T, int CL>
 __global__ void __launch_bounds__(kTournThreads, 1)
-k_tourn(const T *__restrict__ P, int ldp, TournPlan plan, TournWS ws, TournEpilogue ep) {
+k_tourn_level(TournLevel lv, TournWS ws, TournEpilogue ep) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    TournSmem<T> &s = *reinterpret_cast<TournSmem<T> *>(smem_raw);
+    TournSmem &s = *reinterpret_cast<TournSmem *>(smem_raw);
+    double *tile = reinterpret_cast<double *>(smem_raw + ((sizeof(TournSmem) + 15) & ~(size_t)15));   // [column][row], ld odd
     cg::cluster_group cl = cg::this_cluster();
-    const int rank = (CL > 1) ? (int)cl.block_rank() : 0;
-    const int c = blockIdx.x / CL;
-    const int tid = threadIdx.x;
-    const int w = plan.w;
+    const int rank = (int)cl.block_rank(), ncta = (int)cl.num_blocks();
+    const int g = blockIdx.x / ncta;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int w = lv.w, ld = lv.ld;
+    int *dst = ws.node_win + (size_t)(lv.off + g) * kMaxV;
 
-    // ---- leaves
-    const int leaf = c * CL + rank;
-    if (leaf < plan.nleaves) {
-        const int row0 = leaf * plan.h;
-        const int nr = min(plan.h, plan.m - row0);
-        for (int i = tid; i < kMaxV; i += kTournThreads) s.rows[i] = row0 + i;
-        if (tid == 0) s.nrows = nr;
+    // ---- this CTA's rows: stacked positions [rank * per, rank * per + mine)
+    const int p0 = rank * lv.per;
+    int total = 0, mine = 0;
+    if (lv.level == 0) {
+        total = min(lv.h, lv.m - g * lv.h);
+        mine = max(0, min(lv.per, total - p0));
+        if (tid < mine) s.rows[tid] = g * lv.h + p0 + tid;
+    } else {
+        const int child0 = g * lv.arity, nchild = min(lv.arity, lv.cnt_below - child0);
+        if (nchild == 1) {                       // pass-through
+            const int src = lv.off_below + child0, np = ws.node_cnt[src];
+            if (rank == 0) {
+                for (int j = tid; j < np; j += kTournThreads) dst[j] = ws.node_win[(size_t)src * kMaxV + j];
+                if (tid == 0) ws.node_cnt[lv.off + g] = np;
+            }
+            return;
+        }
+        int at = -1, base = 0;
+        for (int q = 0; q < nchild; ++q) {
+            const int c = ws.node_cnt[lv.off_below + child0 + q];
+            if (p0 + tid >= base && p0 + tid < base + c)
+                at = (lv.off_below + child0 + q) * kMaxV + (p0 + tid - base);
+            base += c;
+        }
+        total = base;
+        mine = max(0, min(lv.per, total - p0));
+        if (tid < mine) s.rows[tid] = ws.node_win[at];
+    }
+    if (tid < kMaxV) s.act[tid] = tid;
+    if (tid == 0) { s.nact = mine; s.bad = 0; }
+    __syncthreads();
+    for (int k = warp; k < w; k += kTournThreads / 32)
+        for (int r = lane; r < mine; r += 32) tile[k * ld + r] = lv.P[(size_t)s.rows[r] + (size_t)k * lv.ldp];
+    __syncthreads();
+    const int npiv = min(total, w);
+    const int nslots = 4 * ncta;
+
+    // Candidate of this warp's rows in one column, into every CTA's slots.
+    auto publish = [&](int par, bool have, double a, int row) {
+        const int best = warp_best(have ? piv_key(a) : 0ull, p0 + row);
+        const unsigned owner = __ballot_sync(0xffffffffu, have && p0 + row == best);
+        const double v = __shfl_sync(0xffffffffu, a, owner ? __ffs(owner) - 1 : 0);
+        if (lane < ncta) {
+            TournSmem *rs = cl.map_shared_rank(&s, lane);
+            rs->slotv[par][rank * 4 + warp] = v;
+            rs->sloti[par][rank * 4 + warp] = best;
+        }
+    };
+    if (ncta > 1) cl.sync();                     // every CTA of the cluster runs before it is written to
+    if (warp < 4) publish(0, tid < mine, tid < mine ? tile[tid] : 0.0, tid);
+
+    for (int j = 0; j < npiv; ++j) {
+        if (ncta > 1) cl.sync(); else __syncthreads();
+        // ---- (1) the winner, found by every warp alike
+        const int par = j & 1;
+        int gi;
+        double piv;
+        {
+            const int i0 = lane < nslots ? s.sloti[par][lane] : -1, i1 = lane + 32 < nslots ? s.sloti[par][lane + 32] : -1;
+            const double v0 = i0 >= 0 ? s.slotv[par][lane] : 0.0, v1 = i1 >= 0 ? s.slotv[par][lane + 32] : 0.0;
+            const unsigned long long k0 = i0 >= 0 ? piv_key(v0) : 0ull, k1 = i1 >= 0 ? piv_key(v1) : 0ull;
+            const bool second = k1 > k0 || (k1 == k0 && k1 != 0 && i1 < i0);
+            gi = warp_best(second ? k1 : k0, second ? i1 : i0);
+            const unsigned owner = __ballot_sync(0xffffffffu, (i0 == gi || i1 == gi) && gi >= 0);
+            piv = __shfl_sync(0xffffffffu, i1 == gi ? v1 : v0, owner ? __ffs(owner) - 1 : 0);
+        }
+        const int owner = gi / lv.per, lrow = gi - owner * lv.per;
+        // ---- (2) pivot row from its owner; meanwhile the multipliers
+        double pr = 0.0;
+        const bool pull = tid < w - j;
+        if (pull) {
+            const double *src = ncta > 1 ? cl.map_shared_rank(tile, owner) : tile;
+            pr = src[(size_t)(j + tid) * ld + lrow];
+        }
+        const int nact = s.nact;
+        const bool mine_won = owner == rank;
+        int row = -1;
+        double l = 0.0;
+        if (tid < nact) {
+            row = s.act[tid];
+            if (mine_won && row == lrow) {
+                s.hole = tid;
+                row = -1;
+            }
+            if (row >= 0 && piv != 0.0) {
+                l = div_rn(tile[j * ld + row], piv);
+                tile[j * ld + row] = l;
+                s.mult[row] = l;
+            }
+        }
+        if (pull) s.prow[j + tid] = pr;
+        if (tid == 0) s.order[j] = gi;
+        if (piv == 0.0 && tid == 0) s.bad = 1;
         __syncthreads();
-        load_rows(s, P, ldp, w, nr);
+        const int jn = j + 1;
+        // ---- (3) the next column and its candidates; the chosen row leaves the list
+        if (mine_won && tid == kTournThreads - 1) {
+            s.act[s.hole] = s.act[nact - 1];
+            s.nact = nact - 1;
+        }
+        if (warp < 4 && jn < npiv) {
+            double a = 0.0;
+            if (row >= 0) {
+                a = tile[jn * ld + row];
+                if (piv != 0.0) {
+                    a = sub_rn(a, mul_rn(l, s.prow[jn]));
+                    tile[jn * ld + row] = a;
+                }
+            }
+            publish(jn & 1, row >= 0, a, row);
+        } else if (row >= 0 && jn < w && piv != 0.0) {       // the last pivot of a node with fewer rows than columns
+            tile[jn * ld + row] = sub_rn(tile[jn * ld + row], mul_rn(l, s.prow[jn]));
+        }
         __syncthreads();
-        const int np = min(nr, w);
-        gepp_select<T, false, CL>(s, w, np, rank);
-        int *dst = ws.node_win + (size_t)(plan.off[0] + leaf) * kMaxV;
-        for (int j = tid; j < np; j += kTournThreads) dst[j] = s.rows[s.order[j]];
-        if (tid == 0) ws.node_cnt[plan.off[0] + leaf] = np;
-        if (plan.nlevels == 1) {          // a single leaf is the root
-            __syncthreads();
-            for (int j = tid; j < np; j += kTournThreads) ws.root_win[j] = dst[j];
-            __threadfence();
-            __syncthreads();
-            root_epilogue(s, dst, np, ep);
+        // ---- (4) the other columns
+        if (piv != 0.0) {
+            const int na = s.nact, tot = na * (w - jn - 1);
+            const unsigned inv = na > 1 ? 0xFFFFFFFFu / (unsigned)na + 1u : 0u;
+#pragma unroll 4
+            for (int e = tid; e < tot; e += kTournThreads) {
+                const int c = na > 1 ? (int)__umulhi((unsigned)e, inv) : e;      // e / na
+                const int r = s.act[e - c * na];
+                const int k = jn + 1 + c;
+                tile[k * ld + r] = sub_rn(tile[k * ld + r], mul_rn(s.mult[r], s.prow[k]));
+            }
         }
     }
-    if (plan.nlevels == 1) {
-        if (CL > 1) cl.sync();
-        return;
+    __syncthreads();
+    for (int j = tid; j < npiv; j += kTournThreads) {
+        const int gi = s.order[j];
+        if (gi / lv.per == rank) {
+            const int r = s.rows[gi - rank * lv.per];
+            dst[j] = r;
+            if (lv.root) ws.root_win[j] = r;
+        }
+    }
+    if (rank == 0 && tid == 0) ws.node_cnt[lv.off + g] = npiv;
+    if (lv.root && ep.lu != nullptr) {
+        // the winners' eliminated rows are the LU of A00 in pivot order
+        for (int j = warp; j < npiv; j += kTournThreads / 32) {
+            const int gi = s.order[j];
+            if (gi / lv.per != rank) continue;
+            for (int k = lane; k < w; k += 32) ep.lu[j + (size_t)k * kMaxV] = tile[k * ld + (gi - rank * lv.per)];
+        }
+        if (rank == 0 && tid == 0) *ep.lu_ok = s.bad == 0 && npiv == w;
     }
     __threadfence();
-    if (CL > 1) cl.sync(); else __syncthreads();
-
-    // ---- playoff nodes: level 1 node c has exactly this cluster's leaves.
-    int level = 1, g = c;
-    while (true) {
-        const int child0 = g * CL;
-        const int nchild = min(CL, plan.cnt[level - 1] - child0);
-        const int node = plan.off[level] + g;
-        int *dst = ws.node_win + (size_t)node * kMaxV;
-        int np;
-        if (nchild == 1) {                // pass-through
-            const int src = plan.off[level - 1] + child0;
-            np = __ldcg(ws.node_cnt + src);
-            if (rank == 0) {
-                for (int j = tid; j < np; j += kTournThreads) dst[j] = __ldcg(ws.node_win + (size_t)src * kMaxV + j);
-                if (tid == 0) ws.node_cnt[node] = np;
-            }
-        } else {
-            int total = 0;
-            for (int q = 0; q < nchild; ++q) total += __ldcg(ws.node_cnt + plan.off[level - 1] + child0 + q);
-            np = min(total, w);
-            int nr = 0;
-            if (rank < nchild) {
-                const int src = plan.off[level - 1] + child0 + rank;
-                nr = __ldcg(ws.node_cnt + src);
-                for (int i = tid; i < nr; i += kTournThreads) s.rows[i] = __ldcg(ws.node_win + (size_t)src * kMaxV + i);
-            }
-            if (tid == 0) s.nrows = nr;
-            __syncthreads();
-            load_rows(s, P, ldp, w, nr);
-            __syncthreads();
-            if (CL > 1) gepp_select<T, true, CL>(s, w, np, rank);
-            else gepp_select<T, false, CL>(s, w, np, rank);
-            if (rank == 0) {
-                for (int j = tid; j < np; j += kTournThreads) {
-                    const int gi = s.order[j];
-                    const int owner = (CL > 1) ? gi / kMaxV : 0;
-                    const int lr = (CL > 1) ? gi % kMaxV : gi;
-                    const TournSmem<T> *os = (CL > 1) ? cl.map_shared_rank(&s, owner) : &s;
-                    dst[j] = os->rows[lr];
-                }
-                if (tid == 0) ws.node_cnt[node] = np;
-            }
-        }
-        __threadfence();
-        if (CL > 1) cl.sync(); else __syncthreads();
-        if (level == plan.nlevels - 1) {  // root
-            if (rank == 0) {
-                for (int j = tid; j < np; j += kTournThreads) ws.root_win[j] = dst[j];
-                __syncthreads();
-                root_epilogue(s, dst, np, ep);
-            }
-            break;
-        }
-        // Climb: the last child to finish continues with the parent.
-        const int parent = g / CL;
-        if (rank == 0 && tid == 0) {
-            const int pnode = plan.off[level + 1] + parent;
-            const int pch = min(CL, plan.cnt[level] - parent * CL);
-            const int old = atomicAdd(ws.counter + pnode, 1);
-            const int cont = (old == pch - 1);
-            if (cont) ws.counter[pnode] = 0;   // leave the counter clean
-            __threadfence();
-            if (CL > 1) {
-                for (int q = 0; q < CL; ++q) cl.map_shared_rank(&s, q)->cont = cont;
-            } else {
-                s.cont = cont;
-            }
-        }
-        if (CL > 1) cl.sync(); else __syncthreads();
-        if (!s.cont) break;
-        __threadfence();
-        ++level;
-        g = parent;
+    if (ncta > 1) cl.sync();                     // remote reads of the tiles and the winners' list are done
+    if (lv.root && rank == 0 && ep.ipiv != nullptr) {
+        __syncthreads();
+        for (int j = tid; j < npiv; j += kTournThreads) s.win[j] = __ldcg(ws.root_win + j);
+        __syncthreads();
+        root_epilogue(s, npiv, ep);
     }
-    if (CL > 1) cl.sync();
 }
 
 // LU-2: gather the moved rows of every column (one warp per column) and the
@@ -387,49 +381,93 @@ int tourn_ws_carve(void *work, int m, int h, int arity, TournWS *ws, TournEpilog
     return CF_OK;
 }
 
-template <typename T, int CL>
-static int launch_tourn_cl(const T *P, int ldp, const TournPlan &plan, const TournWS &ws, const TournEpilogue &ep,
-                           cudaStream_t st) {
-    const size_t smem = sizeof(TournSmem<T>);
-    // The attribute belongs to the current device: set it on every call (a
-    // flag kept per process would skip it on the second device).
-    CF_CUDA_TRY(cudaFuncSetAttribute(k_tourn<T, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const int nclusters = ceil_div(plan.nleaves, CL);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(nclusters * CL);
-    cfg.blockDim = dim3(kTournThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = CL;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    CF_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_tourn<T, CL>, P, ldp, plan, ws, ep));
-    count_launches(1);
-    return CF_OK;
+// Largest cluster of the level kernel that the device takes: 16 (not
+// portable) where some GPC has 16 SMs to give, else 8.
+static int tourn_max_cluster() {
+    constexpr int kDevs = 64;
+    static std::atomic<int> cache[kDevs];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevs) {
+        cudaGetLastError();
+        return 8;
+    }
+    int n = cache[dev].load(std::memory_order_relaxed);
+    if (n > 0) return n;
+    n = 8;
+    if (cudaFuncSetAttribute(k_tourn_level, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(kTournMaxCluster);
+        cfg.blockDim = dim3(kTournThreads);
+        cfg.dynamicSmemBytes = kTournMaxSmem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = kTournMaxCluster;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int clusters = 0;
+        if (cudaFuncSetAttribute(k_tourn_level, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTournMaxSmem) ==
+                cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&clusters, k_tourn_level, &cfg) == cudaSuccess && clusters > 0)
+            n = kTournMaxCluster;
+    }
+    cudaGetLastError();
+    cache[dev].store(n, std::memory_order_relaxed);
+    return n;
 }
 
-template <typename T>
-int launch_tourn(const T *P, int ldp, int m, int w, int h, int arity, const TournWS &ws, const TournEpilogue &ep,
+int launch_tourn(const double *P, int ldp, int m, int w, int h, int arity, const TournWS &ws, const TournEpilogue &ep,
                  cudaStream_t st) {
-    if (h > kMaxV) return CF_ERR_UNSUPPORTED;      // a leaf is one tile of kMaxV rows at most
+    if (h > kMaxV || arity > 8) return CF_ERR_UNSUPPORTED;      // a node has at most 8 x kMaxV rows
     TournPlan plan{};
     int rc = make_tourn_plan(m, w, h, arity, &plan);
     if (rc != CF_OK) return rc;
     if (m == 0 || w == 0) return CF_OK;
-    switch (arity) {
-        case 2: return launch_tourn_cl<T, 2>(P, ldp, plan, ws, ep, st);
-        case 3: return launch_tourn_cl<T, 3>(P, ldp, plan, ws, ep, st);
-        case 4: return launch_tourn_cl<T, 4>(P, ldp, plan, ws, ep, st);
-        case 5: return launch_tourn_cl<T, 5>(P, ldp, plan, ws, ep, st);
-        case 6: return launch_tourn_cl<T, 6>(P, ldp, plan, ws, ep, st);
-        case 7: return launch_tourn_cl<T, 7>(P, ldp, plan, ws, ep, st);
-        case 8: return launch_tourn_cl<T, 8>(P, ldp, plan, ws, ep, st);
-        default: return CF_ERR_UNSUPPORTED;
+    const int sms = device_sm_count(), most = tourn_max_cluster();
+    int rows = h < m ? h : m;                    // rows of the level's largest node
+    for (int l = 0; l < plan.nlevels; ++l) {
+        if (l > 0) {
+            const int kids = arity < plan.cnt[l - 1] ? arity : plan.cnt[l - 1];
+            rows = kids * (rows < w ? rows : w);
+        }
+        // as many CTAs per node as leave every CTA of the level an SM of its own,
+        // down to 8 rows each
+        int cta = ceil_div(rows, kMaxV) > 4 ? 8 : (ceil_div(rows, kMaxV) > 2 ? 4 : (rows > kMaxV ? 2 : 1));
+        while (cta < most && 2ll * cta * plan.cnt[l] <= sms && ceil_div(rows, cta) > 8) cta *= 2;
+        TournLevel lv{};
+        lv.P = P;
+        lv.ldp = ldp;
+        lv.m = m;
+        lv.w = w;
+        lv.h = h;
+        lv.arity = arity;
+        lv.level = l;
+        lv.root = l == plan.nlevels - 1;
+        lv.cnt_below = l > 0 ? plan.cnt[l - 1] : 0;
+        lv.off_below = l > 0 ? plan.off[l - 1] : 0;
+        lv.off = plan.off[l];
+        lv.per = ceil_div(rows, cta);
+        lv.ld = lv.per | 1;
+        const size_t smem = align_up(sizeof(TournSmem), 16) + sizeof(double) * (size_t)lv.ld * w;
+        // the attributes belong to the current device: set on every call
+        CF_CUDA_TRY(cudaFuncSetAttribute(k_tourn_level, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTournMaxSmem));
+        if (cta > 8) CF_CUDA_TRY(cudaFuncSetAttribute(k_tourn_level, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(plan.cnt[l] * cta);
+        cfg.blockDim = dim3(kTournThreads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = cta;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        CF_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_tourn_level, lv, ws, ep));
+        count_launches(1);
     }
+    return CF_OK;
 }
 
 template <typename T>
@@ -442,10 +480,6 @@ int launch_apply_swaps(T *A, int lda, int ncols, int k0, const TournEpilogue &ep
     return CF_OK;
 }
 
-template int launch_tourn<double>(const double *, int, int, int, int, int, const TournWS &, const TournEpilogue &,
-                                  cudaStream_t);
-template int launch_tourn<float>(const float *, int, int, int, int, int, const TournWS &, const TournEpilogue &,
-                                 cudaStream_t);
 template int launch_apply_swaps<double>(double *, int, int, int, const TournEpilogue &, int *, cudaStream_t);
 template int launch_apply_swaps<float>(float *, int, int, int, const TournEpilogue &, int *, cudaStream_t);
 
@@ -480,5 +514,5 @@ extern "C" int cf_tourn_select(int m, int w, const double *panel, int ldp, int l
     ep.ipiv = nullptr;
     CF_CUDA_TRY(cudaMemsetAsync(ws.counter, 0, ws.counter_bytes, stream));
     ws.root_win = winners;
-    return launch_tourn<double>(panel, ldp, m, w, leaf_h, arity, ws, ep, stream);
+    return launch_tourn(panel, ldp, m, w, leaf_h, arity, ws, ep, stream);
 }

@@ -113,7 +113,7 @@ def test_minimal_and_null_workspaces_stay_accepted(cf):
     o = ctypes.byref(cf.options())
     assert L.cf_potrf_workspace_size(n, o) == 0
     assert L.cf_getrf_optimal_workspace_size(n, o) > L.cf_getrf_workspace_size(n, o)
-    assert L.cf_getrf_optimal_workspace_size(100, o) == L.cf_getrf_workspace_size(100, o)
+    assert L.cf_getrf_optimal_workspace_size(100, o) < 1 << 20
     A, S = inputs.uniform_pm1(n, seed=1), inputs.spd_gram(n, seed=2)
     dA = _dev(A)
     ipiv, info = cf.getrf(dA, work=_minimal(cf, n))
