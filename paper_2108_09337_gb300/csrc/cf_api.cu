@@ -202,9 +202,9 @@ static int getrf_lookahead(int n, double *A, int lda, int *ipiv, int *info, cons
         if (rest_pending && (rc = L.wait_update())) return fail(rc);
         if ((rc = launch_apply_swaps<double>(A, lda, n, k0, ep, nullptr, sp))) return fail(rc);
         if ((rc = launch_getf2_nopiv(A00, lda, w, k0, info, ep.lu, ep.lu_ok, sp))) return fail(rc);
-        if ((rc = launch_trsm_right_upper<double>(A00 + w, lda, m - w, w, A00, lda, false, nullptr, sp)))
+        if ((rc = launch_trsm_right_upper(A00 + w, lda, m - w, w, A00, lda, false, nullptr, sp)))
             return fail(rc);
-        if ((rc = launch_trsm_left_lower_unit<double>(A00 + w * ld, lda, w, n - k0 - w, A00, lda, sp)))
+        if ((rc = launch_trsm_left_lower_unit(A00 + w * ld, lda, w, n - k0 - w, A00, lda, sp)))
             return fail(rc);
         rest_pending = false;
         const int right = n - k0 - w;
@@ -257,8 +257,8 @@ static int potrf_lookahead(int n, double *A, int lda, int *info, const Opts &o, 
         const int w = o.v < n - k0 ? o.v : n - k0;
         const int m = n - k0;
         double *A00 = A + k0 + k0 * ld;
-        if ((rc = launch_potf2<double>(A00, lda, w, k0, info, sp))) return rc;
-        if ((rc = launch_trsm_right_upper<double>(A00 + w, lda, m - w, w, A00, lda, true, info, sp))) return rc;
+        if ((rc = launch_potf2(A00, lda, w, k0, info, sp))) return rc;
+        if ((rc = launch_trsm_right_upper(A00 + w, lda, m - w, w, A00, lda, true, info, sp))) return rc;
         const int rest = m - w;
         if (rest <= 0) continue;
         if (rest_pending && (rc = L.wait_update())) return rc;
@@ -340,9 +340,9 @@ extern "C" int cf_getrf(int n, double *A, int lda, int *ipiv, int *info, void *w
         // A00 = L00 U00 (no further pivoting)
         if ((rc = launch_getf2_nopiv(A00, lda, w, k0, info, ep.lu, ep.lu_ok, st))) return rc;
         // LU-3 A10 <- A10 U00^{-1}
-        if ((rc = launch_trsm_right_upper<double>(A00 + w, lda, m - w, w, A00, lda, false, nullptr, st))) return rc;
+        if ((rc = launch_trsm_right_upper(A00 + w, lda, m - w, w, A00, lda, false, nullptr, st))) return rc;
         // LU-4 A01 <- L00^{-1} A01
-        if ((rc = launch_trsm_left_lower_unit<double>(A00 + w * ld, lda, w, n - k0 - w, A00, lda, st))) return rc;
+        if ((rc = launch_trsm_left_lower_unit(A00 + w * ld, lda, w, n - k0 - w, A00, lda, st))) return rc;
         // LU-5 A11 <- A11 - A10 A01
         if (sl != nullptr && w >= kSliceMinW && n - k0 - w > 0) {
             const int right = n - k0 - w;
@@ -399,9 +399,9 @@ extern "C" int cf_potrf(int n, double *A, int lda, int *info, void *work, size_t
         const int m = n - k0;
         double *A00 = A + k0 + k0 * ld;
         // CH-1 L00 = chol(A00)
-        if ((rc = launch_potf2<double>(A00, lda, w, k0, info, st))) return rc;
+        if ((rc = launch_potf2(A00, lda, w, k0, info, st))) return rc;
         // CH-2 L10 <- A10 L00^{-T}
-        if ((rc = launch_trsm_right_upper<double>(A00 + w, lda, m - w, w, A00, lda, true, info, st))) return rc;
+        if ((rc = launch_trsm_right_upper(A00 + w, lda, m - w, w, A00, lda, true, info, st))) return rc;
         // CH-3 A11 <- A11 - L10 L10^T (lower)
         if (sl != nullptr && w >= kSliceMinW && m - w > 0) {
             if ((rc = slice64_begin(*sl, nullptr, lda, w, 0, info, st))) return rc;

@@ -122,6 +122,12 @@ bool tourn32_shape_ok(int v, int h, int arity);
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
 __device__ __forceinline__ double div_rn(double a, double b) { return __ddiv_rn(a, b); }
+// The division out of line, for the rare arguments that a reciprocal's quotient
+// does not cover: inlined in a select it would be evaluated for all (an FP64
+// division takes ~560 clocks, a comparison ~100, any other FP64 operation 64).
+static __device__ __noinline__ double div_call(double a, double b) { return __ddiv_rn(a, b); }
+// Biased exponent field of |x| by integer operations.
+__device__ __forceinline__ unsigned exp_bits(double x) { return ((unsigned)__double2hiint(x) >> 20) & 0x7FFu; }
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ float div_rn(float a, float b) { return __fdiv_rn(a, b); }

@@ -58,17 +58,13 @@ int launch_apply_swaps(T *A, int lda, int ncols, int k0, const TournEpilogue &ep
 int launch_getf2_nopiv(double *A00, int lda, int w, int kglob, int *info, const double *lu, const int *lu_ok,
                        cudaStream_t st);
 // A10 <- A10 * U^{-1}: rows x w block X, U upper non-unit w x w (or, with
-// trans_lower, U = L^T for a lower L).  Optional low-precision copy of the
-// result, K-major: lp[(r) * ldlp + c].
-template <typename T>
-int launch_trsm_right_upper(T *X, int ldx, int rows, int w, const T *U, int ldu, bool trans_lower,
+// trans_lower, U = L^T for a lower L).
+int launch_trsm_right_upper(double *X, int ldx, int rows, int w, const double *U, int ldu, bool trans_lower,
                             const int *skip_if_nonzero, cudaStream_t st);
 // A01 <- L^{-1} * A01: w x cols block X, L unit lower w x w.
-template <typename T>
-int launch_trsm_left_lower_unit(T *X, int ldx, int w, int cols, const T *L, int ldl, cudaStream_t st);
+int launch_trsm_left_lower_unit(double *X, int ldx, int w, int cols, const double *L, int ldl, cudaStream_t st);
 // Cholesky of the w x w diagonal block (lower), Listing "Cholesky".
-template <typename T>
-int launch_potf2(T *A00, int lda, int w, int kglob, int *info, cudaStream_t st);
+int launch_potf2(double *A00, int lda, int w, int kglob, int *info, cudaStream_t st);
 
 // ---- FP64 GEMM / SYRK (cf_gemm64.cu)
 // C -= A * op(B); op(B)(p, j) = trans_b ? B[j + p*ldb] : B[p + j*ldb].

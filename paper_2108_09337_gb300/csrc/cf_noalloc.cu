@@ -89,8 +89,8 @@ extern "C" int cf_getrf_noalloc(int n, double *A, int lda, int *ipiv, int *info,
         if ((rc = launch_tourn(A00, lda, m, w, o.leaf_h, o.arity, ws, ep, st))) return rc;
         if ((rc = launch_apply_swaps<double>(A, lda, n, k0, ep, nullptr, st))) return rc;
         if ((rc = launch_getf2_nopiv(A00, lda, w, k0, info, ep.lu, ep.lu_ok, st))) return rc;
-        if ((rc = launch_trsm_right_upper<double>(A00 + w, lda, m - w, w, A00, lda, false, nullptr, st))) return rc;
-        if ((rc = launch_trsm_left_lower_unit<double>(A00 + w * ld, lda, w, n - k0 - w, A00, lda, st))) return rc;
+        if ((rc = launch_trsm_right_upper(A00 + w, lda, m - w, w, A00, lda, false, nullptr, st))) return rc;
+        if ((rc = launch_trsm_left_lower_unit(A00 + w * ld, lda, w, n - k0 - w, A00, lda, st))) return rc;
         const int right = n - k0 - w;
         if (w < kSliceMinW) {
             if ((rc = launch_gemm_f64_sub(m - w, right, w, A00 + w, lda, A00 + w * ld, lda, false, A00 + w + w * ld,

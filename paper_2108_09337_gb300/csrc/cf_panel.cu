@@ -6,20 +6,16 @@
 //         room for it, which saves 0.59 ms of one SM per 128-column panel
 //   CH-1  potrf of A00 (Listing "Cholesky Factorization"; Table 2, v^3/6)
 //   CH-2  L10 <- A10 L00^{-T}      (Table 2: costed like the LU panel solve)
-//   S-1   the same triangular kernels serve the solves.
 //
-// The v x v triangle lives in shared memory; each CTA streams a chunk of
-// rows (right solves) or columns (left solves) of the panel.  Every update
-// is a separately rounded multiply and subtract in the oracle's order, so
-// step 0 of a factorization reproduces the oracle's values bit for bit.
+// The v x v triangle lives in shared memory.  LU's updates are a separately
+// rounded multiply and subtract in the oracle's order, so step 0 of an LU
+// reproduces the oracle's values bit for bit.
 #include "cf_common.cuh"
 #include "cf_kernels.cuh"
 
 namespace cf {
 
 constexpr int kPanelThreads = 256;
-constexpr int kRB = 64;            // rows per CTA, right solves
-constexpr int kCB = 64;            // columns per CTA, left solves
 constexpr int kLdT = kMaxV;        // triangle tile leading dimension
 
 // ---------------------------------------------------------------------------
@@ -68,144 +64,240 @@ k_getf2_nopiv(double *A, int lda, int w, int kglob, int *info, const double *lu,
 // ---------------------------------------------------------------------------
 // A00: Cholesky (lower, w <= 128), one CTA.  Stops at the first pivot that is
 // not positive (or NaN) and records info; later launches see info != 0.
+//
+// Bound by a chain of w pivots (square root, reciprocal, scaling, update of the
+// next pivot: each FP64 operation 64 clocks) and by the FP64 pipe of one SM
+// (w^3 / 6 multiply-adds, two lanes per clock).  Blocks of 16 columns: the
+// rows' block entries live in registers, one row per lane, warp 0 (the block's
+// own rows) runs ahead and hands each finished column, its square root and the
+// root's reciprocal to the warps below through shared memory; then all warps
+// update the columns right of the block.
 // ---------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(kPanelThreads, 1)
-k_potf2(T *A, int lda, int w, int kglob, int *info) {
+constexpr int kPB = 16;            // columns of a block
+constexpr int kPotThreads = 512;
+constexpr int kLdP = kMaxV + 1;
+
+struct PotSmem {
+    double t[kMaxV * kLdP];        // t[column * kLdP + row]
+    double col[kPB][kPB];          // col[c][j]: finished column c at the block's row j
+    double root[kPB], rinv[kPB];   // pivot and its reciprocal
+    int dead[kPB];                 // 1 from the first failed pivot on
+    int fail;                      // column of the failed pivot (-1: none)
+};
+
+// a / l from r ~ 1 / l (to a few ulp), corrected by the exact remainder; what
+// leaves the normal numbers is divided.
+__device__ __forceinline__ double quot1(double a, double l, double r) {
+    const double q0 = a * r;
+    double q = fma(fma(-q0, l, a), r, q0);
+    if (exp_bits(q0) - 100u >= 1900u) q = div_call(a, l);
+    return q;
+}
+
+// Square root of a pivot that is not a positive normal number; false: not positive.
+static __device__ __noinline__ bool odd_root(double d, double *root, double *r) {
+    *root = sqrt(d);
+    *r = 1.0 / *root;
+    return d > 0.0;
+}
+
+__global__ void __launch_bounds__(kPotThreads, 1)
+k_potf2(double *A, int lda, int w, int kglob, int *info) {
     if (*info != 0) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *t = reinterpret_cast<T *>(smem_raw);
-    __shared__ int fail;
-    const int tid = threadIdx.x;
-    for (int idx = tid; idx < w * w; idx += kPanelThreads) {
-        const int k = idx / w, r = idx % w;
-        if (r >= k) t[k * kLdT + r] = A[r + (size_t)k * lda];
-    }
-    if (tid == 0) fail = 0;
+    PotSmem &s = *reinterpret_cast<PotSmem *>(smem_raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int k = warp; k < w; k += kPotThreads / 32)
+        for (int r = lane; r < w; r += 32)
+            if (r >= k) s.t[k * kLdP + r] = A[r + (size_t)k * lda];
+    if (tid == 0) s.fail = -1;
     __syncthreads();
-    const int r = tid & (kMaxV - 1), half = tid / kMaxV;
-    int kdone = w;
-    for (int k = 0; k < w; ++k) {
-        const T d = t[k * kLdT + k];
-        if (!(d > T(0))) {                       // uniform: all threads read d
-            if (tid == 0) atomicCAS(info, 0, kglob + k + 1);
-            kdone = k;
-            break;
+    for (int k0 = 0; k0 < w; k0 += kPB) {
+        const int nb = min(kPB, w - k0);
+        // ---- the block's columns: warps 0..3, one row per lane
+        if (warp < 4 && (warp == 0 || k0 + 32 * warp < w)) {
+            const int row = k0 + 32 * warp + lane;
+            const bool in = row < w;
+            const int warps = min(4, (w - k0 + 31) / 32);
+            double p[kPB];
+#pragma unroll
+            for (int c = 0; c < kPB; ++c) p[c] = (in && c < nb && row >= k0 + c) ? s.t[(k0 + c) * kLdP + row] : 0.0;
+            bool dead = false;
+#pragma unroll
+            for (int c = 0; c < kPB; ++c) {
+                if (warp > 0 && (c & 1) == 0)          // columns c and c + 1 are ready
+                    asm volatile("bar.sync %0, %1;" ::"r"(1 + c / 2), "r"(32 * warps) : "memory");
+                if (warp == 0) {
+                    const double d = __shfl_sync(0xffffffffu, p[c], c);
+                    double r = rsqrt(d);
+                    const double s0 = d * r;
+                    double root = fma(fma(-s0, s0, d), 0.5 * r, s0);
+                    if (c < nb && !dead && (unsigned)__double2hiint(d) - 0x00100000u >= 0x7FE00000u) {
+                        if (!odd_root(d, &root, &r)) {
+                            dead = true;
+                            if (lane == 0) {
+                                s.fail = k0 + c;
+                                atomicCAS(info, 0, kglob + k0 + c + 1);
+                            }
+                        }
+                    }
+                    if (c < nb && !dead) {
+                        if (row > k0 + c) p[c] = quot1(p[c], root, r);
+                        else if (lane == c) p[c] = root;
+                        if (lane < kPB) s.col[c][lane] = p[c];
+                        if (lane == 0) { s.root[c] = root; s.rinv[c] = r; }
+                    }
+                    if (lane == 0) s.dead[c] = dead || c >= nb;
+                    __syncwarp();
+                    if (warps > 1 && (c & 1))
+                        asm volatile("bar.arrive %0, %1;" ::"r"(1 + c / 2), "r"(32 * warps) : "memory");
+                    if (c < nb && !dead) {
+#pragma unroll
+                        for (int j = c + 1; j < kPB; ++j) p[j] = fma(-p[c], s.col[c][j], p[j]);
+                    }
+                } else if (!s.dead[c]) {
+                    p[c] = quot1(p[c], s.root[c], s.rinv[c]);
+#pragma unroll
+                    for (int j = c + 1; j < kPB; ++j) p[j] = fma(-p[c], s.col[c][j], p[j]);
+                }
+            }
+            if (in) {
+#pragma unroll
+                for (int c = 0; c < kPB; ++c)
+                    if (c < nb && row >= k0 + c) s.t[(k0 + c) * kLdP + row] = p[c];
+            }
         }
-        const T lkk = sqrt(d);                                  // the pivot
-        if (half == 0 && r > k && r < w) t[k * kLdT + r] = div_rn(t[k * kLdT + r], lkk);   // column scaling
         __syncthreads();
-        if (tid == 0) t[k * kLdT + k] = lkk;
-        if (r > k && r < w) {                                   // trailing update, j in (k, r]
-            const T lik = t[k * kLdT + r];
-            for (int j = k + 1 + half; j <= r; j += 2)
-                t[j * kLdT + r] = sub_rn(t[j * kLdT + r], mul_rn(lik, t[k * kLdT + j]));
+        if (s.fail >= 0) break;
+        // ---- the columns right of the block: 32 rows x 8 columns per warp and turn
+        const int c1 = k0 + kPB;
+        if (c1 < w) {
+            const int rg = (w - c1 + 31) / 32, cgs = (w - c1 + 7) / 8;
+            for (int u = warp; u < rg * cgs; u += kPotThreads / 32) {
+                const int j0 = c1 + (u / rg) * 8, r = c1 + (u % rg) * 32 + lane;
+                if (c1 + (u % rg) * 32 + 31 < j0) continue;            // above the diagonal
+                double acc[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) acc[q] = (r < w && j0 + q < w) ? s.t[(j0 + q) * kLdP + r] : 0.0;
+#pragma unroll 4
+                for (int c = 0; c < kPB; ++c) {
+                    const double *tc = s.t + (k0 + c) * kLdP;
+                    const double l = r < w ? tc[r] : 0.0;
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) acc[q] = fma(-l, tc[min(j0 + q, w - 1)], acc[q]);
+                }
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    if (r < w && j0 + q <= r) s.t[(j0 + q) * kLdP + r] = acc[q];
+            }
         }
         __syncthreads();
     }
-    (void)fail;
     // Write back the lower triangle (columns past a breakdown keep their
     // partially updated values, as LAPACK leaves them).
-    for (int idx = tid; idx < w * w; idx += kPanelThreads) {
-        const int k = idx / w, rr = idx % w;
-        if (rr >= k) A[rr + (size_t)k * lda] = t[k * kLdT + rr];
-    }
-    (void)kdone;
+    for (int k = warp; k < w; k += kPotThreads / 32)
+        for (int r = lane; r < w; r += 32)
+            if (r >= k) A[r + (size_t)k * lda] = s.t[k * kLdP + r];
 }
 
 // ---------------------------------------------------------------------------
-// Right solve X <- X M^{-1}, M upper non-unit (M(k,j) = U[k + j*ldu]) or, with
-// TRANS, M = L^T for lower L (M(k,j) = L[j + k*ldu]).  X is rows x w.
-// CTA: kRB rows; four lanes of one warp share a row.
+// LU-3, CH-2 and LU-4: lines of X (rows in the right solves, columns in the
+// left one) against the step's w x w triangle:
+//   for k = 0..w-1:  x_k = x_k / M(k,k) (not LU-4);  x_j -= x_k M(k,j), j > k.
+//   kRight  M = U00: M(k, j) = U[k + j ldm]      (a zero pivot divides nothing)
+//   kChol   M = L00^T: M(k, j) = L[j + k ldm]
+//   kLeft   M = L00^T, unit: the columns of A01
+// Bound by the FP64 pipe: an FP64 instruction takes a quarter SM 64 clocks
+// whatever its active lanes, so lines are spread over all SMs (the number per
+// CTA is lines / SMs) and a line over LPR lanes, each holding every LPR-th
+// element in registers: 8 lanes keep four lines per warp and the shuffle of x_k
+// short; 16 where an SM has at most 8 lines, so that its four quarters still
+// have a warp each.  LU's updates are a separately rounded multiply and
+// subtract, and its quotients correctly rounded, in the oracle's order;
+// Cholesky's are fused.
 // ---------------------------------------------------------------------------
-template <typename T, bool TRANS>
-__global__ void __launch_bounds__(kPanelThreads, 1)
-k_trsm_right_upper(T *X, int ldx, int rows, int w, const T *U, int ldu, const int *skip) {
+enum { kRight = 0, kChol = 1, kLeft = 2 };
+constexpr int kLdM = kMaxV + 1;
+
+// LU-3's quotient in full: a zero pivot divides nothing.
+static __device__ __noinline__ double pivot_div(double x, double u) { return u != 0.0 ? __ddiv_rn(x, u) : x; }
+
+// RN(x / u) for u with r = RN(1 / u): two residual corrections (the second one
+// gives the correctly rounded quotient by Markstein's theorem, IBM J. Res. Dev.
+// 34, 1990).  r = 0 marks a u outside 2^+-300; such u, and x outside 2^+-600
+// are divided.
+__device__ __forceinline__ double quot_rn(double x, double u, double r) {
+    const double q0 = x * r;
+    const double q1 = fma(fma(-q0, u, x), r, q0);
+    const double q2 = fma(fma(-q1, u, x), r, q1);
+    double q = q2;
+    if (__double2hiint(r) == 0 || exp_bits(x) - 423u > 1200u) q = pivot_div(x, u);
+    return q;
+}
+
+template <int LPR, int KIND>
+__global__ void __launch_bounds__(512, 1)
+k_panel_solve(double *__restrict__ X, int ldx, int lines, int per, int w, const double *__restrict__ M, int ldm,
+              const int *skip) {
     if (skip != nullptr && *skip != 0) return;
+    constexpr int NI = kMaxV / LPR;                // elements per lane
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *Ms = reinterpret_cast<T *>(smem_raw);     // Ms[j*kLdT + k] = M(k, j)
-    T *Xs = Ms + kLdT * kMaxV;                   // Xs[j*(kRB+1) + r]
-    constexpr int XLD = kRB + 1;
-    const int tid = threadIdx.x;
-    const int r0 = blockIdx.x * kRB;
-    const int nr = min(kRB, rows - r0);
-    for (int idx = tid; idx < w * w; idx += kPanelThreads) {
-        const int k = idx % w, j = idx / w;
-        if (k <= j) Ms[j * kLdT + k] = TRANS ? U[j + (size_t)k * ldu] : U[k + (size_t)j * ldu];
+    double *Ms = reinterpret_cast<double *>(smem_raw);      // Ms[k * kLdM + j] = M(k, j)
+    double *rs = Ms + kMaxV * kLdM;                         // RN(1 / M(k, k)), 0: divide
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    const int sub = tid & (LPR - 1);
+    const int line = blockIdx.x * per + tid / LPR;
+    const bool in = tid / LPR < per && line < lines;
+    double x[NI];
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+        const int e = LPR * i + sub;
+        x[i] = (in && e < w) ? (KIND == kLeft ? X[(size_t)e + (size_t)line * ldx] : X[(size_t)line + (size_t)e * ldx]) : 0.0;
     }
-    for (int idx = tid; idx < kRB * w; idx += kPanelThreads) {
-        const int r = idx % kRB, j = idx / kRB;
-        if (r < nr) Xs[j * XLD + r] = X[(size_t)(r0 + r) + (size_t)j * ldx];
-    }
-    __syncthreads();
-    const int r = tid >> 2, q = tid & 3;
-    if (r < nr) {
-        for (int k = 0; k < w; ++k) {
-            if (q == 0) {
-                const T ukk = Ms[k * kLdT + k];
-                if (ukk != T(0)) Xs[k * XLD + r] = div_rn(Xs[k * XLD + r], ukk);
-            }
-            __syncwarp(0xfu << (tid & 28));
-            const T xk = Xs[k * XLD + r];
-            for (int j = k + 1 + q; j < w; j += 4)
-                Xs[j * XLD + r] = sub_rn(Xs[j * XLD + r], mul_rn(xk, Ms[j * kLdT + k]));
-            __syncwarp(0xfu << (tid & 28));
+    for (int idx = tid; idx < kMaxV * w; idx += nthr) {
+        const int a = idx & (kMaxV - 1), b = idx / kMaxV;   // a runs along the memory of the triangle
+        if (KIND == kRight) {
+            if (a <= b) Ms[a * kLdM + b] = M[a + (size_t)b * ldm];
+        } else {
+            if (a < w && a >= b) Ms[b * kLdM + a] = M[a + (size_t)b * ldm];
         }
     }
     __syncthreads();
-    for (int idx = tid; idx < kRB * w; idx += kPanelThreads) {
-        const int rr = idx % kRB, j = idx / kRB;
-        if (rr < nr) X[(size_t)(r0 + rr) + (size_t)j * ldx] = Xs[j * XLD + rr];
+    if (KIND != kLeft) {
+        for (int k = tid; k < w; k += nthr) {
+            const double u = Ms[k * kLdM + k];
+            rs[k] = exp_bits(u) - 723u <= 600u ? __drcp_rn(u) : (KIND == kChol ? 1.0 / u : 0.0);
+        }
+        __syncthreads();
     }
-}
-
-// ---------------------------------------------------------------------------
-// Left solve X <- M^{-1} X with M = T (TRANS: M = T^T) of size w x w, lower
-// (forward) or upper (backward), unit or non-unit diagonal.  X is w x cols.
-// CTA: kCB columns; four lanes of one warp share a column.
-// ---------------------------------------------------------------------------
-template <typename T, bool LOWER, bool UNIT, bool TRANS>
-__global__ void __launch_bounds__(kPanelThreads, 1)
-k_trsm_left(T *X, int ldx, int w, int cols, const T *Tm, int ldt) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *Ms = reinterpret_cast<T *>(smem_raw);     // Ms[k*kLdT + i] = M(i, k)
-    T *Xs = Ms + kLdT * kMaxV;                   // Xs[c*XLD + i]
-    constexpr int XLD = kMaxV + 1;
-    const int tid = threadIdx.x;
-    const int c0 = blockIdx.x * kCB;
-    const int nc = min(kCB, cols - c0);
-    for (int idx = tid; idx < w * w; idx += kPanelThreads) {
-        const int i = idx % w, k = idx / w;
-        const bool need = LOWER ? (i >= k) : (i <= k);
-        if (need) Ms[k * kLdT + i] = TRANS ? Tm[k + (size_t)i * ldt] : Tm[i + (size_t)k * ldt];
-    }
-    for (int idx = tid; idx < kCB * w; idx += kPanelThreads) {
-        const int i = idx % w, c = idx / w;
-        if (c < nc) Xs[c * XLD + i] = X[(size_t)i + (size_t)(c0 + c) * ldx];
-    }
-    __syncthreads();
-    const int c = tid >> 2, q = tid & 3;
-    if (c < nc) {
-        T *x = Xs + c * XLD;
-        for (int s = 0; s < w; ++s) {
-            const int k = LOWER ? s : (w - 1 - s);
-            if (!UNIT) {
-                if (q == 0) x[k] = div_rn(x[k], Ms[k * kLdT + k]);
-                __syncwarp(0xfu << (tid & 28));
+#pragma unroll
+    for (int kk = 0; kk < NI; ++kk) {
+        if (kk * LPR >= w) break;
+        const int kend = min(LPR, w - kk * LPR);
+        for (int kl = 0; kl < kend; ++kl) {
+            const int k = kk * LPR + kl;
+            const double *m = Ms + k * kLdM + sub;
+            double xk = __shfl_sync(0xffffffffu, x[kk], kl, LPR);
+            if (KIND != kLeft) {
+                const double u = Ms[k * kLdM + k];
+                xk = KIND == kChol ? quot1(xk, u, rs[k]) : quot_rn(xk, u, rs[k]);
+                if (sub == kl) x[kk] = xk;
             }
-            const T xk = x[k];
-            if (LOWER) {
-                for (int i = k + 1 + q; i < w; i += 4) x[i] = sub_rn(x[i], mul_rn(Ms[k * kLdT + i], xk));
-            } else {
-                for (int i = q; i < k; i += 4) x[i] = sub_rn(x[i], mul_rn(Ms[k * kLdT + i], xk));
+            if (sub > kl) {
+                const double mk = m[kk * LPR];
+                x[kk] = KIND == kChol ? fma(-xk, mk, x[kk]) : sub_rn(x[kk], mul_rn(xk, mk));
             }
-            __syncwarp(0xfu << (tid & 28));
+#pragma unroll
+            for (int i = kk + 1; i < NI; ++i) {
+                const double mk = m[i * LPR];
+                x[i] = KIND == kChol ? fma(-xk, mk, x[i]) : sub_rn(x[i], mul_rn(xk, mk));
+            }
         }
     }
-    __syncthreads();
-    for (int idx = tid; idx < kCB * w; idx += kPanelThreads) {
-        const int i = idx % w, cc = idx / w;
-        if (cc < nc) X[(size_t)i + (size_t)(c0 + cc) * ldx] = Xs[cc * XLD + i];
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+        const int e = LPR * i + sub;
+        if (in && e < w) (KIND == kLeft ? X[(size_t)e + (size_t)line * ldx] : X[(size_t)line + (size_t)e * ldx]) = x[i];
     }
 }
 
@@ -229,59 +321,44 @@ int launch_getf2_nopiv(double *A00, int lda, int w, int kglob, int *info, const 
     return CF_OK;
 }
 
-template <typename T>
-int launch_potf2(T *A00, int lda, int w, int kglob, int *info, cudaStream_t st) {
+int launch_potf2(double *A00, int lda, int w, int kglob, int *info, cudaStream_t st) {
     if (w <= 0) return CF_OK;
-    const size_t smem = sizeof(T) * kLdT * kMaxV;
-    int rc = set_smem(k_potf2<T>, smem);
+    int rc = set_smem(k_potf2, sizeof(PotSmem));
     if (rc) return rc;
-    k_potf2<T><<<1, kPanelThreads, smem, st>>>(A00, lda, w, kglob, info);
+    k_potf2<<<1, kPotThreads, sizeof(PotSmem), st>>>(A00, lda, w, kglob, info);
     CF_LAUNCH_CHECK();
     return CF_OK;
 }
 
-template <typename T>
-int launch_trsm_right_upper(T *X, int ldx, int rows, int w, const T *U, int ldu, bool trans_lower,
+template <int LPR, int KIND>
+static int launch_panel_lpr(double *X, int ldx, int lines, int per, int w, const double *M, int ldm, const int *skip,
+                            cudaStream_t st) {
+    const size_t smem = sizeof(double) * (kMaxV * kLdM + kMaxV);
+    int rc = set_smem(k_panel_solve<LPR, KIND>, smem);
+    if (rc) return rc;
+    const int threads = (int)align_up((size_t)per * LPR, 32);
+    k_panel_solve<LPR, KIND><<<ceil_div(lines, per), threads, smem, st>>>(X, ldx, lines, per, w, M, ldm, skip);
+    CF_LAUNCH_CHECK();
+    return CF_OK;
+}
+
+template <int KIND>
+static int launch_panel(double *X, int ldx, int lines, int w, const double *M, int ldm, const int *skip,
+                        cudaStream_t st) {
+    if (lines <= 0 || w <= 0) return CF_OK;
+    const int per = ceil_div(lines, device_sm_count());
+    if (per <= 8) return launch_panel_lpr<16, KIND>(X, ldx, lines, per, w, M, ldm, skip, st);
+    return launch_panel_lpr<8, KIND>(X, ldx, lines, per < 64 ? per : 64, w, M, ldm, skip, st);
+}
+
+int launch_trsm_right_upper(double *X, int ldx, int rows, int w, const double *U, int ldu, bool trans_lower,
                             const int *skip_if_nonzero, cudaStream_t st) {
-    if (rows <= 0 || w <= 0) return CF_OK;
-    const size_t smem = sizeof(T) * ((size_t)kLdT * kMaxV + (size_t)(kRB + 1) * kMaxV);
-    const int grid = ceil_div(rows, kRB);
-    if (trans_lower) {
-        int rc = set_smem(k_trsm_right_upper<T, true>, smem);
-        if (rc) return rc;
-        k_trsm_right_upper<T, true><<<grid, kPanelThreads, smem, st>>>(X, ldx, rows, w, U, ldu, skip_if_nonzero);
-    } else {
-        int rc = set_smem(k_trsm_right_upper<T, false>, smem);
-        if (rc) return rc;
-        k_trsm_right_upper<T, false><<<grid, kPanelThreads, smem, st>>>(X, ldx, rows, w, U, ldu, skip_if_nonzero);
-    }
-    CF_LAUNCH_CHECK();
-    return CF_OK;
+    return trans_lower ? launch_panel<kChol>(X, ldx, rows, w, U, ldu, skip_if_nonzero, st)
+                       : launch_panel<kRight>(X, ldx, rows, w, U, ldu, skip_if_nonzero, st);
 }
 
-template <typename T, bool LOWER, bool UNIT, bool TRANS>
-static int launch_trsm_left_t(T *X, int ldx, int w, int cols, const T *Tm, int ldt, cudaStream_t st) {
-    if (cols <= 0 || w <= 0) return CF_OK;
-    const size_t smem = sizeof(T) * ((size_t)kLdT * kMaxV + (size_t)kCB * (kMaxV + 1));
-    int rc = set_smem(k_trsm_left<T, LOWER, UNIT, TRANS>, smem);
-    if (rc) return rc;
-    k_trsm_left<T, LOWER, UNIT, TRANS><<<ceil_div(cols, kCB), kPanelThreads, smem, st>>>(X, ldx, w, cols, Tm, ldt);
-    CF_LAUNCH_CHECK();
-    return CF_OK;
+int launch_trsm_left_lower_unit(double *X, int ldx, int w, int cols, const double *L, int ldl, cudaStream_t st) {
+    return launch_panel<kLeft>(X, ldx, cols, w, L, ldl, nullptr, st);
 }
-
-template <typename T>
-int launch_trsm_left_lower_unit(T *X, int ldx, int w, int cols, const T *L, int ldl, cudaStream_t st) {
-    return launch_trsm_left_t<T, true, true, false>(X, ldx, w, cols, L, ldl, st);
-}
-
-template int launch_potf2<double>(double *, int, int, int, int *, cudaStream_t);
-template int launch_potf2<float>(float *, int, int, int, int *, cudaStream_t);
-template int launch_trsm_right_upper<double>(double *, int, int, int, const double *, int, bool, const int *,
-                                             cudaStream_t);
-template int launch_trsm_right_upper<float>(float *, int, int, int, const float *, int, bool, const int *,
-                                            cudaStream_t);
-template int launch_trsm_left_lower_unit<double>(double *, int, int, int, const double *, int, cudaStream_t);
-template int launch_trsm_left_lower_unit<float>(float *, int, int, int, const float *, int, cudaStream_t);
 
 }  // namespace cf

@@ -209,8 +209,9 @@ k_tri_solve64(int n, const double *__restrict__ T, int ldt, double *__restrict__
                     // whatever leaves the normal numbers, by the division itself
                     const double d = D[k * LDD + k], r = s.rinv[o][k];
                     const double q0 = xk * r;
-                    const double q1 = fma(fma(-q0, d, xk), r, q0);
-                    xk = isfinite(q1) && fabs(q0) > 1e-290 ? q1 : (xk == 0.0 && isfinite(r) && r != 0.0 ? q0 : xk / d);
+                    double q1 = fma(fma(-q0, d, xk), r, q0);
+                    if (exp_bits(q0) - 100u >= 1900u || exp_bits(r) - 100u >= 1900u) q1 = div_call(xk, d);
+                    xk = q1;
                 }
                 const double da = D[k * LDD + lane], db = D[k * LDD + lane + 32];
                 if (FWD) {
