@@ -128,6 +128,9 @@ __device__ __forceinline__ double div_rn(double a, double b) { return __ddiv_rn(
 static __device__ __noinline__ double div_call(double a, double b) { return __ddiv_rn(a, b); }
 // Biased exponent field of |x| by integer operations.
 __device__ __forceinline__ unsigned exp_bits(double x) { return ((unsigned)__double2hiint(x) >> 20) & 0x7FFu; }
+__device__ __forceinline__ bool is_zero(double x) {
+    return (((unsigned)__double2hiint(x) << 1) | (unsigned)__double2loint(x)) == 0u;
+}
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ float div_rn(float a, float b) { return __fdiv_rn(a, b); }

@@ -67,11 +67,12 @@ k_getf2_nopiv(double *A, int lda, int w, int kglob, int *info, const double *lu,
 //
 // Bound by a chain of w pivots (square root, reciprocal, scaling, update of the
 // next pivot: each FP64 operation 64 clocks) and by the FP64 pipe of one SM
-// (w^3 / 6 multiply-adds, two lanes per clock).  Blocks of 16 columns: the
-// rows' block entries live in registers, one row per lane, warp 0 (the block's
-// own rows) runs ahead and hands each finished column, its square root and the
-// root's reciprocal to the warps below through shared memory; then all warps
-// update the columns right of the block.
+// (w^3 / 6 multiply-adds, two lanes per clock).  Blocks of 16 columns, one row
+// per lane: warp 0 (the block's first rows) runs the chain alone, with nothing
+// else on its quarter of the SM; three helpers bring its later columns up to
+// date and up to three warps follow with the rows below, from the columns, roots
+// and reciprocals it leaves in shared memory; then all warps update the columns
+// right of the block.  w = 128: 0.21 ms (0.56 with one barrier pair per column).
 // ---------------------------------------------------------------------------
 constexpr int kPB = 16;            // columns of a block
 constexpr int kPotThreads = 512;
@@ -85,20 +86,27 @@ struct PotSmem {
     int fail;                      // column of the failed pivot (-1: none)
 };
 
-// a / l from r ~ 1 / l (to a few ulp), corrected by the exact remainder; what
-// leaves the normal numbers is divided.
+// a / l from r ~ 1 / l (to a few ulp), corrected by the exact remainder; a zero
+// is its own product, what else leaves the normal numbers is divided.
 __device__ __forceinline__ double quot1(double a, double l, double r) {
     const double q0 = a * r;
     double q = fma(fma(-q0, l, a), r, q0);
-    if (exp_bits(q0) - 100u >= 1900u) q = div_call(a, l);
+    if (exp_bits(q0) - 100u >= 1900u) q = is_zero(a) && exp_bits(r) - 1u < 2046u ? q0 : div_call(a, l);
     return q;
 }
 
-// Square root of a pivot that is not a positive normal number; false: not positive.
-static __device__ __noinline__ bool odd_root(double d, double *root, double *r) {
-    *root = sqrt(d);
-    *r = 1.0 / *root;
-    return d > 0.0;
+// Square root of a pivot that is not a positive normal number, and its
+// reciprocal; a root of -1: not positive.
+static __device__ __noinline__ double2 odd_root(double d) {
+    const double root = sqrt(d);
+    return d > 0.0 ? make_double2(root, 1.0 / root) : make_double2(-1.0, -1.0);
+}
+
+__device__ __forceinline__ void named_sync(int id, int threads) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void named_arrive(int id, int threads) {
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
 __global__ void __launch_bounds__(kPotThreads, 1)
@@ -114,81 +122,117 @@ k_potf2(double *A, int lda, int w, int kglob, int *info) {
     __syncthreads();
     for (int k0 = 0; k0 < w; k0 += kPB) {
         const int nb = min(kPB, w - k0);
-        // ---- the block's columns: warps 0..3, one row per lane
-        if (warp < 4 && (warp == 0 || k0 + 32 * warp < w)) {
-            const int row = k0 + 32 * warp + lane;
-            const bool in = row < w;
-            const int warps = min(4, (w - k0 + 31) / 32);
-            double p[kPB];
-#pragma unroll
-            for (int c = 0; c < kPB; ++c) p[c] = (in && c < nb && row >= k0 + c) ? s.t[(k0 + c) * kLdP + row] : 0.0;
+        // ---- the block's columns, one row per lane.  (Loops, with the entries in
+        // shared memory: unrolled with the entries in registers, the code outgrew
+        // the instruction caches.)
+        const int below = max(0, (w - k0 - 1) / 32);           // 32-row groups below the first
+        if (warp == 0) {
+            // the chain: pivot, column, the next column's own update
+            const int row = k0 + lane;
+            double *x = s.t + k0 * kLdP + min(row, w - 1);     // x[c * kLdP]: this row's entries
             bool dead = false;
-#pragma unroll
-            for (int c = 0; c < kPB; ++c) {
-                if (warp > 0 && (c & 1) == 0)          // columns c and c + 1 are ready
-                    asm volatile("bar.sync %0, %1;" ::"r"(1 + c / 2), "r"(32 * warps) : "memory");
-                if (warp == 0) {
-                    const double d = __shfl_sync(0xffffffffu, p[c], c);
-                    double r = rsqrt(d);
-                    const double s0 = d * r;
-                    double root = fma(fma(-s0, s0, d), 0.5 * r, s0);
-                    if (c < nb && !dead && (unsigned)__double2hiint(d) - 0x00100000u >= 0x7FE00000u) {
-                        if (!odd_root(d, &root, &r)) {
-                            dead = true;
-                            if (lane == 0) {
-                                s.fail = k0 + c;
-                                atomicCAS(info, 0, kglob + k0 + c + 1);
-                            }
+            double a = x[0];
+#pragma unroll 1
+            for (int c = 0; c < nb; ++c) {
+                const double d = __shfl_sync(0xffffffffu, a, c);
+                double r = rsqrt(d);
+                const double s0 = d * r;
+                double root = fma(fma(-s0, s0, d), 0.5 * r, s0);
+                if (!dead && (unsigned)__double2hiint(d) - 0x00100000u >= 0x7FE00000u) {
+                    const double2 o = odd_root(d);
+                    root = o.x;
+                    r = o.y;
+                    if (__double2hiint(root) < 0) {
+                        dead = true;
+                        if (lane == 0) {
+                            s.fail = k0 + c;
+                            atomicCAS(info, 0, kglob + k0 + c + 1);
                         }
                     }
-                    if (c < nb && !dead) {
-                        if (row > k0 + c) p[c] = quot1(p[c], root, r);
-                        else if (lane == c) p[c] = root;
-                        if (lane < kPB) s.col[c][lane] = p[c];
-                        if (lane == 0) { s.root[c] = root; s.rinv[c] = r; }
-                    }
-                    if (lane == 0) s.dead[c] = dead || c >= nb;
-                    __syncwarp();
-                    if (warps > 1 && (c & 1))
-                        asm volatile("bar.arrive %0, %1;" ::"r"(1 + c / 2), "r"(32 * warps) : "memory");
-                    if (c < nb && !dead) {
-#pragma unroll
-                        for (int j = c + 1; j < kPB; ++j) p[j] = fma(-p[c], s.col[c][j], p[j]);
-                    }
-                } else if (!s.dead[c]) {
-                    p[c] = quot1(p[c], s.root[c], s.rinv[c]);
-#pragma unroll
-                    for (int j = c + 1; j < kPB; ++j) p[j] = fma(-p[c], s.col[c][j], p[j]);
+                }
+                if (!dead) {
+                    if (lane > c) a = quot1(a, root, r);
+                    else if (lane == c) a = root;
+                    if (lane < kPB) s.col[c][lane] = a;
+                    if (lane >= c && row < w) x[c * kLdP] = a;
+                    if (lane == 0) { s.root[c] = root; s.rinv[c] = r; }
+                }
+                if (lane == 0) s.dead[c] = dead;
+                __syncwarp();
+                if (c < nb - 2) named_arrive(9 + (c & 1), 128);
+                if (below > 0 && ((c & 1) || c == nb - 1)) named_arrive(1 + c / 2, 32 * (1 + below));
+                if (c + 1 < nb) {
+                    if (c > 0) named_sync(11 + ((c - 1) & 1), 128);      // column c + 1 has every earlier column's part
+                    const double y = x[(c + 1) * kLdP];
+                    a = dead ? y : fma(-a, s.col[c][c + 1], y);
                 }
             }
-            if (in) {
+        } else if (warp < 4) {
+            // its helpers: the later columns of the same rows, a third each
+            const int row = k0 + lane;
+            double *x = s.t + k0 * kLdP + min(row, w - 1);
+#pragma unroll 1
+            for (int c = 0; c < nb - 2; ++c) {
+                named_sync(9 + (c & 1), 128);
+                if (!s.dead[c]) {
+                    const double a = x[c * kLdP];
+                    for (int q = c + 1 + warp; q < nb; q += 3) {
+                        const double v = fma(-a, s.col[c][q], x[q * kLdP]);
+                        if (lane >= q && row < w) x[q * kLdP] = v;
+                    }
+                }
+                named_arrive(11 + (c & 1), 128);
+            }
+        } else if (warp >= 5 && warp < 5 + below) {
+            // the rows below, one or two columns behind
+            const int row = k0 + 32 * (warp - 4) + lane;
+            const bool in = row < w;
+            double *x = s.t + k0 * kLdP + (in ? row : w - 1);
+#pragma unroll 1
+            for (int c = 0; c < nb; ++c) {
+                if ((c & 1) == 0) named_sync(1 + c / 2, 32 * (1 + below));      // columns c and c + 1 are ready
+                if (s.dead[c]) continue;
+                const double a = quot1(x[c * kLdP], s.root[c], s.rinv[c]);
+                const double *col = s.col[c];
+                if (in) x[c * kLdP] = a;
+                for (int q0 = c + 1; q0 < nb; q0 += 4) {
+                    double v[4];
 #pragma unroll
-                for (int c = 0; c < kPB; ++c)
-                    if (c < nb && row >= k0 + c) s.t[(k0 + c) * kLdP + row] = p[c];
+                    for (int q = 0; q < 4; ++q)
+                        if (q0 + q < nb) v[q] = fma(-a, col[q0 + q], x[(q0 + q) * kLdP]);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (q0 + q < nb && in) x[(q0 + q) * kLdP] = v[q];
+                }
             }
         }
         __syncthreads();
         if (s.fail >= 0) break;
-        // ---- the columns right of the block: 32 rows x 8 columns per warp and turn
+        // ---- the columns right of the block: 16 x 16 tiles on or below the
+        // diagonal (two columns per FP64 instruction: tiles of 32 rows would
+        // spend a third of them above it), round the warps
         const int c1 = k0 + kPB;
         if (c1 < w) {
-            const int rg = (w - c1 + 31) / 32, cgs = (w - c1 + 7) / 8;
-            for (int u = warp; u < rg * cgs; u += kPotThreads / 32) {
-                const int j0 = c1 + (u / rg) * 8, r = c1 + (u % rg) * 32 + lane;
-                if (c1 + (u % rg) * 32 + 31 < j0) continue;            // above the diagonal
+            const int g = (w - c1 + 15) / 16;
+            const int half = lane >> 4;
+            for (int u = warp; u < g * (g + 1) / 2; u += kPotThreads / 32) {
+                int ti = 0, tj = u;                                    // tile row, tile column
+                while (tj > ti) { ++ti; tj -= ti; }
+                const int r = c1 + ti * 16 + (lane & 15), j0 = c1 + tj * 16 + half;
+                const int rr = min(r, w - 1);
                 double acc[8];
 #pragma unroll
-                for (int q = 0; q < 8; ++q) acc[q] = (r < w && j0 + q < w) ? s.t[(j0 + q) * kLdP + r] : 0.0;
+                for (int q = 0; q < 8; ++q) acc[q] = s.t[min(j0 + 2 * q, w - 1) * kLdP + rr];
 #pragma unroll 4
                 for (int c = 0; c < kPB; ++c) {
                     const double *tc = s.t + (k0 + c) * kLdP;
-                    const double l = r < w ? tc[r] : 0.0;
+                    const double l = tc[rr];
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) acc[q] = fma(-l, tc[min(j0 + q, w - 1)], acc[q]);
+                    for (int q = 0; q < 8; ++q) acc[q] = fma(-l, tc[min(j0 + 2 * q, w - 1)], acc[q]);
                 }
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
-                    if (r < w && j0 + q <= r) s.t[(j0 + q) * kLdP + r] = acc[q];
+                    if (r < w && j0 + 2 * q <= r) s.t[(j0 + 2 * q) * kLdP + r] = acc[q];
             }
         }
         __syncthreads();
@@ -225,13 +269,13 @@ static __device__ __noinline__ double pivot_div(double x, double u) { return u !
 // RN(x / u) for u with r = RN(1 / u): two residual corrections (the second one
 // gives the correctly rounded quotient by Markstein's theorem, IBM J. Res. Dev.
 // 34, 1990).  r = 0 marks a u outside 2^+-300; such u, and x outside 2^+-600
-// are divided.
+// other than zero, are divided.
 __device__ __forceinline__ double quot_rn(double x, double u, double r) {
     const double q0 = x * r;
     const double q1 = fma(fma(-q0, u, x), r, q0);
     const double q2 = fma(fma(-q1, u, x), r, q1);
     double q = q2;
-    if (__double2hiint(r) == 0 || exp_bits(x) - 423u > 1200u) q = pivot_div(x, u);
+    if (__double2hiint(r) == 0 || exp_bits(x) - 423u > 1200u) q = __double2hiint(r) != 0 && is_zero(x) ? q0 : pivot_div(x, u);
     return q;
 }
 

@@ -36,7 +36,7 @@
 // columns fill the 512 TMEM columns.  Per tile: 36 digit pairs = 9,200 tensor
 // clocks; sixteen epilogue warps combine the diagonals in integers as they
 // leave TMEM (the accumulators are free again after the read), then do the
-// one FP64 operation per element while the next tile's MMAs run.
+// rounding and the one FP64 operation per element beside the next tile's MMAs.
 #include <climits>
 
 #include <cuda_bf16.h>
@@ -120,33 +120,32 @@ struct Walk {
                  : "=r"(r[o]), "=r"(r[o + 1]), "=r"(r[o + 2]), "=r"(r[o + 3])                       \
                  : "r"(taddr))
 
-// (hi 2^32 + lo) 2^(e - 2112), |hi| < 2^44, |lo| < 2^48, rounded to nearest (a
-// tie between two doubles goes up in magnitude).  Integer operations only: the
-// FP64 pipe has ~2 lanes per clock and is left to the subtraction.
-__device__ __forceinline__ double scaled_double(long long hi, long long lo, int e) {
-    hi += lo >> 32;
-    unsigned l = (unsigned)lo;
-    const bool neg = hi < 0;
-    if (neg) {                                      // negate the 96-bit number
-        l = 0u - l;
-        hi = -hi - (l != 0u ? 1 : 0);
-    }
-    unsigned long long w = ((unsigned long long)hi << 20) | (l >> 12);
-    unsigned long long x = (unsigned long long)l << 52;
-    if (w == 0) {
-        if (x == 0) return 0.0;
-        w = x;
-        x = 0;
-        e -= 64;
-    }
-    const int lz = __clzll((long long)w);
-    const unsigned long long m = lz ? (w << lz) | (x >> (64 - lz)) : w;
-    // value = m 2^(12 - lz) 2^(e - 2112), m in [2^63, 2^64)
-    const int field = e - 2112 + 12 - lz + 63 + 1023;
-    unsigned long long b = (m >> 11) + ((m >> 10) & 1u);      // 53 bits; a carry moves the exponent up by one
-    b += (unsigned long long)(field - 1) << 52;               // the leading bit adds the missing one
-    return __longlong_as_double((long long)(b | (neg ? 0x8000000000000000ull : 0ull)));
+// (hi 2^32 + lo) 2^(e - 2112), |hi| < 2^44, rounded to nearest (a
+// tie between two doubles goes up in magnitude).  32-bit integer operations
+// only (about 30): the FP64 pipe takes 64 clocks per instruction and quarter
+// SM and is left to the subtraction.
+__device__ __forceinline__ double scaled_double(long long hi, unsigned lo, int e) {
+    const unsigned sign = (unsigned)(hi >> 63);               // all ones if negative
+    unsigned long long low = ((unsigned long long)(unsigned)hi << 32) | lo;
+    const unsigned long long mask = ((unsigned long long)sign << 32) | sign;
+    low = (low ^ mask) - mask;
+    unsigned w2 = ((unsigned)(hi >> 32) ^ sign) + ((sign != 0u && low == 0ull) ? 1u : 0u);
+    unsigned w1 = (unsigned)(low >> 32), w0 = (unsigned)low;
+    if (w2 == 0u) { w2 = w1; w1 = w0; w0 = 0u; e -= 32; }
+    if (w2 == 0u) { w2 = w1; w1 = 0u; e -= 32; }
+    const int lz = __clz((int)w2);
+    const unsigned m1 = __funnelshift_lc(w1, w2, lz), m0 = __funnelshift_lc(w0, w1, lz);      // top bit of m1 set
+    const unsigned field = (unsigned)(e - 2112 + 95 - lz + 1023);
+    // 53 bits rounded; the leading bit adds the exponent's missing one, a carry one more
+    unsigned long long b = ((unsigned long long)((m1 >> 11) + ((field - 1u) << 20)) << 32) | __funnelshift_r(m0, m1, 11);
+    b += (m0 >> 10) & 1u;
+    b |= (unsigned long long)(sign & 0x80000000u) << 32;
+    return w2 == 0u ? 0.0 : __longlong_as_double((long long)b);
 }
+
+// An integer of magnitude at most 2^22 held in a float, without the conversion
+// unit (16 lanes per clock).
+__device__ __forceinline__ int small_int(float x) { return __float_as_int(x + 12582912.f) - 0x4B400000; }
 
 __global__ void __launch_bounds__(kThreads, 1)
 k_update_sliced(Problem p) {
@@ -306,12 +305,17 @@ k_update_sliced(Problem p) {
             const int row = wk.rt * BM + quarter * 32 + lane;
             const int col0 = wk.ct * BN + grp * 16;
             const int Ei = row < p.m ? p.E[row] : kCentre;
+            double *Cp = p.C + (size_t)row + (size_t)col0 * p.ldc;
+            auto mine = [&](int c) { return row < p.m && col0 + c >= p.c0 && col0 + c < p.c1 && (!p.lower || row >= col0 + c); };
             if (lane == 0) ok = wait_bounded(&s.acc_full, (uint32_t)n & 1u, abort_flag, &g_slice64_status);
             ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
             if (!ok) break;
             tc_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(grp * 16);
-            double v[16];
+            // the diagonals leave TMEM as one 96-bit integer per element, so that the
+            // accumulators are free for the next tile before the rounding
+            long long hi[16];
+            unsigned lo[16];
 #pragma unroll
             for (int c = 0; c < 16; c += 4) {
                 uint32_t r[4 * ND];
@@ -320,34 +324,33 @@ k_update_sliced(Problem p) {
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
+                    // |S_0| <= 2^19, |S_d| <= d 2^21: S_0 .. S_2 by the FP32 pipe, and the sums
+                    // formed in int32 fit it
+                    const int S0 = small_int(__uint_as_float(r[q])), S1 = small_int(__uint_as_float(r[4 + q])),
+                              S2 = small_int(__uint_as_float(r[8 + q]));
                     int S[ND];
 #pragma unroll
-                    for (int d = 0; d < ND; ++d) S[d] = __float2int_rn(__uint_as_float(r[4 * d + q]));
-                    // |S_d| <= d 2^21 (S_0: 2^19): the pairs below fit int32 where they are formed in int32
-                    const long long hi = (long long)(S[0] * 256 + S[1]) * 65536 + (long long)(S[2] * 256 + S[3]);
-                    const long long lo = (long long)S[4] * 16777216 + (long long)S[5] * 65536 +
-                                         ((long long)S[6] * 256 + S[7]);
-                    const int col = col0 + c + q;
-                    const int Fk = p.same ? (col < p.c1 ? p.E[col] - kCentre : 0) : (col < p.c1 ? p.F[col] : 0);
-                    v[c + q] = scaled_double(hi, lo, Ei + Fk);
+                    for (int d = 3; d < ND; ++d) S[d] = __float2int_rn(__uint_as_float(r[4 * d + q]));
+                    const long long low = (long long)S[4] * 16777216 + ((long long)S[5] * 65536 + ((long long)S[6] * 256 + S[7]));
+                    hi[c + q] = (long long)(S0 * 256 + S1) * 65536 + (long long)(S2 * 256 + S[3]) + (low >> 32);
+                    lo[c + q] = (unsigned)low;
                 }
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&s.acc_empty);
             if (row >= p.m || (any && (p.flagA[wk.rt] || (p.same ? p.flagA[wk.ct / 2] : p.flagB[wk.ct / 2])))) continue;
-            double *Cp = p.C + (size_t)row + (size_t)col0 * p.ldc;
-            double cv[16];
+            const int *Fp = p.same ? p.E + col0 : p.F + col0;
+            const int shift = p.same ? Ei - kCentre : Ei;
 #pragma unroll
-            for (int c = 0; c < 16; ++c) {
-                const int col = col0 + c;
-                const bool in = col >= p.c0 && col < p.c1 && (!p.lower || row >= col);
-                cv[c] = in ? Cp[(size_t)c * p.ldc] : 0.0;
-            }
+            for (int c0 = 0; c0 < 16; c0 += 8) {
+                double cv[8];
 #pragma unroll
-            for (int c = 0; c < 16; ++c) {
-                const int col = col0 + c;
-                if (col >= p.c0 && col < p.c1 && (!p.lower || row >= col)) Cp[(size_t)c * p.ldc] = cv[c] - v[c];
+                for (int c = 0; c < 8; ++c) cv[c] = mine(c0 + c) ? Cp[(size_t)(c0 + c) * p.ldc] : 0.0;
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    if (mine(c0 + c))
+                        Cp[(size_t)(c0 + c) * p.ldc] = cv[c] - scaled_double(hi[c0 + c], lo[c0 + c], shift + Fp[c0 + c]);
             }
         }
     }

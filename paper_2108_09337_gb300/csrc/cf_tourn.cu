@@ -47,7 +47,8 @@ struct TournSmem {
     int sloti[2][4 * kTournMaxCluster];          // their stacked positions (-1: none)
     int act[kMaxV];                              // this CTA's rows still in the race
     int rows[kMaxV];                             // panel row of each tile row
-    int order[kMaxV];                            // stacked position of each pivot
+    int order[kMaxV];                            // stacked position of each pivot, and its CTA
+    int own[kMaxV];
     int nact;
     int hole;                                    // place of the chosen row in act
     int lab_at[2 * kMaxV];                       // root epilogue: swap simulation
@@ -64,10 +65,13 @@ __device__ __forceinline__ unsigned long long piv_key(double a) {
     return b > 0x7FF0000000000000ull ? 1ull : b + 2ull;
 }
 
-// Warp maximum of (key, smallest position); every lane gets the position (-1: none).
+// Warp maximum of (key, smallest position); every lane gets the position (-1:
+// none).  One lane usually has the largest upper word alone.
 __device__ __forceinline__ int warp_best(unsigned long long key, int pos) {
     const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
     const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned tops = __ballot_sync(0xffffffffu, hi == mh);
+    if (mh != 0u && (tops & (tops - 1u)) == 0u) return __shfl_sync(0xffffffffu, pos, __ffs(tops) - 1);
     const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
     const bool top = hi == mh && lo == ml && key != 0;
     return (int)__reduce_min_sync(0xffffffffu, top ? (unsigned)pos : 0xffffffffu);
@@ -164,7 +168,7 @@ k_tourn_level(TournLevel lv, TournWS ws, TournEpilogue ep) {
         for (int r = lane; r < mine; r += 32) tile[k * ld + r] = lv.P[(size_t)s.rows[r] + (size_t)k * lv.ldp];
     __syncthreads();
     const int npiv = min(total, w);
-    const int nslots = 4 * ncta;
+    const int nw = (lv.per + 31) / 32, nslots = nw * ncta;      // a slot per warp that has rows
 
     // Candidate of this warp's rows in one column, into every CTA's slots.
     auto publish = [&](int par, bool have, double a, int row) {
@@ -173,29 +177,36 @@ k_tourn_level(TournLevel lv, TournWS ws, TournEpilogue ep) {
         const double v = __shfl_sync(0xffffffffu, a, owner ? __ffs(owner) - 1 : 0);
         if (lane < ncta) {
             TournSmem *rs = cl.map_shared_rank(&s, lane);
-            rs->slotv[par][rank * 4 + warp] = v;
-            rs->sloti[par][rank * 4 + warp] = best;
+            rs->slotv[par][rank * nw + warp] = v;
+            rs->sloti[par][rank * nw + warp] = best;
         }
     };
     if (ncta > 1) cl.sync();                     // every CTA of the cluster runs before it is written to
-    if (warp < 4) publish(0, tid < mine, tid < mine ? tile[tid] : 0.0, tid);
+    if (warp < nw) publish(0, tid < mine, tid < mine ? tile[tid] : 0.0, tid);
 
     for (int j = 0; j < npiv; ++j) {
         if (ncta > 1) cl.sync(); else __syncthreads();
         // ---- (1) the winner, found by every warp alike
         const int par = j & 1;
-        int gi;
+        int gi, owner;
         double piv;
         {
-            const int i0 = lane < nslots ? s.sloti[par][lane] : -1, i1 = lane + 32 < nslots ? s.sloti[par][lane + 32] : -1;
-            const double v0 = i0 >= 0 ? s.slotv[par][lane] : 0.0, v1 = i1 >= 0 ? s.slotv[par][lane + 32] : 0.0;
-            const unsigned long long k0 = i0 >= 0 ? piv_key(v0) : 0ull, k1 = i1 >= 0 ? piv_key(v1) : 0ull;
-            const bool second = k1 > k0 || (k1 == k0 && k1 != 0 && i1 < i0);
-            gi = warp_best(second ? k1 : k0, second ? i1 : i0);
-            const unsigned owner = __ballot_sync(0xffffffffu, (i0 == gi || i1 == gi) && gi >= 0);
-            piv = __shfl_sync(0xffffffffu, i1 == gi ? v1 : v0, owner ? __ffs(owner) - 1 : 0);
+            int at = lane, pos = lane < nslots ? s.sloti[par][lane] : -1;
+            double v = pos >= 0 ? s.slotv[par][lane] : 0.0;
+            unsigned long long key = pos >= 0 ? piv_key(v) : 0ull;
+            if (nslots > 32) {
+                const int i1 = lane + 32 < nslots ? s.sloti[par][lane + 32] : -1;
+                const double v1 = i1 >= 0 ? s.slotv[par][lane + 32] : 0.0;
+                const unsigned long long k1 = i1 >= 0 ? piv_key(v1) : 0ull;
+                if (k1 > key || (k1 == key && k1 != 0 && i1 < pos)) { key = k1; pos = i1; v = v1; at = lane + 32; }
+            }
+            gi = warp_best(key, pos);
+            const int src = __ffs(__ballot_sync(0xffffffffu, pos == gi)) - 1;
+            piv = __shfl_sync(0xffffffffu, v, src);
+            owner = __shfl_sync(0xffffffffu, at / nw, src);
         }
-        const int owner = gi / lv.per, lrow = gi - owner * lv.per;
+        const bool go = !is_zero(piv);           // a zero pivot eliminates nothing
+        const int lrow = gi - owner * lv.per;
         // ---- (2) pivot row from its owner; meanwhile the multipliers
         double pr = 0.0;
         const bool pull = tid < w - j;
@@ -213,15 +224,15 @@ k_tourn_level(TournLevel lv, TournWS ws, TournEpilogue ep) {
                 s.hole = tid;
                 row = -1;
             }
-            if (row >= 0 && piv != 0.0) {
+            if (row >= 0 && go) {
                 l = div_rn(tile[j * ld + row], piv);
                 tile[j * ld + row] = l;
                 s.mult[row] = l;
             }
         }
         if (pull) s.prow[j + tid] = pr;
-        if (tid == 0) s.order[j] = gi;
-        if (piv == 0.0 && tid == 0) s.bad = 1;
+        if (tid == 0) { s.order[j] = gi; s.own[j] = owner; }
+        if (!go && tid == 0) s.bad = 1;
         __syncthreads();
         const int jn = j + 1;
         // ---- (3) the next column and its candidates; the chosen row leaves the list
@@ -229,22 +240,22 @@ k_tourn_level(TournLevel lv, TournWS ws, TournEpilogue ep) {
             s.act[s.hole] = s.act[nact - 1];
             s.nact = nact - 1;
         }
-        if (warp < 4 && jn < npiv) {
+        if (warp < nw && jn < npiv) {
             double a = 0.0;
             if (row >= 0) {
                 a = tile[jn * ld + row];
-                if (piv != 0.0) {
+                if (go) {
                     a = sub_rn(a, mul_rn(l, s.prow[jn]));
                     tile[jn * ld + row] = a;
                 }
             }
             publish(jn & 1, row >= 0, a, row);
-        } else if (row >= 0 && jn < w && piv != 0.0) {       // the last pivot of a node with fewer rows than columns
+        } else if (row >= 0 && jn < w && go) {       // the last pivot of a node with fewer rows than columns
             tile[jn * ld + row] = sub_rn(tile[jn * ld + row], mul_rn(l, s.prow[jn]));
         }
         __syncthreads();
         // ---- (4) the other columns
-        if (piv != 0.0) {
+        if (go) {
             const int na = s.nact, tot = na * (w - jn - 1);
             const unsigned inv = na > 1 ? 0xFFFFFFFFu / (unsigned)na + 1u : 0u;
 #pragma unroll 4
@@ -259,7 +270,7 @@ k_tourn_level(TournLevel lv, TournWS ws, TournEpilogue ep) {
     __syncthreads();
     for (int j = tid; j < npiv; j += kTournThreads) {
         const int gi = s.order[j];
-        if (gi / lv.per == rank) {
+        if (s.own[j] == rank) {
             const int r = s.rows[gi - rank * lv.per];
             dst[j] = r;
             if (lv.root) ws.root_win[j] = r;
@@ -270,7 +281,7 @@ k_tourn_level(TournLevel lv, TournWS ws, TournEpilogue ep) {
         // the winners' eliminated rows are the LU of A00 in pivot order
         for (int j = warp; j < npiv; j += kTournThreads / 32) {
             const int gi = s.order[j];
-            if (gi / lv.per != rank) continue;
+            if (s.own[j] != rank) continue;
             for (int k = lane; k < w; k += 32) ep.lu[j + (size_t)k * kMaxV] = tile[k * ld + (gi - rank * lv.per)];
         }
         if (rank == 0 && tid == 0) *ep.lu_ok = s.bad == 0 && npiv == w;
