@@ -90,53 +90,81 @@ __device__ __forceinline__ void cta_argmax_1bar(BSmem<T> &s, T &bv, int &bi, int
     for (int q = 1; q < kBT / 32; ++q) bbetter(bv, bi, s.redv2[buf][q], s.redi2[buf][q]);
 }
 
-// C (mm x nn, ldc) -= A (mm x kk, lda) * B (kk x nn, ldb), kk <= kBMaxV; if
-// lower, only i >= j (relative indices, diagonal aligned).  A may be shared.
+// LU-5 / CH-3: C (mm x mm, ldc) -= A B, A (mm x w, lda); B = A01 (w x mm, ld
+// ldb) or, for Cholesky (B null), A^T with only i >= j written.
+//
+// A goes to the panel's shared memory (free after the pivot search) in whole
+// columns, A01 in chunks of 32 columns to the diagonal block's.  A warp takes
+// units of 32 RPT rows x 8 columns, lanes along the rows: per k one load of its
+// rows and broadcast loads of the eight columns, C read and written in whole
+// segments; FP32 takes two rows per lane (the loads bound it), FP64 one (the
+// FP64 pipe bounds it, so a unit past the edge or the diagonal counts).  The
+// operands read from global memory for every multiply-add, 4 + 4 loads per 16,
+// with 64 x 64 tiles: 13.5 ms of a 512 x 512 FP64 LU's 21, 4.1 of the FP32
+// one's 7.5.  Every element's operations and their order are as before.
 template <typename T>
-__device__ void cta_gemm_sub(int mm, int nn, int kk, const T *A, int lda, const T *B, int ldb, T *C, int ldc,
-                             bool lower) {
-    const int tid = threadIdx.x;
-    const int tr = (tid & 15) * 4, tc = (tid >> 4) * 4;      // 64 x 64 tiles, 4 x 4 per thread
-    for (int j0 = 0; j0 < nn; j0 += 64) {
-        for (int i0 = 0; i0 < mm; i0 += 64) {
-            if (lower && j0 > i0 + 63) continue;
-            T acc[4][4];
+__device__ void cta_update(BSmem<T> &s, int mm, int w, const T *A, int lda, const T *B, int ldb, T *C, int ldc) {
+    constexpr int RPT = sizeof(T) == 4 ? 2 : 1, UR = 32 * RPT, UC = 8, CH = 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool lower = B == nullptr;
+    T *Ls = bsmem_panel(s);                        // Ls[p * lm + i]
+    const int lm = (mm + 3) & ~3;                  // w * lm <= vb * kBMaxN
+    for (int p = warp; p < w; p += kBT / 32)
+        for (int i = lane; i < lm; i += 32) Ls[p * lm + i] = i < mm ? A[(size_t)i + (size_t)p * lda] : T(0);
+    __syncthreads();
+    const int rgs = (mm + UR - 1) / UR;
+    for (int j0 = 0; j0 < mm; j0 += lower ? mm : CH) {
+        const int nc = lower ? mm : min(CH, mm - j0);
+        if (!lower) {                              // s.D[p * CH + j]
+            for (int e = tid; e < w * CH; e += kBT) {
+                const int p = e % w, j = e / w;
+                s.D[p * CH + j] = j < nc ? B[(size_t)p + (size_t)(j0 + j) * ldb] : T(0);
+            }
+            __syncthreads();
+        }
+        const int cgs = (nc + UC - 1) / UC;
+        // the units on or below the diagonal, column group by column group, round the
+        // warps with a turn per group
+        for (int cg = 0; cg < cgs; ++cg)
+        for (int rg = (lower ? cg * UC / UR : 0) + ((warp - cg) & (kBT / 32 - 1)); rg < rgs; rg += kBT / 32) {
+            const int c0 = cg * UC;                                  // first column, from j0
+            const int i0 = rg * UR + lane * RPT;
+            const T *Bp = lower ? Ls + c0 : s.D + c0;
+            const int bs = lower ? lm : CH;
+            const int ia = min(i0, lm - RPT);
+            T acc[RPT][UC];
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
+            for (int a = 0; a < RPT; ++a)
 #pragma unroll
-                for (int b = 0; b < 4; ++b) acc[a][b] = T(0);
-            for (int p = 0; p < kk; ++p) {
-                T av[4], bv[4];
+                for (int b = 0; b < UC; ++b) acc[a][b] = T(0);
+            // (columns c0 .. c0 + 7 of Ls past lm: the next row's values, finite or not, in columns not written)
+            const bool whole = !lower || c0 + UC <= lm;
+#pragma unroll 2
+            for (int p = 0; p < w; ++p) {
+                T av[RPT], bv[UC];
 #pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    const int i = i0 + tr + a;
-                    av[a] = i < mm ? A[(size_t)i + (size_t)p * lda] : T(0);
-                }
+                for (int a = 0; a < RPT; ++a) av[a] = Ls[p * lm + ia + a];
 #pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    const int j = j0 + tc + b;
-                    bv[b] = j < nn ? B[(size_t)p + (size_t)j * ldb] : T(0);
-                }
+                for (int b = 0; b < UC; ++b) bv[b] = Bp[p * bs + (whole ? b : min(b, lm - 1 - c0))];
 #pragma unroll
-                for (int a = 0; a < 4; ++a)
+                for (int a = 0; a < RPT; ++a)
 #pragma unroll
-                    for (int b = 0; b < 4; ++b) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
+                    for (int b = 0; b < UC; ++b) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
             }
 #pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const int j = j0 + tc + b;
-                if (j >= nn) continue;
+            for (int b = 0; b < UC; ++b) {
+                const int jc = j0 + c0 + b;
 #pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    const int i = i0 + tr + a;
-                    if (i >= mm || (lower && i < j)) continue;
-                    T *c = C + (size_t)i + (size_t)j * ldc;
+                for (int a = 0; a < RPT; ++a) {
+                    const int ic = i0 + a;
+                    if (ic >= mm || jc >= mm || c0 + b >= nc || (lower && ic < jc)) continue;
+                    T *c = C + (size_t)ic + (size_t)jc * ldc;
                     *c = *c - acc[a][b];
                 }
             }
         }
+        __syncthreads();
     }
-    __syncthreads();
 }
 
 // In-place LU of one n x n matrix (n <= kBMaxN) with the pivot rule of the
@@ -273,8 +301,7 @@ __device__ void cta_getrf(BSmem<T> &s, T *A, int n, int lda, int *ipiv, int *inf
         }
         __syncthreads();
         // ---- LU-5: A11 <- A11 - A10 A01
-        if (m > w) cta_gemm_sub<T>(m - w, m - w, w, A00 + w, lda, A00 + (size_t)w * lda, lda,
-                                   A00 + w + (size_t)w * lda, lda, false);
+        if (m > w) cta_update<T>(s, m - w, w, A00 + w, lda, A00 + (size_t)w * lda, lda, A00 + w + (size_t)w * lda, lda);
         __syncthreads();
     }
 }
@@ -338,49 +365,8 @@ __device__ int cta_potrf(BSmem<T> &s, T *A, int n, int lda, int *info, int vb) {
                 if (k < w) row[(size_t)k * lda] = v[k];
         }
         __syncthreads();
-        // CH-3: A11 <- A11 - L10 L10^T (lower); B operand = L10^T read from A
-        if (m > w) {
-            // stage L10^T? read directly: B(p, j) = L10(j, p) = A00[w + j + p*lda]
-            const int mm = m - w;
-            T *C = A00 + w + (size_t)w * lda;
-            const int tr = (tid & 15) * 4, tc = (tid >> 4) * 4;
-            for (int j0 = 0; j0 < mm; j0 += 64)
-                for (int i0 = j0; i0 < mm; i0 += 64) {
-                    T acc[4][4];
-#pragma unroll
-                    for (int a = 0; a < 4; ++a)
-#pragma unroll
-                        for (int b = 0; b < 4; ++b) acc[a][b] = T(0);
-                    for (int p = 0; p < w; ++p) {
-                        T av[4], bv[4];
-#pragma unroll
-                        for (int a = 0; a < 4; ++a) {
-                            const int i = i0 + tr + a;
-                            av[a] = i < mm ? A00[w + i + (size_t)p * lda] : T(0);
-                        }
-#pragma unroll
-                        for (int b = 0; b < 4; ++b) {
-                            const int j = j0 + tc + b;
-                            bv[b] = j < mm ? A00[w + j + (size_t)p * lda] : T(0);
-                        }
-#pragma unroll
-                        for (int a = 0; a < 4; ++a)
-#pragma unroll
-                            for (int b = 0; b < 4; ++b) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
-                    }
-#pragma unroll
-                    for (int b = 0; b < 4; ++b) {
-                        const int j = j0 + tc + b;
-                        if (j >= mm) continue;
-#pragma unroll
-                        for (int a = 0; a < 4; ++a) {
-                            const int i = i0 + tr + a;
-                            if (i >= mm || i < j) continue;
-                            C[(size_t)i + (size_t)j * lda] -= acc[a][b];
-                        }
-                    }
-                }
-        }
+        // CH-3: A11 <- A11 - L10 L10^T (lower)
+        if (m > w) cta_update<T>(s, m - w, w, A00 + w, lda, (const T *)nullptr, 0, A00 + w + (size_t)w * lda, lda);
         __syncthreads();
     }
     return 0;
