@@ -123,20 +123,20 @@ __global__ void k_iota(int n, int *p) {
 // One pass over A: W = fl32(A) (+ shift on the diagonal) and, if rowsum is
 // set, rowsum[i] += sum_j |a_ij| over this CTA's columns (atomic over column
 // chunks).  CTA: 512 rows, two per thread (16-byte loads when vec: lda even
-// and A 16-byte aligned; W stores as float2, ldw even) x kCvtCols columns.
+// and A 16-byte aligned; W stores as float2, ldw even) x cols columns.
 // The row sums add |fl32(a_ij)| in FP32 over 32 columns and those partial
 // sums in FP64 (relative error ~1e-6, as the norm in eta needs): GB300's
 // FP64 pipe, ~2 operations per clock per SM, would otherwise bound the pass
 // at half the HBM bandwidth (measured 3.95 ms at N = 32768 with FP64 sums,
 // 2.05 ms with these, 92% of the copy bandwidth for its 12 bytes per
 // element).
-constexpr int kCvtCols = 1024;
+constexpr int kCvtColsMax = 1024;
 __global__ void __launch_bounds__(256) k_to_f32_rowsum(int n, const double *__restrict__ A, int lda,
                                                        float *__restrict__ W, int ldw, double shift, double *rowsum,
-                                                       int *ef, int vec) {
+                                                       int *ef, int vec, int cols) {
     const int i = (blockIdx.x * 256 + threadIdx.x) * 2;
     if (i >= n) return;
-    const int j0 = blockIdx.y * kCvtCols, j1 = min(n, j0 + kCvtCols);
+    const int j0 = blockIdx.y * cols, j1 = min(n, j0 + cols);
     const bool two = i + 1 < n;
     double s0 = 0.0, s1 = 0.0;
     int f0 = 0, f1 = 0;        // largest exponent fields (the tensor-core residual's row scales)
@@ -190,8 +190,13 @@ static int launch_to_f32_rowsum(int n, const double *A, int lda, float *W, int l
     if (n <= 0) return CF_OK;
     if (ldw % 2 != 0 || ((uintptr_t)W & 7)) return CF_ERR_UNSUPPORTED;
     const int vec = (lda % 2 == 0 && ((uintptr_t)A & 15) == 0) ? 1 : 0;
-    dim3 g(ceil_div(n, 512), ceil_div(n, kCvtCols));
-    k_to_f32_rowsum<<<g, 256, 0, st>>>(n, A, lda, W, ldw, shift, rowsum, ef, vec);
+    // columns per CTA: a thread walks them one after the other (eight loads in
+    // flight), so fewer of them, down to one FP32 partial sum, until every SM has
+    // eight CTAs (n = 4096: 8 x 4 CTAs of 1024 columns took 0.55 ms)
+    int cols = kCvtColsMax;
+    while (cols > 32 && (long long)ceil_div(n, 512) * ceil_div(n, cols) < 8ll * device_sm_count()) cols /= 2;
+    dim3 g(ceil_div(n, 512), ceil_div(n, cols));
+    k_to_f32_rowsum<<<g, 256, 0, st>>>(n, A, lda, W, ldw, shift, rowsum, ef, vec, cols);
     CF_LAUNCH_CHECK();
     return CF_OK;
 }

@@ -120,13 +120,19 @@ __device__ __forceinline__ int ld_acquire_gpu(const int *p) {
     asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
-__device__ __forceinline__ void st_release_gpu(int *p, int v) {
-    asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+__device__ __forceinline__ void or_release_gpu(int *p, int v) {
+    asm volatile("red.release.gpu.global.or.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
                  "l"(src)
+                 : "memory");
+}
+// The same for the first `bytes` bytes, zeros after them.
+__device__ __forceinline__ void cp_async16_zfill(void *dst, const void *src, int bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src), "r"(bytes)
                  : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
@@ -135,8 +141,10 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 
 // Stages the STORED SB x SB tile whose top-left element is (i0, j0) of T
 // (column-major, ld ldt) into St[col * (SB + 4) + row] with 16-byte async
-// copies when the whole tile is inside the matrix and aligned; element by
-// element otherwise (zero outside).
+// copies, zero-filled outside the matrix, when the matrix is aligned; element
+// by element otherwise.  (The last block row of a ragged matrix took the
+// element loop for every one of its tiles and ended the chain 0.6 ms late at
+// n = 10001.)
 template <int SB>
 __device__ __forceinline__ void stage_tile(float *St, const float *T, int ldt, int n, int i0, int j0, bool fast) {
     constexpr int TLD = SB + 4;
@@ -144,7 +152,9 @@ __device__ __forceinline__ void stage_tile(float *St, const float *T, int ldt, i
     if (fast) {
         for (int e = tid; e < SB * SB / 4; e += 256) {
             const int r4 = e % (SB / 4), c = e / (SB / 4);
-            cp_async16(St + c * TLD + 4 * r4, T + (size_t)(i0 + 4 * r4) + (size_t)(j0 + c) * ldt);
+            const int left = j0 + c < n ? max(0, min(4, n - (i0 + 4 * r4))) : 0;      // rows of the chunk inside
+            cp_async16_zfill(St + c * TLD + 4 * r4, left > 0 ? T + (size_t)(i0 + 4 * r4) + (size_t)(j0 + c) * ldt : T,
+                             4 * left);
         }
     } else {
         for (int e = tid; e < SB * SB; e += 256) {
@@ -193,11 +203,20 @@ __host__ __device__ constexpr size_t trsv_smem_bytes() {
                          (M::RED_IN_TILE ? 0 : (size_t)M::KS * SB * NR));   // partial sums of the k split
 }
 
+// A float as VT.  To double by its bits: the conversion instruction is an FP64
+// one (64 clocks of a quarter SM), half as many as the multiply-adds here.
+__device__ __forceinline__ void widen(float &r, float x) { r = x; }
+__device__ __forceinline__ void widen(double &r, float x) {
+    const unsigned b = __float_as_uint(x), u = b & 0x7FFFFFFFu;
+    r = __hiloint2double((int)((b & 0x80000000u) | ((u >> 3) + 0x38000000u)), (int)(u << 29));
+    if (u - 0x00800000u >= 0x7F000000u) r = (double)x;        // zero, subnormal, not finite
+}
+
 // Four consecutive 16-byte-aligned shared-memory values as VT.
 template <typename VT>
 __device__ __forceinline__ void load4(VT (&m)[4], const float *p) {
     const float4 v = *reinterpret_cast<const float4 *>(p);
-    m[0] = (VT)v.x; m[1] = (VT)v.y; m[2] = (VT)v.z; m[3] = (VT)v.w;
+    widen(m[0], v.x); widen(m[1], v.y); widen(m[2], v.z); widen(m[3], v.w);
 }
 __device__ __forceinline__ void load4(double (&m)[4], const double *p) {
     const double2 a = reinterpret_cast<const double2 *>(p)[0], b = reinterpret_cast<const double2 *>(p)[1];
@@ -292,7 +311,7 @@ __device__ __forceinline__ void trsv_stage_step(float *dst, int step, int s, boo
     }
     const int cb = fwd ? step : nb - 1 - step;
     const int ti = (MODE == 3) ? cb * SB : r0, tj = (MODE == 3) ? r0 : cb * SB;
-    stage_tile<SB>(dst, T, ldt, n, ti, tj, aligned && ti + SB <= n && tj + SB <= n);
+    stage_tile<SB>(dst, T, ldt, n, ti, tj, aligned);
 }
 // Block solve of one ticket.  VT: arithmetic and right-hand-side type
 // (float, or double for FP64 solves with the FP32 factor); the factor tiles
@@ -307,9 +326,10 @@ __device__ __forceinline__ void trsv_stage_step(float *dst, int step, int s, boo
 // partial sums meet in shared memory once per block before the diagonal
 // inverse is applied (and once more for its product).
 template <int SB, int MODE, int NR, typename VT>
-__global__ void __launch_bounds__(256, 1)        // one CTA per SM (shared memory)
+__global__ void __launch_bounds__(256, sizeof(VT) == 8 ? 2 : 1)        // CTAs per SM: shared memory
 k_trsv_blocked(int n, int nrhs, const float *__restrict__ T, int ldt, const VT *__restrict__ Dinv,
-               const float *__restrict__ Gn, VT *X, int ldx, int *flags, int *ticket, long long spin_limit) {
+               const float *__restrict__ Gn, VT *X, int ldx, int *flags, int *ticket, int groups,
+               long long spin_limit) {
     using Map = TrsvMap<SB, NR>;
     constexpr int TLD = SB + 4;
     constexpr int LR = Map::LR, C = Map::C, RW = Map::RW, WR = Map::WR, KS = Map::KS, KW = Map::KW;
@@ -329,8 +349,12 @@ k_trsv_blocked(int n, int nrhs, const float *__restrict__ T, int ldt, const VT *
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) s_ticket = atomicAdd(ticket, 1);
     __syncthreads();
-    const int s = s_ticket;
+    // ticket: step s of the group's own chain (bit of the block's flag)
+    const int s = s_ticket / groups, grp = s_ticket - s * groups;
     if (s >= nb) return;
+    const int bit = 1 << grp;
+    X += (size_t)grp * NR * ldx;
+    nrhs = min(NR, nrhs - grp * NR);
     const int b = fwd ? s : nb - 1 - s;
     const int r0 = b * SB, rb = min(SB, n - r0);
     const int wr = warp % WR, kp = warp / WR;      // row warp, k part
@@ -416,7 +440,7 @@ k_trsv_blocked(int n, int nrhs, const float *__restrict__ T, int ldt, const VT *
             if (lane == 0) {
                 const int *f = flags + (fwd ? from : nb - 1 - from);
                 long long it = 0;
-                while (ld_acquire_gpu(f) == 0 && it < spin_limit) {
+                while ((ld_acquire_gpu(f) & bit) == 0 && it < spin_limit) {
                     ++it;
                     if (it > 64) __nanosleep(20);
                 }
@@ -427,7 +451,7 @@ k_trsv_blocked(int n, int nrhs, const float *__restrict__ T, int ldt, const VT *
 #pragma unroll 1
             for (int chunk = 0; chunk < 2 && u < s; ++chunk) {
                 const int idx = u + lane;
-                const int fl = (idx < s) ? ld_acquire_gpu(flags + (fwd ? idx : nb - 1 - idx)) : 1;
+                const int fl = (idx < s) ? ld_acquire_gpu(flags + (fwd ? idx : nb - 1 - idx)) & bit : bit;
                 const unsigned unset = ~__ballot_sync(0xffffffffu, fl != 0);
                 if (unset == 0u) {
                     u = min(s, u + 32);
@@ -519,9 +543,9 @@ k_trsv_blocked(int n, int nrhs, const float *__restrict__ T, int ldt, const VT *
         if (i < rb && cc < nrhs) X[(size_t)(r0 + i) + (size_t)cc * ldx] = v;
     }
     // publish: the barrier orders every thread's stores of the block before
-    // thread 0's release store of the flag (release is cumulative)
+    // thread 0's release of the flag's bit (release is cumulative)
     __syncthreads();
-    if (tid == 0) st_release_gpu(flags + b, 1);
+    if (tid == 0) or_release_gpu(flags + b, bit);
 }
 
 // Flags for the smaller block size (the larger needs fewer).
@@ -572,12 +596,13 @@ int launch_diag_inverse64(int mode, int n, const float *T, int ldt, double *Dinv
 
 template <int SB, int MODE, int NR, typename VT>
 static int launch_trsv_nr(int n, int nrhs, const float *T, int ldt, const VT *Dinv, const float *Gn, VT *X, int ldx,
-                          int *flags, int *ticket, long long spin, cudaStream_t st) {
+                          int *flags, int *ticket, int groups, long long spin, cudaStream_t st) {
     const int nb = (n + SB - 1) / SB;
     const size_t smem = trsv_smem_bytes<SB, VT, NR>();
     CF_CUDA_TRY(cudaFuncSetAttribute(k_trsv_blocked<SB, MODE, NR, VT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)smem));
-    k_trsv_blocked<SB, MODE, NR, VT><<<nb, 256, smem, st>>>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, flags, ticket, spin);
+    k_trsv_blocked<SB, MODE, NR, VT><<<nb * groups, 256, smem, st>>>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, flags, ticket,
+                                                                    groups, spin);
     CF_LAUNCH_CHECK();
     return CF_OK;
 }
@@ -591,9 +616,20 @@ static int launch_trsv_mode(int n, int nrhs, const float *T, int ldt, const VT *
     CF_CUDA_TRY(cudaMemsetAsync(sync_ws, 0, sizeof(int) * (size_t)(nb + 1), st));
     int *flags = sync_ws, *ticket = sync_ws + nb;
     if (withhold) CF_CUDA_TRY(cudaMemsetAsync(ticket, 1, 1, st));     // ticket = 1 (little-endian low byte)
-    if (nrhs <= 4) return launch_trsv_nr<SB, MODE, 4, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, flags, ticket, spin, st);
-    if (nrhs <= 8) return launch_trsv_nr<SB, MODE, 8, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, flags, ticket, spin, st);
-    return launch_trsv_nr<SB, MODE, 16, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, flags, ticket, spin, st);
+    // FP64 arithmetic: a block's products are bound by one SM's FP64 pipe (64 x 64 x
+    // 16: 16 us each, 40 us per link of the chain), so each group of four
+    // right-hand sides is a chain of its own, side by side with the others
+    // (the factor is read once per group).  FP32: one chain for all.
+    if constexpr (sizeof(VT) == 8) {
+        return launch_trsv_nr<SB, MODE, 4, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, flags, ticket, ceil_div(nrhs, 4), spin,
+                                               st);
+    } else {
+        if (nrhs <= 4)
+            return launch_trsv_nr<SB, MODE, 4, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, flags, ticket, 1, spin, st);
+        if (nrhs <= 8)
+            return launch_trsv_nr<SB, MODE, 8, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, flags, ticket, 1, spin, st);
+        return launch_trsv_nr<SB, MODE, 16, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, flags, ticket, 1, spin, st);
+    }
 }
 
 template <int SB, typename VT>
