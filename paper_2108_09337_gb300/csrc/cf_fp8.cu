@@ -227,11 +227,19 @@ k_schur_fp8(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             }
             if (!ok) break;
             if (row < p.m && half_live) {
-                float *crow = p.C + row;
+                // 32 columns' loads in flight before their stores (one read-modify-write
+                // after the other waited for memory 128 times per tile)
+                const int c0 = n0 + half * 128;
+                const int live = p.lower ? min(p.n, row + 1) : p.n;      // columns this row may touch
+                float *cp = p.C + row + (size_t)c0 * p.ldc;
 #pragma unroll
-                for (int j = 0; j < 128; ++j) {
-                    const int col = n0 + half * 128 + j;
-                    if (col < p.n && (!p.lower || row >= col)) crow[(size_t)col * p.ldc] -= sum[j];
+                for (int j0 = 0; j0 < 128; j0 += 32) {
+                    float v[32];
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) v[j] = c0 + j0 + j < live ? cp[(size_t)(j0 + j) * p.ldc] : 0.f;
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        if (c0 + j0 + j < live) cp[(size_t)(j0 + j) * p.ldc] = v[j] - sum[j0 + j];
                 }
             }
         }
