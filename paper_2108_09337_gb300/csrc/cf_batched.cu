@@ -36,13 +36,15 @@ constexpr int kBMaxV = 32;              // largest block size
 template <typename T>
 struct BSmem {
     T D[kBMaxV * (kBMaxV + 1)];         // diagonal block
-    T redv2[2][kBT / 32];               // the pivot search's warp maxima, alternating by column
-    int redi2[2][kBT / 32];
+    unsigned long long redk[2][kBT / 32];   // the pivot search's warp maxima, alternating by column
+    int redi[2][kBT / 32];
     int used[kBMaxN];
     int order[kBMaxV];
     int lab[kBMaxN];
     int where_[kBMaxN];
     int fail;
+    int cnt;                            // moved rows (their positions in where_)
+    int zero;                           // 1: the panel met a zero pivot
 };
 
 template <typename T>
@@ -58,36 +60,41 @@ __device__ __forceinline__ T *bsmem_panel(BSmem<T> &s) {
     return reinterpret_cast<T *>(reinterpret_cast<unsigned char *>(&s) + bsmem_header_bytes<T>());
 }
 
-template <typename T>
-__device__ __forceinline__ T bkey(T a) {
-    T x = fabs(a);
-    return (x != x) ? T(-0.5) : x;
+// Rank of a pivot candidate as an unsigned key: |a| by its bits, NaN below
+// every number (1), no candidate 0.  Integers, because an FP64 comparison takes
+// a quarter of the SM ~100 clocks.
+__device__ __forceinline__ unsigned long long bkey(double a) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(a) & 0x7FFFFFFFFFFFFFFFull;
+    return b > 0x7FF0000000000000ull ? 1ull : b + 2ull;
+}
+__device__ __forceinline__ unsigned long long bkey(float a) {
+    const unsigned b = __float_as_uint(a) & 0x7FFFFFFFu;
+    return b > 0x7F800000u ? 1ull : (unsigned long long)(b + 2u) << 32;
 }
 
-template <typename T>
-__device__ __forceinline__ void bbetter(T &bv, int &bi, T ov, int oi) {
-    if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
+// Smallest index among the lanes with the largest key; the key in `key`.
+__device__ __forceinline__ int warp_argmax(unsigned long long &key, int idx) {
+    const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+    const bool top = hi == mh && lo == ml && key != 0;
+    key = ((unsigned long long)mh << 32) | ml;
+    return (int)__reduce_min_sync(0xffffffffu, top ? (unsigned)idx : 0x7fffffffu);
 }
 
-// CTA-wide argmax (value, index) with the tie rule of the tournament, one
-// barrier: the warp maxima go to buffer buf (alternating from one call to
-// the next, so the next call's writes never meet this call's reads) and
-// every thread reduces the eight itself.
+// CTA-wide argmax with the tie rule of the tournament (smallest index), one
+// barrier: the warp maxima go to buffer buf (alternating from one call to the
+// next, so the next call's writes never meet this call's reads) and every warp
+// reduces the eight itself.
 template <typename T>
-__device__ __forceinline__ void cta_argmax_1bar(BSmem<T> &s, T &bv, int &bi, int buf) {
+__device__ __forceinline__ int cta_argmax_1bar(BSmem<T> &s, unsigned long long key, int idx, int buf) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const T ov = __shfl_xor_sync(0xffffffffu, bv, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        bbetter(bv, bi, ov, oi);
-    }
-    if (lane == 0) { s.redv2[buf][warp] = bv; s.redi2[buf][warp] = bi; }
+    idx = warp_argmax(key, idx);
+    if (lane == 0) { s.redk[buf][warp] = key; s.redi[buf][warp] = idx; }
     __syncthreads();
-    bv = s.redv2[buf][0];
-    bi = s.redi2[buf][0];
-#pragma unroll
-    for (int q = 1; q < kBT / 32; ++q) bbetter(bv, bi, s.redv2[buf][q], s.redi2[buf][q]);
+    key = lane < kBT / 32 ? s.redk[buf][lane] : 0ull;
+    idx = lane < kBT / 32 ? s.redi[buf][lane] : 0x7fffffff;
+    return warp_argmax(key, idx);
 }
 
 // LU-5 / CH-3: C (mm x mm, ldc) -= A B, A (mm x w, lda); B = A01 (w x mm, ld
@@ -167,6 +174,63 @@ __device__ void cta_update(BSmem<T> &s, int mm, int w, const T *A, int lda, cons
     }
 }
 
+// A00's LU and LU-3 on their own, for a panel that met a zero pivot (which
+// divides nothing).
+template <typename T>
+__device__ __noinline__ void cta_a00_lu3(BSmem<T> &s, T *A00, int lda, int m, int w, int k0, int *info) {
+    const int tid = threadIdx.x;
+            // A00 = L00 U00 (no pivoting) in shared memory
+            for (int e = tid; e < w * w; e += kBT) {
+                const int r = e % w, c = e / w;
+                s.D[c * (kBMaxV + 1) + r] = A00[r + (size_t)c * lda];
+            }
+            __syncthreads();
+            for (int k = 0; k < w; ++k) {
+                const T piv = s.D[k * (kBMaxV + 1) + k];
+                if (piv == T(0) && tid == 0) atomicCAS(info, 0, k0 + k + 1);
+                __syncthreads();
+                for (int e = tid; e < (w - k - 1); e += kBT) {
+                    const int r = k + 1 + e;
+                    if (piv != T(0)) s.D[k * (kBMaxV + 1) + r] = s.D[k * (kBMaxV + 1) + r] / piv;
+                }
+                __syncthreads();
+                const int rem = w - k - 1;
+                for (int e = tid; e < rem * rem; e += kBT) {
+                    const int r = k + 1 + e % rem, c = k + 1 + e / rem;
+                    s.D[c * (kBMaxV + 1) + r] -= s.D[k * (kBMaxV + 1) + r] * s.D[c * (kBMaxV + 1) + k];
+                }
+                __syncthreads();
+            }
+            for (int e = tid; e < w * w; e += kBT) {
+                const int r = e % w, c = e / w;
+                A00[r + (size_t)c * lda] = s.D[c * (kBMaxV + 1) + r];
+            }
+            // LU-3: A10 <- A10 U00^{-1} (one row per thread, held in registers:
+            // every element gets the same operations in the same order as in
+            // place, without a trip through memory per multiply-add)
+            for (int r = w + tid; r < m; r += kBT) {
+                T *row = A00 + r;
+                T v[kBMaxV];
+    #pragma unroll
+                for (int k = 0; k < kBMaxV; ++k) v[k] = k < w ? row[(size_t)k * lda] : T(0);
+    #pragma unroll
+                for (int k = 0; k < kBMaxV; ++k) {
+                    if (k < w) {
+                        const T ukk = s.D[k * (kBMaxV + 1) + k];
+                        T x = v[k];
+                        if (ukk != T(0)) x = x / ukk;
+                        v[k] = x;
+    #pragma unroll
+                        for (int j = k + 1; j < kBMaxV; ++j)
+                            if (j < w) v[j] -= x * s.D[j * (kBMaxV + 1) + k];
+                    }
+                }
+    #pragma unroll
+                for (int k = 0; k < kBMaxV; ++k)
+                    if (k < w) row[(size_t)k * lda] = v[k];
+            }
+}
+
 // In-place LU of one n x n matrix (n <= kBMaxN) with the pivot rule of the
 // tournament for a single leaf (partial pivoting, ties to the smallest
 // position), block size vb.  Same step structure as cf_getrf.
@@ -183,17 +247,24 @@ __device__ void cta_getrf(BSmem<T> &s, T *A, int n, int lda, int *ipiv, int *inf
             P[c * m + r] = A00[r + (size_t)c * lda];
         }
         for (int r = tid; r < m; r += kBT) s.used[r] = 0;
+        if (tid == 0) s.zero = s.cnt = 0;
         __syncthreads();
         // One barrier per column: a thread reads and writes only its own
         // rows (r = tid mod kBT) and marks its own row when it wins; the
         // pivot row, final since its owner's update of the previous column,
         // is read by all after the column's barrier and written by no one.
+        // The multipliers stay in the panel: what the elimination leaves is
+        // A00's LU in the winners' rows and A10 U00^{-1} in the others, the
+        // same operations in the same order as A00 and LU-3 on their own.
         for (int j = 0; j < w; ++j) {
-            T bv = T(-1);
-            int bi = INT_MAX;
+            unsigned long long bk = 0ull;
+            int bi = 0x7fffffff;
             for (int r = tid; r < m; r += kBT)
-                if (!s.used[r]) bbetter(bv, bi, bkey(P[j * m + r]), r);
-            cta_argmax_1bar(s, bv, bi, j & 1);
+                if (!s.used[r]) {
+                    const unsigned long long k = bkey(P[j * m + r]);
+                    if (k > bk) { bk = k; bi = r; }
+                }
+            bi = cta_argmax_1bar(s, bk, bi, j & 1);
             if (tid == 0) s.order[j] = bi;
             if (bi % kBT == tid) s.used[bi] = 1;
             const T piv = P[j * m + bi];
@@ -201,8 +272,11 @@ __device__ void cta_getrf(BSmem<T> &s, T *A, int n, int lda, int *ipiv, int *inf
                 for (int r = tid; r < m; r += kBT) {
                     if (s.used[r]) continue;
                     const T l = P[j * m + r] / piv;
+                    P[j * m + r] = l;
                     for (int c = j + 1; c < w; ++c) P[c * m + r] = P[c * m + r] - l * P[c * m + bi];
                 }
+            } else if (tid == 0) {
+                s.zero = 1;
             }
         }
         __syncthreads();
@@ -213,7 +287,6 @@ __device__ void cta_getrf(BSmem<T> &s, T *A, int n, int lda, int *ipiv, int *inf
             for (int j = 0; j < w; ++j) {
                 const int lab = s.order[j], p = s.where_[lab];
                 ipiv[k0 + j] = k0 + p + 1;
-                s.order[j] = p;                          // the swap partner, for the column loop
                 if (p != j) {
                     const int lj = s.lab[j];
                     s.lab[j] = lab; s.where_[lab] = j;
@@ -222,64 +295,47 @@ __device__ void cta_getrf(BSmem<T> &s, T *A, int n, int lda, int *ipiv, int *inf
             }
         }
         __syncthreads();
-        for (int c = tid; c < n; c += kBT) {
-            T *col = A + (size_t)c * lda;
-            for (int j = 0; j < w; ++j) {
-                const int p = k0 + s.order[j];
-                if (p != k0 + j) { const T t = col[k0 + j]; col[k0 + j] = col[p]; col[p] = t; }
-            }
-        }
+        const bool redo = s.zero != 0;                      // a zero pivot divides nothing: A00 and LU-3 on their own
+        for (int r = tid; r < m; r += kBT)                  // positions whose row moves (at most 2 w)
+            if (s.lab[r] != r) s.where_[atomicAdd(&s.cnt, 1)] = r;
         __syncthreads();
-        // ---- A00 = L00 U00 (no pivoting) in shared memory
-        for (int e = tid; e < w * w; e += kBT) {
-            const int r = e % w, c = e / w;
-            s.D[c * (kBMaxV + 1) + r] = A00[r + (size_t)c * lda];
-        }
-        __syncthreads();
-        for (int k = 0; k < w; ++k) {
-            const T piv = s.D[k * (kBMaxV + 1) + k];
-            if (piv == T(0) && tid == 0) atomicCAS(info, 0, k0 + k + 1);
-            __syncthreads();
-            for (int e = tid; e < (w - k - 1); e += kBT) {
-                const int r = k + 1 + e;
-                if (piv != T(0)) s.D[k * (kBMaxV + 1) + r] = s.D[k * (kBMaxV + 1) + r] / piv;
-            }
-            __syncthreads();
-            const int rem = w - k - 1;
-            for (int e = tid; e < rem * rem; e += kBT) {
-                const int r = k + 1 + e % rem, c = k + 1 + e / rem;
-                s.D[c * (kBMaxV + 1) + r] -= s.D[k * (kBMaxV + 1) + r] * s.D[c * (kBMaxV + 1) + k];
-            }
-            __syncthreads();
-        }
-        for (int e = tid; e < w * w; e += kBT) {
-            const int r = e % w, c = e / w;
-            A00[r + (size_t)c * lda] = s.D[c * (kBMaxV + 1) + r];
-        }
-        // ---- LU-3: A10 <- A10 U00^{-1} (one row per thread, held in registers:
-        // every element gets the same operations in the same order as in
-        // place, without a trip through memory per multiply-add)
-        for (int r = w + tid; r < m; r += kBT) {
-            T *row = A00 + r;
-            T v[kBMaxV];
+        {
+            // every column outside the panel (with redo: inside too) as one gather: a
+            // warp takes four columns, a lane two moved rows of each
+            const int lane = tid & 31, cnt = s.cnt;
+            const int d0 = lane < cnt ? s.where_[lane] : -1, d1 = lane + 32 < cnt ? s.where_[lane + 32] : -1;
+            const int s0 = d0 >= 0 ? s.lab[d0] : 0, s1 = d1 >= 0 ? s.lab[d1] : 0;
+            for (int c0 = (tid >> 5) * 4; c0 < n && cnt > 0; c0 += kBT / 8) {
+                T v[4][2];
 #pragma unroll
-            for (int k = 0; k < kBMaxV; ++k) v[k] = k < w ? row[(size_t)k * lda] : T(0);
+                for (int q = 0; q < 4; ++q) {
+                    const int c = c0 + q;
+                    if (c >= n || (!redo && c >= k0 && c < k0 + w)) continue;
+                    const T *col = A + (size_t)c * lda + k0;
+                    if (d0 >= 0) v[q][0] = col[s0];
+                    if (d1 >= 0) v[q][1] = col[s1];
+                }
+                __syncwarp();
 #pragma unroll
-            for (int k = 0; k < kBMaxV; ++k) {
-                if (k < w) {
-                    const T ukk = s.D[k * (kBMaxV + 1) + k];
-                    T x = v[k];
-                    if (ukk != T(0)) x = x / ukk;
-                    v[k] = x;
-#pragma unroll
-                    for (int j = k + 1; j < kBMaxV; ++j)
-                        if (j < w) v[j] -= x * s.D[j * (kBMaxV + 1) + k];
+                for (int q = 0; q < 4; ++q) {
+                    const int c = c0 + q;
+                    if (c >= n || (!redo && c >= k0 && c < k0 + w)) continue;
+                    T *col = A + (size_t)c * lda + k0;
+                    if (d0 >= 0) col[d0] = v[q][0];
+                    if (d1 >= 0) col[d1] = v[q][1];
                 }
             }
-#pragma unroll
-            for (int k = 0; k < kBMaxV; ++k)
-                if (k < w) row[(size_t)k * lda] = v[k];
         }
+        if (!redo) {
+            for (int c = tid >> 5; c < w; c += kBT / 32)
+                for (int r = tid & 31; r < m; r += 32) {
+                    const T v = P[c * m + s.lab[r]];
+                    A00[r + (size_t)c * lda] = v;
+                    if (r < w) s.D[c * (kBMaxV + 1) + r] = v;
+                }
+        }
+        __syncthreads();
+        if (redo) cta_a00_lu3<T>(s, A00, lda, m, w, k0, info);
         // ---- LU-4: A01 <- L00^{-1} A01 (one column per thread, in registers)
         for (int c = w + tid; c < m; c += kBT) {
             T *col = A00 + (size_t)c * lda;
