@@ -10,9 +10,11 @@
 //   * warp 0 issues TMA loads (128-byte swizzle) into a 4-stage ring of
 //     shared-memory stages, warp 1 (one elected lane) issues tcgen05.mma
 //     (kind::f16, M=128, N=256, K=16) into one of two TMEM accumulators,
-//     warps 2-5 drain the other accumulator with tcgen05.ld and apply
+//     warps 2-9 drain the other accumulator with tcgen05.ld and apply
 //     C -= acc with coalesced column accesses, so the epilogue of tile i
-//     overlaps the MMAs of tile i+1;
+//     overlaps the MMAs of tile i+1.  An update of small K is bound by C's
+//     traffic, so C's columns are loaded ahead: the first group before the
+//     accumulator is ready, the next one before the current one is stored;
 //   * every mbarrier wait is bounded; on expiry the kernel records
 //     CF_ERR_TIMEOUT in a device status word, drains its own copies and
 //     MMAs (again bounded), frees its TMEM and returns.
@@ -38,7 +40,8 @@ using namespace umma;
 
 constexpr int BM = 128, BN = 256, BK = 64, STAGES = 4;
 constexpr int UMMA_K = 16;
-constexpr int kThreads = 192;         // 6 warps
+constexpr int EPI = 8;                // epilogue warps: 4 lane quarters x 2 (32-column groups by turns)
+constexpr int kThreads = 64 + 32 * EPI;
 constexpr uint32_t kStageA = BM * BK * 2;     // 16 KB
 constexpr uint32_t kStageB = BN * BK * 2;     // 32 KB
 constexpr uint32_t kStageBytes = kStageA + kStageB;
@@ -106,7 +109,7 @@ k_schur_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < STAGES; ++i) { mbar_init(&s.full[i], 1); mbar_init(&s.empty[i], 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(&s.acc_full[i], 1); mbar_init(&s.acc_empty[i], 4); }
+        for (int i = 0; i < 2; ++i) { mbar_init(&s.acc_full[i], 1); mbar_init(&s.acc_empty[i], EPI); }
         mbar_init(&s.drain, 1);
         s.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -191,8 +194,9 @@ k_schur_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
             }
         }
     } else {
-        // ------------------------------------------------ epilogue (warps 2..5)
+        // ------------------------------------------------ epilogue (warps 2..9)
         const int quarter = warp & 3;                 // TMEM lanes 32*quarter ..
+        const int half = (warp - 2) >> 2;             // column groups half, half + 2, ...
         int tcount = 0;
         for (int u = blockIdx.x; u < p.nunits; u += gridDim.x) {
             int t, kb0, kb1, m0, n0;
@@ -200,11 +204,6 @@ k_schur_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
             if (!tile_coords(p, t, m0, n0)) continue;
             const int b = tcount & 1;
             const uint32_t aph = (uint32_t)(tcount >> 1) & 1u;
-            bool ok = true;
-            if (lane == 0) ok = wait_bounded(&s.acc_full[b], aph, abort_flag, &g_tc_status);
-            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-            if (!ok) break;
-            tc_fence_after();
             // narrow outputs: the columns of this tile that exist (and, for the
             // lower form, reach the diagonal of the tile's last row)
             int cmax = BN;
@@ -212,11 +211,26 @@ k_schur_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
                 cmax = min(p.nmma, p.n - n0);
                 if (p.lower) cmax = min(cmax, m0 + BM - n0);
             }
+            const int cend = NARROW ? cmax : BN;
+            const int row = m0 + quarter * 32 + lane;
+            const int live = row < p.m ? (p.lower ? min(p.n, row + 1) : p.n) : 0;      // columns this row may touch
+            float *crow = p.C + row;
+            auto load_c = [&](float (&v)[32], int c0) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) v[j] = n0 + c0 + j < live ? crow[(size_t)(n0 + c0 + j) * p.ldc] : 0.f;
+            };
+            float cv[32];
+            if (p.P == nullptr && 32 * half < cend) load_c(cv, 32 * half);
+            bool ok = true;
+            if (lane == 0) ok = wait_bounded(&s.acc_full[b], aph, abort_flag, &g_tc_status);
+            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+            if (!ok) break;
+            tc_fence_after();
             if (p.P != nullptr) {
                 // split-K partial: the accumulator's live columns, column-major
                 float *dst = p.P + ((size_t)(u / p.ntiles) * p.ntiles + t) * (BM * BN) + quarter * 32 + lane;
 #pragma unroll 1
-                for (int c0 = 0; c0 < (NARROW ? cmax : BN); c0 += 32) {
+                for (int c0 = 32 * half; c0 < cend; c0 += 64) {
                     uint32_t r[32];
                     const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * BN + c0);
                     TMEM_LD32(taddr, r);
@@ -230,28 +244,21 @@ k_schur_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
                 ++tcount;
                 continue;
             }
-            const int row = m0 + quarter * 32 + lane;
-            const bool row_ok = row < p.m;
-            float *crow = p.C + row;
 #pragma unroll 1
-            for (int c0 = 0; c0 < (NARROW ? cmax : BN); c0 += 32) {
-                const int colbase = n0 + c0;
-                float cv[32];
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const int col = colbase + j;
-                    const bool ok2 = row_ok && col < p.n && (!p.lower || row >= col);
-                    cv[j] = ok2 ? crow[(size_t)col * p.ldc] : 0.f;
-                }
+            for (int c0 = 32 * half; c0 < cend; c0 += 64) {
                 uint32_t r[32];
                 const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * BN + c0);
                 TMEM_LD32(taddr, r);
+                float nx[32];
+                const bool more = c0 + 64 < cend;
+                if (more) load_c(nx, c0 + 64);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const int col = colbase + j;
-                    const bool ok2 = row_ok && col < p.n && (!p.lower || row >= col);
-                    if (ok2) crow[(size_t)col * p.ldc] = cv[j] - __uint_as_float(r[j]);
+                for (int j = 0; j < 32; ++j)
+                    if (n0 + c0 + j < live) crow[(size_t)(n0 + c0 + j) * p.ldc] = cv[j] - __uint_as_float(r[j]);
+                if (more) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) cv[j] = nx[j];
                 }
             }
             tc_fence_before();
