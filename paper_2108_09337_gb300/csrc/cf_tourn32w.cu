@@ -63,6 +63,8 @@ struct Smem {
     int cont;
     int lab_at[2 * kW];
     int where_[2 * kW];
+    int win[kW];
+    int cnt;
 };
 
 __device__ __forceinline__ unsigned key32u(float a, bool used) {
@@ -277,31 +279,43 @@ __device__ void gepp_select(Smem<NT, RPT> &s, float2 (&a)[RPT][kWP], int w, int 
 // (panel rows in pivot order): winner j moves from its current position to
 // k0 + j.  Positions 0..w-1 are the pivot block, w + j stands for winner j's
 // original row when that row lies below the block.
+// Only the walk over the interchanges is serial (one thread, in shared memory);
+// winners that are all in place already leave nothing to walk.
 template <int NT, int RPT>
-__device__ void root_epilogue(Smem<NT, RPT> &s, const int *win, int np, const TournEpilogue &ep) {
-    if (ep.ipiv == nullptr || threadIdx.x != 0) return;
-    const int w = np;
-    for (int q = 0; q < 2 * w; ++q) { s.lab_at[q] = q; s.where_[q] = q; }
-    for (int j = 0; j < w; ++j) {
-        const int hj = win[j] < w ? win[j] : w + j;
-        const int ps = s.where_[hj];
-        const int p = ps < w ? ps : win[ps - w];
-        ep.ipiv[ep.k0 + j] = ep.k0 + p + 1;
-        if (ps != j) {
-            const int hx = s.lab_at[j];
-            s.lab_at[j] = hj; s.where_[hj] = j;
-            s.lab_at[ps] = hx; s.where_[hx] = ps;
+__device__ void root_epilogue(Smem<NT, RPT> &s, int np, const TournEpilogue &ep) {
+    if (ep.ipiv == nullptr) return;
+    const int w = np, tid = threadIdx.x;
+    if (tid < w) s.win[tid] = s.rows[s.order[tid]];
+    for (int q = tid; q < 2 * w; q += NT) { s.lab_at[q] = q; s.where_[q] = q; }
+    if (tid == 0) s.cnt = 0;
+    if (__syncthreads_and(tid >= w || s.win[tid] == tid)) {
+        if (tid < w) ep.ipiv[ep.k0 + tid] = ep.k0 + tid + 1;
+        if (tid == 0) *ep.swap_cnt = 0;
+        return;
+    }
+    if (tid == 0) {
+        for (int j = 0; j < w; ++j) {
+            const int hj = s.win[j] < w ? s.win[j] : w + j;
+            const int ps = s.where_[hj];
+            const int p = ps < w ? ps : s.win[ps - w];
+            ep.ipiv[ep.k0 + j] = ep.k0 + p + 1;
+            if (ps != j) {
+                const int hx = s.lab_at[j];
+                s.lab_at[j] = hj; s.where_[hj] = j;
+                s.lab_at[ps] = hx; s.where_[hx] = ps;
+            }
         }
     }
-    int cnt = 0;
-    for (int q = 0; q < 2 * w; ++q) {
-        if (s.lab_at[q] == q) continue;
+    __syncthreads();
+    for (int q = tid; q < 2 * w; q += NT) {
         const int hq = s.lab_at[q];
-        ep.swap_dst[cnt] = q < w ? q : win[q - w];
-        ep.swap_src[cnt] = hq < w ? hq : win[hq - w];
-        ++cnt;
+        if (hq == q) continue;
+        const int at = atomicAdd(&s.cnt, 1);     // any order: the moves are applied as one gather
+        ep.swap_dst[at] = q < w ? q : s.win[q - w];
+        ep.swap_src[at] = hq < w ? hq : s.win[hq - w];
     }
-    *ep.swap_cnt = cnt;
+    __syncthreads();
+    if (tid == 0) *ep.swap_cnt = s.cnt;
 }
 
 __device__ __forceinline__ void load_row64(float2 (&a)[kWP], const float *__restrict__ P, int ldp, size_t row, int w,
@@ -353,7 +367,7 @@ k_tourn32w(const float *__restrict__ P, int ldp, TournPlan plan, TournWS ws, Tou
             __syncthreads();
             if (tid < np) ws.root_win[tid] = dst[tid];
             __syncthreads();
-            root_epilogue<NT, RPT>(s, dst, np, ep);
+            root_epilogue<NT, RPT>(s, np, ep);
             return;
         }
     }
@@ -431,7 +445,7 @@ k_tourn32w(const float *__restrict__ P, int ldp, TournPlan plan, TournWS ws, Tou
             __syncthreads();
             if (tid < np) ws.root_win[tid] = dst[tid];
             __syncthreads();
-            root_epilogue<NT, RPT>(s, dst, np, ep);
+            root_epilogue<NT, RPT>(s, np, ep);
             return;
         }
     }
