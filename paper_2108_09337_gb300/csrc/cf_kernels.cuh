@@ -47,6 +47,7 @@ int make_tourn_plan(int m, int w, int h, int arity, TournPlan *plan);
 size_t tourn_ws_bytes(int m, int h, int arity);
 int tourn_ws_carve(void *work, int m, int h, int arity, TournWS *ws, TournEpilogue *ep);
 
+int tourn_take_status(cudaStream_t st, int *status);      // and clears it: a bounded wait ran out
 int launch_tourn(const double *P, int ldp, int m, int w, int h, int arity, const TournWS &ws, const TournEpilogue &ep,
                  cudaStream_t st);
 template <typename T>

@@ -455,7 +455,7 @@ extern "C" int cf_schur_update_lp_splitk(int m, int n, int k, const void *A_lp, 
 }
 
 extern "C" int cf_device_status(cudaStream_t stream) {
-    int s = 0, s8 = 0, st = 0, sr = 0, sl = 0, sv = 0;
+    int s = 0, s8 = 0, st = 0, sr = 0, sl = 0, sv = 0, sw = 0;
     int rc = cf::tc_take_status(stream, &s);
     if (rc != CF_OK) return rc;
     if ((rc = cf::fp8_take_status(stream, &s8)) != CF_OK) return rc;
@@ -463,5 +463,6 @@ extern "C" int cf_device_status(cudaStream_t stream) {
     if ((rc = cf::rtc_take_status(stream, &sr)) != CF_OK) return rc;
     if ((rc = cf::slice64_take_status(stream, &sl)) != CF_OK) return rc;
     if ((rc = cf::solve64_take_status(stream, &sv)) != CF_OK) return rc;
-    return s != 0 ? s : (s8 != 0 ? s8 : (st != 0 ? st : (sr != 0 ? sr : (sl != 0 ? sl : sv))));
+    if ((rc = cf::tourn_take_status(stream, &sw)) != CF_OK) return rc;
+    return s != 0 ? s : (s8 != 0 ? s8 : (st != 0 ? st : (sr != 0 ? sr : (sl != 0 ? sl : (sv != 0 ? sv : sw)))));
 }

@@ -8,19 +8,26 @@
 // equal shares.  The elimination is bound by the FP64 pipe (an element's
 // multiply and subtract take 128 clocks of a quarter SM per 32 lanes), so the
 // cluster size is chosen to put a level on as many SMs as it has: 16 leaves of
-// a 2048-row panel run on 128 SMs, 16 rows each.  Per column:
-//   * the threads that own a row divide by the pivot, update the next column
-//     and take its argmax (redux on the key's bits), which goes straight into
-//     every CTA's slots through distributed shared memory;
-//   * all threads update the other columns, element by element over the rows
-//     still in the race (a list, so that chosen rows cost nothing);
-//   * one cluster barrier; then every warp finds the winner from the slots and
-//     pulls the pivot row from its owner while the multipliers are divided.
-// The eliminated rows of the root's winners are A00's LU, which the root hands
-// to the driver (TournEpilogue::lu).
+// a 2048-row panel run on 128 SMs, 16 rows each.
 //
-// A 2048-row, 128-column panel: 1.0 ms for its three levels (2.5 with one CTA per
-// leaf and all levels in one launch), an 8192-row one 1.9 (3.2).
+// The elimination goes by blocks of 4 columns.  Inside a block only the rows'
+// four entries move, in registers, one row per thread, and nothing but the
+// candidates crosses warps and CTAs: per column each warp sends its best row's
+// four entries (multipliers so far, then the values) and its position into
+// every CTA's slots through distributed shared memory, counted by an mbarrier
+// there; whoever has all slots picks the winner, divides, updates and sends the
+// next.  No barrier over the CTA or the cluster is on this chain, and the warps
+// without rows apply the block before to the other columns beside it.  At the
+// block's end the CTA pulls the four pivot rows' other columns from their
+// owners, brings them up to date among themselves and applies them to the next
+// block's columns; always all four in the order of the columns, so that every
+// element sees the operations of the column-by-column elimination.  The multipliers stay in
+// place: the root's winners carry A00's LU, which the driver takes over
+// (TournEpilogue::lu).
+//
+// Panels of 128 columns: 128 rows 0.28 ms, 2048 rows 1.08 ms, 8192 rows 1.60 ms
+// (column by column, with a cluster barrier and the pivot row pulled per column:
+// 0.32, 1.24, 1.80; one CTA per leaf, all levels in one launch: 0.88, 2.5, 3.2).
 //
 // Every elimination step uses separately rounded multiply and subtract and
 // an IEEE division, in the same order as the FP64 oracle, so a tournament on
@@ -40,17 +47,22 @@ namespace cf {
 constexpr int kTournThreads = 256;
 constexpr int kTournMaxCluster = 16;
 
+constexpr int kTB = 4;                           // columns of a block
+
 struct TournSmem {
-    double prow[kMaxV];                          // pivot row from the current column on
-    double mult[kMaxV];                          // multiplier of each row
-    double slotv[2][4 * kTournMaxCluster];       // candidates of every CTA's warps, by column parity
-    int sloti[2][4 * kTournMaxCluster];          // their stacked positions (-1: none)
-    int act[kMaxV];                              // this CTA's rows still in the race
+    // candidates of every CTA's warps, by column parity: the row's block entries,
+    // then its stacked position (-1: none) as a double's bits
+    alignas(16) double slot[2][4 * kTournMaxCluster][kTB + 2];
+    alignas(16) double stage[4][kTB + 2];        // a warp's candidate on its way out
+    double pin[kTB][kTB];                        // the block's pivots: pin[u][t] = entry t of pivot u
+    double U[kTB][kMaxV];                        // their other columns
+    uint64_t bar[2];                             // all slots of a parity have arrived
+    int act[2][kMaxV];                           // this CTA's rows still in the race, by block parity
     int rows[kMaxV];                             // panel row of each tile row
-    int order[kMaxV];                            // stacked position of each pivot, and its CTA
-    int own[kMaxV];
-    int nact;
-    int hole;                                    // place of the chosen row in act
+    int order[kMaxV];                            // stacked position of each pivot (CTA: modulo the cluster's size)
+    int go[2][kTB];                              // pivot u is not zero, by block parity
+    int nact[2];
+    int out[4];                                  // rows a warp lost in the block
     int lab_at[2 * kMaxV];                       // root epilogue: swap simulation
     int where_[2 * kMaxV];
     int win[kMaxV];
@@ -76,6 +88,50 @@ __device__ __forceinline__ int warp_best(unsigned long long key, int pos) {
     const bool top = hi == mh && lo == ml && key != 0;
     return (int)__reduce_min_sync(0xffffffffu, top ? (unsigned)pos : 0xffffffffu);
 }
+
+__device__ __forceinline__ void named_bar_sync(int id, int threads) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+__device__ int g_tourn_status = 0;               // 0 or CF_ERR_TIMEOUT
+
+// Waits (bounded) until the barrier's phase of this parity has completed; the
+// writes of every arrival are then visible.
+__device__ __forceinline__ void tourn_wait(uint64_t *bar, uint32_t parity) {
+    for (long long i = 0; i < (1ll << 22); ++i) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}\n"
+            : "=r"(ok)
+            : "r"((uint32_t)__cvta_generic_to_shared(bar)), "r"(parity)
+            : "memory");
+        if (ok) return;
+        if (i > 64) __nanosleep(20);
+    }
+    atomicExch(&g_tourn_status, CF_ERR_TIMEOUT);
+}
+
+// One phase more on the barrier: complete once `bytes` have arrived.
+__device__ __forceinline__ void tourn_arm(uint64_t *bar, int bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(bar)),
+                 "r"(bytes)
+                 : "memory");
+}
+// Stores to a CTA of the cluster that count their bytes on its barrier: data and
+// signal in one trip (a release after plain remote stores waits for them first).
+__device__ __forceinline__ void st_async2(uint32_t dst, double a, double b, uint32_t bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(dst),
+                 "l"(__double_as_longlong(a)), "l"(__double_as_longlong(b)), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void st_async1(uint32_t dst, double a, uint32_t bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(dst),
+                 "l"(__double_as_longlong(a)), "r"(bar)
+                 : "memory");
+}
+constexpr int kSlotBytes = 8 * (kTB + 1);
 
 // Shared memory of the largest share (128 rows x 128 columns): the limit that
 // is set for every launch, whatever the launch takes.
@@ -133,13 +189,13 @@ k_tourn_level(TournLevel lv, TournWS ws, TournEpilogue ep) {
     const int w = lv.w, ld = lv.ld;
     int *dst = ws.node_win + (size_t)(lv.off + g) * kMaxV;
 
-    // ---- this CTA's rows: stacked positions [rank * per, rank * per + mine)
-    const int p0 = rank * lv.per;
+    // ---- this CTA's rows: stacked positions rank, rank + ncta, ... (dealt out,
+    // since the rows of one child tend to be chosen together)
     int total = 0, mine = 0;
     if (lv.level == 0) {
         total = min(lv.h, lv.m - g * lv.h);
-        mine = max(0, min(lv.per, total - p0));
-        if (tid < mine) s.rows[tid] = g * lv.h + p0 + tid;
+        mine = total > rank ? (total - rank + ncta - 1) / ncta : 0;
+        if (tid < mine) s.rows[tid] = g * lv.h + rank + tid * ncta;
     } else {
         const int child0 = g * lv.arity, nchild = min(lv.arity, lv.cnt_below - child0);
         if (nchild == 1) {                       // pass-through
@@ -151,138 +207,238 @@ k_tourn_level(TournLevel lv, TournWS ws, TournEpilogue ep) {
             return;
         }
         int at = -1, base = 0;
+        const int want = rank + tid * ncta;
         for (int q = 0; q < nchild; ++q) {
             const int c = ws.node_cnt[lv.off_below + child0 + q];
-            if (p0 + tid >= base && p0 + tid < base + c)
-                at = (lv.off_below + child0 + q) * kMaxV + (p0 + tid - base);
+            if (want >= base && want < base + c) at = (lv.off_below + child0 + q) * kMaxV + (want - base);
             base += c;
         }
         total = base;
-        mine = max(0, min(lv.per, total - p0));
+        mine = total > rank ? (total - rank + ncta - 1) / ncta : 0;
         if (tid < mine) s.rows[tid] = ws.node_win[at];
     }
-    if (tid < kMaxV) s.act[tid] = tid;
-    if (tid == 0) { s.nact = mine; s.bad = 0; }
+    if (tid < kMaxV) s.act[0][tid] = tid;
+    const int npiv = min(total, w);
+    const int nw = (lv.per + 31) / 32, nslots = nw * ncta;      // a slot per warp that has rows
+    if (tid == 0) {
+        s.nact[0] = mine;
+        s.bad = 0;
+        for (int b = 0; b < 2; ++b)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(&s.bar[b])),
+                         "r"(1)
+                         : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
     __syncthreads();
     for (int k = warp; k < w; k += kTournThreads / 32)
         for (int r = lane; r < mine; r += 32) tile[k * ld + r] = lv.P[(size_t)s.rows[r] + (size_t)k * lv.ldp];
-    __syncthreads();
-    const int npiv = min(total, w);
-    const int nw = (lv.per + 31) / 32, nslots = nw * ncta;      // a slot per warp that has rows
+    cl.sync();                                   // every CTA of the cluster is there before it is written to
 
-    // Candidate of this warp's rows in one column, into every CTA's slots.
-    auto publish = [&](int par, bool have, double a, int row) {
-        const int best = warp_best(have ? piv_key(a) : 0ull, p0 + row);
-        const unsigned owner = __ballot_sync(0xffffffffu, have && p0 + row == best);
-        const double v = __shfl_sync(0xffffffffu, a, owner ? __ffs(owner) - 1 : 0);
-        if (lane < ncta) {
-            TournSmem *rs = cl.map_shared_rank(&s, lane);
-            rs->slotv[par][rank * nw + warp] = v;
-            rs->sloti[par][rank * nw + warp] = best;
+    if (tid == 0)
+        for (int b = 0; b < 2; ++b) tourn_arm(&s.bar[b], nslots * kSlotBytes);
+    uint32_t phase = 0;                          // completed phases of the two barriers, bit per parity
+    // Elements [first, last) by `step` of rows list[0 .. na) x columns k0 ..: less the
+    // parts of the four pivots of block jb, in order.
+    auto apply_block = [&](int jb, int par, const int *list, int na, int k0, int ncol, int first, int step) {
+        const unsigned inv = na > 1 ? 0xFFFFFFFFu / (unsigned)na + 1u : 0u;
+        unsigned gos = 0;
+#pragma unroll
+        for (int u = 0; u < kTB; ++u) gos |= s.go[par][u] ? 1u << u : 0u;
+        for (int e = first; e < na * ncol; e += step) {
+            const int c = na > 1 ? (int)__umulhi((unsigned)e, inv) : e;      // e / na
+            const int r = list[e - c * na];
+            const int k = k0 + c;
+            double a = tile[k * ld + r], m[kTB], uk[kTB];
+#pragma unroll
+            for (int u = 0; u < kTB; ++u) {
+                m[u] = tile[(jb + u) * ld + r];
+                uk[u] = s.U[u][k];
+            }
+            if (gos == (1u << kTB) - 1u) {
+#pragma unroll
+                for (int u = 0; u < kTB; ++u) a = sub_rn(a, mul_rn(m[u], uk[u]));
+            } else {
+#pragma unroll
+                for (int u = 0; u < kTB; ++u)
+                    if (gos >> u & 1u) a = sub_rn(a, mul_rn(m[u], uk[u]));
+            }
+            tile[k * ld + r] = a;
         }
     };
-    if (ncta > 1) cl.sync();                     // every CTA of the cluster runs before it is written to
-    if (warp < nw) publish(0, tid < mine, tid < mine ? tile[tid] : 0.0, tid);
-
-    for (int j = 0; j < npiv; ++j) {
-        if (ncta > 1) cl.sync(); else __syncthreads();
-        // ---- (1) the winner, found by every warp alike
-        const int par = j & 1;
-        int gi, owner;
-        double piv;
-        {
-            int at = lane, pos = lane < nslots ? s.sloti[par][lane] : -1;
-            double v = pos >= 0 ? s.slotv[par][lane] : 0.0;
-            unsigned long long key = pos >= 0 ? piv_key(v) : 0ull;
-            if (nslots > 32) {
-                const int i1 = lane + 32 < nslots ? s.sloti[par][lane + 32] : -1;
-                const double v1 = i1 >= 0 ? s.slotv[par][lane + 32] : 0.0;
-                const unsigned long long k1 = i1 >= 0 ? piv_key(v1) : 0ull;
-                if (k1 > key || (k1 == key && k1 != 0 && i1 < pos)) { key = k1; pos = i1; v = v1; at = lane + 32; }
-            }
-            gi = warp_best(key, pos);
-            const int src = __ffs(__ballot_sync(0xffffffffu, pos == gi)) - 1;
-            piv = __shfl_sync(0xffffffffu, v, src);
-            owner = __shfl_sync(0xffffffffu, at / nw, src);
-        }
-        const bool go = !is_zero(piv);           // a zero pivot eliminates nothing
-        const int lrow = gi - owner * lv.per;
-        // ---- (2) pivot row from its owner; meanwhile the multipliers
-        double pr = 0.0;
-        const bool pull = tid < w - j;
-        if (pull) {
-            const double *src = ncta > 1 ? cl.map_shared_rank(tile, owner) : tile;
-            pr = src[(size_t)(j + tid) * ld + lrow];
-        }
-        const int nact = s.nact;
-        const bool mine_won = owner == rank;
-        int row = -1;
-        double l = 0.0;
-        if (tid < nact) {
-            row = s.act[tid];
-            if (mine_won && row == lrow) {
-                s.hole = tid;
-                row = -1;
-            }
-            if (row >= 0 && go) {
-                l = div_rn(tile[j * ld + row], piv);
-                tile[j * ld + row] = l;
-                s.mult[row] = l;
-            }
-        }
-        if (pull) s.prow[j + tid] = pr;
-        if (tid == 0) { s.order[j] = gi; s.own[j] = owner; }
-        if (!go && tid == 0) s.bad = 1;
-        __syncthreads();
-        const int jn = j + 1;
-        // ---- (3) the next column and its candidates; the chosen row leaves the list
-        if (mine_won && tid == kTournThreads - 1) {
-            s.act[s.hole] = s.act[nact - 1];
-            s.nact = nact - 1;
-        }
-        if (warp < nw && jn < npiv) {
-            double a = 0.0;
-            if (row >= 0) {
-                a = tile[jn * ld + row];
-                if (go) {
-                    a = sub_rn(a, mul_rn(l, s.prow[jn]));
-                    tile[jn * ld + row] = a;
+    __syncthreads();
+    for (int j0 = 0, cur = 0; j0 < npiv; j0 += kTB, cur ^= 1) {
+        // Here the rows of act[cur] have every earlier block's part in this block's
+        // columns, and all but the last block's in the columns right of it.
+        const int cb = min(kTB, npiv - j0);
+        const int nact = s.nact[cur];
+        if (warp >= nw) {
+            // ---- the last block's part, beside this block's chain
+            if (j0 > 0)
+                apply_block(j0 - kTB, cur ^ 1, s.act[cur], nact, j0 + kTB, w - j0 - kTB, tid - 32 * nw,
+                            kTournThreads - 32 * nw);
+        } else {
+            // ---- the block's columns: this thread's row, its entries j0 .. j0 + 3
+            bool live = tid < nact;
+            const int row = live ? s.act[cur][tid] : 0;
+            const int pos = rank + row * ncta;
+            double x[kTB];
+#pragma unroll
+            for (int t = 0; t < kTB; ++t) x[t] = (live && j0 + t < w) ? tile[(j0 + t) * ld + row] : 0.0;
+            bool lost = false;
+#pragma unroll 1
+            for (int u = 0; u <= cb; ++u) {
+                double l = 0.0;
+                if (u > 0) {
+                    // ---- the winner of column j0 + u - 1, found by every warp alike
+                    const int par = (j0 + u - 1) & 1;
+                    tourn_wait(&s.bar[par], (phase >> par) & 1u);
+                    phase ^= 1u << par;
+                    // (armed again before this warp's next candidate goes out, which
+                    // every sender of the next but one waits for)
+                    if (tid == 0) tourn_arm(&s.bar[par], nslots * kSlotBytes);
+                    int at = lane, best = lane < nslots ? (int)__double_as_longlong(s.slot[par][lane][kTB]) : -1;
+                    unsigned long long key = best >= 0 ? piv_key(s.slot[par][lane][u - 1]) : 0ull;
+                    if (nslots > 32) {
+                        const int i1 = lane + 32 < nslots ? (int)__double_as_longlong(s.slot[par][lane + 32][kTB]) : -1;
+                        const unsigned long long k1 = i1 >= 0 ? piv_key(s.slot[par][lane + 32][u - 1]) : 0ull;
+                        if (k1 > key || (k1 == key && k1 != 0 && i1 < best)) { key = k1; best = i1; at = lane + 32; }
+                    }
+                    const int gi = warp_best(key, best);
+                    at = __shfl_sync(0xffffffffu, at, __ffs(__ballot_sync(0xffffffffu, best == gi)) - 1);
+                    const double *pv = s.slot[par][at];
+                    const double piv = pv[u - 1];
+                    const bool go = !is_zero(piv);           // a zero pivot eliminates nothing
+                    if (live && pos == gi) {
+                        live = false;
+                        lost = true;
+                    }
+                    if (warp == 0) {
+                        if (lane < kTB) s.pin[u - 1][lane] = pv[lane];
+                        if (lane == 0) {
+                            s.order[j0 + u - 1] = gi;
+                            s.go[cur][u - 1] = go;
+                            if (!go) s.bad = 1;
+                        }
+                    }
+                    // ---- multiplier (kept in the entry) and the later entries
+                    if (live && go) {
+                        double a = x[0];
+#pragma unroll
+                        for (int t = 1; t < kTB; ++t) a = t == u - 1 ? x[t] : a;
+                        l = div_rn(a, piv);
+#pragma unroll
+                        for (int t = 0; t < kTB; ++t) x[t] = t == u - 1 ? l : x[t];
+                        switch (u) {             // entries u .. 3
+                            case 1: x[1] = sub_rn(x[1], mul_rn(l, pv[1])); [[fallthrough]];
+                            case 2: x[2] = sub_rn(x[2], mul_rn(l, pv[2])); [[fallthrough]];
+                            case 3: x[3] = sub_rn(x[3], mul_rn(l, pv[3])); [[fallthrough]];
+                            default: break;
+                        }
+                    }
+                    __syncwarp();
+                }
+                if (u == cb) break;
+                // ---- this warp's candidate for column j0 + u, into every CTA's slots
+                double a = x[0];
+#pragma unroll
+                for (int t = 1; t < kTB; ++t) a = t == u ? x[t] : a;
+                const int best = warp_best(live ? piv_key(a) : 0ull, pos);
+                if (best < 0 ? lane == 0 : (live && pos == best)) {
+#pragma unroll
+                    for (int t = 0; t < kTB; ++t) s.stage[warp][t] = x[t];
+                    s.stage[warp][kTB] = __longlong_as_double((long long)best);
+                }
+                __syncwarp();
+                const int par = (j0 + u) & 1;
+                // lane = (CTA, half): asynchronous stores that count on the CTA's barrier
+                {
+                    const int cta = lane >> 1, half = lane & 1;
+                    if (cta < ncta) {
+                        uint32_t dst, bar;
+                        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                                     : "=r"(dst)
+                                     : "r"((uint32_t)__cvta_generic_to_shared(&s.slot[par][rank * nw + warp][0])), "r"(cta));
+                        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                                     : "=r"(bar)
+                                     : "r"((uint32_t)__cvta_generic_to_shared(&s.bar[par])), "r"(cta));
+                        const double *st = s.stage[warp];
+                        st_async2(dst + 16 * half, st[2 * half], st[2 * half + 1], bar);
+                        if (half == 0) st_async1(dst + 8 * kTB, st[kTB], bar);
+                    }
                 }
             }
-            publish(jn & 1, row >= 0, a, row);
-        } else if (row >= 0 && jn < w && go) {       // the last pivot of a node with fewer rows than columns
-            tile[jn * ld + row] = sub_rn(tile[jn * ld + row], mul_rn(l, s.prow[jn]));
+            // ---- the rows back, the list without the chosen ones
+            if (tid < nact) {
+#pragma unroll
+                for (int t = 0; t < kTB; ++t)
+                    if (j0 + t < w) tile[(j0 + t) * ld + row] = x[t];
+            }
+            const unsigned gone = __ballot_sync(0xffffffffu, lost);
+            if (lane == 0) s.out[warp] = __popc(gone);
+            named_bar_sync(1, 32 * nw);
+            int before = 0;
+            for (int q = 0; q < warp; ++q) before += s.out[q];
+            int all = 0;
+            for (int q = 0; q < nw; ++q) all += s.out[q];
+            if (tid < nact && !lost) s.act[cur ^ 1][tid - before - __popc(gone & ((1u << lane) - 1u))] = row;
+            if (tid == 0) s.nact[cur ^ 1] = nact - all;
         }
         __syncthreads();
-        // ---- (4) the other columns
-        if (go) {
-            const int na = s.nact, tot = na * (w - jn - 1);
-            const unsigned inv = na > 1 ? 0xFFFFFFFFu / (unsigned)na + 1u : 0u;
-#pragma unroll 4
-            for (int e = tid; e < tot; e += kTournThreads) {
-                const int c = na > 1 ? (int)__umulhi((unsigned)e, inv) : e;      // e / na
-                const int r = s.act[e - c * na];
-                const int k = jn + 1 + c;
-                tile[k * ld + r] = sub_rn(tile[k * ld + r], mul_rn(s.mult[r], s.prow[k]));
+        const int k1 = j0 + kTB;                 // first column right of the block
+        if (k1 >= w || k1 >= npiv) {
+            if (lv.root && rank == 0 && ep.lu != nullptr && npiv == w)
+                for (int e = tid; e < kTB * kTB; e += kTournThreads)
+                    if (e / kTB < cb && j0 + e % kTB < w) ep.lu[(j0 + e / kTB) + (size_t)(j0 + e % kTB) * kMaxV] = s.pin[e / kTB][e % kTB];
+            break;                               // no selection left
+        }
+        if (ncta > 1) cl.sync();                 // every CTA's rows have the last block's part
+        // ---- the pivot rows' other columns, a column per thread: as they were at
+        // the block's start, then each less the earlier ones' parts
+        if (tid < w - k1) {
+            const int k = k1 + tid;
+            double v[kTB];
+#pragma unroll
+            for (int u = 0; u < kTB; ++u) {
+                const int own = s.order[j0 + u] % ncta;
+                v[u] = cl.map_shared_rank(tile, own)[(size_t)k * ld + s.order[j0 + u] / ncta];
+            }
+#pragma unroll
+            for (int u = 1; u < kTB; ++u)
+#pragma unroll
+                for (int t = 0; t < u; ++t)
+                    if (s.go[cur][t]) v[u] = sub_rn(v[u], mul_rn(s.pin[u][t], v[t]));
+#pragma unroll
+            for (int u = 0; u < kTB; ++u) s.U[u][k] = v[u];
+            if (lv.root && rank == 0 && ep.lu != nullptr && npiv == w) {
+#pragma unroll
+                for (int u = 0; u < kTB; ++u) ep.lu[(j0 + u) + (size_t)k * kMaxV] = v[u];
             }
         }
+        if (lv.root && rank == 0 && ep.lu != nullptr && npiv == w)
+            for (int e = tid; e < kTB * kTB; e += kTournThreads)
+                ep.lu[(j0 + e / kTB) + (size_t)(j0 + e % kTB) * kMaxV] = s.pin[e / kTB][e % kTB];
+        __syncthreads();
+        // ---- their part in the next block's columns (the rest goes beside its chain)
+        apply_block(j0, cur, s.act[cur ^ 1], s.nact[cur ^ 1], k1, min(kTB, w - k1), tid, kTournThreads);
+        __syncthreads();
     }
     __syncthreads();
     for (int j = tid; j < npiv; j += kTournThreads) {
         const int gi = s.order[j];
-        if (s.own[j] == rank) {
-            const int r = s.rows[gi - rank * lv.per];
+        if (gi % ncta == rank) {
+            const int r = s.rows[gi / ncta];
             dst[j] = r;
             if (lv.root) ws.root_win[j] = r;
         }
     }
     if (rank == 0 && tid == 0) ws.node_cnt[lv.off + g] = npiv;
     if (lv.root && ep.lu != nullptr) {
-        // the winners' eliminated rows are the LU of A00 in pivot order
+        // A00's LU in pivot order: the multipliers of earlier blocks are with the
+        // winners' rows, the rest was written block by block
         for (int j = warp; j < npiv; j += kTournThreads / 32) {
-            const int gi = s.order[j];
-            if (s.own[j] != rank) continue;
-            for (int k = lane; k < w; k += 32) ep.lu[j + (size_t)k * kMaxV] = tile[k * ld + (gi - rank * lv.per)];
+            if (s.order[j] % ncta != rank) continue;
+            const int r = s.order[j] / ncta;
+            for (int k = lane; k < j / kTB * kTB; k += 32) ep.lu[j + (size_t)k * kMaxV] = tile[k * ld + r];
         }
         if (rank == 0 && tid == 0) *ep.lu_ok = s.bad == 0 && npiv == w;
     }
@@ -478,6 +634,19 @@ int launch_tourn(const double *P, int ldp, int m, int w, int h, int arity, const
         CF_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_tourn_level, lv, ws, ep));
         count_launches(1);
     }
+    return CF_OK;
+}
+
+int tourn_take_status(cudaStream_t st, int *status) {
+    int h = 0;
+    CF_CUDA_TRY(cudaMemcpyFromSymbolAsync(&h, g_tourn_status, sizeof(int), 0, cudaMemcpyDeviceToHost, st));
+    CF_CUDA_TRY(cudaStreamSynchronize(st));
+    if (h != 0) {
+        const int zero = 0;
+        CF_CUDA_TRY(cudaMemcpyToSymbolAsync(g_tourn_status, &zero, sizeof(int), 0, cudaMemcpyHostToDevice, st));
+        CF_CUDA_TRY(cudaStreamSynchronize(st));
+    }
+    *status = h;
     return CF_OK;
 }
 
