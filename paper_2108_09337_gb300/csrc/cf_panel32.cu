@@ -1,15 +1,15 @@
 // cf_panel32.cu -- FP32 block routines of the mixed-precision path, built for
 // latency (they sit on the chain of dependent work of every step):
 //
-//   k_a00_lu_q32,   LU of A00 without pivoting (Fig. "prog_rep" on
+//   k_a00_lu_g64,   LU of A00 without pivoting (Fig. "prog_rep" on
 //   k_a00_lu32      the rows TournPivot selected; Sec. 7.2)
 //   k_a00_chol32    Cholesky of A00 (Listing "Cholesky Factorization"; CH-1)
 //   k_rtrsm32(_w)   LU-3  A10 <- A10 U00^{-1}  /  CH-2  L10 <- A10 L00^{-T}
 //   k_ltrsm32(_w)   LU-4  A01 <- L00^{-1} A01
 //
-// The A00 kernels: one thread per row (four lanes per row for LU blocks of
-// up to 64 rows), the row in registers with compile-time indices, one
-// barrier per column.
+// The A00 kernels: a grid of threads with a few rows and columns each in
+// registers, one barrier per column (LU blocks of more than 64 rows: one
+// thread per row).
 // The panel solves: one thread per row (LU-3, CH-2) or column (LU-4), held
 // as float2 pairs updated with packed FMAs, no barrier, results written
 // straight from registers; they also write the BF16/FP16 K-major copies that
@@ -36,81 +36,73 @@ template <>
 __device__ __forceinline__ __half lp_from<__half>(float x) { return __float2half_rn(x); }
 
 // ---------------------------------------------------------------------------
-// A00 LU of blocks of up to 64 rows, four lanes per row: lane q of row r
-// holds the row's columns 16q .. 16q + 15, one barrier per column.  With one
-// thread per row (below) a 64 x 64 LU issued ~10,000 instructions per warp
-// on two warps (ncu: 24 us per launch, 19% issue active, 1.8 cycles of
-// fixed-latency wait per issue); split four ways over eight warps it takes
-// 18.7 us against 26.2 (measured alone).  For 128 rows the quartered rows
-// (32 columns a lane, the column loop unrolled 32 times) measured slower
-// than one thread per row (83 against 53 us), and so did the same form of
-// the Cholesky (108 against 51 us at 128 rows): those keep the kernels
-// below.
+// A00 LU of blocks of up to 64 rows (Fig. "prog_rep" on the rows TournPivot
+// selected, Sec. 7.2), in place, without pivoting: 256 threads hold the block
+// as 4 x 4 elements each, rows ty + 16 i, columns tx + 16 j.  For every column k
+// the threads of column k and of row k publish them as they are, one barrier,
+// and every thread divides its rows' entries by the pivot itself and does
+// a(r, j) -= l a(k, j).  A zero pivot is reported in info and its column is not
+// divided (LAPACK dgetf2); the elimination then goes on with the undivided
+// column.
 //
-// LU without pivoting (Fig. "prog_rep" on the rows TournPivot
-// selected, Sec. 7.2), in place: for every column k, row k (final from
-// column k on) is published in shared memory; every row r > k takes
-// l = a(r, k) / a(k, k) (its lane holding column k divides and hands l to
-// the other three) and does a(r, j) -= l a(k, j) for j > k.  A zero pivot
-// is reported in info and its column is not divided (LAPACK dgetf2); the
-// elimination then goes on with the undivided column.
+// A chain of w column steps on one SM: the barrier, a shared-memory read, the
+// division and the update are what it takes.  The loop over the 16 columns of a
+// column group stays rolled: with the columns unrolled (four lanes per row, 16.4
+// us) every instruction is fetched once and used once.  12.3 us at w = 64.
 // ---------------------------------------------------------------------------
-template <int R>
-__global__ void __launch_bounds__(4 * R, 1) k_a00_lu_q32(float *A00, int lda, int w, int kglob, int *info) {
-    constexpr int T = 4, C = R / T;
-    __shared__ __align__(16) float prow[2][R];
-    const int tid = threadIdx.x, r = tid / T, q = tid % T, lane = tid & 31;
-    const int base = lane - q, c0 = q * C;
-    const bool row_live = r < w;
-    float a[C];
+__global__ void __launch_bounds__(256, 1) k_a00_lu_g64(float *A00, int lda, int w, int kglob, int *info) {
+    __shared__ float col[2][64], row[2][64];
+    const int tid = threadIdx.x, ty = tid & 15, tx = tid >> 4;
+    float a[4][4];
 #pragma unroll
-    for (int jl = 0; jl < C; ++jl) a[jl] = (row_live && c0 + jl < w) ? A00[(size_t)r + (size_t)(c0 + jl) * lda] : 0.f;
-    if (r == 0) {
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int g = 0; g < C / 4; ++g)
-            *reinterpret_cast<float4 *>(&prow[0][c0 + 4 * g]) =
-                make_float4(a[4 * g], a[4 * g + 1], a[4 * g + 2], a[4 * g + 3]);
-    }
-    __syncthreads();
-    for (int qo = 0; qo < T; ++qo) {
-        if (qo * C >= w) break;
+        for (int j = 0; j < 4; ++j) {
+            const int r = ty + 16 * i, c = tx + 16 * j;
+            a[i][j] = (r < w && c < w) ? A00[(size_t)r + (size_t)c * lda] : 0.f;
+        }
 #pragma unroll
-        for (int kl = 0; kl < C; ++kl) {
-            const int k = qo * C + kl;
+    for (int kb = 0; kb < 4; ++kb) {
+#pragma unroll 1
+        for (int kk = 0; kk < 16; ++kk) {
+            const int k = 16 * kb + kk, par = kk & 1;
             if (k >= w) break;
-            const float *u = prow[k & 1];
-            const float piv = u[k];
-            const bool upd = row_live && r > k;
-            float l = 0.f;
-            if (upd && q == qo) l = (piv != 0.f) ? a[kl] / piv : a[kl];
-            l = __shfl_sync(0xffffffffu, l, base + qo);
-            if (upd) {
-                if (q == qo) a[kl] = l;                           // L(r, k)
-                float m[C];
+            if (tx == kk) {
 #pragma unroll
-                for (int g = 0; g < C / 4; ++g) {
-                    const float4 v = *reinterpret_cast<const float4 *>(u + c0 + 4 * g);
-                    m[4 * g] = v.x; m[4 * g + 1] = v.y; m[4 * g + 2] = v.z; m[4 * g + 3] = v.w;
-                }
-#pragma unroll
-                for (int jl = 0; jl < C; ++jl)
-                    if (q > qo || (q == qo && jl > kl)) a[jl] = fmaf(-l, m[jl], a[jl]);
+                for (int i = kb; i < 4; ++i) col[par][ty + 16 * i] = a[i][kb];
             }
-            if (r == k + 1 && k + 1 < w) {                         // the next pivot row, final from k + 1 on
+            if (ty == kk) {
 #pragma unroll
-                for (int g = 0; g < C / 4; ++g)
-                    *reinterpret_cast<float4 *>(&prow[(k + 1) & 1][c0 + 4 * g]) =
-                        make_float4(a[4 * g], a[4 * g + 1], a[4 * g + 2], a[4 * g + 3]);
+                for (int j = kb; j < 4; ++j) row[par][tx + 16 * j] = a[kb][j];
             }
-            if (tid == 0 && piv == 0.f) atomicCAS(info, 0, kglob + k + 1);
             __syncthreads();
+            const float piv = row[par][k];
+            if (tid == 0 && piv == 0.f) atomicCAS(info, 0, kglob + k + 1);
+            float l[4], u[4];
+#pragma unroll
+            for (int i = kb; i < 4; ++i) {
+                l[i] = col[par][ty + 16 * i];
+                if (piv != 0.f) l[i] = l[i] / piv;
+            }
+#pragma unroll
+            for (int j = kb; j < 4; ++j) u[j] = row[par][tx + 16 * j];
+#pragma unroll
+            for (int i = kb; i < 4; ++i) {
+                const bool below = i > kb || ty > kk;
+                if (below && tx == kk) a[i][kb] = l[i];
+#pragma unroll
+                for (int j = kb; j < 4; ++j)
+                    if (below && (j > kb || tx > kk)) a[i][j] = fmaf(-l[i], u[j], a[i][j]);
+            }
         }
     }
-    if (row_live) {
 #pragma unroll
-        for (int jl = 0; jl < C; ++jl)
-            if (c0 + jl < w) A00[(size_t)r + (size_t)(c0 + jl) * lda] = a[jl];
-    }
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int r = ty + 16 * i, c = tx + 16 * j;
+            if (r < w && c < w) A00[(size_t)r + (size_t)c * lda] = a[i][j];
+        }
 }
 
 // ---------------------------------------------------------------------------
@@ -266,107 +258,113 @@ __global__ void __launch_bounds__(kMaxV, 1) k_a00_lu32(float *A00, int lda, int 
 }
 
 // ---------------------------------------------------------------------------
-// A00 = L00 L00^T (lower), in place.  Thread r owns row r (pair row), blocked
-// by 8 columns: for column k = j0 + U every live row r >= k publishes its
-// entry a(r, k) (the column k of the Schur complement, kept for the block);
-// barrier; L(k, k) = sqrt(a(k, k)), every row r > k stores L(r, k) and
-// updates its in-block columns; at the block end every row below the block
-// applies the rank-8 update a(r, t) -= sum_U L(r, U) L(t, U) for the columns
-// t past the block (L(t, U) = the published a(t, U) / L(U, U)), with no
-// barrier (the column buffers alternate between blocks).  Stops at the first
-// pivot that is not positive (info).
+// A00 = L00 L00^T (lower), in place: 512 threads hold the block as 4 x 8 elements
+// each, rows lane + 32 i, columns warp + 16 j.  A column belongs to one warp,
+// which takes its pivot by shuffle, the root, the division of its rows and
+// publishes the column of L; one barrier per column; the warp of the next column
+// updates that one first and goes straight on to its root.  Stops at the first
+// pivot that is not positive (info); then nothing is written.  The loop over the
+// 16 columns of a column group stays rolled (one thread per row with unrolled
+// blocks of 8 columns: 49 us at w = 128; this: 41 us).
 // ---------------------------------------------------------------------------
 struct A00CholSmem {
-    float4 col[2][kBlk][kMaxV / 4 + 1];   // [block parity][U][relative row]
+    float l[2][kMaxV];
+    int fail;       // the column whose pivot failed (w: none yet)
 };
 
-struct CholStep {
-    A00CholSmem &s;
-    float2 (&a)[kPairs];
-    float (&lb)[kBlk];                    // L(r, U) / L(U, U)
-    float *A00;
-    int lda, w, r, kglob;
-    int *info;
-    bool failed;
-    template <int U>
-    __device__ __forceinline__ void step(int j0) {
-        if (failed) return;                          // uniform
-        const int k = j0 + U, bp = (j0 / kBlk) & 1;
-        float *cf = reinterpret_cast<float *>(s.col[bp][U]);
-        const float au = pair_elem<U>(a);
-        if (r >= k && r < w) cf[r - j0] = au;        // column k by relative row
-        __syncthreads();
-        const float d = cf[U];
-        if (!(d > 0.f)) {
-            if (r == 0) atomicCAS(info, 0, kglob + k + 1);
-            failed = true;                           // every thread read the same d
-            return;
+// The finished column k (entries a[.][J] of this warp): root, division, out.
+template <int J>
+__device__ __forceinline__ void chol_column(A00CholSmem &s, float (&a)[4][8], int k, int lane, int kglob, int *info) {
+    float d = 0.f;
+#pragma unroll
+    for (int i = J / 2; i < 4; ++i) {              // rows 16 J .. : the diagonal lies in group i = k / 32 = J / 2
+        if (i == J / 2) d = __shfl_sync(0xffffffffu, a[i][J], k & 31);
+    }
+    if (!(d > 0.f)) {
+        if (lane == 0) {
+            atomicCAS(info, 0, kglob + k + 1);
+            s.fail = k;
         }
-        const float lkk = sqrtf(d);
-        if (r == k) A00[(size_t)k + (size_t)k * lda] = lkk;
-        if (r > k && r < w) {
-            const float l = au / lkk;
-            A00[(size_t)r + (size_t)k * lda] = l;                               // L(r, k)
-            // a(r, j0+t) -= L(r,k) L(j0+t,k) = (l / lkk) col[t]
-            const float cl = l / lkk;
-            lb[U] = cl;
-            const float2 nl = make_float2(-cl, -cl);
-            const float4 u0 = s.col[bp][U][0], u1 = s.col[bp][U][1];
-            if (1 > U) a[0] = __ffma2_rn(nl, make_float2(u0.x, u0.y), a[0]);
-            if (3 > U) a[1] = __ffma2_rn(nl, make_float2(u0.z, u0.w), a[1]);
-            if (5 > U) a[2] = __ffma2_rn(nl, make_float2(u1.x, u1.y), a[2]);
-            if (7 > U) a[3] = __ffma2_rn(nl, make_float2(u1.z, u1.w), a[3]);
+        return;
+    }
+    const float root = sqrtf(d);
+#pragma unroll
+    for (int i = J / 2; i < 4; ++i) {
+        const int r = lane + 32 * i;
+        const float l = r == k ? root : a[i][J] / root;
+        if (r >= k) {
+            a[i][J] = l;
+            s.l[k & 1][r] = l;
         }
     }
-    __device__ __forceinline__ void block_end(int j0) {
-        if (failed) return;
-        const int bp = (j0 / kBlk) & 1;
-        const int lim = r - j0 + 1;                  // columns up to the diagonal
-        if (r >= j0 + kBlk && r < w) {
-#pragma unroll
-            for (int u = 0; u < kBlk; ++u) {
-                const float2 nc = make_float2(-lb[u], -lb[u]);
-#pragma unroll
-                for (int ch = 0; ch < 4; ++ch)
-                    if (ch * 32 < lim) {
-#pragma unroll
-                        for (int q = ch * 8; q < ch * 8 + 8; ++q) {
-                            if (q < 2) continue;
-                            const float4 p = s.col[bp][u][q];
-                            a[2 * q] = __ffma2_rn(nc, make_float2(p.x, p.y), a[2 * q]);
-                            a[2 * q + 1] = __ffma2_rn(nc, make_float2(p.z, p.w), a[2 * q + 1]);
-                        }
-                    }
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < kBlk; ++u) lb[u] = 0.f;
-    }
-};
+}
 
-__global__ void __launch_bounds__(kMaxV, 1) k_a00_chol32(float *A00, int lda, int w, int kglob, int *info) {
+// Column k = 16 KB + kk applied; the next column is entry JN of warp (kk + 1) % 16.
+template <int KB, int JN>
+__device__ __forceinline__ bool chol_step(A00CholSmem &s, float (&a)[4][8], int kk, int w, int lane, int warp, int kglob,
+                                          int *info) {
+    const int k = 16 * KB + kk;
+    __syncthreads();
+    if (s.fail <= k) return false;     // (a failure of column k + 1 may be there already: next step)
+    const float *lc = s.l[k & 1];
+    float lr[4];
+#pragma unroll
+    for (int i = KB / 2; i < 4; ++i) lr[i] = lc[lane + 32 * i];
+    const bool next = warp == ((kk + 1) & 15) && k + 1 < w;
+    if (JN < 8 && next) {
+        const float c = lc[warp + 16 * JN];
+#pragma unroll
+        for (int i = JN / 2; i < 4; ++i) a[i][JN] = fmaf(-lr[i], c, a[i][JN]);
+        chol_column<(JN < 8 ? JN : 7)>(s, a, k + 1, lane, kglob, info);
+    }
+#pragma unroll
+    for (int j = KB; j < 8; ++j) {
+        if (j == JN && next) continue;
+        if (j == KB && warp <= kk) continue;       // finished columns
+        const float c = lc[warp + 16 * j];
+#pragma unroll
+        for (int i = j / 2; i < 4; ++i) a[i][j] = fmaf(-lr[i], c, a[i][j]);
+    }
+    return true;
+}
+
+template <int KB>
+__device__ __forceinline__ bool chol_group(A00CholSmem &s, float (&a)[4][8], int w, int lane, int warp, int kglob,
+                                           int *info) {
+#pragma unroll 1
+    for (int kk = 0; kk < 15; ++kk) {
+        if (16 * KB + kk >= w) return true;
+        if (!chol_step<KB, KB>(s, a, kk, w, lane, warp, kglob, info)) return false;
+    }
+    if (16 * KB + 15 >= w) return true;
+    if (!chol_step<KB, KB + 1>(s, a, 15, w, lane, warp, kglob, info)) return false;
+    if constexpr (KB < 7) return chol_group<KB + 1>(s, a, w, lane, warp, kglob, info);
+    return true;
+}
+
+__global__ void __launch_bounds__(512, 1) k_a00_chol32(float *A00, int lda, int w, int kglob, int *info) {
     if (*info != 0) return;
-    __shared__ __align__(16) A00CholSmem s;
-    const int r = threadIdx.x;
-    float2 a[kPairs];
-    float lb[kBlk];
+    __shared__ A00CholSmem s;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float a[4][8];
 #pragma unroll
-    for (int u = 0; u < kBlk; ++u) lb[u] = 0.f;
-    load_pair_row(a, A00, lda, r, w);
-    CholStep body{s, a, lb, A00, lda, w, r, kglob, info, false};
-    for (int j0 = 0; j0 < w; j0 += kBlk) {
-        body.template step<0>(j0);
-        if (j0 + 1 < w) body.template step<1>(j0);
-        if (j0 + 2 < w) body.template step<2>(j0);
-        if (j0 + 3 < w) body.template step<3>(j0);
-        if (j0 + 4 < w) body.template step<4>(j0);
-        if (j0 + 5 < w) body.template step<5>(j0);
-        if (j0 + 6 < w) body.template step<6>(j0);
-        if (j0 + 7 < w) body.template step<7>(j0);
-        if (j0 + kBlk >= w) break;
-        body.block_end(j0);
-        shift_pairs(a, w - j0 - kBlk);
-    }
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int r = lane + 32 * i, c = warp + 16 * j;
+            a[i][j] = (r < w && c <= r) ? A00[(size_t)r + (size_t)c * lda] : 0.f;
+        }
+    if (threadIdx.x == 0) s.fail = w;
+    __syncthreads();
+    if (warp == 0) chol_column<0>(s, a, 0, lane, kglob, info);
+    if (!chol_group<0>(s, a, w, lane, warp, kglob, info)) return;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int r = lane + 32 * i, c = warp + 16 * j;
+            if (r < w && c <= r) A00[(size_t)r + (size_t)c * lda] = a[i][j];
+        }
 }
 
 // Packs 8 consecutive values as low-precision and stores them as one 16-byte
@@ -745,12 +743,12 @@ k_ltrsm32_w(float *X, int ldx, int cols, const float *__restrict__ L00, int ldl,
 }
 
 // ---------------------------------------------------------------------------
-// One CTA: four lanes per row for LU blocks of up to 64 rows (256 threads),
+// One CTA: a grid of 4 x 4 elements per thread for LU blocks of up to 64 rows,
 // else one thread per row in whole warps.
 int launch_a00_lu32(float *A00, int lda, int w, int kglob, int *info, cudaStream_t st) {
     if (w <= 0) return CF_OK;
     if (w > kMaxV) return CF_ERR_UNSUPPORTED;
-    if (w <= 64) k_a00_lu_q32<64><<<1, 256, 0, st>>>(A00, lda, w, kglob, info);
+    if (w <= 64) k_a00_lu_g64<<<1, 256, 0, st>>>(A00, lda, w, kglob, info);
     else k_a00_lu32<<<1, (w + 31) / 32 * 32, 0, st>>>(A00, lda, w, kglob, info);
     CF_LAUNCH_CHECK();
     return CF_OK;
@@ -759,7 +757,7 @@ int launch_a00_lu32(float *A00, int lda, int w, int kglob, int *info, cudaStream
 int launch_a00_chol32(float *A00, int lda, int w, int kglob, int *info, cudaStream_t st) {
     if (w <= 0) return CF_OK;
     if (w > kMaxV) return CF_ERR_UNSUPPORTED;
-    k_a00_chol32<<<1, (w + 31) / 32 * 32, 0, st>>>(A00, lda, w, kglob, info);
+    k_a00_chol32<<<1, 512, 0, st>>>(A00, lda, w, kglob, info);
     CF_LAUNCH_CHECK();
     return CF_OK;
 }
