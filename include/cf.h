@@ -182,8 +182,8 @@ long long cf_kernel_launches(void);
  * Leaves are leaf_h consecutive rows; each playoff node stacks the winners
  * of `arity` adjacent children (original panel values) and keeps min(rows, w)
  * by partial-pivoting elimination; ties go to the smallest stacked position.
- * w <= 128, 1 <= leaf_h <= 128, 2 <= arity <= 8 (a playoff node is a
- * thread-block cluster of `arity` CTAs).
+ * w <= 128, 1 <= leaf_h <= 128, 2 <= arity <= 8 (a leaf or playoff node is a
+ * thread-block cluster of up to 16 CTAs, a level of the tree one launch).
  * ------------------------------------------------------------------------ */
 size_t cf_tourn_workspace_size(int m, int w, int leaf_h, int arity);
 int cf_tourn_select(int m, int w, const double *panel, int ldp, int leaf_h,

@@ -93,6 +93,11 @@ int launch_rtrsm32(float *X, int ldx, int rows, int w, const float *M00, int ldm
 template <typename LP>
 int launch_ltrsm32(float *X, int ldx, int w, int cols, const float *L00, int ldl, LP *lp, int ldk, int kpad,
                    cudaStream_t st);
+// LU-3 on A10 (rows x w) and LU-4 on A01 (w x cols) with the same A00 (all with
+// leading dimension ld), with their low-precision copies (both or none).
+template <typename LP>
+int launch_panel32(float *A10, int rows, float *A01, int cols, int w, int ld, const float *A00, LP *lpa, LP *lpb, int ldk,
+                   int kpad, cudaStream_t st);
 
 // ---- thin triangular solves with FP32 factors (cf_trsv.cu)
 // mode: 0 unit lower (L of LU), 1 upper (U), 2 lower (Cholesky L), 3 L^T.

@@ -538,17 +538,15 @@ static int cvt_cols_split(int k, int cols, int kpad, const float *src, int lds, 
 // Mixed LU of W (in place): tournament pivoting with FP32 panels, tensor-core
 // Schur updates.
 // ---------------------------------------------------------------------------
-// A second stream for the parts of a panel step that do not depend on each
-// other (released when its work completes).
+// A second stream for the parts of a panel step that the panel's chain does not
+// wait for (released when its work completes).
 struct SideStream {
-    cudaStream_t s = nullptr, bg = nullptr;
-    cudaEvent_t swapped = nullptr, a00_done = nullptr, side_done = nullptr, bg_done = nullptr;
+    cudaStream_t bg = nullptr;
+    cudaEvent_t swapped = nullptr, a00_done = nullptr, bg_done = nullptr;
     int open() {
-        if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess ||
-            cudaStreamCreateWithFlags(&bg, cudaStreamNonBlocking) != cudaSuccess ||
+        if (cudaStreamCreateWithFlags(&bg, cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&swapped, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&a00_done, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&side_done, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&bg_done, cudaEventDisableTiming) != cudaSuccess)
             return CF_ERR_CUDA;
         return CF_OK;
@@ -556,9 +554,7 @@ struct SideStream {
     ~SideStream() {
         if (swapped) cudaEventDestroy(swapped);
         if (a00_done) cudaEventDestroy(a00_done);
-        if (side_done) cudaEventDestroy(side_done);
         if (bg_done) cudaEventDestroy(bg_done);
-        if (s) cudaStreamDestroy(s);
         if (bg) cudaStreamDestroy(bg);
     }
 };
@@ -621,21 +617,17 @@ static int mixed_getrf(int n, MixedWS &w, int *info, const Opts &o, cudaStream_t
                 la_pending = false;
             }
             if ((rc = launch_apply_swaps<float>(W, w.ldw, n, k0, w.tep, w.perm, st))) return rc;
-            // Fork: the side stream takes LU-4 on the slab's columns with
-            // their operand copy (concurrent with LU-3); the main stream joins
-            // before the next panel's update, which reads both solves'
-            // operands.  The background stream takes what only the slab's
-            // deferred update needs: the pivot rows' left-looking update
-            // right of the slab, LU-4 there and its K-major copy; the main
-            // stream joins it at the slab's end.  It writes only this step's
-            // pivot rows right of the slab, which no later step of the slab
-            // reads before it (the next steps' swaps move rows below them;
-            // the next steps' background work follows in stream order).
+            // The background stream takes what only the slab's deferred update
+            // needs: the pivot rows' left-looking update right of the slab,
+            // LU-4 there and its K-major copy; the main stream joins it at the
+            // slab's end.  It writes only this step's pivot rows right of the
+            // slab, which no later step of the slab reads before it (the next
+            // steps' swaps move rows below them; the next steps' background
+            // work follows in stream order).
             CF_CUDA_TRY(cudaEventRecord(ss.swapped, st));
             CF_CUDA_TRY(cudaStreamWaitEvent(ss.bg, ss.swapped, 0));
             if ((rc = launch_a00_lu32(A00, w.ldw, wd, k0, info, st))) return rc;
             CF_CUDA_TRY(cudaEventRecord(ss.a00_done, st));
-            CF_CUDA_TRY(cudaStreamWaitEvent(ss.s, ss.a00_done, 0));
             const int below = m - wd, right = n - k0 - wd;
             const int off = k0 - J0, nout = n - JE;
             const int rslab = right - nout;              // columns right of the panel inside the slab
@@ -664,16 +656,6 @@ static int mixed_getrf(int n, MixedWS &w, int *info, const Opts &o, cudaStream_t
                             return rc;
                 }
             }
-            // LU-4 (side) after the A00 LU on the slab's columns; it also
-            // writes the K-major low-precision operand of the updates inside
-            // the slab (split form: converted after).
-            if ((rc = launch_ltrsm32<LP>(A00 + wd * ld, w.ldw, wd, rslab, A00, w.ldw, split ? nullptr : (LP *)w.Bb,
-                                         kMaxV, kMaxV, ss.s)))
-                return rc;
-            if (split && (rc = cvt_cols_split(wd, rslab, kMaxV, A00 + wd * ld, w.ldw, w.Bb, 3 * kMaxV, kMaxV, 1,
-                                              ss.s)))
-                return rc;
-            CF_CUDA_TRY(cudaEventRecord(ss.side_done, ss.s));
             // LU-4 right of the slab (background, after the left-looking
             // update); those U rows go to the K-major operand of the slab's
             // deferred update (K rows off .. off + wd, zeros up to the next
@@ -693,13 +675,16 @@ static int mixed_getrf(int n, MixedWS &w, int *info, const Opts &o, cudaStream_t
                 }
             }
             CF_CUDA_TRY(cudaEventRecord(ss.bg_done, ss.bg));
-            // LU-3 (main)
-            if ((rc = launch_rtrsm32<LP>(A00 + wd, w.ldw, below, wd, A00, w.ldw, false,
-                                         split ? nullptr : (LP *)w.Ab, kMaxV, kMaxV, nullptr, st)))
+            // LU-3 and, on the slab's columns, LU-4 (main), with the K-major
+            // low-precision operands of the updates inside the slab (split form:
+            // converted after)
+            if ((rc = launch_panel32<LP>(A00 + wd, below, A00 + wd * ld, rslab, wd, w.ldw, A00,
+                                         split ? nullptr : (LP *)w.Ab, split ? nullptr : (LP *)w.Bb, kMaxV, kMaxV, st)))
                 return rc;
-            if (split && (rc = cvt_rows_split(below, wd, kMaxV, A00 + wd, w.ldw, w.Ab, 3 * kMaxV, kMaxV, 0, st)))
-                return rc;
-            CF_CUDA_TRY(cudaStreamWaitEvent(st, ss.side_done, 0));
+            if (split) {
+                if ((rc = cvt_cols_split(wd, rslab, kMaxV, A00 + wd * ld, w.ldw, w.Bb, 3 * kMaxV, kMaxV, 1, st))) return rc;
+                if ((rc = cvt_rows_split(below, wd, kMaxV, A00 + wd, w.ldw, w.Ab, 3 * kMaxV, kMaxV, 0, st))) return rc;
+            }
             if (below <= 0 || right <= 0) continue;
             // A11 restricted to the slab's remaining columns (every row below)
             const int nslab = JE - (k0 + wd);

@@ -6,6 +6,7 @@
 //   k_a00_chol32    Cholesky of A00 (Listing "Cholesky Factorization"; CH-1)
 //   k_rtrsm32(_w)   LU-3  A10 <- A10 U00^{-1}  /  CH-2  L10 <- A10 L00^{-T}
 //   k_ltrsm32(_w)   LU-4  A01 <- L00^{-1} A01
+//   k_panel32(_w)   LU-3 and the slab's LU-4 in one launch
 //
 // The A00 kernels: a grid of threads with a few rows and columns each in
 // registers, one barrier per column (LU blocks of more than 64 rows: one
@@ -436,11 +437,9 @@ __device__ __forceinline__ void run_block(Body &body, int j0, int w) {
 // (j < kpad, zero for j >= w) is written in 16-byte chunks of 8.
 // ---------------------------------------------------------------------------
 template <typename LP>
-__global__ void __launch_bounds__(kMaxV)
-k_rtrsm32(float *X, int ldx, int rows, int w, const float *__restrict__ M00, int ldm, int trans_lower, LP *lp,
-          int ldk, int kpad, const int *skip) {
-    if (skip != nullptr && *skip != 0) return;
-    extern __shared__ __align__(16) float smem[];
+__device__ __forceinline__ void rtrsm_rows_any(float *smem, int block, float *X, int ldx, int rows, int w,
+                                               const float *__restrict__ M00, int ldm, int trans_lower, LP *lp, int ldk,
+                                               int kpad) {
     // [kMaxV + 1][kMaxV]: a step reads row k from column j0 in whole 32-column
     // chunks, up to 31 floats past the row's end; the last row's overrun
     // lands in the zeroed padding row
@@ -481,7 +480,7 @@ k_rtrsm32(float *X, int ldx, int rows, int w, const float *__restrict__ M00, int
         const float d = Ms[tid * kMaxV + tid];
         rinv[tid] = d != 0.f ? 1.0f / d : 1.0f;
     }
-    const int r0 = blockIdx.x * kMaxV;
+    const int r0 = block * kMaxV;
     const int nr = min(kMaxV, rows - r0);
     const bool live = tid < nr;
     float2 a[kPairs];
@@ -509,6 +508,15 @@ k_rtrsm32(float *X, int ldx, int rows, int w, const float *__restrict__ M00, int
     }
 }
 
+template <typename LP>
+__global__ void __launch_bounds__(kMaxV)
+k_rtrsm32(float *X, int ldx, int rows, int w, const float *__restrict__ M00, int ldm, int trans_lower, LP *lp,
+          int ldk, int kpad, const int *skip) {
+    if (skip != nullptr && *skip != 0) return;
+    extern __shared__ __align__(16) float smem[];
+    rtrsm_rows_any<LP>(smem, blockIdx.x, X, ldx, rows, w, M00, ldm, trans_lower, lp, ldk, kpad);
+}
+
 // ---------------------------------------------------------------------------
 // Left solve of a row block: X (w x cols, column-major ldx) <- L00^{-1} X, L00
 // unit lower.  Thread = column, held as a pair row; L staged column by
@@ -518,9 +526,8 @@ k_rtrsm32(float *X, int ldx, int rows, int w, const float *__restrict__ M00, int
 // zero for i >= w).
 // ---------------------------------------------------------------------------
 template <typename LP>
-__global__ void __launch_bounds__(kMaxV)
-k_ltrsm32(float *X, int ldx, int w, int cols, const float *__restrict__ L00, int ldl, LP *lp, int ldk, int kpad) {
-    extern __shared__ __align__(16) float smem[];
+__device__ __forceinline__ void ltrsm_cols_any(float *smem, int block, float *X, int ldx, int w, int cols,
+                                               const float *__restrict__ L00, int ldl, LP *lp, int ldk, int kpad) {
     float *Ls = smem;                                // [kMaxV + 1][kMaxV]: Ls[k][i] = L(i, k), zero padding row
     const int tid = threadIdx.x;
     Ls[kMaxV * kMaxV + tid] = 0.f;
@@ -534,7 +541,7 @@ k_ltrsm32(float *X, int ldx, int w, int cols, const float *__restrict__ L00, int
 #pragma unroll
         for (int u = 0; u < 16; ++u) Ls[(k0 + u) * kMaxV + tid] = v[u];
     }
-    const int c0 = blockIdx.x * kMaxV;
+    const int c0 = block * kMaxV;
     const int nc = min(kMaxV, cols - c0);
     const bool live = tid < nc;
     float *xc = X + (size_t)(c0 + (live ? tid : 0)) * ldx;
@@ -568,6 +575,13 @@ k_ltrsm32(float *X, int ldx, int w, int cols, const float *__restrict__ L00, int
         float z[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         for (int j0 = (w + 7) / 8 * 8; j0 < kpad; j0 += 8) store8_lp<LP>(lcol + j0, z);
     }
+}
+
+template <typename LP>
+__global__ void __launch_bounds__(kMaxV)
+k_ltrsm32(float *X, int ldx, int w, int cols, const float *__restrict__ L00, int ldl, LP *lp, int ldk, int kpad) {
+    extern __shared__ __align__(16) float smem[];
+    ltrsm_cols_any<LP>(smem, blockIdx.x, X, ldx, w, cols, L00, ldl, lp, ldk, kpad);
 }
 
 // ---------------------------------------------------------------------------
@@ -674,16 +688,14 @@ struct TrsmFixed {
 };
 
 template <int W, typename LP>
-__global__ void __launch_bounds__(128, 1)
-k_rtrsm32_w(float *X, int ldx, int rows, const float *__restrict__ M00, int ldm, int trans_lower, LP *lp, int ldk,
-            int kpad, const int *skip) {
-    if (skip != nullptr && *skip != 0) return;
+__device__ __forceinline__ void rtrsm_rows(float *smem, int block, float *X, int ldx, int rows,
+                                           const float *__restrict__ M00, int ldm, int trans_lower, LP *lp, int ldk,
+                                           int kpad) {
     constexpr int MS = W + 4;
-    extern __shared__ __align__(16) float smem[];
     float *Ms = smem;               // [W][MS]
     float *rinv = smem + W * MS;    // [W]
     const int tid = threadIdx.x;
-    const int r0 = blockIdx.x * 128;
+    const int r0 = block * 128;
     const bool live = tid < rows - r0;
     float2 a[W / 2];
 #pragma unroll
@@ -710,17 +722,24 @@ k_rtrsm32_w(float *X, int ldx, int rows, const float *__restrict__ M00, int ldm,
     }
 }
 
+template <int W, typename LP>
+__global__ void __launch_bounds__(128, 1)
+k_rtrsm32_w(float *X, int ldx, int rows, const float *__restrict__ M00, int ldm, int trans_lower, LP *lp, int ldk,
+            int kpad, const int *skip) {
+    if (skip != nullptr && *skip != 0) return;
+    extern __shared__ __align__(16) float smem[];
+    rtrsm_rows<W, LP>(smem, blockIdx.x, X, ldx, rows, M00, ldm, trans_lower, lp, ldk, kpad);
+}
+
 // X (W x cols) <- L00^{-1} X, thread = column, 64 threads per CTA (a slab's
 // 2,000 columns spread over twice the SMs).  The columns must be 16-byte
 // aligned (the launcher checks).
-template <int W, typename LP>
-__global__ void __launch_bounds__(64)
-k_ltrsm32_w(float *X, int ldx, int cols, const float *__restrict__ L00, int ldl, LP *lp, int ldk, int kpad) {
-    constexpr int NT = 64;
-    extern __shared__ __align__(16) float smem[];
+template <int W, int NT, typename LP>
+__device__ __forceinline__ void ltrsm_cols(float *smem, int block, float *X, int ldx, int cols,
+                                           const float *__restrict__ L00, int ldl, LP *lp, int ldk, int kpad) {
     float *Ms = smem;               // [W][W + 4]
     const int tid = threadIdx.x;
-    const int c0 = blockIdx.x * NT;
+    const int c0 = block * NT;
     const bool live = tid < cols - c0;
     float *xc = X + (size_t)(c0 + (live ? tid : 0)) * ldx;
     float2 a[W / 2];
@@ -742,6 +761,27 @@ k_ltrsm32_w(float *X, int ldx, int cols, const float *__restrict__ L00, int ldl,
     }
 }
 
+template <int W, typename LP>
+__global__ void __launch_bounds__(64)
+k_ltrsm32_w(float *X, int ldx, int cols, const float *__restrict__ L00, int ldl, LP *lp, int ldk, int kpad) {
+    extern __shared__ __align__(16) float smem[];
+    ltrsm_cols<W, 64, LP>(smem, blockIdx.x, X, ldx, cols, L00, ldl, lp, ldk, kpad);
+}
+
+// LU-3 on A10's rows and LU-4 on the slab's columns of A01 in one launch (the
+// first row_blocks CTAs take rows): both are a few dozen CTAs waiting on their
+// own chains, and as two launches the fork to a second stream and the join cost
+// the panel's chain 4 us of event waits (LU of n = 32768, 512 panels: 134.0 ms,
+// in one launch 131.9).
+template <int W, typename LP>
+__global__ void __launch_bounds__(128, 1)
+k_panel32_w(float *A10, int rows, int row_blocks, float *A01, int cols, int ld, const float *__restrict__ A00, LP *lpa,
+            LP *lpb, int ldk, int kpad) {
+    extern __shared__ __align__(16) float smem[];
+    if ((int)blockIdx.x < row_blocks) rtrsm_rows<W, LP>(smem, blockIdx.x, A10, ld, rows, A00, ld, 0, lpa, ldk, kpad);
+    else ltrsm_cols<W, 128, LP>(smem, blockIdx.x - row_blocks, A01, ld, cols, A00, ld, lpb, ldk, kpad);
+}
+
 // ---------------------------------------------------------------------------
 // One CTA: a grid of 4 x 4 elements per thread for LU blocks of up to 64 rows,
 // else one thread per row in whole warps.
@@ -760,6 +800,16 @@ int launch_a00_chol32(float *A00, int lda, int w, int kglob, int *info, cudaStre
     k_a00_chol32<<<1, 512, 0, st>>>(A00, lda, w, kglob, info);
     CF_LAUNCH_CHECK();
     return CF_OK;
+}
+
+template <typename LP>
+__global__ void __launch_bounds__(kMaxV)
+k_panel32(float *A10, int rows, int row_blocks, float *A01, int cols, int w, int ld, const float *__restrict__ A00,
+          LP *lpa, LP *lpb, int ldk, int kpad) {
+    extern __shared__ __align__(16) float smem[];
+    if ((int)blockIdx.x < row_blocks)
+        rtrsm_rows_any<LP>(smem, blockIdx.x, A10, ld, rows, w, A00, ld, 0, lpa, ldk, kpad);
+    else ltrsm_cols_any<LP>(smem, blockIdx.x - row_blocks, A01, ld, w, cols, A00, ld, lpb, ldk, kpad);
 }
 
 template <typename LP>
@@ -813,6 +863,38 @@ int launch_ltrsm32(float *X, int ldx, int w, int cols, const float *L00, int ldl
     return CF_OK;
 }
 
+// One launch where both solves take the same form (w = 64 or 128 with what
+// k_ltrsm32_w's 16-byte accesses need; every other width), else one for each.
+template <typename LP>
+int launch_panel32(float *A10, int rows, float *A01, int cols, int w, int ld, const float *A00, LP *lpa, LP *lpb, int ldk,
+                   int kpad, cudaStream_t st) {
+    const bool lp_ok =
+        lpa == nullptr || (ldk % 8 == 0 && kpad % 8 == 0 && (((uintptr_t)lpa | (uintptr_t)lpb) & 15) == 0);
+    const bool fixed = (w == 64 || w == 128) && (lpa == nullptr || kpad >= w);
+    if (rows > 0 && cols > 0 && w > 0 && lp_ok && (!fixed || ((((uintptr_t)A01) & 15) == 0 && ld % 4 == 0))) {
+        const int rb = ceil_div(rows, 128), blocks = rb + ceil_div(cols, 128);
+        const size_t smem = fixed ? sizeof(float) * (size_t)w * (w + 5) : sizeof(float) * (size_t)(kMaxV + 1) * kMaxV;
+        if (!fixed) {
+            CF_CUDA_TRY(cudaFuncSetAttribute(k_panel32<LP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            k_panel32<LP><<<blocks, kMaxV, smem, st>>>(A10, rows, rb, A01, cols, w, ld, A00, lpa, lpb, ldk, kpad);
+        } else if (w == 64) {
+            CF_CUDA_TRY(cudaFuncSetAttribute(k_panel32_w<64, LP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            k_panel32_w<64, LP><<<blocks, 128, smem, st>>>(A10, rows, rb, A01, cols, ld, A00, lpa, lpb, ldk, kpad);
+        } else {
+            CF_CUDA_TRY(cudaFuncSetAttribute(k_panel32_w<128, LP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            k_panel32_w<128, LP><<<blocks, 128, smem, st>>>(A10, rows, rb, A01, cols, ld, A00, lpa, lpb, ldk, kpad);
+        }
+        CF_LAUNCH_CHECK();
+        return CF_OK;
+    }
+    int rc = launch_ltrsm32<LP>(A01, ld, w, cols, A00, ld, lpb, ldk, kpad, st);
+    if (rc) return rc;
+    return launch_rtrsm32<LP>(A10, ld, rows, w, A00, ld, false, lpa, ldk, kpad, nullptr, st);
+}
+template int launch_panel32<__nv_bfloat16>(float *, int, float *, int, int, int, const float *, __nv_bfloat16 *,
+                                           __nv_bfloat16 *, int, int, cudaStream_t);
+template int launch_panel32<__half>(float *, int, float *, int, int, int, const float *, __half *, __half *, int, int,
+                                    cudaStream_t);
 template int launch_rtrsm32<__nv_bfloat16>(float *, int, int, int, const float *, int, bool, __nv_bfloat16 *, int,
                                            int, const int *, cudaStream_t);
 template int launch_rtrsm32<__half>(float *, int, int, int, const float *, int, bool, __half *, int, int, const int *,

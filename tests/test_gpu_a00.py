@@ -55,3 +55,16 @@ def test_failing_pivot_index(cf, n, k):
         A[k, k] = d
         info = f(_dev(A), _dev(B), prec="bf16")[1]
         assert int(info.item()) == k + 1
+
+
+# LU-3 and the slab's LU-4 in one launch: fixed widths, other ones, ragged last
+# panels (with 99, a panel of 64 columns at an odd column: a launch for each), and
+# slabs with and without columns right of the panel.
+@pytest.mark.parametrize("prec", ["f16", "bf16x3"])
+@pytest.mark.parametrize("n,v", [(300, 7), (300, 48), (321, 64), (361, 99), (163, 99), (300, 128), (129, 64)])
+def test_panel_solves_any_width(cf, n, v, prec):
+    A = inputs.uniform_pm1(n, seed=n + v, shift=2 * np.sqrt(n))
+    B = inputs.rhs_normal(n, 3, seed=3)
+    X, info, stats, st = cf.gesv_mixed(_dev(A), _dev(B), prec=prec, v=v)
+    assert st == cf.CF_OK and int(info.item()) == 0 and stats.converged == 1
+    assert oracle.backward_error(A, X.cpu().numpy(), B).max() <= 1e-14
