@@ -618,18 +618,20 @@ static int launch_trsv_mode(int n, int nrhs, const float *T, int ldt, const VT *
     if (withhold) CF_CUDA_TRY(cudaMemsetAsync(ticket, 1, 1, st));     // ticket = 1 (little-endian low byte)
     // FP64 arithmetic: a block's products are bound by one SM's FP64 pipe (64 x 64 x
     // 16: 16 us each, 40 us per link of the chain), so each group of four
-    // right-hand sides is a chain of its own, side by side with the others
-    // (the factor is read once per group).  FP32: one chain for all.
-    if constexpr (sizeof(VT) == 8) {
+    // right-hand sides is a chain of its own, side by side with the others.
+    // Every group reads the factor and widens it to FP64 (on the FP64 pipe too):
+    // once all SMs are busy for most of the solve that costs more than the
+    // shorter links give.  Refinement of an unshifted split-BF16 LU with 16
+    // right-hand sides, in groups / in one chain: n = 16384 331 / 442 ms, n =
+    // 32768 1620 / 1583 ms; the line lies between the two.  FP32: one chain.
+    if (sizeof(VT) == 8 && n <= 24576)
         return launch_trsv_nr<SB, MODE, 4, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, flags, ticket, ceil_div(nrhs, 4), spin,
                                                st);
-    } else {
-        if (nrhs <= 4)
-            return launch_trsv_nr<SB, MODE, 4, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, flags, ticket, 1, spin, st);
-        if (nrhs <= 8)
-            return launch_trsv_nr<SB, MODE, 8, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, flags, ticket, 1, spin, st);
-        return launch_trsv_nr<SB, MODE, 16, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, flags, ticket, 1, spin, st);
-    }
+    if (nrhs <= 4)
+        return launch_trsv_nr<SB, MODE, 4, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, flags, ticket, 1, spin, st);
+    if (nrhs <= 8)
+        return launch_trsv_nr<SB, MODE, 8, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, flags, ticket, 1, spin, st);
+    return launch_trsv_nr<SB, MODE, 16, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, flags, ticket, 1, spin, st);
 }
 
 template <int SB, typename VT>
