@@ -326,7 +326,7 @@ __device__ __forceinline__ void trsv_stage_step(float *dst, int step, int s, boo
 // partial sums meet in shared memory once per block before the diagonal
 // inverse is applied (and once more for its product).
 template <int SB, int MODE, int NR, typename VT>
-__global__ void __launch_bounds__(256, sizeof(VT) == 8 ? 2 : 1)        // CTAs per SM: shared memory
+__global__ void __launch_bounds__(256, sizeof(VT) == 8 && NR == 4 ? 2 : 1)        // CTAs per SM: shared memory
 k_trsv_blocked(int n, int nrhs, const float *__restrict__ T, int ldt, const VT *__restrict__ Dinv,
                const float *__restrict__ Gn, VT *X, int ldx, int *flags, int *ticket, int groups,
                long long spin_limit) {
@@ -623,7 +623,7 @@ static int launch_trsv_mode(int n, int nrhs, const float *T, int ldt, const VT *
     // once all SMs are busy for most of the solve that costs more than the
     // shorter links give.  Refinement of an unshifted split-BF16 LU with 16
     // right-hand sides, in groups / in one chain: n = 16384 331 / 442 ms, n =
-    // 32768 1620 / 1583 ms; the line lies between the two.  FP32: one chain.
+    // 32768 1620 / 1545 ms; the line lies between the two.  FP32: one chain.
     if (sizeof(VT) == 8 && n <= 24576)
         return launch_trsv_nr<SB, MODE, 4, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, flags, ticket, ceil_div(nrhs, 4), spin,
                                                st);
