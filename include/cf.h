@@ -207,14 +207,9 @@ int cf_tourn_select_f32(int m, int w, const float *panel, int ldp, int leaf_h,
  *   ipiv  device int[n], 1-based interchanges (see above).
  *   info  device int[1].
  *   work  at least cf_getrf_workspace_size(n, opt) bytes.  With
- *         cf_getrf_optimal_workspace_size(n, opt) bytes (4 KB per row more)
- *         the Schur updates of steps at least 17 wide run on the tensor cores
- *         from 62-bit digit slices of A10 and A01 (error a few 2^-62 of the
- *         row's and column's largest scaled elements per term and two
- *         roundings per element, where the FP64 loop rounds v partial sums;
- *         rows and columns holding Inf, NaN or scales more than 2^450 from
- *         the rest take the FP64 loop); with less, every update is the FP64
- *         loop.  The two differ by the update's rounding.
+ *         cf_getrf_optimal_workspace_size(n, opt) bytes (130 KB more) A00's LU
+ *         is taken over from the tournament's last elimination, which holds
+ *         the same bits; with less it is computed again.
  * ------------------------------------------------------------------------ */
 size_t cf_getrf_workspace_size(int n, const cf_options *opt);
 size_t cf_getrf_optimal_workspace_size(int n, const cf_options *opt);
@@ -239,8 +234,8 @@ int cf_getrf(int n, double *A, int lda, int *ipiv, int *info, void *work,
  *     (other streams, other host threads) race and corrupt each other.  The
  *     arrival counters are cleared at the start of every call.
  *   - It always runs the one-stream schedule on `stream` (opt->lookahead is
- *     ignored): the results equal cf_getrf's with its optimal workspace; the
- *     Schur update runs in pieces of 384 x 384, more slowly than there.
+ *     ignored): the results equal cf_getrf's, the speed is that of cf_getrf
+ *     with lookahead = 0.
  *   - The looked-up address is kept for the life of the process: after a
  *     cudaDeviceReset (or anything else that destroys the device's primary
  *     context) the next call on that device is invalid. */
@@ -252,8 +247,13 @@ int cf_getrf_noalloc(int n, double *A, int lda, int *ipiv, int *info,
  * Factorization", Sec. 6.2; COnfCHOX, Sec. 7.5 and Table 2: potrf on A00,
  * trsm on the panel, triangular update of A11).  Only the lower triangle is
  * read or written.  work may be NULL (cf_potrf_workspace_size is 0); with
- * cf_potrf_optimal_workspace_size(n, opt) bytes the updates run on the tensor
- * cores as in cf_getrf.
+ * cf_potrf_optimal_workspace_size(n, opt) bytes (2 KB per row) the updates of
+ * steps at least 17 wide run on the tensor cores from 62-bit digit slices of
+ * L10: an error of a few 2^-62 max_j |l_ij| max_j |l_kj|, both at most the
+ * diagonal's square roots, per term and two roundings per element, where the
+ * FP64 loop rounds v partial sums (rows holding Inf, NaN or elements outside
+ * 2^+-450 take that loop).  With less work every update is the FP64 loop; the
+ * two differ by the update's rounding.
  * ------------------------------------------------------------------------ */
 size_t cf_potrf_workspace_size(int n, const cf_options *opt);
 size_t cf_potrf_optimal_workspace_size(int n, const cf_options *opt);

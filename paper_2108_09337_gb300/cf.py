@@ -222,8 +222,8 @@ def getrf(A: torch.Tensor, v=None, leaf_h=None, arity=None, work=None, lookahead
     int32 tensors (ipiv 1-based).  lookahead: 1 (default) overlaps step
     t+1's TournPivot with step t's trailing update, 0 keeps one stream.
     work: at least cf_getrf_workspace_size bytes; from
-    cf_getrf_optimal_workspace_size on (the default buffer's size) the Schur
-    updates run on the tensor cores, below it on the FP64 pipe."""
+    cf_getrf_optimal_workspace_size on (the default buffer's size) A00's LU is
+    taken over from the tournament instead of computed again (the same bits)."""
     assert A.dtype == torch.float64
     n = A.shape[0]
     assert A.shape == (n, n)

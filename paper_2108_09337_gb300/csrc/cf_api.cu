@@ -127,14 +127,10 @@ extern "C" size_t cf_getrf_workspace_size(int n, const cf_options *opt) {
 // A00's LU and its flag.
 static constexpr size_t kLuBytes = sizeof(double) * kMaxV * kMaxV + 1024;
 
-// The minimal workspace plus A00's LU as the tournament leaves it and the digit
-// slices of one step's operands, with which the updates run on the tensor cores.
+// The minimal workspace plus A00's LU as the tournament leaves it.
 extern "C" size_t cf_getrf_optimal_workspace_size(int n, const cf_options *opt) {
     const size_t base = cf_getrf_workspace_size(n, opt);
-    Opts o;
-    if (base == 0 || resolve_options(opt, &o) != CF_OK) return 0;
-    const size_t head = align_up(base, 1024) + kLuBytes;
-    return o.v < kSliceMinW || n <= o.v ? head : head + slice64_bytes(n - o.v, n - o.v);
+    return base == 0 ? 0 : align_up(base, 1024) + kLuBytes;
 }
 
 // LU-6 look-ahead (FP64 path).  Step t runs its panel chain (TournPivot,
@@ -184,7 +180,7 @@ struct LookaheadStreams {
 };
 
 static int getrf_lookahead(int n, double *A, int lda, int *ipiv, int *info, const Opts &o, TournWS &ws,
-                           TournEpilogue &ep, const Slice64 *sl, cudaStream_t st) {
+                           TournEpilogue &ep, cudaStream_t st) {
     LookaheadStreams L;
     int rc = L.open(st);
     if (rc) return rc;
@@ -210,22 +206,6 @@ static int getrf_lookahead(int n, double *A, int lda, int *ipiv, int *info, cons
         const int right = n - k0 - w;
         if (m - w <= 0 || right <= 0) continue;
         const int w1 = o.v < right ? o.v : right;       // the next panel's columns
-        if (sl != nullptr && w >= kSliceMinW) {         // the slices of step t - 1 are free: its wide update is done
-            const double *A10 = A00 + w, *A01 = A00 + w * ld;
-            double *A11 = A00 + w + w * ld;
-            if ((rc = slice64_begin(*sl, A01, lda, w, right, nullptr, sp))) return fail(rc);
-            if ((rc = slice64_operands(*sl, A10, lda, m - w, A01, lda, right, w, nullptr, sp))) return fail(rc);
-            if ((rc = slice64_update(*sl, m - w, 0, w1, w, A10, lda, A01, lda, A11, lda, false, nullptr, sp)))
-                return fail(rc);
-            if (right > w1) {
-                if ((rc = L.panel_to_update())) return fail(rc);
-                if ((rc = slice64_update(*sl, m - w, w1, right, w, A10, lda, A01, lda, A11, lda, false, nullptr, su)))
-                    return fail(rc);
-                if ((rc = L.update_done())) return fail(rc);
-                rest_pending = true;
-            }
-            continue;
-        }
         if ((rc = launch_gemm_f64_sub(m - w, w1, w, A00 + w, lda, A00 + w * ld, lda, false, A00 + w + w * ld, lda,
                                       false, nullptr, sp)))
             return fail(rc);
@@ -265,15 +245,13 @@ static int potrf_lookahead(int n, double *A, int lda, int *info, const Opts &o, 
         rest_pending = false;
         const int w1 = o.v < rest ? o.v : rest;
         if (sl != nullptr && w >= kSliceMinW) {
-            const double *A10 = A00 + w;
+            const double *L10 = A00 + w;
             double *A11 = A00 + w + w * ld;
-            if ((rc = slice64_begin(*sl, nullptr, lda, w, 0, info, sp))) return rc;
-            if ((rc = slice64_operands(*sl, A10, lda, rest, nullptr, lda, 0, w, info, sp))) return rc;
-            if ((rc = slice64_update(*sl, rest, 0, w1, w, A10, lda, nullptr, lda, A11, lda, true, info, sp))) return rc;
+            if ((rc = slice64_operand(*sl, L10, lda, rest, w, info, sp))) return rc;
+            if ((rc = slice64_update(*sl, rest, 0, w1, w, L10, lda, A11, lda, info, sp))) return rc;
             if (rest > w1) {
                 if ((rc = L.panel_to_update())) return rc;
-                if ((rc = slice64_update(*sl, rest, w1, rest, w, A10, lda, nullptr, lda, A11, lda, true, info, su)))
-                    return rc;
+                if ((rc = slice64_update(*sl, rest, w1, rest, w, L10, lda, A11, lda, info, su))) return rc;
                 if ((rc = L.update_done())) return rc;
                 rest_pending = true;
             }
@@ -314,18 +292,12 @@ extern "C" int cf_getrf(int n, double *A, int lda, int *ipiv, int *info, void *w
     rc = tourn_ws_carve(work, n, o.leaf_h, o.arity, &ws, &ep);
     if (rc != CF_OK) return rc;
     CF_CUDA_TRY(cudaMemsetAsync(ws.counter, 0, ws.counter_bytes, st));
-    Slice64 slices;
-    const Slice64 *sl = nullptr;
     const size_t base = align_up(cf_getrf_workspace_size(n, opt), 1024);
     if (lwork >= cf_getrf_optimal_workspace_size(n, opt)) {
         ep.lu_ok = (int *)((char *)work + base);
         ep.lu = (double *)((char *)work + base + 1024);
-        if (o.v >= kSliceMinW && n > o.v) {
-            slices = slice64_carve((char *)work + base + kLuBytes, n - o.v, n - o.v);
-            sl = &slices;
-        }
     }
-    if (o.lookahead) return getrf_lookahead(n, A, lda, ipiv, info, o, ws, ep, sl, st);
+    if (o.lookahead) return getrf_lookahead(n, A, lda, ipiv, info, o, ws, ep, st);
     const size_t ld = (size_t)lda;
     for (int k0 = 0; k0 < n; k0 += o.v) {
         const int w = o.v < n - k0 ? o.v : n - k0;
@@ -344,16 +316,6 @@ extern "C" int cf_getrf(int n, double *A, int lda, int *ipiv, int *info, void *w
         // LU-4 A01 <- L00^{-1} A01
         if ((rc = launch_trsm_left_lower_unit(A00 + w * ld, lda, w, n - k0 - w, A00, lda, st))) return rc;
         // LU-5 A11 <- A11 - A10 A01
-        if (sl != nullptr && w >= kSliceMinW && n - k0 - w > 0) {
-            const int right = n - k0 - w;
-            const double *A10 = A00 + w, *A01 = A00 + w * ld;
-            if ((rc = slice64_begin(*sl, A01, lda, w, right, nullptr, st))) return rc;
-            if ((rc = slice64_operands(*sl, A10, lda, right, A01, lda, right, w, nullptr, st))) return rc;
-            if ((rc = slice64_update(*sl, right, 0, right, w, A10, lda, A01, lda, A00 + w + w * ld, lda, false, nullptr,
-                                     st)))
-                return rc;
-            continue;
-        }
         if ((rc = launch_gemm_f64_sub(m - w, n - k0 - w, w, A00 + w, lda, A00 + w * ld, lda, false,
                                       A00 + w + w * ld, lda, false, nullptr, st)))
             return rc;
@@ -372,7 +334,7 @@ extern "C" size_t cf_potrf_workspace_size(int n, const cf_options *opt) {
 extern "C" size_t cf_potrf_optimal_workspace_size(int n, const cf_options *opt) {
     Opts o;
     if (n < 0 || resolve_options(opt, &o) != CF_OK) return 0;
-    return o.v < kSliceMinW || n <= o.v ? 0 : 1024 + slice64_bytes(n - o.v, 0);
+    return o.v < kSliceMinW || n <= o.v ? 0 : 1024 + slice64_bytes(n - o.v);
 }
 
 extern "C" int cf_potrf(int n, double *A, int lda, int *info, void *work, size_t lwork, const cf_options *opt,
@@ -389,7 +351,7 @@ extern "C" int cf_potrf(int n, double *A, int lda, int *info, void *work, size_t
     const Slice64 *sl = nullptr;
     const size_t need = cf_potrf_optimal_workspace_size(n, opt);
     if (need > 0 && work != nullptr && lwork >= need) {
-        slices = slice64_carve((void *)align_up((size_t)work, 1024), n - o.v, 0);
+        slices = slice64_carve((void *)align_up((size_t)work, 1024), n - o.v);
         sl = &slices;
     }
     if (o.lookahead && n > 0) return potrf_lookahead(n, A, lda, info, o, sl, st);
@@ -404,11 +366,8 @@ extern "C" int cf_potrf(int n, double *A, int lda, int *info, void *work, size_t
         if ((rc = launch_trsm_right_upper(A00 + w, lda, m - w, w, A00, lda, true, info, st))) return rc;
         // CH-3 A11 <- A11 - L10 L10^T (lower)
         if (sl != nullptr && w >= kSliceMinW && m - w > 0) {
-            if ((rc = slice64_begin(*sl, nullptr, lda, w, 0, info, st))) return rc;
-            if ((rc = slice64_operands(*sl, A00 + w, lda, m - w, nullptr, lda, 0, w, info, st))) return rc;
-            if ((rc = slice64_update(*sl, m - w, 0, m - w, w, A00 + w, lda, nullptr, lda, A00 + w + w * ld, lda, true,
-                                     info, st)))
-                return rc;
+            if ((rc = slice64_operand(*sl, A00 + w, lda, m - w, w, info, st))) return rc;
+            if ((rc = slice64_update(*sl, m - w, 0, m - w, w, A00 + w, lda, A00 + w + w * ld, lda, info, st))) return rc;
             continue;
         }
         if ((rc = launch_gemm_f64_sub(m - w, m - w, w, A00 + w, lda, A00 + w, lda, true, A00 + w + w * ld, lda,

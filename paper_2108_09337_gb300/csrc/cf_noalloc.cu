@@ -10,21 +10,16 @@
 // For them this variant keeps the scratch in a fixed array that the library
 // itself places in device memory when it is loaded (kNoAllocScratchBytes on
 // every GPU that loads the library, held until the process exits).  It runs
-// cf_getrf's kernels; the Schur update goes in pieces whose digit slices fit
-// the array.
+// cf_getrf's kernels on one stream.
 #include <mutex>
 
 #include "cf_common.cuh"
 #include "cf_kernels.cuh"
-#include "cf_slice64.cuh"
 
 namespace cf {
 
 constexpr size_t kNoAllocScratchBytes = (size_t)2 << 20;   // 2 MiB
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
-
-// Rows and columns of one piece of the update: 2 KB of digit slices each.
-constexpr int kPiece = 384;
 
 constexpr int kMaxDevices = 64;
 static std::mutex g_noalloc_mu;
@@ -91,30 +86,9 @@ extern "C" int cf_getrf_noalloc(int n, double *A, int lda, int *ipiv, int *info,
         if ((rc = launch_getf2_nopiv(A00, lda, w, k0, info, ep.lu, ep.lu_ok, st))) return rc;
         if ((rc = launch_trsm_right_upper(A00 + w, lda, m - w, w, A00, lda, false, nullptr, st))) return rc;
         if ((rc = launch_trsm_left_lower_unit(A00 + w * ld, lda, w, n - k0 - w, A00, lda, st))) return rc;
-        const int right = n - k0 - w;
-        if (w < kSliceMinW) {
-            if ((rc = launch_gemm_f64_sub(m - w, right, w, A00 + w, lda, A00 + w * ld, lda, false, A00 + w + w * ld,
-                                          lda, false, nullptr, st)))
-                return rc;
-            continue;
-        }
-        if (right <= 0) continue;
-        // The update in pieces whose digit slices fit the scratch (the
-        // tournament's part of it is free until the next step): every piece
-        // gives its elements the values cf_getrf's whole update gives them.
-        const Slice64 sl = slice64_carve(scratch, kPiece, kPiece);
-        if ((rc = slice64_begin(sl, A00 + w * ld, lda, w, right, nullptr, st))) return rc;
-        for (int c = 0; c < right; c += kPiece)
-            for (int r = 0; r < m - w; r += kPiece) {
-                const double *A10 = A00 + w + r, *A01 = A00 + (w + c) * ld;
-                const int rows = m - w - r < kPiece ? m - w - r : kPiece, cols = right - c < kPiece ? right - c : kPiece;
-                if ((rc = slice64_clear_flags(sl, st))) return rc;
-                if ((rc = slice64_operands(sl, A10, lda, rows, A01, lda, cols, w, nullptr, st))) return rc;
-                if ((rc = slice64_update(sl, rows, 0, cols, w, A10, lda, A01, lda, A00 + w + r + (w + c) * ld, lda,
-                                         false, nullptr, st)))
-                    return rc;
-            }
-        CF_CUDA_TRY(cudaMemsetAsync(ws.counter, 0, ws.counter_bytes, st));
+        if ((rc = launch_gemm_f64_sub(m - w, n - k0 - w, w, A00 + w, lda, A00 + w * ld, lda, false,
+                                      A00 + w + w * ld, lda, false, nullptr, st)))
+            return rc;
     }
     return CF_OK;
 }

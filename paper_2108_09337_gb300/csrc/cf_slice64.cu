@@ -1,37 +1,35 @@
-// cf_slice64.cu -- LU-5 / CH-3 of the FP64 path on the tensor cores:
-//     C -= A10 A01   (LU; A10 m x w, A01 w x n)     C -= L10 L10^T   (Cholesky, lower)
+// cf_slice64.cu -- CH-3 of the FP64 path on the tensor cores:
+//     C -= L10 L10^T (lower), L10 m x w
 //
 // GB300 runs FP64 at ~2 fused multiply-adds per clock per SM (1.20 TFLOP/s
 // measured), so the update as FP64 code is bound by that pipe; the BF16 tensor
 // cores run 1500 times faster and form the same product exactly from small
 // integers:
-//   * inner scale: rho_j is the largest exponent in row j of A01.  A10's
-//     column j is scaled up and A01's row j down by 2^rho_j (exact; the
-//     product does not change), so that a row scaling of the matrix, which
-//     partial pivoting turns into opposite gradings of A10's columns and
-//     A01's rows, costs no accuracy.  Cholesky needs none (L10 is both sides);
-//   * per row of A10 (column of A01) the elements become integers of at most
-//     62 bits relative to the row's (column's) largest exponent and eight
-//     balanced base-256 digits (the top one in [-64, 64], the others in
-//     [-128, 127]), exact in BF16;
-//   * Q_d = sum_{s+t=d} sum_j d_s e_t, d = 0..7: for every A10 digit s one
-//     chain of tcgen05 MMAs against the A01 digits t = 0..7-s, accumulating
+//   * per row of L10 the elements become integers of at most 62 bits relative
+//     to the row's largest exponent and eight balanced base-256 digits (the top
+//     one in [-64, 64], the others in [-128, 127]), exact in BF16;
+//   * Q_d = sum_{s+t=d} sum_j d_s e_t, d = 0..7: for every row digit s one
+//     chain of tcgen05 MMAs against the column digits t = 0..7-s, accumulating
 //     into the TMEM columns of diagonal s + t.  A sum holds at most 128
 //     products of each of at most 8 digit pairs, two of them with a top digit:
 //     at most 7 x 2^21 < 2^24, so the FP32 accumulation is exact in any order;
-//   * C -= 2^(E_i + F_k - 2112) sum_d Q_d 256^(7-d): the 76-bit integer sum is
+//   * C -= 2^(E_i + E_k - 4158) sum_d Q_d 256^(7-d): the 76-bit integer sum is
 //     rounded to FP64 once and subtracted with a second rounding.
-// The error is a few 2^-62 of (max of the row) x (max of the column) per term
-// and one rounding of the sum, where the FP64 loop rounds w partial sums.
-// Every C element's value is a function of its row, its column and the inner
-// exponents alone, so it does not depend on how the update is cut into pieces.
+// The error is a few 2^-62 of (max of row i) x (max of row k) per term and one
+// rounding of the sum, where the FP64 loop rounds w partial sums.  A Cholesky
+// factor's rows are bounded by the diagonal, |l_ij| <= sqrt(a_ii), so this is
+// below the factorization's own error u sqrt(a_ii a_kk) whatever the rows'
+// scales.  LU has no such bound (one large element of U in one column would take
+// the bits of all others): its update is the FP64 loop.
+// Every C element's value is a function of its row and its column alone, so it
+// does not depend on how the update is cut into pieces.
 //
-// Rows (columns) with an infinity, a NaN or scales whose product could leave
-// the normal range flag their tile, and flagged tiles are done by the FP64 loop
+// Rows with an infinity, a NaN or scales whose product could leave the normal
+// range flag their tile, and flagged tiles are done by the FP64 loop
 // (k_gemm_flagged), with that loop's results.
 //
 // Kernel layout: persistent CTAs over 128 x 64 tiles of C, column-tile major,
-// so that a CTA's A01 digits (128 KB) stay in shared memory while the A10
+// so that a CTA's column digits (128 KB) stay in shared memory while the row
 // digits (16 KB tiles, six in flight) stream through from L2; 8 diagonals x 64
 // columns fill the 512 TMEM columns.  Per tile: 36 digit pairs = 9,200 tensor
 // clocks; sixteen epilogue warps combine the diagonals in integers as they
@@ -58,7 +56,7 @@ using namespace umma;
 constexpr int ND = 8;                  // digits per element
 constexpr int BM = 128, BN = 64, BK = 64;
 constexpr int UMMA_K = 16;
-constexpr int AST = 6;                 // A10 digit tiles in flight
+constexpr int AST = 6;                 // row digit tiles in flight
 constexpr int EPI = 16;                // epilogue warps: 4 lane quarters x 4 groups of 16 columns
 constexpr int kThreads = 64 + 32 * EPI;
 constexpr uint32_t kABytes = BM * BK * 2;          // one digit of 128 rows x 64 k
@@ -66,8 +64,7 @@ constexpr uint32_t kBHalf = BN * BK * 2;           // one digit of 64 rows x 64 
 constexpr uint32_t kBBytes = 2 * ND * kBHalf;      // all digits of 64 columns x 128 k
 constexpr uint32_t kTmemCols = 512;
 constexpr int kCentre = 2046;          // E of a row whose largest scaled element is in [1, 2)
-constexpr int kSpan = 450;             // E and F may be this far from their centres (below), E this far ...
-constexpr int kSpanUp = 900;           // ... above its centre when F <= 0: E + F - 994 - 95 >= 1, E + F - 994 <= 2046
+constexpr int kSpan = 450;             // E may be this far from it: E_i + E_k - kCentre - 994 - 95 >= 1, ... - 994 <= 2046
 
 struct Smem {
     uint64_t afull[AST], aempty[AST];
@@ -77,14 +74,13 @@ struct Smem {
 };
 
 struct Problem {
-    int m, c0, c1;                     // rows, columns [c0, c1) of the sliced operands
+    int m, c0, c1;                     // rows; columns [c0, c1), rows of the slices too; i >= j only
     int nkb;                           // K blocks of 64 (1 or 2)
-    int lower, same;                   // Cholesky: triangle only; one set of slices for both operands
     int ct0, ct1, nrt;                 // column tiles of 64, row tiles of 128
     long long units;
-    const uint8_t *SA, *SB;
-    const int *E, *F;
-    const int *any, *flagA, *flagB;
+    const uint8_t *S;
+    const int *E;
+    const int *any, *flag;
     const int *skip;
     double *C;
     int ldc;
@@ -99,19 +95,13 @@ __host__ __device__ __forceinline__ size_t tile_offset(int rt, int kb, int d) {
 // The units of a CTA: (column tile, row tile) pairs, row tiles fastest.
 struct Walk {
     int ct, rt;
-    __device__ static int first_rt(const Problem &p, int ct) { return p.lower ? ct / 2 : 0; }
     __device__ void seek(const Problem &p, long long u) {
         ct = p.ct0;
-        if (!p.lower) {
-            ct += (int)(u / p.nrt);
-            rt = (int)(u % p.nrt);
-            return;
-        }
         while (u >= p.nrt - ct / 2) { u -= p.nrt - ct / 2; ++ct; }
         rt = ct / 2 + (int)u;
     }
     __device__ void next(const Problem &p) {
-        if (++rt >= p.nrt) { ++ct; rt = first_rt(p, ct); }
+        if (++rt >= p.nrt) { ++ct; rt = ct / 2; }
     }
 };
 
@@ -196,13 +186,12 @@ k_update_sliced(Problem p) {
                         break;
                     }
                     mbar_arrive_expect_tx(&s.bfull, (uint32_t)p.nkb * ND * kBHalf);
-                    const uint8_t *S = (p.same ? p.SA : p.SB);
                     for (int kb = 0; kb < p.nkb; ++kb)
                         for (int d = 0; d < ND; ++d)
                             asm volatile(
                                 "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, "
                                 "[%3];" ::"r"(smem_u32(sB + (kb * ND + d) * kBHalf)),
-                                "l"(S + tile_offset(ct / 2, kb, d) + (size_t)(ct & 1) * kBHalf), "r"(kBHalf),
+                                "l"(p.S + tile_offset(ct / 2, kb, d) + (size_t)(ct & 1) * kBHalf), "r"(kBHalf),
                                 "r"(smem_u32(&s.bfull))
                                 : "memory");
                     ++nb;
@@ -219,7 +208,7 @@ k_update_sliced(Problem p) {
                         asm volatile(
                             "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                                 smem_u32(sA + st * kABytes)),
-                            "l"(p.SA + tile_offset(wk.rt, kb, d)), "r"(kABytes), "r"(smem_u32(&s.afull[st]))
+                            "l"(p.S + tile_offset(wk.rt, kb, d)), "r"(kABytes), "r"(smem_u32(&s.afull[st]))
                             : "memory");
                         ++ia;
                     }
@@ -263,7 +252,7 @@ k_update_sliced(Problem p) {
                         }
                         tc_fence_after();
                         const uint64_t ad = make_sw128_desc(smem_u32(sA + as * kABytes));
-                        // A10 digit d times A01 digits t = 0..7-d into the columns of diagonals d..7
+                        // row digit d times column digits t = 0..7-d into the columns of diagonals d..7
                         const int ncol = BN * (ND - d);
                         const int n1 = ncol < 256 ? ncol : 256, n2 = ncol - n1;
                         const uint32_t id1 = make_idesc(true, BM, n1);
@@ -306,7 +295,7 @@ k_update_sliced(Problem p) {
             const int col0 = wk.ct * BN + grp * 16;
             const int Ei = row < p.m ? p.E[row] : kCentre;
             double *Cp = p.C + (size_t)row + (size_t)col0 * p.ldc;
-            auto mine = [&](int c) { return row < p.m && col0 + c >= p.c0 && col0 + c < p.c1 && (!p.lower || row >= col0 + c); };
+            auto mine = [&](int c) { return row < p.m && col0 + c >= p.c0 && col0 + c < p.c1 && row >= col0 + c; };
             if (lane == 0) ok = wait_bounded(&s.acc_full, (uint32_t)n & 1u, abort_flag, &g_slice64_status);
             ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
             if (!ok) break;
@@ -339,9 +328,9 @@ k_update_sliced(Problem p) {
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&s.acc_empty);
-            if (row >= p.m || (any && (p.flagA[wk.rt] || (p.same ? p.flagA[wk.ct / 2] : p.flagB[wk.ct / 2])))) continue;
-            const int *Fp = p.same ? p.E + col0 : p.F + col0;
-            const int shift = p.same ? Ei - kCentre : Ei;
+            if (row >= p.m || (any && (p.flag[wk.rt] || p.flag[wk.ct / 2]))) continue;
+            const int *Ek = p.E + col0;
+            const int shift = Ei - kCentre;
 #pragma unroll
             for (int c0 = 0; c0 < 16; c0 += 8) {
                 double cv[8];
@@ -350,7 +339,7 @@ k_update_sliced(Problem p) {
 #pragma unroll
                 for (int c = 0; c < 8; ++c)
                     if (mine(c0 + c))
-                        Cp[(size_t)(c0 + c) * p.ldc] = cv[c] - scaled_double(hi[c0 + c], lo[c0 + c], shift + Fp[c0 + c]);
+                        Cp[(size_t)(c0 + c) * p.ldc] = cv[c] - scaled_double(hi[c0 + c], lo[c0 + c], shift + Ek[c0 + c]);
             }
         }
     }
@@ -364,36 +353,8 @@ k_update_sliced(Problem p) {
 }
 
 // ---------------------------------------------------------------------------
-// Inner exponents: rho[j] = max over the columns of the exponent field of
-// A01(j, k); zero before.  A warp takes whole columns (w contiguous values).
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_inner_exp(const double *__restrict__ U, int ldu, int w, int cols, int *rho) {
-    __shared__ int red[kMaxV];
-    const int lane = threadIdx.x & 31;
-    if (threadIdx.x < kMaxV) red[threadIdx.x] = 0;
-    __syncthreads();
-    int f[4] = {0, 0, 0, 0};
-    for (int c = blockIdx.x * 8 + (threadIdx.x >> 5); c < cols; c += gridDim.x * 8) {
-        const double *u = U + (size_t)c * ldu;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int j = lane + 32 * q;
-            if (j < w) {
-                const int e = (int)((__double_as_longlong(u[j]) >> 52) & 0x7FF);
-                if (e != 0x7FF) f[q] = max(f[q], e);
-            }
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-        if (f[q] > 0) atomicMax(red + lane + 32 * q, f[q]);
-    __syncthreads();
-    if (threadIdx.x < kMaxV && red[threadIdx.x] > 0) atomicMax(rho + threadIdx.x, red[threadIdx.x]);
-}
-
-// ---------------------------------------------------------------------------
-// Digit slices of rows of A10 (A[i + j lda]) and columns of A01 (B[j + i ldb]).
-// CTA: 32 rows x 128 j; the row's largest scaled exponent, the digits, then
+// Digit slices of the rows of L10 (A[i + j lda]).
+// CTA: 32 rows x 128 j; the row's largest exponent, the digits, then
 // each slice through shared memory as whole 128-byte tile rows.  Bound by the
 // memory traffic of 24 bytes per element and ~40 integer operations.
 // ---------------------------------------------------------------------------
@@ -422,57 +383,32 @@ __device__ __forceinline__ void digits8(double x, int sh, __nv_bfloat16 (&dg)[ND
 }
 
 struct SliceArgs {
-    const double *A, *B;
-    int lda, ldb, rows, cols, w, nkb;
-    int blocks_a;                       // CTAs of the A side; the rest cut B
-    uint8_t *SA, *SB;
-    int *E, *F;
-    const int *rho;                     // null: Cholesky (no inner scale)
-    int *any, *flagA, *flagB;
+    const double *A;
+    int lda, rows, w, nkb;
+    uint8_t *S;
+    int *E;
+    int *any, *flag;
     const int *skip;
 };
 
-__global__ void __launch_bounds__(256) k_slice_operands(SliceArgs a) {
+__global__ void __launch_bounds__(256) k_slice_rows(SliceArgs a) {
     if (a.skip != nullptr && *a.skip != 0) return;
-    __shared__ double xs[kRows][2 * BK + 1];
     __shared__ __align__(16) __nv_bfloat16 tile[kRows * kPitch];
     __shared__ int gmax[8][kRows];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const bool side_b = (int)blockIdx.x >= a.blocks_a;
-    const int i0 = (side_b ? blockIdx.x - a.blocks_a : blockIdx.x) * kRows;
-    const int m = side_b ? a.cols : a.rows;
+    const int i0 = blockIdx.x * kRows;
     const int i = i0 + lane, j0 = warp * 16;
     double x[16];
-    if (!side_b) {
 #pragma unroll
-        for (int c = 0; c < 16; ++c)
-            x[c] = (i < m && j0 + c < a.w) ? a.A[(size_t)i + (size_t)(j0 + c) * a.lda] : 0.0;
-    } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int col = i0 + warp * 4 + q;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int j = lane + 32 * e;
-                xs[warp * 4 + q][j] = (col < m && j < a.w) ? a.B[(size_t)j + (size_t)col * a.ldb] : 0.0;
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int c = 0; c < 16; ++c) x[c] = xs[lane][j0 + c];
-    }
+    for (int c = 0; c < 16; ++c)
+        x[c] = (i < a.rows && j0 + c < a.w) ? a.A[(size_t)i + (size_t)(j0 + c) * a.lda] : 0.0;
     int g[16];
     int top = INT_MIN;
     bool bad = false;
 #pragma unroll
     for (int c = 0; c < 16; ++c) {
         const int f = (int)((__double_as_longlong(x[c]) >> 52) & 0x7FF);
-        int r = 1023;
-        if (a.rho != nullptr && j0 + c < a.w) {
-            r = a.rho[j0 + c];
-            if (r == 0) r = 1023;
-        }
-        g[c] = max(f, 1) + (side_b ? -r : r);
+        g[c] = max(f, 1) + 1023;
         bad |= f == 0x7FF;
         if (x[c] != 0.0) top = max(top, g[c]);
     }
@@ -480,13 +416,12 @@ __global__ void __launch_bounds__(256) k_slice_operands(SliceArgs a) {
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < 8; ++q) top = max(top, gmax[q][lane]);
-    const int centre = side_b ? 0 : kCentre;
-    if (top == INT_MIN) top = centre;                   // a zero row: all digits zero
-    bad |= top < centre - kSpan || top > centre + (a.rho == nullptr || side_b ? kSpan : kSpanUp);
-    if (i < m) {
-        if (warp == 0) (side_b ? a.F : a.E)[i] = top;
+    if (top == INT_MIN) top = kCentre;                  // a zero row: all digits zero
+    bad |= top < kCentre - kSpan || top > kCentre + kSpan;
+    if (i < a.rows) {
+        if (warp == 0) a.E[i] = top;
         if (bad) {
-            atomicOr((side_b ? a.flagB : a.flagA) + i / BM, 1);
+            atomicOr(a.flag + i / BM, 1);
             atomicOr(a.any, 1);
         }
     }
@@ -504,7 +439,6 @@ __global__ void __launch_bounds__(256) k_slice_operands(SliceArgs a) {
             pk[d][c / 2] = *reinterpret_cast<const uint32_t *>(&h);
         }
     }
-    uint8_t *S = side_b ? a.SB : a.SA;
 #pragma unroll
     for (int d = 0; d < ND; ++d) {
         uint4 *sdst = reinterpret_cast<uint4 *>(tile + lane * kPitch + warp * 16);
@@ -519,7 +453,7 @@ __global__ void __launch_bounds__(256) k_slice_operands(SliceArgs a) {
             const int gi = i0 + r, rl = gi & (BM - 1);
             if (kb < a.nkb) {       // rows past m: zero digits, inside the padded tile
                 const uint4 v = *reinterpret_cast<const uint4 *>(tile + r * kPitch + q * 8);
-                *reinterpret_cast<uint4 *>(S + tile_offset(gi / BM, kb, d) + (size_t)rl * 128 +
+                *reinterpret_cast<uint4 *>(a.S + tile_offset(gi / BM, kb, d) + (size_t)rl * 128 +
                                            (size_t)((ch ^ (rl & 7)) * 16)) = v;
             }
         }
@@ -533,20 +467,19 @@ __global__ void __launch_bounds__(256) k_slice_operands(SliceArgs a) {
 // flagged: one load per CTA.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
-k_gemm_flagged(Problem p, int w, const double *__restrict__ A, int lda, const double *__restrict__ B, int ldb) {
+k_gemm_flagged(Problem p, int w, const double *__restrict__ A, int lda) {
     if (p.skip != nullptr && *p.skip != 0) return;
     if (*p.any == 0) return;
     const int nrt = (p.m + 63) / 64, ct0 = p.c0 / 64, ct1 = (p.c1 + 63) / 64;
     for (long long t = blockIdx.x; t < (long long)nrt * (ct1 - ct0); t += gridDim.x) {
         const int rt = (int)(t % nrt), ct = ct0 + (int)(t / nrt);
-        if (!(p.flagA[rt / 2] || (p.same ? p.flagA[ct / 2] : p.flagB[ct / 2]))) continue;
+        if (!(p.flag[rt / 2] || p.flag[ct / 2])) continue;
         for (int e = threadIdx.x; e < 64 * 64; e += 256) {
             const int i = rt * 64 + (e & 63), j = ct * 64 + (e >> 6);
-            if (i >= p.m || j < p.c0 || j >= p.c1 || (p.lower && i < j)) continue;
+            if (i >= p.m || j < p.c0 || j >= p.c1 || i < j) continue;
             double acc = 0.0;
             for (int k = 0; k < w; ++k)
-                acc = fma(A[(size_t)i + (size_t)k * lda],
-                          p.same ? A[(size_t)j + (size_t)k * lda] : B[(size_t)k + (size_t)j * ldb], acc);
+                acc = fma(A[(size_t)i + (size_t)k * lda], A[(size_t)j + (size_t)k * lda], acc);
             double *c = p.C + (size_t)i + (size_t)j * p.ldc;
             *c = *c - acc;
         }
@@ -558,78 +491,50 @@ k_gemm_flagged(Problem p, int w, const double *__restrict__ A, int lda, const do
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
-Slice64 slice64_carve(void *work, int rows, int cols) {
-    Slice64 s;
+static void carve(Carver &cv, int rows, Slice64 &s) {
+    const size_t r = align_up((size_t)rows, s64::BM);
     s.rows = rows;
-    s.cols = cols;
+    s.S = cv.take<uint8_t>(r * 2 * s64::ND * 128, 1024);
+    s.E = cv.take<int>(r);
+    s.nflags = 4 + r / s64::BM;
+    s.flags = cv.take<int>(s.nflags);
+}
+
+Slice64 slice64_carve(void *work, int rows) {
     Carver cv(work);
-    const size_t ra = align_up((size_t)rows, s64::BM), rb = align_up((size_t)cols, s64::BM);
-    s.SA = cv.take<uint8_t>(ra * 2 * s64::ND * 128, 1024);
-    s.SB = cols ? cv.take<uint8_t>(rb * 2 * s64::ND * 128, 1024) : nullptr;
-    s.E = cv.take<int>(ra);
-    s.F = cols ? cv.take<int>(rb) : nullptr;
-    s.nflags = 4 + ra / s64::BM + rb / s64::BM;
-    s.head = cv.take<int>(kMaxV + s.nflags);
+    Slice64 s;
+    carve(cv, rows, s);
     return s;
 }
 
-size_t slice64_bytes(int rows, int cols) {
-    const Slice64 s = slice64_carve(nullptr, rows, cols);
+size_t slice64_bytes(int rows) {
     Carver cv(nullptr);
-    const size_t ra = align_up((size_t)rows, s64::BM), rb = align_up((size_t)cols, s64::BM);
-    cv.take<uint8_t>(ra * 2 * s64::ND * 128, 1024);
-    if (cols) cv.take<uint8_t>(rb * 2 * s64::ND * 128, 1024);
-    cv.take<int>(ra);
-    if (cols) cv.take<int>(rb);
-    cv.take<int>(kMaxV + s.nflags);
+    Slice64 s;
+    carve(cv, rows, s);
     return cv.size();
 }
 
-int slice64_begin(const Slice64 &s, const double *A01, int lda, int w, int cols, const int *skip, cudaStream_t st) {
-    (void)skip;
-    CF_CUDA_TRY(cudaMemsetAsync(s.head, 0, sizeof(int) * (kMaxV + s.nflags), st));
-    if (A01 == nullptr || cols <= 0) return CF_OK;
-    const int want = ceil_div(cols, 8), most = 2 * device_sm_count();     // eight columns per CTA and pass
-    s64::k_inner_exp<<<want < most ? want : most, 256, 0, st>>>(A01, lda, w, cols, s.rho());
-    CF_LAUNCH_CHECK();
-    return CF_OK;
-}
-
-int slice64_clear_flags(const Slice64 &s, cudaStream_t st) {
-    CF_CUDA_TRY(cudaMemsetAsync(s.any(), 0, sizeof(int) * s.nflags, st));
-    return CF_OK;
-}
-
-int slice64_operands(const Slice64 &s, const double *A10, int lda, int rows, const double *A01, int ldb, int cols,
-                     int w, const int *skip, cudaStream_t st) {
+int slice64_operand(const Slice64 &s, const double *L10, int lda, int rows, int w, const int *skip, cudaStream_t st) {
+    CF_CUDA_TRY(cudaMemsetAsync(s.flags, 0, sizeof(int) * s.nflags, st));
+    if (rows <= 0) return CF_OK;
     s64::SliceArgs a{};
-    a.A = A10;
-    a.B = A01;
+    a.A = L10;
     a.lda = lda;
-    a.ldb = ldb;
     a.rows = rows;
-    a.cols = A01 ? cols : 0;
     a.w = w;
     a.nkb = ceil_div(w, s64::BK);
-    a.blocks_a = ceil_div(rows, s64::kRows);
-    a.SA = s.SA;
-    a.SB = s.SB;
+    a.S = s.S;
     a.E = s.E;
-    a.F = s.F;
-    a.rho = s.cols ? s.rho() : nullptr;
     a.any = s.any();
-    a.flagA = s.flagA();
-    a.flagB = s.flagB();
+    a.flag = s.flag();
     a.skip = skip;
-    const int blocks = a.blocks_a + ceil_div(a.cols, s64::kRows);
-    if (blocks == 0) return CF_OK;
-    s64::k_slice_operands<<<blocks, 256, 0, st>>>(a);
+    s64::k_slice_rows<<<ceil_div(rows, s64::kRows), 256, 0, st>>>(a);
     CF_LAUNCH_CHECK();
     return CF_OK;
 }
 
-int slice64_update(const Slice64 &s, int rows, int c0, int c1, int w, const double *A10, int lda, const double *A01,
-                   int ldb, double *C, int ldc, bool lower, const int *skip, cudaStream_t st) {
+int slice64_update(const Slice64 &s, int rows, int c0, int c1, int w, const double *L10, int lda, double *C, int ldc,
+                   const int *skip, cudaStream_t st) {
     using namespace s64;
     if (rows <= 0 || c1 <= c0 || w <= 0) return CF_OK;
     Problem p{};
@@ -637,20 +542,15 @@ int slice64_update(const Slice64 &s, int rows, int c0, int c1, int w, const doub
     p.c0 = c0;
     p.c1 = c1;
     p.nkb = ceil_div(w, BK);
-    p.lower = lower ? 1 : 0;
-    p.same = s.cols == 0 ? 1 : 0;
     p.ct0 = c0 / BN;
     p.ct1 = ceil_div(c1, BN);
     p.nrt = ceil_div(rows, BM);
     p.units = 0;
-    for (int ct = p.ct0; ct < p.ct1; ++ct) p.units += lower ? p.nrt - ct / 2 : p.nrt;
-    p.SA = s.SA;
-    p.SB = s.SB;
+    for (int ct = p.ct0; ct < p.ct1; ++ct) p.units += p.nrt - ct / 2;
+    p.S = s.S;
     p.E = s.E;
-    p.F = s.F;
     p.any = s.any();
-    p.flagA = s.flagA();
-    p.flagB = s.flagB();
+    p.flag = s.flag();
     p.skip = skip;
     p.C = C;
     p.ldc = ldc;
@@ -659,7 +559,7 @@ int slice64_update(const Slice64 &s, int rows, int c0, int c1, int w, const doub
     CF_CUDA_TRY(cudaFuncSetAttribute(k_update_sliced, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     k_update_sliced<<<(int)(p.units < sms ? p.units : sms), kThreads, smem, st>>>(p);
     CF_LAUNCH_CHECK();
-    k_gemm_flagged<<<sms, 256, 0, st>>>(p, w, A10, lda, A01, ldb);
+    k_gemm_flagged<<<sms, 256, 0, st>>>(p, w, L10, lda);
     CF_LAUNCH_CHECK();
     return CF_OK;
 }
