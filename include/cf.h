@@ -209,7 +209,8 @@ int cf_tourn_select_f32(int m, int w, const float *panel, int ldp, int leaf_h,
  *   work  at least cf_getrf_workspace_size(n, opt) bytes.  With
  *         cf_getrf_optimal_workspace_size(n, opt) bytes (130 KB more) A00's LU
  *         is taken over from the tournament's last elimination, which holds
- *         the same bits; with less it is computed again.
+ *         the same bits; with less it is computed again.  Any 4-byte-aligned
+ *         address will do.
  * ------------------------------------------------------------------------ */
 size_t cf_getrf_workspace_size(int n, const cf_options *opt);
 size_t cf_getrf_optimal_workspace_size(int n, const cf_options *opt);

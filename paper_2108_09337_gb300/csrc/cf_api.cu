@@ -124,7 +124,7 @@ extern "C" size_t cf_getrf_workspace_size(int n, const cf_options *opt) {
     return tourn_ws_bytes(n > 0 ? n : 1, o.leaf_h, o.arity);
 }
 
-// A00's LU and its flag.
+// A00's LU and its flag, with room to align the LU whatever work's alignment.
 static constexpr size_t kLuBytes = sizeof(double) * kMaxV * kMaxV + 1024;
 
 // The minimal workspace plus A00's LU as the tournament leaves it.
@@ -295,7 +295,7 @@ extern "C" int cf_getrf(int n, double *A, int lda, int *ipiv, int *info, void *w
     const size_t base = align_up(cf_getrf_workspace_size(n, opt), 1024);
     if (lwork >= cf_getrf_optimal_workspace_size(n, opt)) {
         ep.lu_ok = (int *)((char *)work + base);
-        ep.lu = (double *)((char *)work + base + 1024);
+        ep.lu = (double *)align_up((size_t)work + base + sizeof(int), 256);
     }
     if (o.lookahead) return getrf_lookahead(n, A, lda, ipiv, info, o, ws, ep, st);
     const size_t ld = (size_t)lda;

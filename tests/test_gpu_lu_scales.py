@@ -1,7 +1,10 @@
 """cf_getrf on matrices whose elements differ by many orders of magnitude in a
 way that no row or column scaling takes out: every element of P A - L U stays
 within the FP64 update's own bound, whatever else the matrix holds, and the
-factors do not depend on the workspace given or on the schedule."""
+factors do not depend on the workspace given (its size, its alignment) or on the
+schedule."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -71,3 +74,20 @@ def test_elements_of_two_magnitudes(cf, kind, t, n, v):
     for LU, ip in out[1:]:
         np.testing.assert_array_equal(LU, out[0][0])
         np.testing.assert_array_equal(ip, out[0][1])
+
+
+@pytest.mark.parametrize("offset", [4, 8, 12, 16, 500])
+@pytest.mark.parametrize("lookahead", [0, 1])
+def test_work_of_any_int_alignment(cf, offset, lookahead):
+    n = 300
+    A = inputs.uniform_pm1(n, seed=2)
+    ref = _dev(A)
+    ipiv_ref, _ = cf.getrf(ref)
+    size = cf.lib().cf_getrf_optimal_workspace_size(n, ctypes.byref(cf.options()))
+    work = torch.empty(size + offset + 4, dtype=torch.uint8, device="cuda")
+    work[offset + size:] = 77                        # nothing is written past the size asked for
+    dA = _dev(A)
+    ipiv, info = cf.getrf(dA, work=work[offset:offset + size], lookahead=lookahead)
+    assert int(info.item()) == 0 and bool((work[offset + size:] == 77).all())
+    np.testing.assert_array_equal(dA.cpu().numpy(), ref.cpu().numpy())
+    np.testing.assert_array_equal(ipiv.cpu().numpy(), ipiv_ref.cpu().numpy())
