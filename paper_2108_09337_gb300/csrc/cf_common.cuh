@@ -131,6 +131,19 @@ __device__ __forceinline__ unsigned exp_bits(double x) { return ((unsigned)__dou
 __device__ __forceinline__ bool is_zero(double x) {
     return (((unsigned)__double2hiint(x) << 1) | (unsigned)__double2loint(x)) == 0u;
 }
+// RN(x / u) from r = quot_recip(u) = RN(1 / u): two residual corrections (the
+// second one gives the correctly rounded quotient by Markstein's theorem, IBM
+// J. Res. Dev. 34, 1990).  r = 0 marks a u outside 2^+-300; where quot_odd
+// says so (such a u, an x outside 2^+-600 other than zero) the caller divides.
+__device__ __forceinline__ double quot_recip(double u) { return exp_bits(u) - 723u <= 600u ? __drcp_rn(u) : 0.0; }
+__device__ __forceinline__ bool quot_odd(double x, double r) {
+    return __double2hiint(r) == 0 || (exp_bits(x) - 423u > 1200u && !is_zero(x));
+}
+__device__ __forceinline__ double quot_from(double x, double u, double r) {
+    const double q0 = x * r;
+    const double q1 = fma(fma(-q0, u, x), r, q0);
+    return is_zero(x) ? q0 : fma(fma(-q1, u, x), r, q1);
+}
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ float div_rn(float a, float b) { return __fdiv_rn(a, b); }

@@ -266,16 +266,10 @@ constexpr int kLdM = kMaxV + 1;
 // LU-3's quotient in full: a zero pivot divides nothing.
 static __device__ __noinline__ double pivot_div(double x, double u) { return u != 0.0 ? __ddiv_rn(x, u) : x; }
 
-// RN(x / u) for u with r = RN(1 / u): two residual corrections (the second one
-// gives the correctly rounded quotient by Markstein's theorem, IBM J. Res. Dev.
-// 34, 1990).  r = 0 marks a u outside 2^+-300; such u, and x outside 2^+-600
-// other than zero, are divided.
+// RN(x / u) with r = quot_recip(u).
 __device__ __forceinline__ double quot_rn(double x, double u, double r) {
-    const double q0 = x * r;
-    const double q1 = fma(fma(-q0, u, x), r, q0);
-    const double q2 = fma(fma(-q1, u, x), r, q1);
-    double q = q2;
-    if (__double2hiint(r) == 0 || exp_bits(x) - 423u > 1200u) q = __double2hiint(r) != 0 && is_zero(x) ? q0 : pivot_div(x, u);
+    double q = quot_from(x, u, r);
+    if (quot_odd(x, r)) q = pivot_div(x, u);
     return q;
 }
 
@@ -310,7 +304,7 @@ k_panel_solve(double *__restrict__ X, int ldx, int lines, int per, int w, const 
     if (KIND != kLeft) {
         for (int k = tid; k < w; k += nthr) {
             const double u = Ms[k * kLdM + k];
-            rs[k] = exp_bits(u) - 723u <= 600u ? __drcp_rn(u) : (KIND == kChol ? 1.0 / u : 0.0);
+            rs[k] = KIND == kRight ? quot_recip(u) : (exp_bits(u) - 723u <= 600u ? __drcp_rn(u) : 1.0 / u);
         }
         __syncthreads();
     }
