@@ -19,9 +19,10 @@ namespace cf {
 constexpr int kBM = 64, kBN = 64, kBK = 16;
 constexpr int kGemmThreads = 256;
 
-// C[m x n] -= A[m x k] * op(B)[k x n]
+// C[m x n] -= op(A)[m x k] * op(B)[k x n]
+//   op(A)(i, p) = TA ? A[p + i*lda] : A[i + p*lda]
 //   op(B)(p, j) = TB ? B[j + p*ldb] : B[p + j*ldb]
-template <bool TB, bool LOWER>
+template <bool TA, bool TB, bool LOWER>
 __global__ void __launch_bounds__(kGemmThreads)
 k_gemm_sub(int m, int n, int k, const double *__restrict__ A, int lda, const double *__restrict__ B, int ldb,
            double *__restrict__ C, int ldc, const int *skip) {
@@ -43,10 +44,11 @@ k_gemm_sub(int m, int n, int k, const double *__restrict__ A, int lda, const dou
 #pragma unroll
         for (int e = 0; e < (kBM * kBK) / kGemmThreads; ++e) {
             const int idx = tid + e * kGemmThreads;
-            const int i = idx % kBM, p = idx / kBM;
+            int i, p;
+            if (!TA) { i = idx % kBM; p = idx / kBM; } else { p = idx % kBK; i = idx / kBK; }
             const int gi = bm + i, gp = p0 + p;
             double v = 0.0;
-            if (gi < m && gp < k) v = A[(size_t)gi + (size_t)gp * lda];
+            if (gi < m && gp < k) v = TA ? A[(size_t)gp + (size_t)gi * lda] : A[(size_t)gi + (size_t)gp * lda];
             As[p][i] = v;
         }
 #pragma unroll
@@ -95,11 +97,22 @@ int launch_gemm_f64_sub(int m, int n, int k, const double *A, int lda, const dou
     dim3 grid(ceil_div(m, kBM), ceil_div(n, kBN));
     if (grid.y > 65535) return CF_ERR_UNSUPPORTED;
     if (trans_b && lower)
-        k_gemm_sub<true, true><<<grid, kGemmThreads, 0, st>>>(m, n, k, A, lda, B, ldb, C, ldc, skip);
+        k_gemm_sub<false, true, true><<<grid, kGemmThreads, 0, st>>>(m, n, k, A, lda, B, ldb, C, ldc, skip);
     else if (!trans_b && !lower)
-        k_gemm_sub<false, false><<<grid, kGemmThreads, 0, st>>>(m, n, k, A, lda, B, ldb, C, ldc, skip);
+        k_gemm_sub<false, false, false><<<grid, kGemmThreads, 0, st>>>(m, n, k, A, lda, B, ldb, C, ldc, skip);
     else
         return CF_ERR_UNSUPPORTED;
+    CF_LAUNCH_CHECK();
+    return CF_OK;
+}
+
+// C -= A^T B, A k x m.
+int launch_gemm_f64_sub_at(int m, int n, int k, const double *A, int lda, const double *B, int ldb, double *C, int ldc,
+                           cudaStream_t st) {
+    if (m <= 0 || n <= 0 || k <= 0) return CF_OK;
+    dim3 grid(ceil_div(m, kBM), ceil_div(n, kBN));
+    if (grid.y > 65535) return CF_ERR_UNSUPPORTED;
+    k_gemm_sub<true, false, false><<<grid, kGemmThreads, 0, st>>>(m, n, k, A, lda, B, ldb, C, ldc, nullptr);
     CF_LAUNCH_CHECK();
     return CF_OK;
 }

@@ -73,6 +73,8 @@ int launch_potf2(double *A00, int lda, int w, int kglob, int *info, cudaStream_t
 // whose nonzero value turns the launch into a no-op (Cholesky breakdown).
 int launch_gemm_f64_sub(int m, int n, int k, const double *A, int lda, const double *B, int ldb, bool trans_b,
                         double *C, int ldc, bool lower, const int *skip_if_nonzero, cudaStream_t st);
+int launch_gemm_f64_sub_at(int m, int n, int k, const double *A, int lda, const double *B, int ldb, double *C, int ldc,
+                           cudaStream_t st);
 // ---- FP32 panel kernels of the mixed path (cf_tourn32.cu, cf_panel32.cu)
 int launch_tourn32(const float *P, int ldp, int m, int w, int h, int arity, const TournWS &ws, const TournEpilogue &ep,
                    cudaStream_t st);

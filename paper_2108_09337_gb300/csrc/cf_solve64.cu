@@ -4,7 +4,8 @@
 // A solve with an n x n triangle is a chain of n dependent steps; its bytes
 // (4 n^2 per direction) and its 2 lanes of FP64 per clock and SM are far from
 // binding for a few right-hand sides.  So the chain is what counts:
-//   * the triangle is cut into super-blocks of 2048 rows.  One thread-block
+//   * the triangle is cut into super-blocks of 2048 rows.  (Up to some 200
+//     right-hand sides; more go block by block over all of them.)  One thread-block
 //     cluster per right-hand side solves a super-block; its rows beyond take
 //     one launch over the whole GPU;
 //   * inside the cluster, a solved block is written into every CTA's shared
@@ -550,12 +551,8 @@ static int chol_mode(int n, int nrhs, const double *T, int ldt, double *X, int l
     for (int q = 0; q < ns; ++q) {
         const int k0 = (FWD ? q : ns - 1 - q) * kSuper;
         const int w = kSuper < n - k0 ? kSuper : n - k0;
-        for (int c0 = 0; c0 < nrhs; c0 += 65535) {
-            const int nc = nrhs - c0 < 65535 ? nrhs - c0 : 65535;
-            k_tri_solve64<MODE><<<dim3(CL, nc), kThreads, sizeof(Smem), st>>>(w, T + k0 + k0 * ld, ldt,
-                                                                            X + k0 + (size_t)c0 * ldx, ldx);
-            CF_LAUNCH_CHECK();
-        }
+        k_tri_solve64<MODE><<<dim3(CL, nrhs), kThreads, sizeof(Smem), st>>>(w, T + k0 + k0 * ld, ldt, X + k0, ldx);
+        CF_LAUNCH_CHECK();
         if (FWD) {
             const int r0 = k0 + w;
             const int rc = launch_residual_f64(n - r0, w, nrhs, T + r0 + k0 * ld, ldt, X + k0, ldx, X + r0, ldx, X + r0,
@@ -577,30 +574,114 @@ static int lu_mode(int n, int nrhs, const double *T, int ldt, double *X, int ldx
         const int k0 = (FWD ? q : ns - 1 - q) * kSuper;
         const int w = kSuper < n - k0 ? kSuper : n - k0;
         const int r0 = FWD ? k0 + w : 0, m = FWD ? n - r0 : k0;      // the rows beyond
-        for (int c0 = 0; c0 < nrhs; c0 += 65535) {
-            const int nc = nrhs - c0 < 65535 ? nrhs - c0 : 65535;
-            double *Xc = X + (size_t)c0 * ldx;
-            k_lu_solve64<FWD><<<dim3(CL, nc), kThreads, 0, st>>>(w, T + k0 + k0 * ld, ldt, Xc + k0, ldx);
-            CF_LAUNCH_CHECK();
-            if (m <= 0) continue;
-            k_lu_rows_sub<<<dim3(ceil_div(m, 32), nc), 32, 0, st>>>(m, w, T + r0 + k0 * ld, ldt, Xc + k0, Xc + r0, ldx,
-                                                                   FWD ? 0 : 1);
-            CF_LAUNCH_CHECK();
+        k_lu_solve64<FWD><<<dim3(CL, nrhs), kThreads, 0, st>>>(w, T + k0 + k0 * ld, ldt, X + k0, ldx);
+        CF_LAUNCH_CHECK();
+        if (m <= 0) continue;
+        k_lu_rows_sub<<<dim3(ceil_div(m, 32), nrhs), 32, 0, st>>>(m, w, T + r0 + k0 * ld, ldt, X + k0, X + r0, ldx,
+                                                                 FWD ? 0 : 1);
+        CF_LAUNCH_CHECK();
+    }
+    return CF_OK;
+}
+
+// ---------------------------------------------------------------------------
+// Many right-hand sides: per block of 128 rows one left solve over all columns
+// and one product over the whole GPU, with k_lu_solve64's order of operations.
+// Its time hardly grows with their number, the clusters' does (every one reads
+// the triangle and takes 8 CTAs).  Both directions, blocked / clusters, ms:
+//   LU        n = 130: 128 rhs 0.72 / 0.66, 160 0.72 / 0.81; n = 300: 192 1.64 /
+//             1.44, 256 1.64 / 1.91; n = 2048: 256 12.3 / 10.9, 320 12.0 / 12.7;
+//             n = 8192: 256 71.6 / 66.7, 320 76.6 / 79.3, 512 96.5 / 127.9
+//   Cholesky  n = 130: 64 0.99 / 0.94, 96 0.99 / 1.30; n = 300: 160 2.24 / 2.05,
+//             192 2.25 / 2.43; n = 2048: 192 17.2 / 13.0, 256 17.2 / 18.0;
+//             n = 8192: 192 83.3 / 75.5, 256 89.4 / 103.1
+//
+// X <- M^{-1} X with M = T (TRANS: T^T) of size w x w, lower (forward) or upper
+// (backward), non-unit.  CTA: 64 columns, four lanes of one warp each.
+// ---------------------------------------------------------------------------
+constexpr int kCB = 64;
+constexpr size_t kBlockSmem = sizeof(double) * ((size_t)kMaxV * kMaxV + (size_t)kCB * (kMaxV + 1));
+
+template <bool LOWER, bool TRANS>
+__global__ void __launch_bounds__(kThreads, 1)
+k_block_solve(double *X, int ldx, int w, int cols, const double *__restrict__ T, int ldt) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double *Ms = reinterpret_cast<double *>(smem_raw);        // Ms[k * kMaxV + i] = M(i, k)
+    double *Xs = Ms + kMaxV * kMaxV;                          // Xs[c * XLD + i]
+    constexpr int XLD = kMaxV + 1;
+    const int tid = threadIdx.x;
+    const int c0 = blockIdx.x * kCB, nc = min(kCB, cols - c0);
+    for (int e = tid; e < w * w; e += kThreads) {
+        const int a = e % w, b = e / w;                       // a runs along the memory
+        const int i = TRANS ? b : a, k = TRANS ? a : b;
+        if (LOWER ? i >= k : i <= k) Ms[k * kMaxV + i] = T[(size_t)a + (size_t)b * ldt];
+    }
+    for (int e = tid; e < nc * w; e += kThreads) Xs[e / w * XLD + e % w] = X[(size_t)(e % w) + (size_t)(c0 + e / w) * ldx];
+    __syncthreads();
+    const int c = tid >> 2, q = tid & 3;
+    if (c < nc) {
+        double *x = Xs + c * XLD;
+        const unsigned mask = 0xfu << (tid & 28);
+        for (int s = 0; s < w; ++s) {
+            const int k = LOWER ? s : w - 1 - s;
+            if (q == 0) x[k] = div_rn(x[k], Ms[k * kMaxV + k]);
+            __syncwarp(mask);
+            const double xk = x[k];
+            for (int i = LOWER ? k + 1 + q : q; i < (LOWER ? w : k); i += 4) x[i] = sub_rn(x[i], mul_rn(Ms[k * kMaxV + i], xk));
+            __syncwarp(mask);
         }
+    }
+    __syncthreads();
+    for (int e = tid; e < nc * w; e += kThreads) X[(size_t)(e % w) + (size_t)(c0 + e / w) * ldx] = Xs[e / w * XLD + e % w];
+}
+
+template <bool LOWER, bool TRANS>
+static int block_solve(double *X, int ldx, int w, int cols, const double *T, int ldt, cudaStream_t st) {
+    CF_CUDA_TRY(cudaFuncSetAttribute(k_block_solve<LOWER, TRANS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)kBlockSmem));
+    k_block_solve<LOWER, TRANS><<<ceil_div(cols, kCB), kThreads, kBlockSmem, st>>>(X, ldx, w, cols, T, ldt);
+    CF_LAUNCH_CHECK();
+    return CF_OK;
+}
+
+static int blocked_solve(int mode, int n, int nrhs, const double *T, int ldt, double *X, int ldx, cudaStream_t st) {
+    const bool fwd = mode == 0 || mode == 2;
+    const size_t ld = (size_t)ldt;
+    const int nb = ceil_div(n, LB);
+    for (int b = 0; b < nb; ++b) {
+        const int k0 = (fwd ? b : nb - 1 - b) * LB, w = LB < n - k0 ? LB : n - k0;
+        const double *D = T + k0 + k0 * ld;
+        double *Y = X + k0;
+        int rc = mode == 0   ? launch_trsm_left_lower_unit(Y, ldx, w, nrhs, D, ldt, st)
+                 : mode == 1 ? block_solve<false, false>(Y, ldx, w, nrhs, D, ldt, st)
+                 : mode == 2 ? block_solve<true, false>(Y, ldx, w, nrhs, D, ldt, st)
+                             : block_solve<false, true>(Y, ldx, w, nrhs, D, ldt, st);
+        if (rc) return rc;
+        if (fwd)
+            rc = launch_gemm_f64_sub(n - k0 - w, nrhs, w, D + w, ldt, Y, ldx, false, Y + w, ldx, false, nullptr, st);
+        else if (mode == 1)
+            rc = launch_gemm_f64_sub(k0, nrhs, w, T + k0 * ld, ldt, Y, ldx, false, X, ldx, false, nullptr, st);
+        else
+            rc = launch_gemm_f64_sub_at(k0, nrhs, w, T + k0, ldt, Y, ldx, X, ldx, st);
+        if (rc) return rc;
     }
     return CF_OK;
 }
 
 }  // namespace sv
 
+// Right-hand sides up to which a cluster takes each (measured above).
+static int most_clusters(int mode, int n) { return mode < 2 ? (n > 256 ? 256 : 128) : (n > 256 ? 160 : 64); }
+
 int launch_tri_solve64(int mode, int n, int nrhs, const double *T, int ldt, double *X, int ldx, cudaStream_t st) {
     if (n <= 0 || nrhs <= 0) return CF_OK;
+    if (mode < 0 || mode > 3) return CF_ERR_UNSUPPORTED;
+    if (nrhs > most_clusters(mode, n)) return sv::blocked_solve(mode, n, nrhs, T, ldt, X, ldx, st);
     switch (mode) {
         case 0: return sv::lu_mode<true>(n, nrhs, T, ldt, X, ldx, st);
         case 1: return sv::lu_mode<false>(n, nrhs, T, ldt, X, ldx, st);
         case 2: return sv::chol_mode<2>(n, nrhs, T, ldt, X, ldx, st);
-        case 3: return sv::chol_mode<3>(n, nrhs, T, ldt, X, ldx, st);
-        default: return CF_ERR_UNSUPPORTED;
+        default: return sv::chol_mode<3>(n, nrhs, T, ldt, X, ldx, st);
     }
 }
 

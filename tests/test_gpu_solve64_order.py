@@ -76,3 +76,23 @@ def test_operation_order(cf, n, scale):
     X = cf.getrs(_dev(L + np.eye(n)), ident, _dev(b[:, None], n + 3)).cpu().numpy()      # U = I
     np.testing.assert_array_equal(X[:, 0], _solve(L, b, True))
     assert cf.device_status() == cf.CF_OK
+
+
+@pytest.mark.parametrize("n,nrhs", [(1, 129), (65, 129), (256, 200), (257, 257), (300, 300), (577, 1025), (2200, 260)])
+def test_many_right_hand_sides(cf, n, nrhs):
+    """Above a few hundred right-hand sides the solves go block by block over
+    all of them: the same bits with LU factors, substitution's bound with Cholesky's."""
+    u = 2.0 ** -53
+    rng = np.random.default_rng(n)
+    L, Um, _ = _factors(n, rng, False)
+    B = rng.standard_normal((n, nrhs))
+    ip = torch.from_numpy(np.arange(n, 0, -1).astype(np.int32)).cuda()        # any list is played
+    LU = _dev(L + Um, n + 2)
+    X = cf.getrs(LU, ip, _dev(B, n + 1)).cpu().numpy()
+    for c in (0, nrhs // 2, nrhs - 1):
+        np.testing.assert_array_equal(X[:, [c]], cf.getrs(LU, ip, _dev(B[:, [c]])).cpu().numpy())
+    Lc = np.tril(Um.T)
+    X = cf.potrs(_dev(Lc, n + 2), _dev(B, n + 1)).cpu().numpy()
+    R = np.abs(B - Lc @ (Lc.T @ X))
+    assert (R <= 6 * (n + 4) * u * (np.abs(Lc) @ (np.abs(Lc.T) @ np.abs(X)))).all()
+    assert cf.device_status() == cf.CF_OK
