@@ -69,6 +69,7 @@ _SIG = {
     "cf_kernel_launches": (ctypes.c_longlong, []),
     "cf_tourn_workspace_size": (_S, [_I, _I, _I, _I]),
     "cf_tourn_select": (_I, [_I, _I, _P, _I, _I, _I, _P, _P, _S, _P]),
+    "cf_tourn_select_withheld": (_I, [_I, _I, _P, _I, _I, _I, _P, ctypes.c_longlong, _P, _S, _P]),
     "cf_tourn_select_f32": (_I, [_I, _I, _P, _I, _I, _I, _P, _P, _S, _P]),
     "cf_getrf_workspace_size": (_S, [_I, _OPT]),
     "cf_getrf_optimal_workspace_size": (_S, [_I, _OPT]),
@@ -214,6 +215,19 @@ def tourn_select(panel: torch.Tensor, leaf_h: int = 128, arity: int = 2) -> torc
     fn, name = ((_lib.cf_tourn_select, "cf_tourn_select") if panel.dtype == torch.float64
                 else (_lib.cf_tourn_select_f32, "cf_tourn_select_f32"))
     _check(name, fn(m, w, _ptr(panel), ld, leaf_h, arity, _ptr(win), _ptr(ws), ws.numel(), _stream()))
+    return win[:min(m, w)]
+
+
+def tourn_select_withheld(panel: torch.Tensor, leaf_h: int = 128, arity: int = 2, spin_limit: int = 0) -> torch.Tensor:
+    """cf_tourn_select_withheld: the FP64 selection with a candidate withheld, so
+    that the wait for it runs out (failure-detection test; the winners are rows
+    in range and cf_device_status reports CF_ERR_TIMEOUT)."""
+    m, w = panel.shape
+    win = torch.empty(max(min(m, w), 1), dtype=torch.int32, device=panel.device)
+    ws = _workspace(_lib.cf_tourn_workspace_size(m, w, leaf_h, arity), panel.device)
+    _check("cf_tourn_select_withheld",
+           _lib.cf_tourn_select_withheld(m, w, _ptr(panel), _ld(panel, "panel"), leaf_h, arity, _ptr(win), spin_limit,
+                                         _ptr(ws), ws.numel(), _stream()))
     return win[:min(m, w)]
 
 

@@ -68,6 +68,7 @@ struct TournSmem {
     int win[kMaxV];
     int cnt;
     int bad;
+    int abort_flag;                              // 1: a wait in the cluster ran out
 };
 
 // Rank of a candidate as an unsigned key: |a| by its bits, NaN below every
@@ -95,10 +96,14 @@ __device__ __forceinline__ void named_bar_sync(int id, int threads) {
 
 __device__ int g_tourn_status = 0;               // 0 or CF_ERR_TIMEOUT
 
+constexpr long long kTournSpin = 1ll << 17;      // polls: half a second (a poll that finds nothing takes 3.9 us)
+
 // Waits (bounded) until the barrier's phase of this parity has completed; the
-// writes of every arrival are then visible.
-__device__ __forceinline__ void tourn_wait(uint64_t *bar, uint32_t parity) {
-    for (long long i = 0; i < (1ll << 22); ++i) {
+// writes of every arrival are then visible.  False where the wait, or any other
+// of the cluster, ran out: the abort flags of all its CTAs are set then.
+__device__ __forceinline__ bool tourn_wait(TournSmem &s, uint64_t *bar, uint32_t parity, long long limit) {
+    volatile int *abort_flag = &s.abort_flag;
+    for (long long i = 0; i < limit; ++i) {
         uint32_t ok;
         asm volatile(
             "{\n\t.reg .pred p;\n\t"
@@ -107,10 +112,16 @@ __device__ __forceinline__ void tourn_wait(uint64_t *bar, uint32_t parity) {
             : "=r"(ok)
             : "r"((uint32_t)__cvta_generic_to_shared(bar)), "r"(parity)
             : "memory");
-        if (ok) return;
-        if (i > 64) __nanosleep(20);
+        if (ok) return true;
+        if (i > 64) {
+            if (*abort_flag) return false;
+            __nanosleep(20);
+        }
     }
+    cg::cluster_group cl = cg::this_cluster();
+    for (unsigned p = 0; p < cl.num_blocks(); ++p) *(volatile int *)cl.map_shared_rank(&s.abort_flag, p) = 1;
     atomicExch(&g_tourn_status, CF_ERR_TIMEOUT);
+    return false;
 }
 
 // One phase more on the barrier: complete once `bytes` have arrived.
@@ -142,6 +153,8 @@ struct TournLevel {
     int ldp, m, w, h, arity, level, root;
     int cnt_below, off_below, off;               // nodes of the level below, first node indexes
     int per, ld;                                 // rows per CTA at most; leading dimension of the tile (odd)
+    long long spin;                              // polls of a wait
+    int withhold;                                // failure test: the first candidate of node 0 does not go out
 };
 
 // Root epilogue: LAPACK ipiv and the list of moved rows (relative positions)
@@ -222,7 +235,7 @@ k_tourn_level(TournLevel lv, TournWS ws, TournEpilogue ep) {
     const int nw = (lv.per + 31) / 32, nslots = nw * ncta;      // a slot per warp that has rows
     if (tid == 0) {
         s.nact[0] = mine;
-        s.bad = 0;
+        s.bad = s.abort_flag = 0;
         for (int b = 0; b < 2; ++b)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(&s.bar[b])),
                          "r"(1)
@@ -291,11 +304,11 @@ k_tourn_level(TournLevel lv, TournWS ws, TournEpilogue ep) {
                 if (u > 0) {
                     // ---- the winner of column j0 + u - 1, found by every warp alike
                     const int par = (j0 + u - 1) & 1;
-                    tourn_wait(&s.bar[par], (phase >> par) & 1u);
+                    const bool ok = __all_sync(0xffffffffu, tourn_wait(s, &s.bar[par], (phase >> par) & 1u, lv.spin));
                     phase ^= 1u << par;
                     // (armed again before this warp's next candidate goes out, which
                     // every sender of the next but one waits for)
-                    if (tid == 0) tourn_arm(&s.bar[par], nslots * kSlotBytes);
+                    if (tid == 0 && ok && !*(volatile int *)&s.abort_flag) tourn_arm(&s.bar[par], nslots * kSlotBytes);
                     int at = lane, best = lane < nslots ? (int)__double_as_longlong(s.slot[par][lane][kTB]) : -1;
                     unsigned long long key = best >= 0 ? piv_key(s.slot[par][lane][u - 1]) : 0ull;
                     if (nslots > 32) {
@@ -303,8 +316,11 @@ k_tourn_level(TournLevel lv, TournWS ws, TournEpilogue ep) {
                         const unsigned long long k1 = i1 >= 0 ? piv_key(s.slot[par][lane + 32][u - 1]) : 0ull;
                         if (k1 > key || (k1 == key && k1 != 0 && i1 < best)) { key = k1; best = i1; at = lane + 32; }
                     }
-                    const int gi = warp_best(key, best);
-                    at = __shfl_sync(0xffffffffu, at, __ffs(__ballot_sync(0xffffffffu, best == gi)) - 1);
+                    // (after a wait that ran out the slots hold anything: any row in range will do, the
+                    // order is replaced at the end)
+                    int gi = warp_best(key, best);
+                    if (!ok || (unsigned)gi >= (unsigned)total) gi = j0 + u - 1;
+                    at = __shfl_sync(0xffffffffu, at, max(__ffs(__ballot_sync(0xffffffffu, best == gi)) - 1, 0));
                     const double *pv = s.slot[par][at];
                     const double piv = pv[u - 1];
                     const bool go = !is_zero(piv);           // a zero pivot eliminates nothing
@@ -353,7 +369,7 @@ k_tourn_level(TournLevel lv, TournWS ws, TournEpilogue ep) {
                 // lane = (CTA, half): asynchronous stores that count on the CTA's barrier
                 {
                     const int cta = lane >> 1, half = lane & 1;
-                    if (cta < ncta) {
+                    if (cta < ncta && !(lv.withhold && g == 0 && rank == 0 && warp == 0 && j0 + u == 0)) {
                         uint32_t dst, bar;
                         asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
                                      : "=r"(dst)
@@ -444,6 +460,20 @@ k_tourn_level(TournLevel lv, TournWS ws, TournEpilogue ep) {
     }
     __threadfence();
     if (ncta > 1) cl.sync();                     // remote reads of the tiles and the winners' list are done
+    else __syncthreads();
+    if (s.abort_flag) {
+        // A wait ran out: the CTAs may have followed different winners.  The first
+        // rows instead, so that every list that others index with is whole; the
+        // host learns of it from the status.  What is still on its way lands first.
+        for (int j = rank + tid * ncta; j < npiv; j += kTournThreads * ncta) {
+            dst[j] = s.rows[j / ncta];
+            if (lv.root) ws.root_win[j] = s.rows[j / ncta];
+        }
+        if (lv.root && ep.lu != nullptr && rank == 0 && tid == 0) *ep.lu_ok = 0;
+        __nanosleep(20000);
+        __threadfence();
+        cl.sync();
+    }
     if (lv.root && rank == 0 && ep.ipiv != nullptr) {
         __syncthreads();
         for (int j = tid; j < npiv; j += kTournThreads) s.win[j] = __ldcg(ws.root_win + j);
@@ -583,8 +613,8 @@ static int tourn_max_cluster() {
     return n;
 }
 
-int launch_tourn(const double *P, int ldp, int m, int w, int h, int arity, const TournWS &ws, const TournEpilogue &ep,
-                 cudaStream_t st) {
+static int run_tourn(const double *P, int ldp, int m, int w, int h, int arity, const TournWS &ws,
+                     const TournEpilogue &ep, long long spin, bool withhold, cudaStream_t st) {
     if (h > kMaxV || arity > 8) return CF_ERR_UNSUPPORTED;      // a node has at most 8 x kMaxV rows
     TournPlan plan{};
     int rc = make_tourn_plan(m, w, h, arity, &plan);
@@ -615,6 +645,8 @@ int launch_tourn(const double *P, int ldp, int m, int w, int h, int arity, const
         lv.off = plan.off[l];
         lv.per = ceil_div(rows, cta);
         lv.ld = lv.per | 1;
+        lv.spin = spin;
+        lv.withhold = withhold && l == 0;
         const size_t smem = align_up(sizeof(TournSmem), 16) + sizeof(double) * (size_t)lv.ld * w;
         // the attributes belong to the current device: set on every call
         CF_CUDA_TRY(cudaFuncSetAttribute(k_tourn_level, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTournMaxSmem));
@@ -635,6 +667,11 @@ int launch_tourn(const double *P, int ldp, int m, int w, int h, int arity, const
         count_launches(1);
     }
     return CF_OK;
+}
+
+int launch_tourn(const double *P, int ldp, int m, int w, int h, int arity, const TournWS &ws, const TournEpilogue &ep,
+                 cudaStream_t st) {
+    return run_tourn(P, ldp, m, w, h, arity, ws, ep, kTournSpin, false, st);
 }
 
 int tourn_take_status(cudaStream_t st, int *status) {
@@ -675,8 +712,8 @@ extern "C" size_t cf_tourn_workspace_size(int m, int w, int leaf_h, int arity) {
     return cf::tourn_ws_bytes(m > 0 ? m : 1, 1, arity < 2 ? 2 : arity);
 }
 
-extern "C" int cf_tourn_select(int m, int w, const double *panel, int ldp, int leaf_h, int arity, int *winners,
-                               void *work, size_t lwork, cudaStream_t stream) {
+static int tourn_select_api(int m, int w, const double *panel, int ldp, int leaf_h, int arity, int *winners, void *work,
+                            size_t lwork, long long spin, bool withhold, cudaStream_t stream) {
     using namespace cf;
     if (m < 0) return -1;
     if (w < 0 || w > kMaxV) return -2;
@@ -694,5 +731,20 @@ extern "C" int cf_tourn_select(int m, int w, const double *panel, int ldp, int l
     ep.ipiv = nullptr;
     CF_CUDA_TRY(cudaMemsetAsync(ws.counter, 0, ws.counter_bytes, stream));
     ws.root_win = winners;
-    return launch_tourn(panel, ldp, m, w, leaf_h, arity, ws, ep, stream);
+    return run_tourn(panel, ldp, m, w, leaf_h, arity, ws, ep, spin, withhold, stream);
+}
+
+extern "C" int cf_tourn_select(int m, int w, const double *panel, int ldp, int leaf_h, int arity, int *winners,
+                               void *work, size_t lwork, cudaStream_t stream) {
+    return tourn_select_api(m, w, panel, ldp, leaf_h, arity, winners, work, lwork, cf::kTournSpin, false, stream);
+}
+
+// Failure-detection test of the bounded waits, not part of the API: the first
+// candidate of the first leaf is withheld, so that the wait for it gives up
+// after spin_limit polls (0: the usual number).
+extern "C" int cf_tourn_select_withheld(int m, int w, const double *panel, int ldp, int leaf_h, int arity, int *winners,
+                                        long long spin_limit, void *work, size_t lwork, cudaStream_t stream) {
+    if (spin_limit < 0) return -8;
+    return tourn_select_api(m, w, panel, ldp, leaf_h, arity, winners, work, lwork,
+                            spin_limit > 0 ? spin_limit : cf::kTournSpin, true, stream);
 }
