@@ -92,6 +92,7 @@ _SIG = {
     "cf_device_status": (_I, [_P]),
     "cf_trsv_f32_workspace_size": (_S, [_I]),
     "cf_trsv_f32": (_I, [_I, _I, _I, _P, _I, _P, _I, _P, _S, _P]),
+    "cf_tri_solve64_withheld": (_I, [_I, _I, _I, _P, _I, _P, _I, ctypes.c_longlong, _P]),
     "cf_trsv_f32_withheld": (_I, [_I, _I, _I, _P, _I, _P, _I, ctypes.c_longlong, _P, _S, _P]),
     "cf_factor_batched_workspace_size": (_S, [_I, _OPT]),
     "cf_factor_batched": (_I, [_I, _P, _I, _P, _P, _P, _P, _P, _P, _S, _OPT, _P]),
@@ -301,6 +302,16 @@ def potrs(L: torch.Tensor, B: torch.Tensor):
     nrhs = B.shape[1] if B.dim() == 2 else 1
     _check("cf_potrs", _lib.cf_potrs(n, nrhs, _ptr(L), _ld(L, "L"), _ptr(B), _ld(B, "B"), _stream()))
     return B
+
+
+def tri_solve64_withheld(T: torch.Tensor, X: torch.Tensor, mode: int, spin_limit: int = 0):
+    """cf_tri_solve64_withheld: one direction of the FP64 solves with its first
+    block withheld, so that the waits for it run out (failure-detection test; X
+    comes back wrong and cf_device_status reports CF_ERR_TIMEOUT)."""
+    n, nrhs = X.shape
+    _check("cf_tri_solve64_withheld", _lib.cf_tri_solve64_withheld(mode, n, nrhs, _ptr(T), _ld(T, "T"), _ptr(X),
+                                                                   _ld(X, "X"), spin_limit, _stream()))
+    return X
 
 
 def residual(A: torch.Tensor, X: torch.Tensor, B: torch.Tensor, R: torch.Tensor | None = None):

@@ -53,12 +53,17 @@ struct Smem {
     double part[4 * NB];
     double pub[NB];
     uint64_t bar[MAXB];
+    int dead;                          // a wait ran out
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-__device__ __forceinline__ void wait_block(uint64_t *bar) {
-    for (long long i = 0; i < (1ll << 22); ++i) {
+constexpr long long kSpin = 1ll << 17;      // polls: half a second (a poll that finds nothing takes 3.9 us)
+
+// Waits (bounded) for a solved block; where one wait ran out (*dead) the CTA's
+// others give up too, and the solve ends with X wrong and the status set.
+__device__ __forceinline__ void wait_block(uint64_t *bar, volatile int *dead, long long limit) {
+    for (long long i = 0; i < limit; ++i) {
         uint32_t ok;
         asm volatile(
             "{\n\t.reg .pred p;\n\t"
@@ -68,8 +73,12 @@ __device__ __forceinline__ void wait_block(uint64_t *bar) {
             : "r"(smem_u32(bar))
             : "memory");
         if (ok) return;
-        if (i > 64) __nanosleep(20);
+        if (i > 64) {
+            if (*dead) return;
+            __nanosleep(20);
+        }
     }
+    *dead = 1;
     atomicExch(&g_solve64_status, CF_ERR_TIMEOUT);
 }
 
@@ -80,6 +89,7 @@ static_assert(LBLK == 2 * CL, "a half CTA owns one block");
 struct LuSmem {
     double xs[LBLK][LB];               // solved blocks, in solving order
     uint64_t bar[LBLK][LB / 32];       // their 32-row parts
+    int dead;                          // a wait ran out
 };
 
 // L y = b (FWD, unit lower) or U x = y with a super-block of the LU factors.
@@ -93,7 +103,7 @@ struct LuSmem {
 // 48.5).
 template <bool FWD>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(kThreads)
-k_lu_solve64(int n, const double *__restrict__ T, int ldt, double *__restrict__ X, int ldx) {
+k_lu_solve64(int n, const double *__restrict__ T, int ldt, double *__restrict__ X, int ldx, long long spin, int withhold) {
     __shared__ LuSmem s;
     cg::cluster_group cl = cg::this_cluster();
     const int tid = threadIdx.x, lane = tid & 31, q = (tid & (LB - 1)) >> 5;      // q: part of the block
@@ -104,7 +114,10 @@ k_lu_solve64(int n, const double *__restrict__ T, int ldt, double *__restrict__ 
     auto row0 = [&](int b) { return (FWD ? b : nb - 1 - b) * LB; };
     if (tid < LBLK * (LB / 32))
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s.bar[0][0] + tid)) : "memory");
-    if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (tid == 0) {
+        s.dead = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
     cl.sync();
     if (t < nb) {
         const int r0 = row0(t), row = r0 + 32 * q + lane;
@@ -132,7 +145,7 @@ k_lu_solve64(int n, const double *__restrict__ T, int ldt, double *__restrict__ 
             if (c + 1 < last) load(c + 1, nxt);
             if (c < own0) {                                   // a block solved before: one FMA chain
                 const int b = c >> 3, kk = c & 7;
-                if ((kk & 1) == 0) wait_block(&s.bar[b][kk >> 1]);
+                if ((kk & 1) == 0) wait_block(&s.bar[b][kk >> 1], &s.dead, spin);
 #pragma unroll
                 for (int a = 0; a < 16; ++a) acc = fma(cur[a], s.xs[b][16 * kk + a], acc);
                 if (kk == 7) {
@@ -141,7 +154,7 @@ k_lu_solve64(int n, const double *__restrict__ T, int ldt, double *__restrict__ 
                 }
             } else if (c < last - 2) {                        // a part of this block solved before
                 const int k0 = first_col(c) - r0;
-                if (((c - own0) & 1) == 0) wait_block(&s.bar[t][k0 >> 5]);
+                if (((c - own0) & 1) == 0) wait_block(&s.bar[t][k0 >> 5], &s.dead, spin);
 #pragma unroll
                 for (int a = 0; a < 16; ++a) {
                     const int e = FWD ? a : 15 - a;
@@ -169,7 +182,7 @@ k_lu_solve64(int n, const double *__restrict__ T, int ldt, double *__restrict__ 
         }
         for (int p = 0; p < CL; ++p) cl.map_shared_rank(&s, p)->xs[t][32 * q + lane] = x;
         __syncwarp();
-        if (lane < CL) {
+        if (lane < CL && !(withhold && t == 0)) {
             uint32_t remote;
             asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(&s.bar[t][q])), "r"(lane));
             asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
@@ -220,7 +233,7 @@ k_lu_rows_sub(int m, int len, const double *__restrict__ T, int ldt, const doubl
 // MODE 2: lower, 3: transposed lower (M = T^T)
 template <int MODE>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(kThreads, 1)
-k_tri_solve64(int n, const double *__restrict__ T, int ldt, double *__restrict__ X, int ldx) {
+k_tri_solve64(int n, const double *__restrict__ T, int ldt, double *__restrict__ X, int ldx, long long spin, int withhold) {
     constexpr bool FWD = MODE == 2, TRANS = MODE == 3;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem &s = *reinterpret_cast<Smem *>(smem_raw);
@@ -233,7 +246,10 @@ k_tri_solve64(int n, const double *__restrict__ T, int ldt, double *__restrict__
     auto row0 = [&](int t) { return (FWD ? t : nb - 1 - t) * NB; };   // first row of the t-th block solved
 
     if (tid < MAXB) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s.bar[tid])) : "memory");
-    if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (tid == 0) {
+        s.dead = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
     for (int t = rank, o = 0; t < nb; t += CL, ++o) {
         const int r0 = row0(t), nr = min(NB, n - r0);
         for (int e = tid; e < NB * NB; e += kThreads) {
@@ -383,7 +399,7 @@ k_tri_solve64(int n, const double *__restrict__ T, int ldt, double *__restrict__
             rs->xs[t][lane] = s.pub[lane];
             rs->xs[t][lane + 32] = s.pub[lane + 32];
             __syncwarp();
-            if (lane == 0) {
+            if (lane == 0 && !(withhold && t == 0)) {
                 uint32_t remote;
                 asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(&s.bar[t])), "r"(warp));
                 asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
@@ -403,7 +419,7 @@ k_tri_solve64(int n, const double *__restrict__ T, int ldt, double *__restrict__
         int j2 = j, t2 = t + CL;
         while (j2 < nb - 1 && t2 >= nb) { ++j2; t2 = first_own(j2); }
         if (j2 < nb - 1) load_tile(t2, j2, nxt);
-        wait_block(&s.bar[j]);
+        wait_block(&s.bar[j], &s.dead, spin);
         mac(t, j, cur);
         if (t == j + 1) solve_block(t);
 #pragma unroll
@@ -543,7 +559,8 @@ __global__ void k_gather_rows(int n, int nrhs, const int *perm, const double *In
 }
 
 template <int MODE>
-static int chol_mode(int n, int nrhs, const double *T, int ldt, double *X, int ldx, cudaStream_t st) {
+static int chol_mode(int n, int nrhs, const double *T, int ldt, double *X, int ldx, long long spin, int withhold,
+                     cudaStream_t st) {
     constexpr bool FWD = MODE == 2;
     const size_t ld = (size_t)ldt;
     CF_CUDA_TRY(cudaFuncSetAttribute(k_tri_solve64<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem)));
@@ -551,7 +568,7 @@ static int chol_mode(int n, int nrhs, const double *T, int ldt, double *X, int l
     for (int q = 0; q < ns; ++q) {
         const int k0 = (FWD ? q : ns - 1 - q) * kSuper;
         const int w = kSuper < n - k0 ? kSuper : n - k0;
-        k_tri_solve64<MODE><<<dim3(CL, nrhs), kThreads, sizeof(Smem), st>>>(w, T + k0 + k0 * ld, ldt, X + k0, ldx);
+        k_tri_solve64<MODE><<<dim3(CL, nrhs), kThreads, sizeof(Smem), st>>>(w, T + k0 + k0 * ld, ldt, X + k0, ldx, spin, withhold);
         CF_LAUNCH_CHECK();
         if (FWD) {
             const int r0 = k0 + w;
@@ -567,14 +584,15 @@ static int chol_mode(int n, int nrhs, const double *T, int ldt, double *X, int l
 }
 
 template <bool FWD>
-static int lu_mode(int n, int nrhs, const double *T, int ldt, double *X, int ldx, cudaStream_t st) {
+static int lu_mode(int n, int nrhs, const double *T, int ldt, double *X, int ldx, long long spin, int withhold,
+                   cudaStream_t st) {
     const size_t ld = (size_t)ldt;
     const int ns = ceil_div(n, kSuper);
     for (int q = 0; q < ns; ++q) {
         const int k0 = (FWD ? q : ns - 1 - q) * kSuper;
         const int w = kSuper < n - k0 ? kSuper : n - k0;
         const int r0 = FWD ? k0 + w : 0, m = FWD ? n - r0 : k0;      // the rows beyond
-        k_lu_solve64<FWD><<<dim3(CL, nrhs), kThreads, 0, st>>>(w, T + k0 + k0 * ld, ldt, X + k0, ldx);
+        k_lu_solve64<FWD><<<dim3(CL, nrhs), kThreads, 0, st>>>(w, T + k0 + k0 * ld, ldt, X + k0, ldx, spin, withhold);
         CF_LAUNCH_CHECK();
         if (m <= 0) continue;
         k_lu_rows_sub<<<dim3(ceil_div(m, 32), nrhs), 32, 0, st>>>(m, w, T + r0 + k0 * ld, ldt, X + k0, X + r0, ldx,
@@ -673,16 +691,21 @@ static int blocked_solve(int mode, int n, int nrhs, const double *T, int ldt, do
 // Right-hand sides up to which a cluster takes each (measured above).
 static int most_clusters(int mode, int n) { return mode < 2 ? (n > 256 ? 256 : 128) : (n > 256 ? 160 : 64); }
 
+static int cluster_solve(int mode, int n, int nrhs, const double *T, int ldt, double *X, int ldx, long long spin,
+                         int withhold, cudaStream_t st) {
+    switch (mode) {
+        case 0: return sv::lu_mode<true>(n, nrhs, T, ldt, X, ldx, spin, withhold, st);
+        case 1: return sv::lu_mode<false>(n, nrhs, T, ldt, X, ldx, spin, withhold, st);
+        case 2: return sv::chol_mode<2>(n, nrhs, T, ldt, X, ldx, spin, withhold, st);
+        default: return sv::chol_mode<3>(n, nrhs, T, ldt, X, ldx, spin, withhold, st);
+    }
+}
+
 int launch_tri_solve64(int mode, int n, int nrhs, const double *T, int ldt, double *X, int ldx, cudaStream_t st) {
     if (n <= 0 || nrhs <= 0) return CF_OK;
     if (mode < 0 || mode > 3) return CF_ERR_UNSUPPORTED;
     if (nrhs > most_clusters(mode, n)) return sv::blocked_solve(mode, n, nrhs, T, ldt, X, ldx, st);
-    switch (mode) {
-        case 0: return sv::lu_mode<true>(n, nrhs, T, ldt, X, ldx, st);
-        case 1: return sv::lu_mode<false>(n, nrhs, T, ldt, X, ldx, st);
-        case 2: return sv::chol_mode<2>(n, nrhs, T, ldt, X, ldx, st);
-        default: return sv::chol_mode<3>(n, nrhs, T, ldt, X, ldx, st);
-    }
+    return cluster_solve(mode, n, nrhs, T, ldt, X, ldx, sv::kSpin, 0, st);
 }
 
 int launch_permute_rhs(int n, int nrhs, const int *ipiv, int *perm, const double *B, int ldb, double *T, cudaStream_t st) {
@@ -717,3 +740,20 @@ int solve64_take_status(cudaStream_t st, int *status) {
 }
 
 }  // namespace cf
+
+// Failure-detection test of the bounded waits, not part of the API: one direction
+// of the cluster solves whose first block of every super-block is withheld from
+// the others, so that each wait for it gives up after spin_limit polls (0: the
+// usual number).
+extern "C" int cf_tri_solve64_withheld(int mode, int n, int nrhs, const double *T, int ldt, double *X, int ldx,
+                                       long long spin_limit, cudaStream_t stream) {
+    if (mode < 0 || mode > 3) return -1;
+    if (n < 1) return -2;
+    if (nrhs < 1 || nrhs > 64) return -3;
+    if (T == nullptr) return -4;
+    if (ldt < n) return -5;
+    if (X == nullptr) return -6;
+    if (ldx < n) return -7;
+    if (spin_limit < 0) return -8;
+    return cf::cluster_solve(mode, n, nrhs, T, ldt, X, ldx, spin_limit > 0 ? spin_limit : cf::sv::kSpin, 1, stream);
+}

@@ -46,3 +46,24 @@ def test_tournament_wait_runs_out(cf, m, w, leaf_h, arity, spin):
     assert win.min() >= 0 and win.max() < m and len(set(win.tolist())) == min(m, w)
     np.testing.assert_array_equal(cf.tourn_select(P, leaf_h, arity).cpu().numpy(), ref)
     assert cf.device_status() == cf.CF_OK
+
+
+@pytest.mark.parametrize("mode", [0, 1, 2, 3])
+@pytest.mark.parametrize("n,nrhs,spin", [(130, 1, 1 << 10), (300, 3, 1 << 10), (2048, 1, 1 << 10), (2048, 2, 0),
+                                         (2500, 1, 1 << 10)])
+def test_solve_wait_runs_out(cf, mode, n, nrhs, spin):
+    rng = np.random.default_rng(n)
+    T = rng.uniform(-1, 1, (n, n)) / n + 2 * np.eye(n)
+    X = _dev(rng.standard_normal((n, nrhs)))
+    _times_out_once(cf, lambda: cf.tri_solve64_withheld(_dev(T), X, mode, spin))
+    # the next solve is right
+    b = rng.standard_normal((n, nrhs))
+    if mode < 2:
+        ident = torch.arange(1, n + 1, dtype=torch.int32, device="cuda")
+        x = cf.getrs(_dev(T), ident, _dev(b)).cpu().numpy()
+        r = (np.tril(T, -1) + np.eye(n)) @ (np.triu(T) @ x) - b
+    else:
+        x = cf.potrs(_dev(T), _dev(b)).cpu().numpy()
+        r = np.tril(T) @ (np.tril(T).T @ x) - b
+    assert cf.device_status() == cf.CF_OK
+    assert np.abs(r).max() <= 6 * (n + 4) * 2.0 ** -53 * 16 * np.abs(b).max()
