@@ -10,10 +10,10 @@
 //   * warp 0 issues TMA loads (128-byte swizzle) into a 4-stage ring of
 //     shared-memory stages, warp 1 (one elected lane) issues tcgen05.mma
 //     (kind::f16, M=128, N=256, K=16) into one of two TMEM accumulators,
-//     warps 2-9 drain the other accumulator with tcgen05.ld and apply
+//     four or eight warps drain the other accumulator with tcgen05.ld and apply
 //     C -= acc with coalesced column accesses, so the epilogue of tile i
 //     overlaps the MMAs of tile i+1.  An update of small K is bound by C's
-//     traffic, so C's columns are loaded ahead: the first group before the
+//     traffic, so there C's columns are loaded ahead: the first group before the
 //     accumulator is ready, the next one before the current one is stored;
 //   * every mbarrier wait is bounded; on expiry the kernel records
 //     CF_ERR_TIMEOUT in a device status word, drains its own copies and
@@ -40,8 +40,10 @@ using namespace umma;
 
 constexpr int BM = 128, BN = 256, BK = 64, STAGES = 4;
 constexpr int UMMA_K = 16;
-constexpr int EPI = 8;                // epilogue warps: 4 lane quarters x 2 (32-column groups by turns)
-constexpr int kThreads = 64 + 32 * EPI;
+// Epilogue warps.  8: 4 lane quarters x 2 (32-column groups by turns), C loaded
+// ahead; 4: a quarter each, C loaded as it is needed.
+constexpr int kEpiMost = 8;
+constexpr int threads_of(int epi) { return 64 + 32 * epi; }
 constexpr uint32_t kStageA = BM * BK * 2;     // 16 KB
 constexpr uint32_t kStageB = BN * BK * 2;     // 32 KB
 constexpr uint32_t kStageBytes = kStageA + kStageB;
@@ -87,8 +89,8 @@ __device__ __forceinline__ bool tile_coords(const Problem &p, int t, int &m0, in
 // MMA and the epilogue cover only those); the wide form keeps compile-time
 // 256-column loops (measured 7-20% faster for wide outputs than the same
 // loops with run-time bounds).
-template <bool NARROW>
-__global__ void __launch_bounds__(kThreads, 1)
+template <bool NARROW, int EPI>
+__global__ void __launch_bounds__(threads_of(EPI), 1)
 k_schur_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, Problem p,
            uint32_t idesc) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -194,9 +196,11 @@ k_schur_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
             }
         }
     } else {
-        // ------------------------------------------------ epilogue (warps 2..9)
+        // ------------------------------------------------ epilogue (warps 2..)
         const int quarter = warp & 3;                 // TMEM lanes 32*quarter ..
-        const int half = (warp - 2) >> 2;             // column groups half, half + 2, ...
+        constexpr bool AHEAD = EPI == kEpiMost;
+        constexpr int STEP = 8 * EPI;                 // columns of one round
+        const int half = (warp - 2) >> 2;             // column groups half, half + STEP / 32, ...
         int tcount = 0;
         for (int u = blockIdx.x; u < p.nunits; u += gridDim.x) {
             int t, kb0, kb1, m0, n0;
@@ -220,7 +224,7 @@ k_schur_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
                 for (int j = 0; j < 32; ++j) v[j] = n0 + c0 + j < live ? crow[(size_t)(n0 + c0 + j) * p.ldc] : 0.f;
             };
             float cv[32];
-            if (p.P == nullptr && 32 * half < cend) load_c(cv, 32 * half);
+            if (AHEAD && p.P == nullptr && 32 * half < cend) load_c(cv, 32 * half);
             bool ok = true;
             if (lane == 0) ok = wait_bounded(&s.acc_full[b], aph, abort_flag, &g_tc_status);
             ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
@@ -230,7 +234,7 @@ k_schur_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
                 // split-K partial: the accumulator's live columns, column-major
                 float *dst = p.P + ((size_t)(u / p.ntiles) * p.ntiles + t) * (BM * BN) + quarter * 32 + lane;
 #pragma unroll 1
-                for (int c0 = 32 * half; c0 < cend; c0 += 64) {
+                for (int c0 = 32 * half; c0 < cend; c0 += STEP) {
                     uint32_t r[32];
                     const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * BN + c0);
                     TMEM_LD32(taddr, r);
@@ -245,13 +249,14 @@ k_schur_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
                 continue;
             }
 #pragma unroll 1
-            for (int c0 = 32 * half; c0 < cend; c0 += 64) {
+            for (int c0 = 32 * half; c0 < cend; c0 += STEP) {
+                if (!AHEAD) load_c(cv, c0);
                 uint32_t r[32];
                 const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * BN + c0);
                 TMEM_LD32(taddr, r);
                 float nx[32];
-                const bool more = c0 + 64 < cend;
-                if (more) load_c(nx, c0 + 64);
+                const bool more = AHEAD && c0 + STEP < cend;
+                if (more) load_c(nx, c0 + STEP);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
                 for (int j = 0; j < 32; ++j)
@@ -348,6 +353,22 @@ size_t schur_tc_splitk_bytes(int m, int n, int ksplit) {
     return sizeof(float) * (size_t)ksplit * ceil_div(m, tc::BM) * ceil_div(n, tc::BN) * tc::BM * tc::BN;
 }
 
+// K of a unit from which four epilogue warps serve a wide output better than
+// eight: a tile's MMAs then outlast its epilogue, and loads of C far ahead only
+// compete with the operands'.  24576 x 24576 in FP16, four / eight, ms: K = 64 1.36 /
+// 1.05, 1024 1.65 / 1.25, 1536 1.62 / 1.56, 1792 1.73 / 1.85, 2048 2.13 / 2.18;
+// 16384 x 16384: 2048 0.93 / 1.01, 4096 1.73 / 1.82.
+constexpr int kDeepK = 1664;
+
+template <bool NARROW, int EPI>
+static int start_schur_tc(int grid, size_t smem, const CUtensorMap &ta, const CUtensorMap &tb, const tc::Problem &p,
+                          uint32_t idesc, cudaStream_t st) {
+    CF_CUDA_TRY(cudaFuncSetAttribute(tc::k_schur_tc<NARROW, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    tc::k_schur_tc<NARROW, EPI><<<grid, tc::threads_of(EPI), smem, st>>>(ta, tb, p, idesc);
+    CF_LAUNCH_CHECK();
+    return CF_OK;
+}
+
 int launch_schur_tc(int m, int n, int k, const void *A, int lda_k, const void *B, int ldb_k, float *C, int ldc,
                     bool bf16, bool lower, cudaStream_t st, int max_ctas) {
     return launch_schur_tc_splitk(m, n, k, A, lda_k, B, ldb_k, C, ldc, bf16, lower, 1, nullptr, st, max_ctas);
@@ -384,14 +405,14 @@ int launch_schur_tc_splitk(int m, int n, int k, const void *A, int lda_k, const 
     int grid = num_sms();
     if (max_ctas > 0 && grid > max_ctas) grid = max_ctas;
     if (grid > p.nunits) grid = p.nunits;
-    if (nmma < tc::BN) {
-        CF_CUDA_TRY(cudaFuncSetAttribute(tc::k_schur_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        tc::k_schur_tc<true><<<grid, tc::kThreads, smem, st>>>(ta, tb, p, tc::make_idesc(bf16, tc::BM, nmma));
-    } else {
-        CF_CUDA_TRY(cudaFuncSetAttribute(tc::k_schur_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        tc::k_schur_tc<false><<<grid, tc::kThreads, smem, st>>>(ta, tb, p, tc::make_idesc(bf16, tc::BM, nmma));
-    }
-    CF_LAUNCH_CHECK();
+    const uint32_t idesc = tc::make_idesc(bf16, tc::BM, nmma);
+    if (nmma < tc::BN)
+        rc = start_schur_tc<true, 8>(grid, smem, ta, tb, p, idesc, st);
+    else if (p.kps * tc::BK < kDeepK)
+        rc = start_schur_tc<false, 8>(grid, smem, ta, tb, p, idesc, st);
+    else
+        rc = start_schur_tc<false, 4>(grid, smem, ta, tb, p, idesc, st);
+    if (rc) return rc;
     if (p.P != nullptr) {
         tc::k_splitk_reduce<<<dim3(8, p.ntiles), 256, 0, st>>>(p);
         CF_LAUNCH_CHECK();
