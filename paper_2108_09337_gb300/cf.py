@@ -92,6 +92,8 @@ _SIG = {
     "cf_device_status": (_I, [_P]),
     "cf_trsv_f32_workspace_size": (_S, [_I]),
     "cf_trsv_f32": (_I, [_I, _I, _I, _P, _I, _P, _I, _P, _S, _P]),
+    "cf_trsv_f32_f64x_workspace_size": (_S, [_I]),
+    "cf_trsv_f32_f64x": (_I, [_I, _I, _I, _P, _I, _P, _I, _I, _P, _S, _P]),
     "cf_tri_solve64_withheld": (_I, [_I, _I, _I, _P, _I, _P, _I, ctypes.c_longlong, _P]),
     "cf_trsv_f32_withheld": (_I, [_I, _I, _I, _P, _I, _P, _I, ctypes.c_longlong, _P, _S, _P]),
     "cf_factor_batched_workspace_size": (_S, [_I, _OPT]),
@@ -408,6 +410,18 @@ def trsv_f32(T: torch.Tensor, X: torch.Tensor, mode: int):
     ws = _workspace(_lib.cf_trsv_f32_workspace_size(n), T.device)
     _check("cf_trsv_f32", _lib.cf_trsv_f32(mode, n, nrhs, _ptr(T), _ld(T, "T"), _ptr(X), _ld(X, "X"), _ptr(ws),
                                            ws.numel(), _stream()))
+    return X
+
+
+def trsv_f32_f64x(T: torch.Tensor, X: torch.Tensor, mode: int, chains: int = 0):
+    """cf_trsv_f32_f64x: the refinement's solve with the FP32 factor T and FP64
+    right-hand sides and arithmetic, in place; chains 0: as the refinement
+    chooses, 1: one chain, 2: one per four right-hand sides."""
+    assert T.dtype == torch.float32 and X.dtype == torch.float64
+    n, nrhs = X.shape
+    ws = _workspace(_lib.cf_trsv_f32_f64x_workspace_size(n), T.device)
+    _check("cf_trsv_f32_f64x", _lib.cf_trsv_f32_f64x(mode, n, nrhs, _ptr(T), _ld(T, "T"), _ptr(X), _ld(X, "X"), chains,
+                                                     _ptr(ws), ws.numel(), _stream()))
     return X
 
 

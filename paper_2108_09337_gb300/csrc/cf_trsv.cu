@@ -607,11 +607,13 @@ static int launch_trsv_nr(int n, int nrhs, const float *T, int ldt, const VT *Di
     return CF_OK;
 }
 
+enum class Chains { kRule = 0, kOne = 1, kGroups = 2 };      // FP64 arithmetic: one chain, or one per four right-hand sides
+
 // withhold: the first ticket is taken before the launch (failure-detection
 // test: the first block is never solved and every wait for it runs out).
 template <int SB, int MODE, typename VT>
 static int launch_trsv_mode(int n, int nrhs, const float *T, int ldt, const VT *Dinv, const float *Gn, VT *X, int ldx,
-                            int *sync_ws, bool withhold, long long spin, cudaStream_t st) {
+                            int *sync_ws, bool withhold, long long spin, Chains chains, cudaStream_t st) {
     const int nb = (n + SB - 1) / SB;
     CF_CUDA_TRY(cudaMemsetAsync(sync_ws, 0, sizeof(int) * (size_t)(nb + 1), st));
     int *flags = sync_ws, *ticket = sync_ws + nb;
@@ -619,12 +621,15 @@ static int launch_trsv_mode(int n, int nrhs, const float *T, int ldt, const VT *
     // FP64 arithmetic: a block's products are bound by one SM's FP64 pipe (64 x 64 x
     // 16: 16 us each, 40 us per link of the chain), so each group of four
     // right-hand sides is a chain of its own, side by side with the others.
-    // Every group reads the factor and widens it to FP64 (on the FP64 pipe too):
-    // once all SMs are busy for most of the solve that costs more than the
-    // shorter links give.  Refinement of an unshifted split-BF16 LU with 16
-    // right-hand sides, in groups / in one chain: n = 16384 331 / 442 ms, n =
-    // 32768 1620 / 1545 ms; the line lies between the two.  FP32: one chain.
-    if (sizeof(VT) == 8 && n <= 24576)
+    // Every group reads the factor and widens it to FP64 again: with four groups
+    // on a large factor, when all SMs are busy for most of the solve, that costs
+    // what the shorter links give.  One direction (U), one chain / groups, ms:
+    //   5..8 right-hand sides    n = 4096 1.59 / 1.00, 16384 7.0 / 5.6, 24576 11.2 / 9.9, 32768 18.1 / 16.1
+    //   9..12                    n = 4096 2.73 / 1.11, 16384 10.6 / 6.6, 24576 16.9 / 12.9, 32768 25.4 / 21.5
+    //   13..16                   n = 4096 2.76 / 1.19, 16384 10.7 / 7.9, 24576 17.0 / 16.0, 28672 20.9 / 20.9,
+    //                            32768 25.5 / 26.7
+    // FP32: one chain.
+    if (sizeof(VT) == 8 && (chains == Chains::kGroups || (chains == Chains::kRule && (nrhs <= 12 || n <= 28672))))
         return launch_trsv_nr<SB, MODE, 4, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, flags, ticket, ceil_div(nrhs, 4), spin,
                                                st);
     if (nrhs <= 4)
@@ -637,14 +642,14 @@ static int launch_trsv_mode(int n, int nrhs, const float *T, int ldt, const VT *
 template <int SB, typename VT>
 static int launch_trsv_t(int mode, int n, int nrhs, const float *T, int ldt, const VT *Dinv, const float *Gn, VT *X,
                          int ldx, int *sync_ws, cudaStream_t st, bool withhold = false,
-                         long long spin = kFlagSpin) {
+                         long long spin = kFlagSpin, Chains chains = Chains::kRule) {
     if (n <= 0 || nrhs <= 0) return CF_OK;
     if (nrhs > 16) return CF_ERR_UNSUPPORTED;
     switch (mode) {
-        case 0: return launch_trsv_mode<SB, 0, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, sync_ws, withhold, spin, st);
-        case 1: return launch_trsv_mode<SB, 1, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, sync_ws, withhold, spin, st);
-        case 2: return launch_trsv_mode<SB, 2, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, sync_ws, withhold, spin, st);
-        case 3: return launch_trsv_mode<SB, 3, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, sync_ws, withhold, spin, st);
+        case 0: return launch_trsv_mode<SB, 0, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, sync_ws, withhold, spin, chains, st);
+        case 1: return launch_trsv_mode<SB, 1, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, sync_ws, withhold, spin, chains, st);
+        case 2: return launch_trsv_mode<SB, 2, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, sync_ws, withhold, spin, chains, st);
+        case 3: return launch_trsv_mode<SB, 3, VT>(n, nrhs, T, ldt, Dinv, Gn, X, ldx, sync_ws, withhold, spin, chains, st);
         default: return CF_ERR_UNSUPPORTED;
     }
 }
@@ -746,3 +751,35 @@ extern "C" int cf_trsv_f32_withheld(int mode, int n, int nrhs, const float *T, i
                         lwork, stream);
 }
 
+
+// The refinement's solve with FP64 arithmetic and the FP32 factor on its own, with
+// the form of its chains given (0: as the refinement chooses, 1: one, 2: one per
+// four right-hand sides): for tests and measurements, not part of the API.
+extern "C" size_t cf_trsv_f32_f64x_workspace_size(int n) {
+    cf::Carver cv(nullptr);
+    cv.take<double>(cf::diag_inverse64_elems(n > 0 ? n : 1));
+    cv.take<int>(cf::trsv_ws_bytes(n > 0 ? n : 1) / sizeof(int) + 1);
+    return cv.size();
+}
+
+extern "C" int cf_trsv_f32_f64x(int mode, int n, int nrhs, const float *T, int ldt, double *X, int ldx, int chains,
+                                void *work, size_t lwork, cudaStream_t stream) {
+    using namespace cf;
+    if (mode < 0 || mode > 3) return -1;
+    if (n < 0) return -2;
+    if (nrhs < 0 || nrhs > 16) return -3;
+    if (n > 0 && T == nullptr) return -4;
+    if (ldt < (n > 1 ? n : 1)) return -5;
+    if (n > 0 && nrhs > 0 && X == nullptr) return -6;
+    if (ldx < (n > 1 ? n : 1)) return -7;
+    if (chains < 0 || chains > 2) return -8;
+    if (n == 0 || nrhs == 0) return CF_OK;
+    if (work == nullptr || lwork < cf_trsv_f32_f64x_workspace_size(n)) return CF_ERR_WORKSPACE;
+    Carver cv(work);
+    double *Dinv = cv.take<double>(diag_inverse64_elems(n));
+    int *sync = cv.take<int>(trsv_ws_bytes(n) / sizeof(int) + 1);
+    const int rc = launch_diag_inverse64(mode == 3 ? 2 : mode, n, T, ldt, Dinv, stream);
+    if (rc != CF_OK) return rc;
+    return launch_trsv_t<kSB64, double>(mode, n, nrhs, T, ldt, Dinv, nullptr, X, ldx, sync, stream, false, kFlagSpin,
+                                        (Chains)chains);
+}
