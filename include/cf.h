@@ -232,8 +232,7 @@ int cf_getrf(int n, double *A, int lda, int *ipiv, int *info, void *work,
  *     with that device current); make that first call before any stream
  *     capture on that device.
  *   - All calls share the one array: calls whose work overlaps on the GPU
- *     (other streams, other host threads) race and corrupt each other.  The
- *     arrival counters are cleared at the start of every call.
+ *     (other streams, other host threads) race and corrupt each other.
  *   - It always runs the one-stream schedule on `stream` (opt->lookahead is
  *     ignored): the results equal cf_getrf's, the speed is that of cf_getrf
  *     with lookahead = 0.

@@ -291,7 +291,6 @@ extern "C" int cf_getrf(int n, double *A, int lda, int *ipiv, int *info, void *w
     TournEpilogue ep{};
     rc = tourn_ws_carve(work, n, o.leaf_h, o.arity, &ws, &ep);
     if (rc != CF_OK) return rc;
-    CF_CUDA_TRY(cudaMemsetAsync(ws.counter, 0, ws.counter_bytes, st));
     const size_t base = align_up(cf_getrf_workspace_size(n, opt), 1024);
     if (lwork >= cf_getrf_optimal_workspace_size(n, opt)) {
         ep.lu_ok = (int *)((char *)work + base);

@@ -1,8 +1,8 @@
 // cf_noalloc.cu -- cf_getrf_noalloc: the FP64 LU of cf_getrf for callers that
 // cannot allocate device memory.
 //
-// cf_getrf needs a small scratch area (the tournament's candidate lists, its
-// arrival counters and the list of moved rows) and takes it from the caller
+// cf_getrf needs a small scratch area (the tournament's candidate lists and the
+// list of moved rows) and takes it from the caller
 // as `work`.  Some callers have no way to provide it: code that runs while a
 // stream is being captured into a CUDA graph (where cudaMalloc is not
 // allowed), plugins that live inside a host framework whose allocator owns
@@ -65,9 +65,6 @@ extern "C" int cf_getrf_noalloc(int n, double *A, int lda, int *ipiv, int *info,
     TournWS ws{};
     TournEpilogue ep{};
     if ((rc = tourn_ws_carve(scratch, n, o.leaf_h, o.arity, &ws, &ep))) return rc;
-    // The array keeps whatever the previous call left: the arrival counters
-    // must start at zero.
-    CF_CUDA_TRY(cudaMemsetAsync(ws.counter, 0, ws.counter_bytes, st));
     // A00's LU beside the tournament's part, where the array has room for it
     const size_t used = align_up(tourn_ws_bytes(n, o.leaf_h, o.arity), 256);
     if (used + 256 + sizeof(double) * kMaxV * kMaxV <= kNoAllocScratchBytes) {

@@ -52,7 +52,7 @@ constexpr int kTB = 4;                           // columns of a block
 struct TournSmem {
     // candidates of every CTA's warps, by column parity: the row's block entries,
     // then its stacked position (-1: none) as a double's bits
-    alignas(16) double slot[2][4 * kTournMaxCluster][kTB + 2];
+    alignas(16) double slot[2][32][kTB + 2];
     alignas(16) double stage[4][kTB + 2];        // a warp's candidate on its way out
     double pin[kTB][kTB];                        // the block's pivots: pin[u][t] = entry t of pivot u
     double U[kTB][kMaxV];                        // their other columns
@@ -309,18 +309,13 @@ k_tourn_level(TournLevel lv, TournWS ws, TournEpilogue ep) {
                     // (armed again before this warp's next candidate goes out, which
                     // every sender of the next but one waits for)
                     if (tid == 0 && ok && !*(volatile int *)&s.abort_flag) tourn_arm(&s.bar[par], nslots * kSlotBytes);
-                    int at = lane, best = lane < nslots ? (int)__double_as_longlong(s.slot[par][lane][kTB]) : -1;
-                    unsigned long long key = best >= 0 ? piv_key(s.slot[par][lane][u - 1]) : 0ull;
-                    if (nslots > 32) {
-                        const int i1 = lane + 32 < nslots ? (int)__double_as_longlong(s.slot[par][lane + 32][kTB]) : -1;
-                        const unsigned long long k1 = i1 >= 0 ? piv_key(s.slot[par][lane + 32][u - 1]) : 0ull;
-                        if (k1 > key || (k1 == key && k1 != 0 && i1 < best)) { key = k1; best = i1; at = lane + 32; }
-                    }
+                    const int best = lane < nslots ? (int)__double_as_longlong(s.slot[par][lane][kTB]) : -1;
+                    const unsigned long long key = best >= 0 ? piv_key(s.slot[par][lane][u - 1]) : 0ull;
                     // (after a wait that ran out the slots hold anything: any row in range will do, the
                     // order is replaced at the end)
                     int gi = warp_best(key, best);
                     if (!ok || (unsigned)gi >= (unsigned)total) gi = j0 + u - 1;
-                    at = __shfl_sync(0xffffffffu, at, max(__ffs(__ballot_sync(0xffffffffu, best == gi)) - 1, 0));
+                    const int at = max(__ffs(__ballot_sync(0xffffffffu, best == gi)) - 1, 0);
                     const double *pv = s.slot[par][at];
                     const double piv = pv[u - 1];
                     const bool go = !is_zero(piv);           // a zero pivot eliminates nothing
@@ -560,8 +555,9 @@ size_t tourn_ws_bytes(int m, int h, int arity) {
     return cv.size();
 }
 
-// Counters must be zero before the first tournament; the tournament leaves
-// them zero.
+// The counters are the FP32 tournaments', whose nodes climb the tree in one
+// launch: zero before the first, left zero.  The FP64 one (a launch per level)
+// has none.
 int tourn_ws_carve(void *work, int m, int h, int arity, TournWS *ws, TournEpilogue *ep) {
     TournPlan p{};
     int st = make_tourn_plan(m, 1, h, arity, &p);
@@ -645,6 +641,7 @@ static int run_tourn(const double *P, int ldp, int m, int w, int h, int arity, c
         lv.off = plan.off[l];
         lv.per = ceil_div(rows, cta);
         lv.ld = lv.per | 1;
+        if (ceil_div(lv.per, 32) * cta > 32) return CF_ERR_UNSUPPORTED;      // a slot per lane (1024 rows: 4 x 8, 2 x 16)
         lv.spin = spin;
         lv.withhold = withhold && l == 0;
         const size_t smem = align_up(sizeof(TournSmem), 16) + sizeof(double) * (size_t)lv.ld * w;
@@ -729,7 +726,6 @@ static int tourn_select_api(int m, int w, const double *panel, int ldp, int leaf
     int rc = tourn_ws_carve(work, m, 1, arity, &ws, &ep);
     if (rc != CF_OK) return rc;
     ep.ipiv = nullptr;
-    CF_CUDA_TRY(cudaMemsetAsync(ws.counter, 0, ws.counter_bytes, stream));
     ws.root_win = winners;
     return run_tourn(panel, ldp, m, w, leaf_h, arity, ws, ep, spin, withhold, stream);
 }
