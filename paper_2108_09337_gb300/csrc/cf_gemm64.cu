@@ -1,9 +1,10 @@
-// cf_gemm64.cu -- SIMT Schur-complement update (FP64; where cf_slice64.cu has no
-// scratch or the step is narrow) and the FP64 residual.
+// cf_gemm64.cu -- SIMT Schur-complement update (FP64: LU; Cholesky where
+// cf_slice64.cu has no scratch or the step is narrow) and the FP64 residual.
 //
 //   LU-5 (FP64 path)  A11 <- A11 - A10 A01      (Alg. 1; Table 2 gemm)
 //   CH-3 (FP64 path)  A11 <- A11 - L10 L10^T    (Table 2 gemmt, lower only)
-//   S-1               products between super-blocks of the triangular solves
+//   S-1               products of the triangular solves: between blocks of many
+//                     right-hand sides, between Cholesky's super-blocks
 //   R-1               R = B - A X
 //
 // GB300 executes FP64 at about 1.2 TFLOP/s (measured: ~1.9 DFMA per clock per
